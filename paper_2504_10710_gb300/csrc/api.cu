@@ -275,21 +275,9 @@ glls_status upload_levels(glls_problem* P, const std::vector<LevelHost>& H, std:
             d.band[a] = dptr;
         }
         if (h.lblock) {
-            using V2 = typename Vec2Of<T>::type;
             for (int a = 0; a < h.dim; ++a) {
                 CK(P->upload(&d.blk[a], h.blk[a]));
-                const size_t nv = h.vband[a].size() / 2;
-                std::vector<V2> packed(nv ? nv : 1);
-                for (size_t i = 0; i < nv; ++i) {
-                    packed[i].x = (T)h.vband[a][2 * i];
-                    packed[i].y = (T)h.vband[a][2 * i + 1];
-                }
-                void* p_ = nullptr;
-                CK(dev_malloc(&p_, sizeof(V2) * packed.size()));
-                P->shared->allocs.push_back(p_);
-                P->shared->bytes += sizeof(V2) * packed.size();
-                CK(cudaMemcpy(p_, packed.data(), sizeof(V2) * packed.size(), cudaMemcpyHostToDevice));
-                d.vband[a] = static_cast<const V2*>(p_);
+                CK(P->upload(&d.vcr[a], h.vcr[a]));
             }
         }
         if (l > 0) {
@@ -877,7 +865,7 @@ enum WlKind { WL_APPLY = 0, WL_LINE, WL_T2, WL_BCR_F, WL_COARSE, WL_BCR_B, WL_FC
 struct WlRecord {
     int kind = 0;
     bool dbl = false;                  // FP64 items
-    int p = 0, cv = 1, wb = 0, ty = 0, l = 0, step = 0;
+    int p = 0, s = 0, cv = 1, wb = 0, ty = 0, l = 0, step = 0;
     bool mask = false, dot = false, add = false;
     bool ff = false;                   // the float-float form of the FP64 outer apply
     int blocks = 0, threads = 256, nitems = 0;
@@ -979,6 +967,7 @@ struct WlBuilder {
         WlRecord r;
         r.kind = WL_LINE;
         r.dbl = sizeof(T) == 8;
+        r.s = s;
         r.threads = 32;
         std::vector<size_t> sm0, sm1;
         std::vector<unsigned char> buf(line_block_item_bytes<T>());
@@ -1248,9 +1237,9 @@ cudaError_t replay(const WlRecord& r, const unsigned char* base, int flexible, c
                                                   r.mask, r.dot, st);
             break;
         case WL_LINE:
-            ok = r.dbl ? launch_line_block_list<double>(r.p, r.cv, items, start, r.nitems, r.blocks, r.threads, r.smem,
+            ok = r.dbl ? launch_line_block_list<double>(r.p, r.s, r.cv, items, start, r.nitems, r.blocks, r.threads, r.smem,
                                                         st)
-                       : launch_line_block_list<float>(r.p, r.cv, items, start, r.nitems, r.blocks, r.threads, r.smem,
+                       : launch_line_block_list<float>(r.p, r.s, r.cv, items, start, r.nitems, r.blocks, r.threads, r.smem,
                                                        st);
             break;
         case WL_T2:
@@ -1895,12 +1884,12 @@ glls_status glls_estimate_bytes(const glls_mesh_desc* desc, size_t* bytes) {
         if (c == 0 && p >= 2 && p <= (d == 2 ? 16 : 8)) total += 4.0 * ncomp * E * nloc;   // float-float G remainders
         total += 2.0 * d * (12.0 * (2 * p + 2) * (double)(ne[0] * p + 1) + 4.0 * (ne[0] * p + 1));
         if (desc->smoother == GLLS_SMOOTHER_GLL && p >= 2) {
-            // condensed line blocks: per segment (p-1)p/2 + 2(p-1) values, per vertex 2 (FP64 + FP32)
+            // condensed line blocks: per segment (p-1)p/2 + 2(p-1) values, per vertex 3 (FP64 + FP32)
             for (int s = 0; s < d; ++s) {
                 double lines = 1.0;
                 for (int a = 0; a < d; ++a)
                     if (a != s) lines *= (double)(ne[a] * p - 1);
-                total += 12.0 * lines * ne[s] * ((p - 1) * p / 2.0 + 2.0 * (p - 1)) + 24.0 * lines * ne[s];
+                total += 12.0 * lines * ne[s] * ((p - 1) * p / 2.0 + 2.0 * (p - 1)) + 36.0 * lines * ne[s];
             }
         }
     }

@@ -7,7 +7,7 @@
 //                     node index q = (k*(p+1) + j)*(p+1) + i
 //   diag, off[s]    : band-1 line-system coefficients on the global grid;
 //                     off[s][node] couples node and node + e_s
-//   blk[s], vband[s]: Def. 3.2 line blocks condensed per element segment
+//   blk[s], vcr[s]  : Def. 3.2 line blocks condensed per element segment
 //                     (GLL smoother, p >= 2), see DevLevel
 //   D               : (p+1)^2 derivative matrix, D[i*(p+1)+j] = pi_j'(xi_i)
 //   P[a], R[a]      : fixed-width row bands of the 1-D transfer matrices
@@ -97,10 +97,11 @@ struct DevLevel {
     const float* Glo = nullptr;
     // Def. 3.2 line blocks condensed per element segment (GLL smoother, p >= 2;
     // null otherwise): blk[s] [ncoef][nlines * ne[s]] = packed K_I^-1, w_L,
-    // w_R per segment; vband[s] [nlines][ne[s] - 1] = vertex Schur complement
-    // (diagonal, coupling to the next vertex).  See lines_block.cu.
+    // w_R per segment (x-lines: segment fastest; other directions: line
+    // fastest); vcr[s] [3][nlines * (ne[s] - 1)] = multipliers l/a, u/a, 1/a
+    // of the vertex cyclic reduction.  See lines_block.cu.
     const T* blk[3] = {nullptr, nullptr, nullptr};
-    const typename Vec2Of<T>::type* vband[3] = {nullptr, nullptr, nullptr};
+    const T* vcr[3] = {nullptr, nullptr, nullptr};
 };
 
 // Exact coarsest solve: cr_levels levels of block cyclic reduction over the
@@ -234,7 +235,7 @@ int line_block_list_item(const DevLevel<T>& L, int s, int mode, const T* g, cons
                          void* item, int* blocks, int* threads, size_t smem[2], int* cv);
 bool line_block_list_specialised(int p, int cv);
 template <typename T>
-bool launch_line_block_list(int p, int cv, const void* items, const int* start, int nitems, int blocks, int threads,
+bool launch_line_block_list(int p, int s, int cv, const void* items, const int* start, int nitems, int blocks, int threads,
                             size_t smem, cudaStream_t st);
 
 // Opt every kernel into up to 200 KB of dynamic shared memory (call once per
@@ -265,7 +266,12 @@ bool line_block_supported(int n, int E);
 template <typename T>
 bool launch_line_block(const DevLevel<T>& L, int s, int mode, const T* g, const T* r, T* y, T* x, T alpha,
                        cudaStream_t st, int nrhs = 1);
+template <typename T>
 bool init_line_block_attributes();
+template <>
+bool init_line_block_attributes<float>();
+template <>
+bool init_line_block_attributes<double>();
 // 3-D FP32 apply with one thread per element column (apply_col.cu), p <= 3
 // (the orders the even-odd kernel does not take); no x.(A x) product.
 // Returns false outside that range.

@@ -1440,7 +1440,8 @@ bool init_kernel_attributes() {
     for (const void* f : fns)
         if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem) != cudaSuccess)
             return false;
-    return init_line_warp_attributes() && init_line_block_attributes() && init_apply_col_attributes() &&
+    return init_line_warp_attributes() && init_line_block_attributes<float>() &&
+           init_line_block_attributes<double>() && init_apply_col_attributes() &&
            init_apply_eo_attributes();
 }
 

@@ -9,24 +9,29 @@
 // the Schur complement on the vertices (Prop. 3.7), which is tridiagonal and
 // is solved by cyclic reduction (Cor. 3.9).  Per segment the set-up stores
 // K_I^-1 (upper triangle) and w_L, w_R = K_I^-1 K_{I,v} for its two vertices;
-// per line the vertex system.  One application of the block inverse to g:
+// per vertex the multipliers of its elimination (Prop. 3.10, first variant).
+// One application of the block inverse to g:
 //   z   = K_I^-1 g_I                          every segment
 //   c_v = g_v - w_R(v-1) . g_I(v-1) - w_L(v) . g_I(v)     (c = R (g - K x))
-//   S nu = c                                  vertex CR, one warp per line
+//   S nu = c                                  vertex CR, one lane group per line
 //   x_I = z - w_L nu_left - w_R nu_right,  x_v = nu_v       (y = x + P e)
 //
-// A CTA owns LPC <= min(16, 256 / E) lines of one direction (E segments
-// each) with LPC E threads (rounded up to a warp), one segment task per
-// thread; small levels take fewer lines per CTA so that every SM gets work.  All
-// global loads are issued at entry: the line values (coalesced: along the
-// line for x-lines, across adjacent lines for strided directions), the
-// vertex systems, and each thread's segment operator into registers; after
-// one barrier the segment work, the vertex CR (one warp per line, warps
-// taking a second line when LPC > 8) and the back substitution run in
-// registers and shared memory, and the results are stored.  P is the
-// compile-time order (2..8); P = 0 takes the order at run time, reads its
-// operator from global memory inside the loops and accumulates K_I^-1 g_I in
-// shared memory.
+// A CTA owns LPC lines of one direction (a power of two, at most 16 lines and
+// 256 segments), one segment task per thread (line_seg_body).  What bounds
+// it: on levels far above L2 the bytes of the segment operators and the
+// vectors, elsewhere the chain of dependent phases.  A thread reads its own
+// nodes of r, y and x straight into registers, all loads back to back, and
+// shared memory only carries the two dots and the vertex value of each
+// segment.  In strided directions adjacent threads hold adjacent lines
+// (coalesced across the lines; the operators are stored line fastest).  On
+// x-lines adjacent threads hold adjacent segments (operators stored segment
+// fastest): their loads share cache lines, which L1 serves, and the results
+// go out through shared memory, coalesced along the line.
+// The segment operators and the vertex multipliers are mesh data that no
+// kernel writes, so they are loaded before the wait on the preceding kernel
+// and overlap its end.
+// P is the compile-time order (2..12); line_any_body takes the order at run
+// time with the operators in shared memory.
 #include "async_copy.cuh"
 #include "cr_warp.cuh"
 #include "device.cuh"
@@ -36,18 +41,27 @@
 #include <cstring>
 
 namespace glls {
+
+// The precision of this translation unit: FP32 here, FP64 in
+// lines_block_f64.cu, which includes this file.
+#ifdef GLLS_LINES_F64
+using LineT = double;
+#else
+using LineT = float;
+#endif
+
 namespace {
 
 template <typename T>
 struct BlockLineArgs {
     int n, nlines, stride, m1, st1, st2, contiguous, mode;
-    int p, E, span, cv, lpc;
+    int p, E, span, cv, lpc, sub;   // sub: lanes per line of the vertex CR (a power of two, sub cv >= E - 1)
     int nrhs;           // right-hand sides (vectors of N values each)
     long long N;
     long long ntask;
     T alpha;
     const T* blk;                              // [ncoef][ntask]
-    const typename Vec2Of<T>::type* vband;     // [nlines][E - 1]
+    const T* vcr;                              // [3][nlines (E - 1)]
     const T* g;
     const T* r;
     T* y;
@@ -71,140 +85,376 @@ int sm_count() {
 // shared-memory index with one pad word per 32
 __device__ __forceinline__ int padk(int k) { return k + (k >> 5); }
 
+// Threads of a CTA of lpc lines of E segments.
+__host__ __device__ __forceinline__ int block_threads(int lpc, int E) {
+    const int t = (lpc * E + 31) / 32 * 32;
+    return t > kBlockThreads ? kBlockThreads : t;
+}
 
-
-// Vertex system of one line (E - 1 unknowns; vertex k is line unknown
-// (k + 1) p - 1), right-hand side c_k = g_v - dr[k] - dl[k + 1], operator
-// from shared memory (vb: diagonal and coupling to the next vertex per
-// vertex); the solution overwrites the vertex entries of `line`.
+// ---- vertex systems -------------------------------------------------------
+// Multipliers of a lane's C vertices (vertex k = C lane + j of the line):
+// l/a, u/a and 1/a at the level that eliminates the vertex; zero past the end.
 template <typename T, int C>
-__device__ __forceinline__ void vertex_solve(T* line, const T* dl, const T* dr, const T* vb, int E, int p,
-                                             int lane) {
-    const int nv = E - 1;
-    T a[C], l[C], u[C], g[C];
+struct VertexCr {
+    T la[C], ua[C], ia[C];
+    __device__ __forceinline__ void load(const BlockLineArgs<T>& A, int line, bool valid, int slane) {
+        const int nv = A.E - 1;
+        const long long tot = (long long)A.nlines * nv;
+        const T* v = A.vcr + (long long)line * nv;
 #pragma unroll
-    for (int j = 0; j < C; ++j) {
-        const int k = C * lane + j;
-        if (k < nv) {
-            a[j] = vb[2 * k];
-            u[j] = k < nv - 1 ? vb[2 * k + 1] : T(0);
-            l[j] = k > 0 ? vb[2 * k - 1] : T(0);
-            g[j] = line[padk((k + 1) * p - 1)] - dr[k] - dl[k + 1];
-        } else {
-            a[j] = T(1); l[j] = T(0); u[j] = T(0); g[j] = T(0);
+        for (int j = 0; j < C; ++j) {
+            const int k = C * slane + j;
+            const bool ok = valid && k < nv;
+            la[j] = ok ? __ldg(v + k) : T(0);
+            ua[j] = ok ? __ldg(v + tot + k) : T(0);
+            ia[j] = ok ? __ldg(v + 2 * tot + k) : T(0);
         }
     }
-    warp_cr_solve<T, C>(a, l, u, g, lane);
+};
+
+// Cyclic reduction with stored multipliers, W lanes per system (W a power of
+// two, several systems per warp): at level h the odd multiples of h are
+// eliminated into the even ones (g_i -= (u/a)_{i-h} g_{i-h} + (l/a)_{i+h}
+// g_{i+h}; the system is symmetric, so l_i = u_{i-h}), then restored
+// (x_i = g_i/a_i - (l/a)_i x_{i-h} - (u/a)_i x_{i+h}).  A level costs two
+// shuffles each way and no reciprocal; the coefficients' own recursion, which
+// took six shuffles and a reciprocal a level, ran once at set-up.  All 32
+// lanes of the warp take part.
+template <typename T, int C>
+__device__ __forceinline__ void vertex_cr(const VertexCr<T, C>& m, T (&g)[C], int slane, int W) {
 #pragma unroll
-    for (int j = 0; j < C; ++j) {
-        const int k = C * lane + j;
-        if (k < nv) line[padk((k + 1) * p - 1)] = g[j];
+    for (int h = 1; h < C; h *= 2) {
+        T gr = __shfl_down_sync(kFullMask, m.la[h - 1] * g[h - 1], 1, W);
+        if (slane == W - 1) gr = T(0);
+#pragma unroll
+        for (int j = 2 * h - 1; j < C; j += 2 * h) {
+            const int jr = j + h < C ? j + h : 0;
+            g[j] = g[j] - m.ua[j - h] * g[j - h] - (j + h < C ? m.la[jr] * g[jr] : gr);
+        }
+    }
+    T G = g[C - 1];
+    for (int d = 1; d < W; d *= 2) {
+        const T fl = __shfl_up_sync(kFullMask, m.ua[C - 1] * G, d, W);
+        const T fr = __shfl_down_sync(kFullMask, m.la[C - 1] * G, d, W);
+        if (((slane + 1) & (2 * d - 1)) == 0) G -= fl + (slane + d < W ? fr : T(0));
+    }
+    const T Gi = G * m.ia[C - 1];
+    T X = slane == W - 1 ? Gi : T(0);
+    for (int d = W / 2; d >= 1; d /= 2) {
+        T xl = __shfl_up_sync(kFullMask, X, d, W);
+        const T xr = __shfl_down_sync(kFullMask, X, d, W);
+        if (slane < d) xl = T(0);
+        if (((slane + 1) & (2 * d - 1)) == d) X = Gi - m.la[C - 1] * xl - m.ua[C - 1] * xr;
+    }
+    g[C - 1] = X;
+    if constexpr (C > 1) {
+        T xprev = __shfl_up_sync(kFullMask, X, 1, W);
+        if (slane == 0) xprev = T(0);
+#pragma unroll
+        for (int h = C / 2; h >= 1; h /= 2) {
+#pragma unroll
+            for (int j = h - 1; j < C; j += 2 * h) {
+                const T xl = j - h >= 0 ? g[j - h >= 0 ? j - h : 0] : xprev;
+                const T xr = g[j + h < C ? j + h : C - 1];
+                g[j] = g[j] * m.ia[j] - m.la[j] * xl - m.ua[j] * xr;
+            }
+        }
     }
 }
 
-// Segment operator of one task in registers (compile-time order).
+// The vertex phase of a CTA: sh[w SE + v] holds g_v - w_L . g_I of segment v
+// (v >= 1) and sdr[w SE + v] w_R . g_I of segment v; the solution of vertex v
+// replaces sh[w SE + v].  `first`: the multipliers of the lane group's first
+// line, loaded at entry.
+template <typename T, int C>
+__device__ __forceinline__ void vertex_phase(const BlockLineArgs<T>& A, VertexCr<T, C>& first, T* sh, const T* sdr,
+                                             int SE, int l0, int Wc) {
+    const int W = A.sub, nv = A.E - 1;
+    const int groups = (int)blockDim.x / W, slane = threadIdx.x & (W - 1);
+    for (int w0 = 0; w0 < Wc; w0 += groups) {
+        const int w = w0 + (int)threadIdx.x / W;
+        if (w0 > 0) first.load(A, l0 + w, w < Wc, slane);
+        T g[C];
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+            const int k = C * slane + j;
+            g[j] = w < Wc && k < nv ? sh[w * SE + k + 1] - sdr[w * SE + k] : T(0);
+        }
+        vertex_cr<T, C>(first, g, slane, W);
+#pragma unroll
+        for (int j = 0; j < C; ++j) {
+            const int k = C * slane + j;
+            if (w < Wc && k < nv) sh[w * SE + k + 1] = g[j];
+        }
+    }
+}
+
+// ---- segments ----------------------------------------------------------------
+// Segment operator of one task, in registers from the kernel's entry (FP64 up
+// to order 8; above, the values are read where they are used, K_I^-1 once and
+// w_L, w_R twice).
 template <typename T, int P>
 struct SegOp {
     static constexpr int MI = P > 1 ? P - 1 : 1;
     static constexpr int NPK = MI * (MI + 1) / 2;
-    T t[NPK], wl[MI], wr[MI];
+    static constexpr bool HELD = P <= (sizeof(T) == 8 ? 8 : 12);
+    T t[HELD ? NPK : 1], wl[HELD ? MI : 1], wr[HELD ? MI : 1];
+    const T* bp;
+    long long nt;
+    __device__ __forceinline__ void load(const T* p, long long ntask, bool valid) {
+        bp = p;
+        nt = ntask;
+        if constexpr (HELD) {
+            if (valid) {
+#pragma unroll
+                for (int c = 0; c < NPK; ++c) t[c] = __ldg(p + (long long)c * ntask);
+#pragma unroll
+                for (int i = 0; i < MI; ++i) {
+                    wl[i] = __ldg(p + (long long)(NPK + i) * ntask);
+                    wr[i] = __ldg(p + (long long)(NPK + MI + i) * ntask);
+                }
+            }
+        }
+    }
+    __device__ __forceinline__ T tri(int c) const {
+        if constexpr (HELD) return t[c];
+        else return __ldg(bp + (long long)c * nt);
+    }
+    __device__ __forceinline__ T left(int i) const {
+        if constexpr (HELD) return wl[i];
+        else return __ldg(bp + (long long)(NPK + i) * nt);
+    }
+    __device__ __forceinline__ T right(int i) const {
+        if constexpr (HELD) return wr[i];
+        else return __ldg(bp + (long long)(NPK + MI + i) * nt);
+    }
+    // z = K_I^-1 g, dl = w_L . g, dr = w_R . g
+    __device__ __forceinline__ void solve(const T (&g)[MI], T (&z)[MI], T& dl, T& dr) const {
+#pragma unroll
+        for (int i = 0; i < MI; ++i) z[i] = T(0);
+        int c = 0;
+#pragma unroll
+        for (int i = 0; i < MI; ++i)
+#pragma unroll
+            for (int j = i; j < MI; ++j) {
+                const T v = tri(c++);
+                z[i] += v * g[j];
+                if (j != i) z[j] += v * g[i];
+            }
+        dl = dr = T(0);
+#pragma unroll
+        for (int i = 0; i < MI; ++i) {
+            dl += left(i) * g[i];
+            dr += right(i) * g[i];
+        }
+    }
 };
+
+// The right-hand side of a CTA (fastest in the CTA order, see device.cuh: the
+// nrhs CTAs of one line group read the same segment operators) and its lines.
+template <typename T>
+__device__ __forceinline__ int enter(BlockLineArgs<T>& A, int blk) {
+    const int rhs = A.nrhs == 1 ? 0 : blk % A.nrhs, bx = A.nrhs == 1 ? blk : blk / A.nrhs;
+    const long long vo = (long long)rhs * A.N;
+    if (A.g) A.g += vo;
+    if (A.r) A.r += vo;
+    if (A.y) A.y += vo;
+    A.x += vo;
+    return bx * A.lpc;
+}
+
+// Waits for the preceding kernel; false when the item's problem has stopped.
+template <typename T>
+__device__ __forceinline__ bool ready(const BlockLineArgs<T>& A) {
+    grid_dep_sync();
+    return !(A.done && *A.done != 0.0);
+}
 
 // MODE 0: x = B^-1 g.  MODE 1: x += alpha B^-1 (r - y), and y is reset to 0
 // on element-boundary nodes (the apply that produced y plain-stores element-
 // interior nodes and adds into element-boundary ones).  MODE 2: x += alpha
 // B^-1 r.  MODE 3: x = alpha B^-1 r.
-// Register budget: FP32 four CTAs per SM (<= 64 registers), three for order 8
-// and the run-time order (<= 85: the 42 operator values of a segment stay in
-// registers), FP64 two (<= 128).
-// The CTA body for block `blk` of the launch of A (any block size of at
-// least lpc E threads, rounded to whole warps).
-template <typename T, int P, int CV>
-__device__ __forceinline__ void line_block_body(BlockLineArgs<T> A, int blk) {
-    // right-hand side fastest in the CTA order (see device.cuh): the nrhs CTAs
-    // of one line group read the same segment operators
-    const int rhs = blk % A.nrhs, bx = blk / A.nrhs;
-    {
-        const long long vo = (long long)rhs * A.N;
-        if (A.g) A.g += vo;
-        if (A.r) A.r += vo;
-        if (A.y) A.y += vo;
-        A.x += vo;
-    }
+template <typename T, int P, int C, bool CONTIG>
+__device__ __forceinline__ void line_seg_body(BlockLineArgs<T>& A, int blk) {
+    constexpr int MI = SegOp<T, P>::MI;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int n = A.n, E = A.E, span = A.span, mode = A.mode, LPC = A.lpc;
-    const int p = P > 0 ? P : A.p;
-    const int mi = p - 1, npk = mi * (mi + 1) / 2;
+    const int E = A.E, LPC = A.lpc, SE = E | 1, mode = A.mode;
+    T* sh = reinterpret_cast<T*>(smem_raw);   // [LPC][SE]
+    T* sdr = sh + LPC * SE;                   // [LPC][SE]
+    T* so = sdr + LPC * SE;                   // [padk(LPC n)]: new x (CONTIG)
+    const int l0 = enter(A, blk);
+    const int Wc = min(LPC, A.nlines - l0);
+    const int tid = threadIdx.x;
+    // this thread's line w and segment e: segments adjacent for x-lines,
+    // lines adjacent for strided directions
+    int w, e;
+    if constexpr (CONTIG) {
+        w = tid / E;
+        e = tid - w * E;
+    } else {
+        w = tid & (LPC - 1);
+        e = tid >> (31 - __clz(LPC));
+    }
+    const bool act = w < Wc && e < E;
+    const int li = l0 + (act ? w : 0);
+    SegOp<T, P> op;
+    op.load(A.blk + (CONTIG ? (long long)li * E + e : (long long)(act ? e : 0) * A.nlines + li), A.ntask, act);
+    VertexCr<T, C> vc;
+    {
+        const int wg = tid / A.sub;
+        vc.load(A, l0 + wg, wg < Wc, tid & (A.sub - 1));
+    }
+    const int stride = CONTIG ? 1 : A.stride;
+    const int c2 = li / A.m1 + 1, c1 = li - (c2 - 1) * A.m1 + 1;
+    const int v0 = c1 * A.st1 + c2 * A.st2 + e * P * stride;   // the segment's left vertex
+    if (!ready(A)) return;
+
+    T gi[MI], xi[MI], gv = T(0), xv = T(0);
+    const bool vertex = act && e > 0;
+    // one branch per mode, so that a thread's loads are issued back to back
+    const T* src = mode == 0 ? A.g : A.r;
+#pragma unroll
+    for (int i = 0; i < MI; ++i) gi[i] = xi[i] = T(0);
+    if (act) {
+        if (vertex) gv = src[v0];
+#pragma unroll
+        for (int i = 0; i < MI; ++i) gi[i] = src[v0 + (i + 1) * stride];
+        if (mode == 1) {
+            T yi[MI], yv = T(0);
+            if (vertex) yv = A.y[v0];
+#pragma unroll
+            for (int i = 0; i < MI; ++i) yi[i] = A.y[v0 + (i + 1) * stride];
+            if (vertex) xv = A.x[v0];
+#pragma unroll
+            for (int i = 0; i < MI; ++i) xi[i] = A.x[v0 + (i + 1) * stride];
+            gv -= yv;
+#pragma unroll
+            for (int i = 0; i < MI; ++i) gi[i] -= yi[i];
+        } else if (mode == 2) {
+            if (vertex) xv = A.x[v0];
+#pragma unroll
+            for (int i = 0; i < MI; ++i) xi[i] = A.x[v0 + (i + 1) * stride];
+        }
+    }
+    T z[MI], nl = T(0), nr = T(0);
+    T dl, dr;
+    op.solve(gi, z, dl, dr);
+    if (E > 1) {
+        if (act) {
+            sdr[w * SE + e] = dr;
+            sh[w * SE + e] = gv - dl;
+        }
+        __syncthreads();
+        vertex_phase<T, C>(A, vc, sh, sdr, SE, l0, Wc);
+        __syncthreads();
+        if (act) {
+            if (e > 0) nl = sh[w * SE + e];
+            if (e < E - 1) nr = sh[w * SE + e + 1];
+        }
+    }
+    const T scale = mode == 0 ? T(1) : A.alpha;
+    // the next apply stores element-interior nodes and adds into the element-
+    // boundary ones: only those must be reset
+    const bool seam = mode == 1 && (c1 % P == 0 || (A.st2 != 0 && c2 % P == 0));
+    if constexpr (!CONTIG) {
+        if (!act) return;
+#pragma unroll
+        for (int i = 0; i < MI; ++i) {
+            const int node = v0 + (i + 1) * stride;
+            A.x[node] = xi[i] + scale * (z[i] - (op.left(i) * nl + op.right(i) * nr));
+            if (seam) A.y[node] = T(0);
+        }
+        if (vertex) {
+            A.x[v0] = xv + scale * nl;
+            if (mode == 1) A.y[v0] = T(0);
+        }
+    } else {
+        // a segment's nodes are adjacent: through shared memory, so that whole
+        // warps write along the lines
+        const int n = A.n, k0 = w * n + e * P;
+        if (act) {
+#pragma unroll
+            for (int i = 0; i < MI; ++i)
+                so[padk(k0 + i)] = xi[i] + scale * (z[i] - (op.left(i) * nl + op.right(i) * nr));
+            if (vertex) {
+                so[padk(k0 - 1)] = xv + scale * nl;
+                if (mode == 1) A.y[v0] = T(0);
+            }
+            if (seam) {
+#pragma unroll
+                for (int i = 0; i < MI; ++i) A.y[v0 + i + 1] = T(0);
+            }
+        }
+        __syncthreads();
+        // value idx lies on line idx / n: exact by the rounded-up reciprocal
+        // for idx < 2^15, n < 2^11
+        const unsigned magic = n > 1 ? 0xffffffffu / (unsigned)n + 1u : 0u;
+        const int total = Wc * n;
+        const int q0 = l0 / A.m1, r0 = l0 - q0 * A.m1;      // plane and row of the CTA's first line
+#pragma unroll
+        for (int it = 0; it < P; ++it) {
+            const int idx = tid + it * (int)blockDim.x;
+            if (idx < total) {
+                const int wl = n > 1 ? (int)__umulhi((unsigned)idx, magic) : idx;
+                int row = r0 + wl, plane = q0;
+                while (row >= A.m1) {
+                    row -= A.m1;
+                    ++plane;
+                }
+                A.x[(row + 1) * A.st1 + (plane + 1) * A.st2 + 1 + idx - wl * n] = so[padk(idx)];
+            }
+        }
+    }
+}
+
+// Any order and line length: the line values and the segment operators in
+// shared memory (cp.async), z accumulated there.
+template <typename T, int C>
+__device__ __forceinline__ void line_any_body(BlockLineArgs<T>& A, int blk) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const int n = A.n, E = A.E, span = A.span, mode = A.mode, LPC = A.lpc, SE = E | 1;
+    const int p = A.p, mi = p - 1, npk = mi * (mi + 1) / 2;
     const long long ntask = A.ntask;
     T* sg = reinterpret_cast<T*>(smem_raw);   // [LPC][span]: g, then z / nu, then B^-1 g
     T* sx = sg + LPC * span;                  // [LPC][span]: x on entry (MODE 1, 2)
     T* sy = sx + LPC * span;                  // [LPC][span]: y on entry (MODE 1)
-    T* sdl = sy + LPC * span;                 // [LPC][E]: w_L . g_I per segment
-    T* sdr = sdl + LPC * E;                   // [LPC][E]: w_R . g_I
-    T* svb = sdr + LPC * E;                   // [LPC][2 (E - 1)]: vertex systems
-    T* sz = svb + 2 * LPC * (E - 1);          // [LPC][span]: z accumulation (P = 0)
-    // orders above 8 keep the segment operators in shared memory (too many
-    // for registers): the run-time order, and compile-time orders 9..12
-    constexpr bool SMOP = P == 0 || P > 8;
-    T* sop = P == 0 ? sz + LPC * span : sz;   // [ncoef][blockDim]: segment operators (SMOP)
-    const int l0 = bx * LPC;
+    T* sz = sy + LPC * span;                  // [LPC][span]: z accumulation
+    T* sh = sz + LPC * span;                  // [LPC][SE]
+    T* sdr = sh + LPC * SE;                   // [LPC][SE]
+    T* sop = sdr + LPC * SE;                  // [ncoef][threads of the item]: segment operators
+    const int l0 = enter(A, blk);
     const int Wc = min(LPC, A.nlines - l0);
     const int tid = threadIdx.x;
-    // first node of line w of this CTA (interior indices c1, c2 of the other axes)
     auto line_base = [&](int w) {
         const int li = l0 + w;
         return (li % A.m1 + 1) * A.st1 + (li / A.m1 + 1) * A.st2;
     };
-    // this thread's segment task and its operator, loaded before anything waits
-    const int ntk = Wc * E;
-    const bool has_task = tid < ntk;
+    const bool has_task = tid < Wc * E;
     const int tw = has_task ? tid / E : 0, te = has_task ? tid - tw * E : 0;
-    const T* bp = A.blk + ((long long)(l0 + tw) * E + te);
-    SegOp<T, SMOP ? 2 : P> op;            // registers (orders 2..8 only)
-    if constexpr (P > 0 && !SMOP) {
-        if (has_task) {
-#pragma unroll
-            for (int c = 0; c < SegOp<T, P>::NPK; ++c) op.t[c] = __ldg(bp + (long long)c * ntask);
-#pragma unroll
-            for (int i = 0; i < P - 1; ++i) {
-                op.wl[i] = __ldg(bp + (long long)(npk + i) * ntask);
-                op.wr[i] = __ldg(bp + (long long)(npk + mi + i) * ntask);
-            }
-        }
-    }
+    const bool contig = A.contiguous != 0;
+    const T* bp = A.blk + (contig ? (long long)(l0 + tw) * E + te : (long long)te * A.nlines + l0 + tw);
     // operator rows are as long as this launch item's own thread count (a
     // work-list block may be larger; its extra threads have no segment)
-    const int opstride = min(kBlockThreads, max(32, (LPC * E + 31) / 32 * 32));
-    if constexpr (SMOP) {
-        // the thread's segment operator is copied to shared memory with the
-        // line values and read from there in the loops
-        if (has_task) {
-            const int ncoef = npk + 2 * mi;
-            for (int c = 0; c < ncoef; ++c) cp_async(sop + c * opstride + tid, bp + (long long)c * ntask);
-        }
+    const int opstride = block_threads(LPC, E);
+    VertexCr<T, C> vc;
+    {
+        const int wg = tid / A.sub;
+        vc.load(A, l0 + wg, wg < Wc, tid & (A.sub - 1));
     }
-    auto opc = [&](int c) { return sop[c * opstride + tid]; };   // coefficient c of this thread's segment (SMOP)
-    auto op_t = [&](int c) -> T {
-        if constexpr (SMOP) return opc(c);
-        else return op.t[c];
-    };
-    auto op_wl = [&](int i) -> T {
-        if constexpr (SMOP) return opc(npk + i);
-        else return op.wl[i];
-    };
-    auto op_wr = [&](int i) -> T {
-        if constexpr (SMOP) return opc(npk + mi + i);
-        else return op.wr[i];
-    };
-
-    // line values, staged without divisions by asynchronous copies (every
-    // copy of the tile in flight at once): x-lines are walked along the line
-    // by whole warps (coalesced along x); strided directions by threads that
-    // each keep one line of the CTA and step over its rows, adjacent threads
-    // on adjacent lines (coalesced across the lines)
-    const bool contig = A.contiguous != 0;
+    if (has_task) {
+        const int ncoef = npk + 2 * mi;
+        for (int c = 0; c < ncoef; ++c) cp_async(sop + c * opstride + tid, bp + (long long)c * ntask);
+    }
+    auto opc = [&](int c) { return sop[c * opstride + tid]; };   // coefficient c of this thread's segment
+    if (!ready(A)) {
+        cp_async_wait_all();
+        return;
+    }
+    // x-lines are walked along the line by whole warps; strided directions by
+    // threads that each keep one line of the CTA and step over its rows,
+    // adjacent threads on adjacent lines
     const int nthr = blockDim.x, nwarp = nthr >> 5;
-    const int rows_per_pass = nthr / LPC;     // strided: rows covered per pass
+    const int rows_per_pass = nthr / LPC;
     const int sw = contig ? 0 : tid % LPC, sk0 = contig ? 0 : tid / LPC;
     const bool s_active = !contig && sw < Wc && sk0 < rows_per_pass;
     const int s_base = s_active ? line_base(sw) : 0;
@@ -217,18 +467,10 @@ __device__ __forceinline__ void line_block_body(BlockLineArgs<T> A, int blk) {
     if (contig) {
         for (int w = tid >> 5; w < Wc; w += nwarp) {
             const int b = line_base(w);
-#pragma unroll 2
             for (int k = tid & 31; k < n; k += 32) stage(w, k, b + (k + 1) * A.stride);
         }
     } else if (s_active) {
-#pragma unroll 2
         for (int k = sk0; k < n; k += rows_per_pass) stage(sw, k, s_base + (k + 1) * A.stride);
-    }
-    // vertex systems of the CTA's lines (contiguous in global memory)
-    if (E > 1) {
-        const T* vsrc = reinterpret_cast<const T*>(A.vband + (long long)l0 * (E - 1));
-        const int nvb = 2 * Wc * (E - 1);
-        for (int i = tid; i < nvb; i += nthr) cp_async(svb + i, vsrc + i);
     }
     cp_async_wait_all();
     __syncthreads();
@@ -236,103 +478,51 @@ __device__ __forceinline__ void line_block_body(BlockLineArgs<T> A, int blk) {
         for (int i = tid; i < Wc * span; i += nthr) sg[i] -= sy[i];
         __syncthreads();
     }
-
-    // ---- segments: z = K_I^-1 g_I and the two vertex dots
-    T z[P > 1 ? P - 1 : 1];
     if (has_task) {
         T* line = sg + tw * span;
+        T* zz = sz + tw * span;
         const int base = te * p;   // line unknown of the segment's first interior node
         T dl = T(0), dr = T(0);
-        if constexpr (P > 0) {
-            T gi[P - 1];
-#pragma unroll
-            for (int i = 0; i < P - 1; ++i) {
-                gi[i] = line[padk(base + i)];
-                z[i] = T(0);
+        for (int i = 0; i < mi; ++i) zz[padk(base + i)] = T(0);
+        int c = 0;
+        for (int i = 0; i < mi; ++i) {
+            const T gi_ = line[padk(base + i)];
+            T zi = T(0);
+            for (int j = i; j < mi; ++j) {
+                const T t = opc(c);
+                ++c;
+                zi += t * line[padk(base + j)];
+                if (j != i) zz[padk(base + j)] += t * gi_;
             }
-            int c = 0;
-#pragma unroll
-            for (int i = 0; i < P - 1; ++i)
-#pragma unroll
-                for (int j = i; j < P - 1; ++j) {
-                    const T t = op_t(c++);
-                    z[i] += t * gi[j];
-                    if (j != i) z[j] += t * gi[i];
-                }
-#pragma unroll
-            for (int i = 0; i < P - 1; ++i) {
-                dl += op_wl(i) * gi[i];
-                dr += op_wr(i) * gi[i];
-            }
-        } else {
-            T* zz = sz + tw * span;
-            for (int i = 0; i < mi; ++i) zz[padk(base + i)] = T(0);
-            int c = 0;
-            for (int i = 0; i < mi; ++i) {
-                const T gi_ = line[padk(base + i)];
-                T zi = T(0);
-                for (int j = i; j < mi; ++j) {
-                    const T t = opc(c);
-                    ++c;
-                    zi += t * line[padk(base + j)];
-                    if (j != i) zz[padk(base + j)] += t * gi_;
-                }
-                zz[padk(base + i)] += zi;
-                dl += opc(npk + i) * gi_;
-                dr += opc(npk + mi + i) * gi_;
-            }
+            zz[padk(base + i)] += zi;
+            dl += opc(npk + i) * gi_;
+            dr += opc(npk + mi + i) * gi_;
         }
-        // each task reads and writes only its own segment's interior nodes
-        if constexpr (P > 0) {
-#pragma unroll
-            for (int i = 0; i < P - 1; ++i) line[padk(base + i)] = z[i];
-        } else {
-            const T* zz = sz + tw * span;
-            for (int i = 0; i < mi; ++i) line[padk(base + i)] = zz[padk(base + i)];
-        }
-        sdl[tw * E + te] = dl;
-        sdr[tw * E + te] = dr;
+        sdr[tw * SE + te] = dr;
+        sh[tw * SE + te] = (te > 0 ? line[padk(base - 1)] : T(0)) - dl;
     }
     __syncthreads();
-
-    // ---- vertex systems, one warp per line
-    const int warp = tid >> 5, lane = tid & 31;
     if (E > 1) {
-        for (int w = warp; w < Wc; w += nwarp) {
-            T* line = sg + w * span;
-            const T* vb = svb + 2 * w * (E - 1);
-            vertex_solve<T, CV>(line, sdl + w * E, sdr + w * E, vb, E, p, lane);
-        }
+        vertex_phase<T, C>(A, vc, sh, sdr, SE, l0, Wc);
+        __syncthreads();
     }
-    __syncthreads();
-
-    // ---- segments: x_I = z - w_L nu_left - w_R nu_right
     if (has_task) {
         T* line = sg + tw * span;
+        const T* zz = sz + tw * span;
         const int base = te * p;
-        const T nl = te > 0 ? line[padk(base - 1)] : T(0);
-        const T nr = te < E - 1 ? line[padk(base + mi)] : T(0);
-        if constexpr (P > 0) {
-#pragma unroll
-            for (int i = 0; i < P - 1; ++i) line[padk(base + i)] = z[i] - (op_wl(i) * nl + op_wr(i) * nr);
-        } else {
-            for (int i = 0; i < mi; ++i) {
-                const T wl = opc(npk + i);
-                const T wr = opc(npk + mi + i);
-                line[padk(base + i)] -= wl * nl + wr * nr;
-            }
-        }
+        const T nl = te > 0 ? sh[tw * SE + te] : T(0);
+        const T nr = te < E - 1 ? sh[tw * SE + te + 1] : T(0);
+        for (int i = 0; i < mi; ++i)
+            line[padk(base + i)] = zz[padk(base + i)] - (opc(npk + i) * nl + opc(npk + mi + i) * nr);
+        if (te > 0) line[padk(base - 1)] = nl;
     }
     __syncthreads();
-
     // seam test: the line lies on an element boundary of another axis, or the
     // node is a vertex of the line
     auto put = [&](int w, int k, int base, bool line_seam) {
         const int node = base + (k + 1) * A.stride;
         const T v = sg[w * span + padk(k)];
         A.x[node] = mode == 0 ? v : (mode == 3 ? A.alpha * v : sx[w * span + padk(k)] + A.alpha * v);
-        // the next apply stores element-interior nodes and adds into the
-        // element-boundary ones: only those must be reset
         if (mode == 1 && (line_seam || (k + 1) % p == 0)) A.y[node] = T(0);
     };
     auto seam_of = [&](int w) {
@@ -343,37 +533,50 @@ __device__ __forceinline__ void line_block_body(BlockLineArgs<T> A, int blk) {
         for (int w = tid >> 5; w < Wc; w += nwarp) {
             const int b = line_base(w);
             const bool ls = seam_of(w);
-#pragma unroll 2
             for (int k = tid & 31; k < n; k += 32) put(w, k, b, ls);
         }
     } else if (s_active) {
         const bool ls = seam_of(sw);
-#pragma unroll 2
         for (int k = sk0; k < n; k += rows_per_pass) put(sw, k, s_base, ls);
     }
 }
 
-template <typename T, int P, int CV>
-__global__ void __launch_bounds__(kBlockThreads, sizeof(T) == 8 ? 2 : (P >= 8 || P == 0 ? 3 : 4))
-    line_block_kernel(BlockLineArgs<T> A) {
-    grid_dep_sync();
-    line_block_body<T, P, CV>(A, blockIdx.x);
+template <typename T, int P, int CV, bool CONTIG>
+__device__ __forceinline__ void line_block_body(BlockLineArgs<T>& A, int blk) {
+    if constexpr (P == 0) line_any_body<T, CV>(A, blk);
+    else line_seg_body<T, P, CV, CONTIG>(A, blk);
+}
+
+// Resident CTAs the registers must allow.
+template <typename T, int P>
+constexpr int line_min_ctas() {
+    return sizeof(T) == 8 ? 2 : P == 0 ? 2 : P >= 9 ? 1 : 3;
+}
+
+template <typename T, int P, int CV, bool CONTIG>
+__global__ void __launch_bounds__(kBlockThreads, line_min_ctas<T, P>())
+    line_block_kernel(const __grid_constant__ BlockLineArgs<T> A0) {
+    BlockLineArgs<T> A = A0;
+    line_block_body<T, P, CV, CONTIG>(A, blockIdx.x);
 }
 
 // Work-list form: item j (one problem's level, direction and vectors) owns
 // the CTAs [start[j], start[j + 1]).
-template <typename T, int P, int CV>
-__global__ void __launch_bounds__(kBlockThreads, sizeof(T) == 8 ? 2 : (P >= 8 || P == 0 ? 3 : 4))
+template <typename T, int P, int CV, bool CONTIG>
+__global__ void __launch_bounds__(kBlockThreads, line_min_ctas<T, P>())
     line_block_list_kernel(const BlockLineArgs<T>* __restrict__ items, const int* __restrict__ start, int nitems) {
-    grid_dep_sync();
     const int j = work_item(start, nitems, blockIdx.x);
-    if (items[j].done && *items[j].done != 0.0) return;
-    line_block_body<T, P, CV>(items[j], blockIdx.x - start[j]);
+    BlockLineArgs<T> A = items[j];
+    line_block_body<T, P, CV, CONTIG>(A, blockIdx.x - start[j]);
 }
 
-template <typename T, int P>
-size_t block_smem(int lpc, int span, int E) {
-    return sizeof(T) * ((size_t)lpc * span * (P == 0 ? 4 : 3) + 2 * (size_t)lpc * E + 2 * (size_t)lpc * (E - 1));
+// Shared memory of a CTA of lpc lines: the vertex arrays, with the line
+// values once (x-lines) or four times (run-time order).
+template <typename T>
+size_t block_smem(int lpc, int n, int span, int E, bool contiguous, bool any_order) {
+    const size_t tile = (size_t)lpc * n;
+    const size_t values = any_order ? 4 * (size_t)lpc * span : contiguous ? tile + tile / 32 + 1 : 0;
+    return sizeof(T) * (values + 2 * (size_t)lpc * (E | 1));
 }
 
 // Shared memory of the run-time-order instance's segment operators for a
@@ -382,6 +585,13 @@ template <typename T>
 size_t op_smem(int p, int threads) {
     const size_t mi = (size_t)(p - 1);
     return sizeof(T) * (mi * (mi + 1) / 2 + 2 * mi) * (size_t)threads;
+}
+
+// Most lines of a CTA: a power of two, at most 16 lines and 256 segments.
+int most_lines(int E) {
+    int lpc = 1;
+    while (2 * lpc <= kMaxLinesPerCta && 2 * lpc * E <= kBlockThreads) lpc *= 2;
+    return lpc;
 }
 
 // Orders 2..12 are compiled for vertex chunks of 1 and 2 per lane (lines of
@@ -393,23 +603,31 @@ bool launch_pc(BlockLineArgs<T> A, cudaStream_t st) {
     // else fewer while the level would have less than about four CTAs per SM
     // (small levels are latency bound: more, smaller CTAs run their phases
     // side by side)
-    const int most = std::min(kMaxLinesPerCta, std::max(1, kBlockThreads / A.E));
+    const int most = most_lines(A.E);
     int lpc = most;
-    if (A.lpc > 0) lpc = std::min(A.lpc, most);
-    else
-        while (lpc > 1 && (long long)(A.nlines + lpc - 1) / lpc * A.nrhs < 4 * sm_count()) lpc /= 2;
-    auto thr = [&](int c) { return std::min(kBlockThreads, std::max(32, (c * A.E + 31) / 32 * 32)); };
+    if (A.lpc > 0) {
+        while (lpc > A.lpc) lpc /= 2;
+    } else {
+        // strided directions keep four adjacent lines, half a 32-byte sector
+        // of FP32 a row: below that the row reads, not the CTA count, bound
+        // the launch (64 x 64 elements, p = 8: 4.7 us with four lines, 11 with one)
+        const int least = A.contiguous ? 1 : 4;
+        while (lpc > least && (long long)(A.nlines + lpc - 1) / lpc * A.nrhs < 4 * sm_count()) lpc /= 2;
+    }
     auto sm = [&](int c) {
-        return block_smem<T, P>(c, A.span, A.E) + (P == 0 || P > 8 ? op_smem<T>(A.p, thr(c)) : 0);
+        return block_smem<T>(c, A.n, A.span, A.E, A.contiguous != 0, P == 0) +
+               (P == 0 ? op_smem<T>(A.p, block_threads(c, A.E)) : 0);
     };
     while (lpc > 1 && sm(lpc) > kMaxDynSmemBytes) lpc /= 2;
     const size_t smem = sm(lpc);
     if (smem > kMaxDynSmemBytes) return false;
     A.lpc = lpc;
-    const int threads = thr(lpc);
+    const int threads = block_threads(lpc, A.E);
     const long long blocks = (long long)(A.nlines + lpc - 1) / lpc * A.nrhs;
     if (blocks > 0x7fffffffLL) return false;
-    return launch_k(line_block_kernel<T, P, CV>, (unsigned)blocks, threads, smem, st, A) == cudaSuccess;
+    if (P > 0 && !A.contiguous)
+        return launch_k(line_block_kernel<T, P, CV, false>, (unsigned)blocks, threads, smem, st, A) == cudaSuccess;
+    return launch_k(line_block_kernel<T, P, CV, true>, (unsigned)blocks, threads, smem, st, A) == cudaSuccess;
 }
 
 template <typename T, int P>
@@ -428,41 +646,35 @@ bool launch_p(BlockLineArgs<T> A, cudaStream_t st) {
     }
 }
 
-template <typename T, int P>
-bool set_attr_p() {
-    const int lim = (int)kMaxDynSmemBytes;
-    if constexpr (P > 0) {
-        const void* fns[] = {(const void*)line_block_kernel<T, P, 1>, (const void*)line_block_kernel<T, P, 2>,
-                             (const void*)line_block_list_kernel<T, P, 1>,
-                             (const void*)line_block_list_kernel<T, P, 2>};
-        for (const void* f : fns)
-            if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) != cudaSuccess) return false;
-        return true;
-    } else {
-        const void* fns[] = {(const void*)line_block_kernel<T, 0, 1>, (const void*)line_block_kernel<T, 0, 2>,
-                             (const void*)line_block_kernel<T, 0, 4>, (const void*)line_block_kernel<T, 0, 8>,
-                             (const void*)line_block_list_kernel<T, 0, 1>,
-                             (const void*)line_block_list_kernel<T, 0, 2>,
-                             (const void*)line_block_list_kernel<T, 0, 4>,
-                             (const void*)line_block_list_kernel<T, 0, 8>};
-        for (const void* f : fns)
-            if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) != cudaSuccess) return false;
-        return true;
-    }
-}
-
+// Dynamic shared memory above 48 KB (the run-time order; the others stay below).
 template <typename T>
-bool set_attr_t() {
-    return set_attr_p<T, 0>() && set_attr_p<T, 2>() && set_attr_p<T, 3>() && set_attr_p<T, 4>() &&
-           set_attr_p<T, 5>() && set_attr_p<T, 6>() && set_attr_p<T, 7>() && set_attr_p<T, 8>() &&
-           set_attr_p<T, 9>() && set_attr_p<T, 10>() && set_attr_p<T, 11>() && set_attr_p<T, 12>();
+bool set_attr_any() {
+    const int lim = (int)kMaxDynSmemBytes;
+    const void* fns[] = {(const void*)line_block_kernel<T, 0, 1, true>, (const void*)line_block_kernel<T, 0, 2, true>,
+                         (const void*)line_block_kernel<T, 0, 4, true>, (const void*)line_block_kernel<T, 0, 8, true>,
+                         (const void*)line_block_list_kernel<T, 0, 1, true>,
+                         (const void*)line_block_list_kernel<T, 0, 2, true>,
+                         (const void*)line_block_list_kernel<T, 0, 4, true>,
+                         (const void*)line_block_list_kernel<T, 0, 8, true>};
+    for (const void* f : fns)
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, lim) != cudaSuccess) return false;
+    return true;
 }
 
 }  // namespace
 
-bool init_line_block_attributes() { return set_attr_t<float>() && set_attr_t<double>(); }
+template <>
+bool init_line_block_attributes<LineT>() {
+    return set_attr_any<LineT>();
+}
 
+#ifndef GLLS_LINES_F64
 bool line_block_supported(int n, int E) { return n <= kMaxBlockLine && E <= kMaxBlockSegments; }
+
+// Whether launch_line_block_list(p, cv, ...) runs the order-specialised
+// instance (smem[0] of the items) or the run-time-order one (smem[1]).
+bool line_block_list_specialised(int p, int cv) { return p >= 2 && p <= 12 && cv <= 2; }
+#endif
 
 namespace {
 
@@ -496,9 +708,11 @@ int make_args(BlockLineArgs<T>& A, const DevLevel<T>& L, int s, int mode, const 
     A.lpc = L.lbc[s];                  // 0: the launch heuristic
     const int nv = A.E - 1;
     A.cv = nv <= 32 ? 1 : (nv <= 64 ? 2 : (nv <= 128 ? 4 : 8));
+    A.sub = 1;                         // lanes per line of the vertex CR
+    while (A.sub * A.cv < nv) A.sub *= 2;
     A.alpha = alpha;
     A.blk = L.blk[s];
-    A.vband = L.vband[s];
+    A.vcr = L.vcr[s];
     A.g = g;
     A.r = r;
     A.y = y;
@@ -508,25 +722,29 @@ int make_args(BlockLineArgs<T>& A, const DevLevel<T>& L, int s, int mode, const 
 }
 
 template <typename T, int P, int CV>
-bool launch_list_pc(const void* items, const int* start, int nitems, int blocks, int threads, size_t smem,
+bool launch_list_pc(int s, const void* items, const int* start, int nitems, int blocks, int threads, size_t smem,
                     cudaStream_t st) {
-    return launch_k(line_block_list_kernel<T, P, CV>, (unsigned)blocks, threads, smem, st,
-                    static_cast<const BlockLineArgs<T>*>(items), start, nitems) == cudaSuccess;
+    const BlockLineArgs<T>* it = static_cast<const BlockLineArgs<T>*>(items);
+    if (P > 0 && s != 0)
+        return launch_k(line_block_list_kernel<T, P, CV, false>, (unsigned)blocks, threads, smem, st, it, start,
+                        nitems) == cudaSuccess;
+    return launch_k(line_block_list_kernel<T, P, CV, true>, (unsigned)blocks, threads, smem, st, it, start, nitems) ==
+           cudaSuccess;
 }
 
 template <typename T, int P>
-bool launch_list_p(int cv, const void* items, const int* start, int nitems, int blocks, int threads, size_t smem,
+bool launch_list_p(int s, int cv, const void* items, const int* start, int nitems, int blocks, int threads, size_t smem,
                    cudaStream_t st) {
     if constexpr (P > 0) {
-        if (cv == 1) return launch_list_pc<T, P, 1>(items, start, nitems, blocks, threads, smem, st);
-        if (cv == 2) return launch_list_pc<T, P, 2>(items, start, nitems, blocks, threads, smem, st);
-        return launch_list_p<T, 0>(cv, items, start, nitems, blocks, threads, smem, st);
+        if (cv == 1) return launch_list_pc<T, P, 1>(s, items, start, nitems, blocks, threads, smem, st);
+        if (cv == 2) return launch_list_pc<T, P, 2>(s, items, start, nitems, blocks, threads, smem, st);
+        return launch_list_p<T, 0>(s, cv, items, start, nitems, blocks, threads, smem, st);
     } else {
         switch (cv) {
-            case 1: return launch_list_pc<T, 0, 1>(items, start, nitems, blocks, threads, smem, st);
-            case 2: return launch_list_pc<T, 0, 2>(items, start, nitems, blocks, threads, smem, st);
-            case 4: return launch_list_pc<T, 0, 4>(items, start, nitems, blocks, threads, smem, st);
-            default: return launch_list_pc<T, 0, 8>(items, start, nitems, blocks, threads, smem, st);
+            case 1: return launch_list_pc<T, 0, 1>(s, items, start, nitems, blocks, threads, smem, st);
+            case 2: return launch_list_pc<T, 0, 2>(s, items, start, nitems, blocks, threads, smem, st);
+            case 4: return launch_list_pc<T, 0, 4>(s, items, start, nitems, blocks, threads, smem, st);
+            default: return launch_list_pc<T, 0, 8>(s, items, start, nitems, blocks, threads, smem, st);
         }
     }
 }
@@ -556,59 +774,52 @@ int line_block_list_item(const DevLevel<T>& L, int s, int mode, const T* g, cons
     BlockLineArgs<T> A;
     const int k = make_args<T>(A, L, s, mode, g, r, y, x, alpha, 1);
     if (k <= 0) return k;
-    // the run-time-order instance and orders 9..12 also hold the segment
-    // operators of the item's own threads
-    auto thr = [&](int c) { return std::min(kBlockThreads, std::max(32, (c * A.E + 31) / 32 * 32)); };
-    auto sm1 = [&](int c) { return block_smem<T, 0>(c, A.span, A.E) + op_smem<T>(A.p, thr(c)); };
-    int lpc = std::min(kMaxLinesPerCta, std::max(1, kBlockThreads / A.E));
+    // the run-time-order instance also holds the segment operators of the
+    // item's own threads
+    auto sm1 = [&](int c) {
+        return block_smem<T>(c, A.n, A.span, A.E, true, true) + op_smem<T>(A.p, block_threads(c, A.E));
+    };
+    int lpc = most_lines(A.E);
     while (lpc > 1 && sm1(lpc) > kMaxDynSmemBytes) lpc /= 2;
     if (sm1(lpc) > kMaxDynSmemBytes) return -1;
     A.lpc = lpc;
-    smem[0] = block_smem<T, 2>(lpc, A.span, A.E) + (A.p > 8 ? op_smem<T>(A.p, thr(lpc)) : 0);
+    smem[0] = block_smem<T>(lpc, A.n, A.span, A.E, A.contiguous != 0, false);
     smem[1] = sm1(lpc);
-    *threads = thr(lpc);
+    *threads = block_threads(lpc, A.E);
     *blocks = (A.nlines + lpc - 1) / lpc;
     *cv = A.cv;
     std::memcpy(item, &A, sizeof(A));
     return 1;
 }
 
-// Whether launch_line_block_list(p, cv, ...) runs the order-specialised
-// instance (smem[0] of the items) or the run-time-order one (smem[1]).
-bool line_block_list_specialised(int p, int cv) { return p >= 2 && p <= 12 && cv <= 2; }
-
-// One launch over the items (all of order p; cv: the largest vertex chunk of
-// the items).
+// One launch over the items (all along axis s and of order p; cv: the largest
+// vertex chunk of the items).
 template <typename T>
-bool launch_line_block_list(int p, int cv, const void* items, const int* start, int nitems, int blocks, int threads,
+bool launch_line_block_list(int p, int s, int cv, const void* items, const int* start, int nitems, int blocks, int threads,
                             size_t smem, cudaStream_t st) {
     if (nitems < 1 || blocks < 1) return true;
     switch (line_block_list_specialised(p, cv) ? p : 0) {
-        case 2: return launch_list_p<T, 2>(cv, items, start, nitems, blocks, threads, smem, st);
-        case 3: return launch_list_p<T, 3>(cv, items, start, nitems, blocks, threads, smem, st);
-        case 4: return launch_list_p<T, 4>(cv, items, start, nitems, blocks, threads, smem, st);
-        case 5: return launch_list_p<T, 5>(cv, items, start, nitems, blocks, threads, smem, st);
-        case 6: return launch_list_p<T, 6>(cv, items, start, nitems, blocks, threads, smem, st);
-        case 7: return launch_list_p<T, 7>(cv, items, start, nitems, blocks, threads, smem, st);
-        case 8: return launch_list_p<T, 8>(cv, items, start, nitems, blocks, threads, smem, st);
-        case 9: return launch_list_p<T, 9>(cv, items, start, nitems, blocks, threads, smem, st);
-        case 10: return launch_list_p<T, 10>(cv, items, start, nitems, blocks, threads, smem, st);
-        case 11: return launch_list_p<T, 11>(cv, items, start, nitems, blocks, threads, smem, st);
-        case 12: return launch_list_p<T, 12>(cv, items, start, nitems, blocks, threads, smem, st);
-        default: return launch_list_p<T, 0>(cv, items, start, nitems, blocks, threads, smem, st);
+        case 2: return launch_list_p<T, 2>(s, cv, items, start, nitems, blocks, threads, smem, st);
+        case 3: return launch_list_p<T, 3>(s, cv, items, start, nitems, blocks, threads, smem, st);
+        case 4: return launch_list_p<T, 4>(s, cv, items, start, nitems, blocks, threads, smem, st);
+        case 5: return launch_list_p<T, 5>(s, cv, items, start, nitems, blocks, threads, smem, st);
+        case 6: return launch_list_p<T, 6>(s, cv, items, start, nitems, blocks, threads, smem, st);
+        case 7: return launch_list_p<T, 7>(s, cv, items, start, nitems, blocks, threads, smem, st);
+        case 8: return launch_list_p<T, 8>(s, cv, items, start, nitems, blocks, threads, smem, st);
+        case 9: return launch_list_p<T, 9>(s, cv, items, start, nitems, blocks, threads, smem, st);
+        case 10: return launch_list_p<T, 10>(s, cv, items, start, nitems, blocks, threads, smem, st);
+        case 11: return launch_list_p<T, 11>(s, cv, items, start, nitems, blocks, threads, smem, st);
+        case 12: return launch_list_p<T, 12>(s, cv, items, start, nitems, blocks, threads, smem, st);
+        default: return launch_list_p<T, 0>(s, cv, items, start, nitems, blocks, threads, smem, st);
     }
 }
 
-template size_t line_block_item_bytes<float>();
-template size_t line_block_item_bytes<double>();
-template size_t line_block_item_done_offset<float>();
-template size_t line_block_item_done_offset<double>();
-template int line_block_list_item<float>(const DevLevel<float>&, int, int, const float*, const float*, float*, float*,
-                                         float, void*, int*, int*, size_t*, int*);
-template int line_block_list_item<double>(const DevLevel<double>&, int, int, const double*, const double*, double*,
-                                          double*, double, void*, int*, int*, size_t*, int*);
-template bool launch_line_block_list<float>(int, int, const void*, const int*, int, int, int, size_t, cudaStream_t);
-template bool launch_line_block_list<double>(int, int, const void*, const int*, int, int, int, size_t, cudaStream_t);
+template size_t line_block_item_bytes<LineT>();
+template size_t line_block_item_done_offset<LineT>();
+template int line_block_list_item<LineT>(const DevLevel<LineT>&, int, int, const LineT*, const LineT*, LineT*, LineT*,
+                                         LineT, void*, int*, int*, size_t*, int*);
+template bool launch_line_block_list<LineT>(int, int, int, const void*, const int*, int, int, int, size_t,
+                                            cudaStream_t);
 
 template <typename T>
 bool launch_line_block(const DevLevel<T>& L, int s, int mode, const T* g, const T* r, T* y, T* x, T alpha,
@@ -632,9 +843,7 @@ bool launch_line_block(const DevLevel<T>& L, int s, int mode, const T* g, const 
     }
 }
 
-template bool launch_line_block<float>(const DevLevel<float>&, int, int, const float*, const float*, float*, float*,
-                                       float, cudaStream_t, int);
-template bool launch_line_block<double>(const DevLevel<double>&, int, int, const double*, const double*, double*,
-                                        double*, double, cudaStream_t, int);
+template bool launch_line_block<LineT>(const DevLevel<LineT>&, int, int, const LineT*, const LineT*, LineT*, LineT*,
+                                       LineT, cudaStream_t, int);
 
 }  // namespace glls

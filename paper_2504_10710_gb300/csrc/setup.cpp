@@ -410,15 +410,23 @@ std::string line_blocks(LevelHost& lv) {
         const long long nlines = (long long)std::max(m1, 0) * std::max(m2, 0);
         const long long ntask = nlines * E;
         lv.blk[s].assign((size_t)ncoef * ntask, 0.0);
-        lv.vband[s].assign((size_t)nlines * std::max(E - 1, 0) * 2, 0.0);
+        const int nv = std::max(E - 1, 0);
+        lv.vcr[s].assign(3 * (size_t)nlines * nv, 0.0);
         SegBuilder sb{lv, s, o1, o2, p, n1, E};
         std::atomic<long long> next(0);
         std::atomic<bool> bad(false);
         auto work = [&]() {
             std::vector<double> M((size_t)E * n1 * n1), K((size_t)mi * mi);
             std::vector<double> wl((size_t)E * mi), wr((size_t)E * mi);
-            for (;;) {
-                const long long li = next.fetch_add(1);
+            std::vector<double> va(nv + 2), vl(nv + 2), vu(nv + 2);
+            // whole runs of lines per thread: neighbouring lines share the
+            // cache lines of the line-fastest arrays
+            constexpr long long kRun = 32;
+            for (long long l1 = 0, li = 0;; ++li) {
+                if (li >= l1) {
+                    li = next.fetch_add(kRun);
+                    l1 = std::min(nlines, li + kRun);
+                }
                 if (li >= nlines || bad.load()) break;
                 const int c1 = (int)(li % m1) + 1, c2 = (int)(li / m1) + 1;
                 for (int e = 0; e < E; ++e) sb.segment(c1, c2, e, &M[(size_t)e * n1 * n1]);
@@ -427,7 +435,7 @@ std::string line_blocks(LevelHost& lv) {
                     for (int i = 0; i < mi; ++i)
                         for (int j = 0; j < mi; ++j) K[i * mi + j] = Me[(i + 1) * n1 + j + 1];
                     if (!spd_inverse_small(K.data(), mi)) { bad = true; break; }
-                    const long long t = li * E + e;
+                    const long long t = s == 0 ? li * E + e : e * nlines + li;
                     int c = 0;
                     for (int i = 0; i < mi; ++i)
                         for (int j = i; j < mi; ++j) lv.blk[s][(size_t)(c++) * ntask + t] = K[i * mi + j];
@@ -460,8 +468,32 @@ std::string line_blocks(LevelHost& lv) {
                         of = Mr[0 * n1 + p];
                         for (int i = 0; i < mi; ++i) of -= Mr[0 * n1 + i + 1] * wr[(size_t)v * mi + i];
                     }
-                    lv.vband[s][((size_t)li * (E - 1) + (v - 1)) * 2 + 0] = dg;
-                    lv.vband[s][((size_t)li * (E - 1) + (v - 1)) * 2 + 1] = of;
+                    va[v] = dg;
+                    vu[v] = of;
+                    vl[v] = v > 1 ? vu[v - 1] : 0.0;
+                }
+                // cyclic reduction (Prop. 3.7 at every level): the odd multiples
+                // of h are eliminated into the even ones
+                double* out = &lv.vcr[s][(size_t)li * nv];
+                const size_t tot = (size_t)nlines * nv;
+                for (int h = 1; h <= nv; h *= 2) {
+                    for (int v = h; v <= nv; v += 2 * h) {
+                        const double ia = 1.0 / va[v];
+                        out[v - 1] = vl[v] * ia;
+                        out[tot + v - 1] = vu[v] * ia;
+                        out[2 * tot + v - 1] = ia;
+                    }
+                    for (int v = 2 * h; v <= nv; v += 2 * h) {
+                        const int a = v - h, b = v + h;
+                        double dg = va[v] - vl[v] * out[tot + a - 1], of = 0.0;
+                        if (b <= nv) {
+                            dg -= vu[v] * out[b - 1];
+                            of = -vu[v] * out[tot + b - 1];
+                        }
+                        vl[v] = -vl[v] * out[a - 1];
+                        vu[v] = of;
+                        va[v] = dg;
+                    }
                 }
             }
         };

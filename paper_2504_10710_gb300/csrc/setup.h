@@ -36,16 +36,19 @@ struct LevelHost {
     // numbered li = (c2 - 1) * (n[o1] - 2) + (c1 - 1) over the interior
     // indices c1, c2 of the other axes o1 < o2; segment e = 0 .. ne[s]-1 holds
     // the p - 1 element-interior nodes e p + 1 .. e p + p - 1 of the line, and
-    // vertex v = 1 .. ne[s]-1 is the node v p.  Task t = li * ne[s] + e.
+    // vertex v = 1 .. ne[s]-1 is the node v p.  Task t = li * ne[s] + e for
+    // x-lines (s = 0) and t = e * nlines + li for the others (neighbouring
+    // lines adjacent).
     //   blk[s]   [ncoef][ntask]: inverse of the segment's interior block K_I
     //            (upper triangle, row-major: (p-1)p/2 values), then
     //            w_L = K_I^-1 K_{I,v=e}, then w_R = K_I^-1 K_{I,v=e+1}
     //            (zero where that vertex is a boundary node)
-    //   vband[s] [nlines][ne[s]-1][2]: the Schur complement on the vertices
-    //            (tridiagonal): diagonal, coupling to the next vertex
+    //   vcr[s]   [3][nlines][ne[s]-1]: the cyclic reduction of the Schur
+    //            complement on the vertices (tridiagonal, symmetric), per
+    //            vertex at the level that eliminates it: l/a, u/a, 1/a
     int lblock = 0;
     std::vector<double> blk[3];
-    std::vector<double> vband[3];
+    std::vector<double> vcr[3];
     Band1D P[3];                  // prolongation (this level <- level-1), per axis
     Band1D R[3];                  // restriction  (this level -> level-1), per axis
 };
