@@ -16,8 +16,8 @@ __device__ __forceinline__ bool on_boundary32(int I, int J, int K, const int n[3
 
 // DOT: also sum_e x_e^T (A_e x_e) over all elements into *dot (last block).
 // Each thread owns ITEMS local nodes (t = threadIdx.x + 256 * it); its
-// geometry factors are loaded into registers before the x gather, so the two
-// global-memory latencies overlap.
+// geometry factors and D are loaded before the wait on the preceding kernel,
+// so that only the x gather's latency follows it.
 // sum_m a[m] b[m] and sum_m a[m] b[m * stride] over N terms with a (and, in
 // the first form, b) contiguous and 16-byte aligned: float4 loads, the terms
 // added in m order.
@@ -59,7 +59,7 @@ __device__ __forceinline__ float dot_cs(const float* a, const float* b) {
 template <typename T, int DIM, int P, bool DOT>
 __device__ __forceinline__ void apply_p_body(const DevLevel<T>& L, const T* __restrict__ x, T* __restrict__ y,
                                              int mask, double* dot, double* part, unsigned* ticket, int nrhs, int blk,
-                                             int nblk) {
+                                             int nblk, const double* done) {
     const int rhs = blk % nrhs, bx = blk / nrhs, nbx = nblk / nrhs;
     x += (long long)rhs * L.N;
     y += (long long)rhs * L.N;
@@ -104,6 +104,7 @@ __device__ __forceinline__ void apply_p_body(const DevLevel<T>& L, const T* __re
         if constexpr (VEC) sDT[t] = L.D[(t % N1) * N1 + t / N1];
     }
     __syncthreads();
+    if (!grid_dep_ready(done)) return;
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
         const int t = threadIdx.x + 256 * it;
@@ -197,8 +198,7 @@ template <typename T, int DIM, int P, bool DOT>
 __global__ void __launch_bounds__(256, 1) apply_p_kernel(DevLevel<T> L, const T* __restrict__ x, T* __restrict__ y,
                                                          int mask, double* dot, double* part, unsigned* ticket,
                                                          int nrhs) {
-    grid_dep_sync();
-    apply_p_body<T, DIM, P, DOT>(L, x, y, mask, dot, part, ticket, nrhs, blockIdx.x, gridDim.x);
+    apply_p_body<T, DIM, P, DOT>(L, x, y, mask, dot, part, ticket, nrhs, blockIdx.x, gridDim.x, nullptr);
 }
 
 // Work-list form: item j (its own level, vectors and partials) owns the CTAs
@@ -206,12 +206,10 @@ __global__ void __launch_bounds__(256, 1) apply_p_kernel(DevLevel<T> L, const T*
 template <typename T, int DIM, int P, bool DOT>
 __global__ void __launch_bounds__(256, 1) apply_p_list_kernel(const ApplyItem<T>* __restrict__ items,
                                                               const int* __restrict__ start, int nitems, int mask) {
-    grid_dep_sync();
     const int j = work_item(start, nitems, blockIdx.x);
     const ApplyItem<T>& it = items[j];
-    if (it.done && *it.done != 0.0) return;
     apply_p_body<T, DIM, P, DOT>(it.L, it.x, it.y, mask, nullptr, it.part, nullptr, 1, blockIdx.x - start[j],
-                                 start[j + 1] - start[j]);
+                                 start[j + 1] - start[j], it.done);
 }
 
 // Number of CTAs (= dot partials) the specialised apply launches for L.

@@ -53,7 +53,7 @@ __device__ __forceinline__ double block_sum_lean(double v, double* sv) {
 template <int P>
 __device__ __forceinline__ void apply_ff_body(const DevLevel<double>& L, const double* __restrict__ x,
                                               double* __restrict__ y, int mask, double* part, int nrhs, int blk,
-                                              int nblk) {
+                                              int nblk, const double* done) {
     const int rhs = blk % nrhs, bx = blk / nrhs, nbx = nblk / nrhs;
     x += (long long)rhs * L.N;
     y += (long long)rhs * L.N;
@@ -89,6 +89,7 @@ __device__ __forceinline__ void apply_ff_body(const DevLevel<double>& L, const d
     }
     for (int t = threadIdx.x; t < N1 * N1; t += 256) sD[t] = ff_from_double(L.D[t]);
     __syncthreads();
+    if (!grid_dep_ready(done)) return;   // G and D above are mesh data: loaded ahead of the wait
     double xd[ITEMS];
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
@@ -165,19 +166,16 @@ __device__ __forceinline__ void apply_ff_body(const DevLevel<double>& L, const d
 template <int P>
 __global__ void __launch_bounds__(256, 1) apply_ff_kernel(DevLevel<double> L, const double* __restrict__ x,
                                                           double* __restrict__ y, int mask, double* part, int nrhs) {
-    grid_dep_sync();
-    apply_ff_body<P>(L, x, y, mask, part, nrhs, blockIdx.x, gridDim.x);
+    apply_ff_body<P>(L, x, y, mask, part, nrhs, blockIdx.x, gridDim.x, nullptr);
 }
 
 // Work-list form: item j owns the CTAs [start[j], start[j + 1]).
 template <int P>
 __global__ void __launch_bounds__(256, 1) apply_ff_list_kernel(const ApplyItem<double>* __restrict__ items,
                                                                const int* __restrict__ start, int nitems, int mask) {
-    grid_dep_sync();
     const int j = work_item(start, nitems, blockIdx.x);
     const ApplyItem<double>& it = items[j];
-    if (it.done && *it.done != 0.0) return;
-    apply_ff_body<P>(it.L, it.x, it.y, mask, it.part, 1, blockIdx.x - start[j], start[j + 1] - start[j]);
+    apply_ff_body<P>(it.L, it.x, it.y, mask, it.part, 1, blockIdx.x - start[j], start[j + 1] - start[j], it.done);
 }
 
 template <int P>

@@ -39,6 +39,15 @@ __device__ __forceinline__ void grid_dep_sync() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
+// grid_dep_sync() for a CTA body that has already loaded mesh data (arrays no
+// kernel writes: geometry factors, operators, transfer bands, work-list
+// items), so that those loads overlap the end of the preceding kernel; false
+// when the work-list item's problem has stopped (done: its stop flag or null).
+__device__ __forceinline__ bool grid_dep_ready(const double* done) {
+    grid_dep_sync();
+    return !(done && *done != 0.0);
+}
+
 // False when GLLS_PDL=0 is set in the environment (plain stream order).
 bool pdl_enabled();
 

@@ -339,7 +339,7 @@ template <typename T>
 __device__ __forceinline__ void coarse_body(long long n, long long ld, const long long* __restrict__ index,
                                             const T* __restrict__ inv, const T* __restrict__ src,
                                             const long long* __restrict__ src_index, int m, int H, T* __restrict__ e,
-                                            int nrhs, long long vstride, int blk, int nblk) {
+                                            int nrhs, long long vstride, int blk, int nblk, const double* done) {
     // right-hand side fastest in the CTA order (see device.cuh); src and e
     // hold vstride values per right-hand side
     const int rhs = blk % nrhs;
@@ -348,36 +348,44 @@ __device__ __forceinline__ void coarse_body(long long n, long long ld, const lon
     e += rhs * vstride;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* rs = reinterpret_cast<T*>(smem_raw);
-    for (long long t = threadIdx.x; t < ld; t += blockDim.x) {
-        T v = T(0);
-        if (t < n) {
-            const long long q = reduced_pos(t, m, H);
-            v = src_index ? src[src_index[q]] : src[q];
-        }
-        rs[t] = v;
-    }
-    __syncthreads();
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
     const int wpb = blockDim.x / 32;
     constexpr int V = 16 / sizeof(T);   // elements per 16-byte vector
     using Vec = typename std::conditional<sizeof(T) == 4, float4, double2>::type;
     // each lane keeps U row chunks in flight (independent loads and partial
-    // sums), so a row costs about one memory latency instead of one per chunk
+    // sums), so a row costs about one memory latency instead of one per
+    // chunk; the first row's first chunks are loaded before the wait on the
+    // preceding kernel (the inverse is mesh data)
     constexpr int U = sizeof(T) == 4 ? 16 : 8;
     const long long nvec = ld / V;
-    for (long long row = bx * wpb + warp; row < n; row += nbx * wpb) {
+    Vec v[U];
+    auto fetch = [&](const Vec* a, long long j0) {
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const long long j = j0 + 32LL * u;
+            if (j < nvec) v[u] = __ldg(a + j);
+        }
+    };
+    const long long row0 = bx * wpb + warp;
+    if (row0 < n) fetch(reinterpret_cast<const Vec*>(inv + row0 * ld), lane);
+    if (!grid_dep_ready(done)) return;
+    for (long long t = threadIdx.x; t < ld; t += blockDim.x) {
+        T w = T(0);
+        if (t < n) {
+            const long long q = reduced_pos(t, m, H);
+            w = src_index ? src[src_index[q]] : src[q];
+        }
+        rs[t] = w;
+    }
+    __syncthreads();
+    for (long long row = row0; row < n; row += nbx * wpb) {
         const long long out = lane == 0 ? index[reduced_pos(row, m, H)] : 0;   // in flight with the row
         const Vec* a = reinterpret_cast<const Vec*>(inv + row * ld);
         T part[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) part[u] = T(0);
         for (long long j0 = lane; j0 < nvec; j0 += 32 * U) {
-            Vec v[U];
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                const long long j = j0 + 32LL * u;
-                if (j < nvec) v[u] = __ldg(a + j);
-            }
+            if (row != row0 || j0 != lane) fetch(a, j0);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const long long j = j0 + 32LL * u;
@@ -401,24 +409,24 @@ __global__ void __launch_bounds__(256) coarse_kernel(long long n, long long ld, 
                                                      const T* __restrict__ inv, const T* __restrict__ src,
                                                      const long long* __restrict__ src_index, int m, int H,
                                                      T* __restrict__ e, int nrhs, long long vstride) {
-    grid_dep_sync();
-    coarse_body<T>(n, ld, index, inv, src, src_index, m, H, e, nrhs, vstride, blockIdx.x, gridDim.x);
+    coarse_body<T>(n, ld, index, inv, src, src_index, m, H, e, nrhs, vstride, blockIdx.x, gridDim.x, nullptr);
 }
 
 template <typename T>
 __global__ void __launch_bounds__(256) coarse_list_kernel(const CoarseItem<T>* __restrict__ items,
                                                           const int* __restrict__ start, int nitems) {
-    grid_dep_sync();
     const int j = work_item(start, nitems, blockIdx.x);
     const CoarseItem<T>& it = items[j];
-    if (it.done && *it.done != 0.0) return;
     coarse_body<T>(it.n, it.ld, it.index, it.inv, it.src, it.src_index, it.m, it.H, it.e, 1, 0,
-                   blockIdx.x - start[j], start[j + 1] - start[j]);
+                   blockIdx.x - start[j], start[j + 1] - start[j], it.done);
 }
 
 // Rows of a block per CTA in the block-CR kernels: one per warp, so that a
 // level with few blocks still spreads over many CTAs.
 constexpr int kBcrRows = 8;
+// Row chunks of 32 columns that a warp loads ahead (blocks of up to 128
+// unknowns wholly; FP64 shares the count).
+constexpr int kBcrAhead = 4;
 
 // Block CR forward step at level l (h = 2^l), one CTA per (kept block,
 // kBcrRows rows): for kept block b = (2q + 2) h - 1,
@@ -430,7 +438,7 @@ constexpr int kBcrRows = 8;
 template <typename T>
 __device__ __forceinline__ void bcr_forward_body(const T* __restrict__ FH, int l, int nb, int m, int ldm,
                                                  const long long* __restrict__ index, const T* __restrict__ r, T* w,
-                                                 int nrhs, long long nvec, int bx, int by) {
+                                                 int nrhs, long long nvec, int bx, int by, const double* done) {
     const int rhs = bx % nrhs;
     r += rhs * nvec;
     w += rhs * nvec;
@@ -442,6 +450,7 @@ __device__ __forceinline__ void bcr_forward_body(const T* __restrict__ FH, int l
     const bool lvl0 = l == 0;
     const int q = bx / nrhs;
     if (q >= nk) {                                   // level 0: copy eliminated block 2 (q - nk)
+        if (!grid_dep_ready(done)) return;
         const long long b = 2LL * (q - nk);
         for (int rr = threadIdx.x; rr < kBcrRows; rr += blockDim.x) {
             const int row = row0 + rr;
@@ -451,33 +460,46 @@ __device__ __forceinline__ void bcr_forward_body(const T* __restrict__ FH, int l
     }
     const long long b = (2LL * q + 2) * h - 1, lb = b - h, rb = b + h;
     const bool right = rb < nb;
+    const T* F = FH + (size_t)q * 2 * m * ldm;
+    const T* Hm = F + (size_t)m * ldm;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int row = row0 + warp;                      // one row per warp
+    // the row's first kBcrAhead chunks, loaded before the wait (mesh data)
+    T f[kBcrAhead], hh[kBcrAhead];
+#pragma unroll
+    for (int u = 0; u < kBcrAhead; ++u) {
+        const int c = lane + 32 * u;
+        const bool ok = row < m && c < m;
+        f[u] = ok ? __ldg(F + (size_t)row * ldm + c) : T(0);
+        hh[u] = ok ? __ldg(Hm + (size_t)row * ldm + c) : T(0);
+    }
+    if (!grid_dep_ready(done)) return;
     for (int c = threadIdx.x; c < m; c += blockDim.x) {
         xl[c] = lvl0 ? r[index[lb * m + c]] : w[lb * m + c];
         xr[c] = right ? (lvl0 ? r[index[rb * m + c]] : w[rb * m + c]) : T(0);
     }
+    const long long o = b * m + row;
+    T own = T(0);
+    if (lane == 0 && row < m) own = lvl0 ? r[index[o]] : w[o];
     __syncthreads();
-    const T* F = FH + (size_t)q * 2 * m * ldm;
-    const T* Hm = F + (size_t)m * ldm;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int rr = warp; rr < kBcrRows; rr += 8) {
-        const int row = row0 + rr;
-        if (row >= m) break;
-        T s = T(0);
-        for (int c = lane; c < m; c += 32) s += F[(size_t)row * ldm + c] * xl[c] + Hm[(size_t)row * ldm + c] * xr[c];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-        if (lane == 0) {
-            const long long o = b * m + row;
-            w[o] = (lvl0 ? r[index[o]] : w[o]) - s;
-        }
+    if (row >= m) return;
+    T s = T(0);
+#pragma unroll
+    for (int u = 0; u < kBcrAhead; ++u) {
+        const int c = lane + 32 * u;
+        if (c < m) s += f[u] * xl[c] + hh[u] * xr[c];
     }
+    for (int c = lane + 32 * kBcrAhead; c < m; c += 32)
+        s += F[(size_t)row * ldm + c] * xl[c] + Hm[(size_t)row * ldm + c] * xr[c];
+    for (int k = 16; k > 0; k >>= 1) s += __shfl_down_sync(0xffffffffu, s, k);
+    if (lane == 0) w[o] = own - s;
 }
 
 template <typename T>
 __global__ void __launch_bounds__(256) bcr_forward_kernel(const T* __restrict__ FH, int l, int nb, int m, int ldm,
                                                           const long long* __restrict__ index,
                                                           const T* __restrict__ r, T* w, int nrhs, long long nvec) {
-    grid_dep_sync();
-    bcr_forward_body<T>(FH, l, nb, m, ldm, index, r, w, nrhs, nvec, blockIdx.x, blockIdx.y);
+    bcr_forward_body<T>(FH, l, nb, m, ldm, index, r, w, nrhs, nvec, blockIdx.x, blockIdx.y, nullptr);
 }
 
 // Block CR back substitution at level l, one CTA per (eliminated block,
@@ -488,7 +510,7 @@ __global__ void __launch_bounds__(256) bcr_forward_kernel(const T* __restrict__ 
 template <typename T>
 __device__ __forceinline__ void bcr_backward_body(const T* __restrict__ AGK, int l, int nb, int m, int ldm,
                                                   const long long* __restrict__ index, const T* __restrict__ w, T* e,
-                                                  int nrhs, long long nvec, int bx, int by) {
+                                                  int nrhs, long long nvec, int bx, int by, const double* done) {
     const int rhs = bx % nrhs;
     w += rhs * nvec;
     e += rhs * nvec;
@@ -501,35 +523,49 @@ __device__ __forceinline__ void bcr_backward_body(const T* __restrict__ AGK, int
     const long long s_ = bx / nrhs;
     const long long b = (2 * s_ + 1) * h - 1, lb = b - h, rb = b + h;
     const bool left = lb >= 0, right = rb < nb;
+    const T* Ai = AGK + (size_t)s_ * 3 * m * ldm;
+    const T* G = Ai + (size_t)m * ldm;
+    const T* K = G + (size_t)m * ldm;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int row = row0 + warp;                      // one row per warp
+    T fa[kBcrAhead], fg[kBcrAhead], fk[kBcrAhead];    // as in the forward step
+#pragma unroll
+    for (int u = 0; u < kBcrAhead; ++u) {
+        const int c = lane + 32 * u;
+        const bool ok = row < m && c < m;
+        const size_t o = (size_t)row * ldm + c;
+        fa[u] = ok ? __ldg(Ai + o) : T(0);
+        fg[u] = ok ? __ldg(G + o) : T(0);
+        fk[u] = ok ? __ldg(K + o) : T(0);
+    }
+    const long long out = row < m ? index[b * m + row] : 0;
+    if (!grid_dep_ready(done)) return;
     for (int c = threadIdx.x; c < m; c += blockDim.x) {
         xw[c] = w[b * m + c];
         xl[c] = left ? e[index[lb * m + c]] : T(0);
         xr[c] = right ? e[index[rb * m + c]] : T(0);
     }
     __syncthreads();
-    const T* Ai = AGK + (size_t)s_ * 3 * m * ldm;
-    const T* G = Ai + (size_t)m * ldm;
-    const T* K = G + (size_t)m * ldm;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    for (int rr = warp; rr < kBcrRows; rr += 8) {
-        const int row = row0 + rr;
-        if (row >= m) break;
-        T v = T(0);
-        for (int c = lane; c < m; c += 32) {
-            const size_t o = (size_t)row * ldm + c;
-            v += Ai[o] * xw[c] - G[o] * xl[c] - K[o] * xr[c];
-        }
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-        if (lane == 0) e[index[b * m + row]] = v;
+    if (row >= m) return;
+    T v = T(0);
+#pragma unroll
+    for (int u = 0; u < kBcrAhead; ++u) {
+        const int c = lane + 32 * u;
+        if (c < m) v += fa[u] * xw[c] - fg[u] * xl[c] - fk[u] * xr[c];
     }
+    for (int c = lane + 32 * kBcrAhead; c < m; c += 32) {
+        const size_t o = (size_t)row * ldm + c;
+        v += Ai[o] * xw[c] - G[o] * xl[c] - K[o] * xr[c];
+    }
+    for (int k = 16; k > 0; k >>= 1) v += __shfl_down_sync(0xffffffffu, v, k);
+    if (lane == 0) e[out] = v;
 }
 
 template <typename T>
 __global__ void __launch_bounds__(256) bcr_backward_kernel(const T* __restrict__ AGK, int l, int nb, int m, int ldm,
                                                            const long long* __restrict__ index,
                                                            const T* __restrict__ w, T* e, int nrhs, long long nvec) {
-    grid_dep_sync();
-    bcr_backward_body<T>(AGK, l, nb, m, ldm, index, w, e, nrhs, nvec, blockIdx.x, blockIdx.y);
+    bcr_backward_body<T>(AGK, l, nb, m, ldm, index, w, e, nrhs, nvec, blockIdx.x, blockIdx.y, nullptr);
 }
 
 // Work-list forms of both block-CR steps: item j owns the CTAs [start[j],
@@ -537,16 +573,14 @@ __global__ void __launch_bounds__(256) bcr_backward_kernel(const T* __restrict__
 template <typename T>
 __global__ void __launch_bounds__(256) bcr_list_kernel(const BcrItem<T>* __restrict__ items,
                                                        const int* __restrict__ start, int nitems, int l, int forward) {
-    grid_dep_sync();
     const int j = work_item(start, nitems, blockIdx.x);
     const BcrItem<T>& it = items[j];
-    if (it.done && *it.done != 0.0) return;
     const int local = blockIdx.x - start[j];
     const int bx = local % it.gx, by = local / it.gx;
     if (forward)
-        bcr_forward_body<T>(it.ops, l, it.nb, it.m, it.ldm, it.index, it.src, it.dst, 1, 0, bx, by);
+        bcr_forward_body<T>(it.ops, l, it.nb, it.m, it.ldm, it.index, it.src, it.dst, 1, 0, bx, by, it.done);
     else
-        bcr_backward_body<T>(it.ops, l, it.nb, it.m, it.ldm, it.index, it.src, it.dst, 1, 0, bx, by);
+        bcr_backward_body<T>(it.ops, l, it.nb, it.m, it.ldm, it.index, it.src, it.dst, 1, 0, bx, by, it.done);
 }
 
 // Fused two-factor transfer: a CTA of 32 x 8 threads computes a 32 x TY tile
@@ -559,7 +593,7 @@ template <typename T, int WB, int TY>
 __device__ __forceinline__ void transfer2_body(const DevBand<T>& M0, const DevBand<T>& M1, int3 nin, int3 nout,
                                                const T* __restrict__ in, const T* __restrict__ in2,
                                                T* __restrict__ out, int add, int mask, T* __restrict__ clear, int bx,
-                                               int by, int z) {
+                                               int by, int z, const double* done) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int win[4];                       // column lo, column count, row lo, row count
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -593,6 +627,7 @@ __device__ __forceinline__ void transfer2_body(const DevBand<T>& M0, const DevBa
         }
     }
     __syncthreads();
+    if (!grid_dep_ready(done)) return;            // the bands above are mesh data
     const int clo = win[0], ncol = win[1], rlo = win[2], nrow = win[3];
     T* sin = reinterpret_cast<T*>(smem_raw);      // nrow x ncol
     T* st = sin + (size_t)M1.span8 * M0.span32;   // nrow x 32
@@ -663,8 +698,8 @@ template <typename T, int WB, int TY>
 __global__ void __launch_bounds__(256) transfer2_kernel(DevBand<T> M0, DevBand<T> M1, int3 nin, int3 nout,
                                                         const T* __restrict__ in, const T* __restrict__ in2,
                                                         T* __restrict__ out, int add, int mask, T* __restrict__ clear) {
-    grid_dep_sync();
-    transfer2_body<T, WB, TY>(M0, M1, nin, nout, in, in2, out, add, mask, clear, blockIdx.x, blockIdx.y, blockIdx.z);
+    transfer2_body<T, WB, TY>(M0, M1, nin, nout, in, in2, out, add, mask, clear, blockIdx.x, blockIdx.y, blockIdx.z,
+                              nullptr);
 }
 
 // Work-list form: item j owns the CTAs [start[j], start[j + 1]), its
@@ -673,14 +708,12 @@ template <typename T, int WB, int TY>
 __global__ void __launch_bounds__(256) transfer2_list_kernel(const Transfer2Item<T>* __restrict__ items,
                                                              const int* __restrict__ start, int nitems, int add,
                                                              int mask) {
-    grid_dep_sync();
     const int j = work_item(start, nitems, blockIdx.x);
     const Transfer2Item<T>& it = items[j];
-    if (it.done && *it.done != 0.0) return;
     const int local = blockIdx.x - start[j];
     const int bx = local % it.gx, rest = local / it.gx;
     transfer2_body<T, WB, TY>(it.M0, it.M1, it.nin, it.nout, it.in, it.in2, it.out, add, mask, it.clear, bx,
-                              rest % it.gy, rest / it.gy);
+                              rest % it.gy, rest / it.gy, it.done);
 }
 
 // ---------------------------------------------------------------------------

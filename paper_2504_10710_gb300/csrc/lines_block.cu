@@ -263,13 +263,6 @@ __device__ __forceinline__ int enter(BlockLineArgs<T>& A, int blk) {
     return bx * A.lpc;
 }
 
-// Waits for the preceding kernel; false when the item's problem has stopped.
-template <typename T>
-__device__ __forceinline__ bool ready(const BlockLineArgs<T>& A) {
-    grid_dep_sync();
-    return !(A.done && *A.done != 0.0);
-}
-
 // MODE 0: x = B^-1 g.  MODE 1: x += alpha B^-1 (r - y), and y is reset to 0
 // on element-boundary nodes (the apply that produced y plain-stores element-
 // interior nodes and adds into element-boundary ones).  MODE 2: x += alpha
@@ -307,7 +300,7 @@ __device__ __forceinline__ void line_seg_body(BlockLineArgs<T>& A, int blk) {
     const int stride = CONTIG ? 1 : A.stride;
     const int c2 = li / A.m1 + 1, c1 = li - (c2 - 1) * A.m1 + 1;
     const int v0 = c1 * A.st1 + c2 * A.st2 + e * P * stride;   // the segment's left vertex
-    if (!ready(A)) return;
+    if (!grid_dep_ready(A.done)) return;
 
     T gi[MI], xi[MI], gv = T(0), xv = T(0);
     const bool vertex = act && e > 0;
@@ -446,7 +439,7 @@ __device__ __forceinline__ void line_any_body(BlockLineArgs<T>& A, int blk) {
         for (int c = 0; c < ncoef; ++c) cp_async(sop + c * opstride + tid, bp + (long long)c * ntask);
     }
     auto opc = [&](int c) { return sop[c * opstride + tid]; };   // coefficient c of this thread's segment
-    if (!ready(A)) {
+    if (!grid_dep_ready(A.done)) {
         cp_async_wait_all();
         return;
     }
