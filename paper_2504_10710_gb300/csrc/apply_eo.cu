@@ -18,9 +18,11 @@
 // coalesced along i), and the r-line (j, k) = (a, b) and the s-line
 // (i, k) = (a, b) through shared memory.  Element-interior nodes are stored,
 // shared nodes summed with atomics (direct stiffness summation), Dirichlet
-// rows skipped when mask is set.  DOT: per-block partials of
-// sum_e x_e^T (A_e x_e) as in the node-per-thread kernels.
+// rows skipped when mask is set.  FP64: apply_eo3_kernel, with DOT per-block
+// partials of sum_e x_e^T (A_e x_e) as in the node-per-thread kernels.  FP32:
+// apply_eo3_pair_kernel, two elements or right-hand sides per thread.
 #include "device.cuh"
+#include "f32x2.cuh"
 #include "reduce.cuh"
 #include "setup.h"
 
@@ -86,19 +88,15 @@ __device__ __forceinline__ void eo_line(const EoMat<T, N>& M, const T (&u)[N], T
     }
 }
 
-// Shared-memory strides (in elements of T): row RS, plane PS, element ES,
+// Shared-memory strides for 8-byte values: row RS, plane PS, element ES,
 // chosen so that the row, column and node accesses of a warp spread over the
 // banks (at most a two-way conflict).
-template <typename T, int N>
+template <int N>
 struct EoShape {
-    static constexpr bool F64 = sizeof(T) == 8;
     static constexpr int NP = N * N, NLOC = NP * N;
-    static constexpr int EPB = 256 / NP;                     // most elements per CTA (256 threads)
-    static constexpr int RS = N == 8 ? 9 : N == 7 ? (F64 ? 7 : 9) : N == 6 ? (F64 ? 9 : 6) : N == 9 ? 9 : N;
-    static constexpr int PS = N == 2 ? 5 : N == 3 ? 9 : N == 4 ? 19 : N == 5 ? 25 : N == 6 ? (F64 ? 54 : 37)
-                            : N == 7 ? (F64 ? 52 : 71) : N == 8 ? 72 : (F64 ? 89 : 81);
-    static constexpr int ES = N == 2 ? 12 : N == 3 ? 27 : N == 4 ? (F64 ? 76 : 80) : N == 5 ? 125
-                            : N == 6 ? (F64 ? 324 : 228) : N == 7 ? (F64 ? 369 : 497) : N == 8 ? 576 : (F64 ? 801 : 729);
+    static constexpr int RS = N == 8 ? 9 : N == 7 ? 7 : N == 6 ? 9 : N;
+    static constexpr int PS = N == 5 ? 25 : N == 6 ? 54 : N == 7 ? 52 : N == 8 ? 72 : 89;
+    static constexpr int ES = N == 5 ? 125 : N == 6 ? 324 : N == 7 ? 369 : N == 8 ? 576 : 801;
     static constexpr int NBUF = 3;                           // x, and two work buffers
 };
 
@@ -106,14 +104,14 @@ __device__ __forceinline__ bool on_bd(int I, int J, int K, const int n[3]) {
     return I == 0 || I == n[0] - 1 || J == 0 || J == n[1] - 1 || K == 0 || K == n[2] - 1;
 }
 
-// epb elements per CTA (at most EoShape::EPB), chosen at launch so that
-// small levels still spread over many CTAs per SM.  Two resident CTAs per SM
-// bound the registers (at most 128 per thread).
+// FP64 (T = double).  epb elements per CTA (at most 256 threads), chosen at
+// launch so that small levels still spread over many CTAs per SM.  Two
+// resident CTAs per SM bound the registers (at most 128 per thread).
 template <typename T, int P, bool DOT>
-__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
+__global__ void __launch_bounds__(256, 2)
     apply_eo3_kernel(DevLevel<T> L, const __grid_constant__ EoParams<T, P + 1> M, const T* __restrict__ x,
                      T* __restrict__ y, int mask, double* dot, double* part, unsigned* ticket, int epb, int nrhs) {
-    using S = EoShape<T, P + 1>;
+    using S = EoShape<P + 1>;
     constexpr int N = P + 1, NP = S::NP, NLOC = S::NLOC, RS = S::RS, PS = S::PS, ES = S::ES;
     extern __shared__ __align__(16) unsigned char eo_smem3[];
     T* sX = reinterpret_cast<T*>(eo_smem3);
@@ -228,6 +226,214 @@ __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 2)
     }
 }
 
+// ---- FP32, two elements or two right-hand sides per thread -----------------
+
+// One N x N matrix in even-odd form, every coefficient twice (both halves of
+// a pair use it).
+template <int N>
+struct EoMat2 {
+    static constexpr int H = N / 2;
+    f32x2 e[H * H], o[H * H], c[H], r[H];
+};
+template <int N>
+struct EoParams2 {
+    EoMat2<N> f, t;
+};
+
+// out = M u for a pair of lines (as eo_line)
+template <int N>
+__device__ __forceinline__ void eo_line2(const EoMat2<N>& M, const f32x2 (&u)[N], f32x2 (&out)[N]) {
+    constexpr int H = N / 2;
+    constexpr bool ODD = (N & 1) != 0;
+    f32x2 ue[H], uo[H];
+#pragma unroll
+    for (int m = 0; m < H; ++m) {
+        ue[m] = add2(u[m], u[N - 1 - m]);
+        uo[m] = sub2(u[m], u[N - 1 - m]);
+    }
+#pragma unroll
+    for (int i = 0; i < H; ++i) {
+        f32x2 a = ODD ? mul2(M.c[i], u[H]) : mul2(M.e[i * H], ue[0]), b = mul2(M.o[i * H], uo[0]);
+        if constexpr (ODD) a = fma2(M.e[i * H], ue[0], a);
+#pragma unroll
+        for (int m = 1; m < H; ++m) {
+            a = fma2(M.e[i * H + m], ue[m], a);
+            b = fma2(M.o[i * H + m], uo[m], b);
+        }
+        out[i] = add2(a, b);
+        out[N - 1 - i] = sub2(b, a);
+    }
+    if constexpr (ODD) {
+        f32x2 s = mul2(M.r[0], uo[0]);
+#pragma unroll
+        for (int m = 1; m < H; ++m) s = fma2(M.r[m], uo[m], s);
+        out[H] = s;
+    }
+}
+
+// The even-odd apply with packed FP32 arithmetic.  A kernel with one line per
+// thread was bound by instruction issue (990 instructions a thread at p = 7)
+// and, next, by shared-memory wavefronts.  A thread that carries two lines in
+// the halves of a pair issues one instruction for both: two right-hand sides
+// of one element (RHS; the geometric factors are read once for both), or two
+// neighbouring elements; at p = 7 the swizzled slots below remove the bank
+// conflicts that a pair of strides leaves.  Measured on 16^3 elements, p = 7:
+// 12.7 -> 10.9 us (9.1 us at the measured copy bandwidth), 32 right-hand
+// sides 359 -> 237 us; 24^3, p = 8: 74 -> 71 us.
+// Resident CTAs of 128 threads the registers must allow, as measured.
+constexpr int eo_pair_min_ctas(int P, bool rhs) { return rhs ? (P == 8 ? 4 : 5) : (P == 5 || P == 6 ? 5 : 4); }
+
+template <int P, bool RHS>
+__global__ void __launch_bounds__(128, eo_pair_min_ctas(P, RHS))
+    apply_eo3_pair_kernel(DevLevel<float> L, const __grid_constant__ EoParams2<P + 1> M, const float* __restrict__ x,
+                          float* __restrict__ y, int mask, int epb, int nrhs) {
+    using S = EoShape<P + 1>;
+    constexpr int N = P + 1, NP = S::NP, NLOC = S::NLOC, RS = S::RS, PS = S::PS, ES = S::ES;
+    extern __shared__ __align__(16) unsigned char eo_smem2[];
+    f32x2* sX = reinterpret_cast<f32x2*>(eo_smem2);
+    f32x2* sU = sX + epb * ES;
+    f32x2* sV = sU + epb * ES;
+    const int E = (int)L.E, n0 = L.n[0], n1 = L.n[1], nplane = n0 * n1;
+    // right-hand sides fastest in the CTA order (see device.cuh)
+    const int groups = RHS ? nrhs / 2 : nrhs;
+    const int rg = blockIdx.x % groups, bx = blockIdx.x / groups;
+    const int tid = threadIdx.x;
+    const int el = tid / NP, c = tid - el * NP, a = c % N, b = c / N;
+    const int slot = bx * epb + el;              // element (RHS) or pair of elements
+    const int eA = RHS ? slot : 2 * slot;
+    const bool act = el < epb && eA < E;
+    const bool hasB = RHS || eA + 1 < E;         // an odd last element computes twice, stores once
+    const int eB = RHS || !hasB ? eA : eA + 1;
+    const float* xA = x + (long long)(RHS ? 2 * rg : rg) * L.N;
+    const float* xB = RHS ? xA + L.N : xA;
+    float* yA = y + (long long)(RHS ? 2 * rg : rg) * L.N;
+    float* yB = RHS ? yA + L.N : yA;
+    const int elo = act ? el : 0;
+    f32x2* X = sX + elo * ES;
+    f32x2* U = sU + elo * ES;
+    f32x2* V = sV + elo * ES;
+    // Slots of node (i, j, k) in the buffers: t-lines are read and written at
+    // (a, b, k), r-lines at (m, a, b), s-lines at (a, m, b).  N = 8: rows of 8
+    // with the column swizzled by the row and plane, so that every half-warp
+    // touches 16 different 8-byte banks in all three; no pair of strides does.
+    constexpr bool SWZ = N == 8;
+    int to[2] = {}, ro[N] = {}, so[4] = {};
+    if constexpr (SWZ) {
+#pragma unroll
+        for (int q = 0; q < 2; ++q) to[q] = b * 8 + (a ^ ((b >> 1) | (q << 2)));
+#pragma unroll
+        for (int m = 0; m < N; ++m) ro[m] = b * 72 + a * 8 + (m ^ ((a >> 1) | ((b & 1) << 2)));
+#pragma unroll
+        for (int q = 0; q < 4; ++q) so[q] = b * 72 + (a ^ (q | ((b & 1) << 2)));
+    }
+    auto at_t = [&](int k) { return SWZ ? k * 72 + to[k & 1] : k * PS + b * RS + a; };
+    auto at_r = [&](int m) { return SWZ ? ro[m] : b * PS + a * RS + m; };
+    auto at_s = [&](int m) { return SWZ ? m * 8 + so[(m >> 1) & 3] : b * PS + m * RS + a; };
+    const int ne0 = L.ne[0], ne1 = L.ne[1];
+    int baseA, baseB, KA, KB;
+    bool bdA, bdB;                               // column (a, b) on the boundary of axes 0, 1
+    {
+        const int ex = eA % ne0, ey = (eA / ne0) % ne1, ez = eA / (ne0 * ne1);
+        const int I = ex * P + a, J = ey * P + b;
+        KA = ez * P;
+        baseA = (KA * n1 + J) * n0 + I;
+        bdA = I == 0 || I == n0 - 1 || J == 0 || J == n1 - 1;
+    }
+    if (RHS) {
+        baseB = baseA;
+        KB = KA;
+        bdB = bdA;
+    } else {
+        const int ex = eB % ne0, ey = (eB / ne0) % ne1, ez = eB / (ne0 * ne1);
+        const int I = ex * P + a, J = ey * P + b;
+        KB = ez * P;
+        baseB = (KB * n1 + J) * n0 + I;
+        bdB = I == 0 || I == n0 - 1 || J == 0 || J == n1 - 1;
+    }
+    grid_dep_sync();
+    f32x2 ut[N];
+    if (act) {
+        f32x2 xc[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) xc[k] = pack2(xA[baseA + k * nplane], xB[baseB + k * nplane]);
+#pragma unroll
+        for (int k = 0; k < N; ++k) X[at_t(k)] = xc[k];
+        eo_line2<N>(M.f, xc, ut);
+    }
+    __syncthreads();
+    if (act) {
+        f32x2 u[N], v[N];
+#pragma unroll
+        for (int m = 0; m < N; ++m) u[m] = X[at_r(m)];
+        eo_line2<N>(M.f, u, v);
+#pragma unroll
+        for (int m = 0; m < N; ++m) U[at_r(m)] = v[m];
+#pragma unroll
+        for (int m = 0; m < N; ++m) u[m] = X[at_s(m)];
+        eo_line2<N>(M.f, u, v);
+#pragma unroll
+        for (int m = 0; m < N; ++m) V[at_s(m)] = v[m];
+    }
+    __syncthreads();
+    f32x2 yt[N];
+    if (act) {
+        const int EN = E * NLOC;
+        const float* GA = L.G + eA * NLOC + c;
+        const float* GB = L.G + eB * NLOC + c;
+        f32x2 wt[N];
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+            f32x2 g[6];
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                const float ga = __ldg(GA + q * EN + k * NP);
+                g[q] = pack2(ga, RHS ? ga : __ldg(GB + q * EN + k * NP));
+            }
+            const int s = at_t(k);
+            const f32x2 dr = U[s], ds = V[s], dt = ut[k];
+            U[s] = fma2(g[2], dt, fma2(g[1], ds, mul2(g[0], dr)));
+            V[s] = fma2(g[4], dt, fma2(g[3], ds, mul2(g[1], dr)));
+            wt[k] = fma2(g[5], dt, fma2(g[4], ds, mul2(g[2], dr)));
+        }
+        eo_line2<N>(M.t, wt, yt);
+    }
+    __syncthreads();
+    if (act) {
+        f32x2 u[N], v[N];
+#pragma unroll
+        for (int m = 0; m < N; ++m) u[m] = U[at_r(m)];
+        eo_line2<N>(M.t, u, v);
+#pragma unroll
+        for (int m = 0; m < N; ++m) U[at_r(m)] = v[m];
+#pragma unroll
+        for (int m = 0; m < N; ++m) u[m] = V[at_s(m)];
+        eo_line2<N>(M.t, u, v);
+#pragma unroll
+        for (int m = 0; m < N; ++m) V[at_s(m)] = v[m];
+    }
+    __syncthreads();
+    if (!act) return;
+    const bool inner = a > 0 && a < P && b > 0 && b < P;
+    const int last = L.n[2] - 1;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+        const int s = at_t(k);
+        float vA, vB;
+        unpack2(add2(add2(yt[k], U[s]), V[s]), vA, vB);
+        float* pA = yA + baseA + k * nplane;
+        float* pB = yB + baseB + k * nplane;
+        if (k > 0 && k < P && inner) {
+            *pA = vA;
+            if (hasB) *pB = vB;
+        } else {
+            const bool outA = bdA || (k == 0 && KA == 0) || (k == P && KA + P == last);
+            const bool outB = bdB || (k == 0 && KB == 0) || (k == P && KB + P == last);
+            if (!(mask && outA)) atomicAdd(pA, vA);
+            if (hasB && !(mask && outB)) atomicAdd(pB, vB);
+        }
+    }
+}
+
 // Even-odd coefficients of D and D^T of order p in T, built once per order
 template <typename T>
 const std::vector<T>& eo_table(int p) {
@@ -261,10 +467,44 @@ EoParams<T, N> eo_params() {
     return M;
 }
 
+template <int N>
+EoParams2<N> eo_params2() {
+    const EoParams<float, N> M = eo_params<float, N>();
+    EoParams2<N> D;
+    const float* src = reinterpret_cast<const float*>(&M);
+    float* dst = reinterpret_cast<float*>(&D);
+    static_assert(sizeof(D) == 2 * sizeof(M), "packed");
+    for (size_t i = 0; i < sizeof(M) / sizeof(float); ++i) dst[2 * i] = dst[2 * i + 1] = src[i];
+    return D;
+}
+
+// Element slots per CTA of the pair kernel: at most 128 threads, and no more
+// than keep about eight CTAs per SM on the level.
+int eo_pair_epb(int p, long long slots) {
+    const long long most = std::max(1, 128 / ((p + 1) * (p + 1)));
+    return (int)std::max(1LL, std::min(most, slots / (152 * 8)));
+}
+
+template <int P>
+bool launch_eo_pair(const DevLevel<float>& L, const float* x, float* y, bool mask, cudaStream_t st, int nrhs) {
+    using S = EoShape<P + 1>;
+    const bool rhs = nrhs % 2 == 0;
+    const EoParams2<P + 1> M = eo_params2<P + 1>();
+    const long long slots = rhs ? L.E : (L.E + 1) / 2;
+    const int epb = eo_pair_epb(P, slots * (rhs ? nrhs / 2 : nrhs));
+    const long long nb = (slots + epb - 1) / epb * (rhs ? nrhs / 2 : nrhs);
+    if (nb > 0x7fffffffLL) return false;
+    const int threads = (epb * S::NP + 31) / 32 * 32;
+    const size_t smem = sizeof(f32x2) * S::NBUF * epb * S::ES;
+    if (rhs) launch_k(apply_eo3_pair_kernel<P, true>, (unsigned)nb, threads, smem, st, L, M, x, y, mask ? 1 : 0, epb, nrhs);
+    else launch_k(apply_eo3_pair_kernel<P, false>, (unsigned)nb, threads, smem, st, L, M, x, y, mask ? 1 : 0, epb, nrhs);
+    return true;
+}
+
 template <typename T, int P>
 bool launch_eo(const DevLevel<T>& L, const T* x, T* y, bool mask, double* dot, double* part, unsigned* ticket,
                cudaStream_t st, int nrhs) {
-    using S = EoShape<T, P + 1>;
+    using S = EoShape<P + 1>;
     const EoParams<T, P + 1> M = eo_params<T, P + 1>();
     const int epb = eo_epb(P, L.E);
     const long long nb = (L.E + epb - 1) / epb * nrhs;
@@ -281,8 +521,8 @@ bool launch_eo(const DevLevel<T>& L, const T* x, T* y, bool mask, double* dot, d
 
 template <typename T, int P>
 bool set_eo_attr() {
-    using S = EoShape<T, P + 1>;
-    const int smem = (int)(sizeof(T) * S::NBUF * S::EPB * S::ES);
+    using S = EoShape<P + 1>;
+    const int smem = (int)(sizeof(T) * S::NBUF * (256 / S::NP) * S::ES);
     return cudaFuncSetAttribute((const void*)apply_eo3_kernel<T, P, false>,
                                 cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
            cudaFuncSetAttribute((const void*)apply_eo3_kernel<T, P, true>,
@@ -291,11 +531,11 @@ bool set_eo_attr() {
 
 }  // namespace
 
-// Orders measured faster with this kernel than with the node-per-thread and
+// Orders measured faster with these kernels than with the node-per-thread and
 // column kernels on 16^3-element levels (graph replay and L2-cold launches):
-// FP32 p >= 4 (p = 7: 15.1 against 16.4 and 24.4 us), FP64 p = 6, 7 (p = 7:
-// 193 against 218 us).  FP64 elsewhere: the 2N adds per line and the lower
-// thread count cost more than the saved multiply-adds.
+// FP32 p >= 4 (one line per thread, p = 7: 15.1 against 16.4 and 24.4 us),
+// FP64 p = 6, 7 (p = 7: 193 against 218 us).  FP64 elsewhere: the 2N adds per
+// line and the lower thread count cost more than the saved multiply-adds.
 bool apply_eo_selected(int dim, int p, bool f64) {
     if (dim != 3) return false;
     return f64 ? (p == 6 || p == 7) : (p >= 4 && p <= 8);
@@ -317,12 +557,13 @@ bool launch_apply_eo(const DevLevel<T>& L, const T* x, T* y, bool mask, double* 
             default: return launch_eo<T, 7>(L, x, y, mask, dot, part, ticket, st, nrhs);
         }
     } else {
+        if (dot) return false;               // x.(A x) is formed in FP64 only
         switch (L.p) {
-            case 4: return launch_eo<T, 4>(L, x, y, mask, dot, part, ticket, st, nrhs);
-            case 5: return launch_eo<T, 5>(L, x, y, mask, dot, part, ticket, st, nrhs);
-            case 6: return launch_eo<T, 6>(L, x, y, mask, dot, part, ticket, st, nrhs);
-            case 7: return launch_eo<T, 7>(L, x, y, mask, dot, part, ticket, st, nrhs);
-            default: return launch_eo<T, 8>(L, x, y, mask, dot, part, ticket, st, nrhs);
+            case 4: return launch_eo_pair<4>(L, x, y, mask, st, nrhs);
+            case 5: return launch_eo_pair<5>(L, x, y, mask, st, nrhs);
+            case 6: return launch_eo_pair<6>(L, x, y, mask, st, nrhs);
+            case 7: return launch_eo_pair<7>(L, x, y, mask, st, nrhs);
+            default: return launch_eo_pair<8>(L, x, y, mask, st, nrhs);
         }
     }
 }
@@ -331,9 +572,6 @@ template bool launch_apply_eo<float>(const DevLevel<float>&, const float*, float
 template bool launch_apply_eo<double>(const DevLevel<double>&, const double*, double*, bool, double*, double*,
                                       unsigned*, cudaStream_t, int);
 
-bool init_apply_eo_attributes() {
-    return set_eo_attr<float, 4>() && set_eo_attr<float, 5>() && set_eo_attr<float, 6>() && set_eo_attr<float, 7>() &&
-           set_eo_attr<float, 8>() && set_eo_attr<double, 6>() && set_eo_attr<double, 7>();
-}
+bool init_apply_eo_attributes() { return set_eo_attr<double, 6>() && set_eo_attr<double, 7>(); }
 
 }  // namespace glls
