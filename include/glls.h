@@ -96,17 +96,20 @@ enum { GLLS_COARSE_AUTO = 0, GLLS_COARSE_DENSE = 1, GLLS_COARSE_BLOCK_CR = 2 };
  *   ATOMIC   one launch; nodes shared by elements are accumulated with atomic
  *            adds, so their summation order, and with it the last bits of an
  *            FP32 or FP64 result, follows the GPU's scheduling.
- *   COLORED  one launch per element colour (the 2^dim parity classes of the
- *            element coordinates, no two elements of a class share a node)
- *            in a fixed order: every shared node sums its contributions in the
- *            same order on every run.  A solve is then the same bits alone, in
- *            a graph-branch batch and in the serving loop, at the cost of the
- *            node-per-thread apply kernel (not the specialised ones) and 2^dim
- *            launches per apply.  A multi-right-hand-side solve gives each
- *            right-hand side the bits of its single solve (every kernel does
- *            the same arithmetic per right-hand side), so grouped requests in
- *            the serving loop keep them too.  Work-list batches refuse such
- *            problems. */
+ *   COLORED  a fixed order on every run: inside solves, cycles and smoothing
+ *            steps the element results go to a scratch array of the instance
+ *            and a second launch adds each node's contributions in element
+ *            order; the single applies (glls_apply, glls_apply_multi,
+ *            glls_apply_partials) and orders outside the specialised kernels
+ *            run one launch per element colour (the 2^dim parity classes of
+ *            the element coordinates, no two elements of a class share a
+ *            node).  A solve is then the same bits alone, in a graph-branch
+ *            batch and in the serving loop, at the cost of the scratch (one
+ *            value per element node, level and precision) and its traffic.  A
+ *            multi-right-hand-side solve gives each right-hand side the bits
+ *            of its single solve (every kernel does the same arithmetic per
+ *            right-hand side), so grouped requests in the serving loop keep
+ *            them too.  Work-list batches refuse such problems. */
 enum { GLLS_SUM_ATOMIC = 0, GLLS_SUM_COLORED = 1 };
 
 typedef struct glls_problem glls_problem;   /* opaque, library-owned */

@@ -84,6 +84,7 @@ struct LevelStore {
     T* y = nullptr;    // A x scratch
     T* t1 = nullptr;   // transfer temporaries
     T* t2 = nullptr;
+    T* loc = nullptr;  // element results of the applies (fixed-order summation only)
 };
 
 }  // namespace
@@ -188,6 +189,7 @@ glls_status alloc_level_vectors(glls_problem* P, std::vector<LevelStore<T>>& Ls)
         CK(P->alloc(&s.y, n));
         CK(P->alloc(&s.t1, n));
         CK(P->alloc(&s.t2, n));
+        if (s.dev.colored) CK(P->alloc(&s.loc, (size_t)s.dev.E * s.dev.nloc * P->nrhs));
         CK(cudaMemset(s.r, 0, sizeof(T) * n));
         CK(cudaMemset(s.x, 0, sizeof(T) * n));
         CK(cudaMemset(s.y, 0, sizeof(T) * n));
@@ -240,7 +242,8 @@ int band_span(const Band1D& b, int tile) {
 }
 
 template <typename T>
-glls_status upload_levels(glls_problem* P, const std::vector<LevelHost>& H, std::vector<LevelStore<T>>& out) {
+glls_status upload_levels(glls_problem* P, const std::vector<LevelHost>& H, bool colored,
+                          std::vector<LevelStore<T>>& out) {
     out.assign(H.size(), LevelStore<T>());
     for (size_t l = 0; l < H.size(); ++l) {
         const LevelHost& h = H[l];
@@ -254,6 +257,7 @@ glls_status upload_levels(glls_problem* P, const std::vector<LevelHost>& H, std:
         for (int a = 0; a < 3; ++a) { d.ne[a] = h.ne[a]; d.n[a] = h.n[a]; }
         d.N = h.N;
         d.E = h.E;
+        d.colored = colored;
         CK(P->upload(&d.G, h.G));
         CK(P->upload(&d.D, h.D));
         CK(P->upload(&d.diag, h.diag));
@@ -410,7 +414,7 @@ void smooth(glls_problem* P, int l, int s, T alpha, const T* r, T* x, bool x_is_
     if (x_is_zero) {
         launch_line_solve<T>(Ls[l].dev, s, 3, nullptr, r, nullptr, x, alpha, st, nrhs);
     } else {
-        launch_apply<T>(Ls[l].dev, x, Ls[l].y, true, st, true, nullptr, nullptr, nullptr, nrhs);
+        launch_apply<T>(Ls[l].dev, x, Ls[l].y, true, st, true, nullptr, nullptr, nullptr, nrhs, Ls[l].loc);
         launch_line_solve<T>(Ls[l].dev, s, 1, nullptr, r, Ls[l].y, x, alpha, st, nrhs);
     }
 }
@@ -432,7 +436,7 @@ void cycle(glls_problem* P, int l, const T* r, T* x, int gamma, int m, T alpha, 
             zero = false;
         }
     for (int g = 0; g < gamma; ++g) {
-        launch_apply<T>(Ls[l].dev, x, Ls[l].y, true, st, true, nullptr, nullptr, nullptr, nrhs);
+        launch_apply<T>(Ls[l].dev, x, Ls[l].y, true, st, true, nullptr, nullptr, nullptr, nrhs, Ls[l].loc);
         restrict_residual<T>(P, l, r, Ls[l].y, Ls[l - 1].r, st, nrhs);
         cycle<T>(P, l - 1, Ls[l - 1].r, Ls[l - 1].x, gamma, m, alpha, st, nrhs);
         prolong_add<T>(P, l, Ls[l - 1].x, x, st, Ls[l].y, nrhs);
@@ -462,8 +466,9 @@ glls_status check_opts(const glls_solve_opts* o) {
     return GLLS_OK;
 }
 
-// Dot partials written by launch_apply for L (coloured summation runs the
-// node-per-thread kernel and a separate dot over kDotBlocks CTAs).
+// Dot partials written by launch_apply for L without scratch (fixed-order
+// summation then runs the colour launches and a separate dot over kDotBlocks
+// CTAs).
 static int dot_partials_of(const DevLevel<double>& L) {
     return L.colored ? kDotBlocks : apply_dot_partials<double>(L);
 }
@@ -493,12 +498,13 @@ void outer_iteration(glls_problem* P, const glls_solve_opts* o, cudaStream_t st)
     // mixed precision: q = A p in float-float arithmetic where the level allows
     // it (apply_ff.cu), else in FP64
     const bool ff = mixed && o->tol >= kFfMinTol && apply_ff_supported(P->L64[L].dev);
-    const int npq = ff ? apply_ff_partials(P->L64[L].dev) : dot_partials_of(P->L64[L].dev);
+    const int npq = ff ? apply_ff_partials(P->L64[L].dev) : apply_dot_partials<double>(P->L64[L].dev);
     launch_dots_rz_zq(P->rk, P->zk, mixed ? P->z32 : nullptr, P->qk, N, prz, pzq, st, k);
     const int nb = fcg_blocks(N);            // the dots' CTAs: partials of r.z, z.q, r.r per right-hand side
     launch_fcg_direction(P->pk, P->zk, N, prz, pzq, nb, P->S, o->krylov == GLLS_KRYLOV_FCG ? 1 : 0, st, k);
     if (ff) launch_apply_ff(P->L64[L].dev, P->pk, P->qk, true, ppq, st, k);
-    else launch_apply<double>(P->L64[L].dev, P->pk, P->qk, true, st, true, P->S + S_PQ, ppq, nullptr, k);
+    else launch_apply<double>(P->L64[L].dev, P->pk, P->qk, true, st, true, P->S + S_PQ, ppq, nullptr, k,
+                              P->L64[L].loc);
     launch_fcg_update(P->xk, P->rk, P->pk, P->qk, N, ppq, npq, prz, nb, prr, P->S, P->ticket,
                       mixed ? P->r32 : nullptr, st, k);
 }
@@ -511,7 +517,7 @@ void solve_prologue(glls_problem* P, const glls_solve_opts* o, cudaStream_t st) 
     const int L = (int)P->L64.size() - 1;
     const DevLevel<double>& F = P->L64[L].dev;
     launch_boundary_only(P->g, P->v, F.n, F.dim, st);
-    launch_apply<double>(F, P->v, P->yk, false, st);
+    launch_apply<double>(F, P->v, P->yk, false, st, false, nullptr, nullptr, nullptr, 1, P->L64[L].loc);
     launch_lift_rhs(P->mass, P->f, P->yk, P->f0, F.n, F.dim, st, P->nrhs);
     cudaMemsetAsync(P->xk, 0, sizeof(double) * NK, st);
     cudaMemsetAsync(P->pk, 0, sizeof(double) * NK, st);
@@ -795,7 +801,7 @@ glls_status gmres_solve(glls_problem* P, const glls_solve_opts* o, cudaStream_t 
         } else {
             cycle<double>(P, L, vk, zk, o->gamma, o->m, o->alpha, st);
         }
-        launch_apply<double>(F, zk, w, true, st);
+        launch_apply<double>(F, zk, w, true, st, false, nullptr, nullptr, nullptr, 1, P->L64[L].loc);
         for (int pass = 0; pass < 2; ++pass) {
             launch_multidot(P->gV, N, k + 1, w, N, P->gpart, P->gh + pass * (m + 1), P->ticket, st);
             launch_gs_update(w, P->gV, N, k + 1, P->gh + pass * (m + 1), N, -1.0, st);
@@ -1541,12 +1547,11 @@ static glls_status problem_create(const glls_mesh_desc* desc, int nrhs, glls_pro
     P->setup_phase_ms[4] = std::chrono::duration<double, std::milli>(t_upload - t_coarse).count();
 
     std::lock_guard<std::recursive_mutex> dev_lock(g_device_mutex);
-    glls_status st = upload_levels<double>(P.get(), H, P->L64);
+    const bool colored = desc->summation == GLLS_SUM_COLORED;
+    glls_status st = upload_levels<double>(P.get(), H, colored, P->L64);
     if (st != GLLS_OK) return st;
-    st = upload_levels<float>(P.get(), H, P->L32);
+    st = upload_levels<float>(P.get(), H, colored, P->L32);
     if (st != GLLS_OK) return st;
-    for (auto& l : P->L64) l.dev.colored = desc->summation == GLLS_SUM_COLORED;
-    for (auto& l : P->L32) l.dev.colored = desc->summation == GLLS_SUM_COLORED;
     {
         // float-float outer apply: the FP32 rounding remainders of the finest
         // level's FP64 geometric factors (the FP32 level holds the rounded
@@ -1711,7 +1716,7 @@ glls_status glls_lift_f64(glls_problem* P, const double* f, const double* g, dou
     const int L = (int)P->L64.size() - 1;
     const DevLevel<double>& F = P->L64[L].dev;
     launch_boundary_only(g, P->v, F.n, F.dim, st);
-    launch_apply<double>(F, P->v, P->yk, false, st);
+    launch_apply<double>(F, P->v, P->yk, false, st, false, nullptr, nullptr, nullptr, 1, P->L64[L].loc);
     launch_lift_rhs(P->mass, f, P->yk, f0, F.n, F.dim, st);
     CK(cudaGetLastError());
     return GLLS_OK;
@@ -1881,6 +1886,7 @@ glls_status glls_estimate_bytes(const glls_mesh_desc* desc, size_t* bytes) {
         // vectors in each precision; transfer bands
         total += 12.0 * ((double)ncomp * E * nloc + (1 + d) * (double)N + (p + 1) * (p + 1)) + 12.0 * 5 * N;
         total += 24.0 * d * (double)N;
+        if (desc->summation == GLLS_SUM_COLORED) total += 12.0 * E * nloc;   // element results, both precisions
         if (c == 0 && p >= 2 && p <= (d == 2 ? 16 : 8)) total += 4.0 * ncomp * E * nloc;   // float-float G remainders
         total += 2.0 * d * (12.0 * (2 * p + 2) * (double)(ne[0] * p + 1) + 4.0 * (ne[0] * p + 1));
         if (desc->smoother == GLLS_SMOOTHER_GLL && p >= 2) {
@@ -2226,7 +2232,8 @@ glls_status glls_apply_partials_ff(glls_problem* P, int level, const double* x, 
         DeviceScope scope(P->device);                                                                           \
         CK(scope.err);                                                                                          \
         auto& Ls = levels_of<T>(P);                                                                             \
-        launch_apply<T>(Ls[level].dev, x, Ls[level].y, true, (cudaStream_t)stream, true);                       \
+        launch_apply<T>(Ls[level].dev, x, Ls[level].y, true, (cudaStream_t)stream, true, nullptr, nullptr,      \
+                        nullptr, 1, Ls[level].loc);                                                             \
         restrict_residual<T>(P, level, r, Ls[level].y, rc, (cudaStream_t)stream);                               \
         CK(cudaMemsetAsync(Ls[level].y, 0, sizeof(T) * Ls[level].dev.N, (cudaStream_t)stream));                 \
         CK(cudaGetLastError());                                                                                 \

@@ -56,13 +56,14 @@ __device__ __forceinline__ float dot_cs(const float* a, const float* b) {
 // 0.5-1 % slower than the 48 registers the compiler picks with one.)
 // The CTA body: block `blk` of `nblk` (per right-hand side: the right-hand
 // side fastest in the CTA order, see device.cuh).
-template <typename T, int DIM, int P, bool DOT>
+template <typename T, int DIM, int P, bool DOT, bool LOC>
 __device__ __forceinline__ void apply_p_body(const DevLevel<T>& L, const T* __restrict__ x, T* __restrict__ y,
                                              int mask, double* dot, double* part, unsigned* ticket, int nrhs, int blk,
-                                             int nblk, const double* done) {
+                                             int nblk, const double* done, T* loc) {
     const int rhs = blk % nrhs, bx = blk / nrhs, nbx = nblk / nrhs;
     x += (long long)rhs * L.N;
     y += (long long)rhs * L.N;
+    if constexpr (LOC) loc += (long long)rhs * L.E * L.nloc;
     constexpr int N1 = P + 1;
     constexpr int NLOC = DIM == 2 ? N1 * N1 : N1 * N1 * N1;
     constexpr int EPB = NLOC >= 256 ? 1 : 256 / NLOC;
@@ -173,6 +174,10 @@ __device__ __forceinline__ void apply_p_body(const DevLevel<T>& L, const T* __re
         const int I = (exyz & 1023) * P + i, J = ((exyz >> 10) & 1023) * P + j, K = (exyz >> 20) * P + k;
         const int g = sbase[el] + (k * n1 + j) * n0 + i;
         if (DOT) local += (double)sx[t] * (double)v;
+        if constexpr (LOC) {             // element values; summed by gather_kernel in a fixed order
+            loc[e0 * NLOC + t] = v;
+            continue;
+        }
         const bool inner = i > 0 && i < P && j > 0 && j < P && (DIM == 2 || (k > 0 && k < P));
         if (inner) {
             y[g] = v;
@@ -194,11 +199,12 @@ __device__ __forceinline__ void apply_p_body(const DevLevel<T>& L, const T* __re
     }
 }
 
-template <typename T, int DIM, int P, bool DOT>
+template <typename T, int DIM, int P, bool DOT, bool LOC>
 __global__ void __launch_bounds__(256, 1) apply_p_kernel(DevLevel<T> L, const T* __restrict__ x, T* __restrict__ y,
                                                          int mask, double* dot, double* part, unsigned* ticket,
-                                                         int nrhs) {
-    apply_p_body<T, DIM, P, DOT>(L, x, y, mask, dot, part, ticket, nrhs, blockIdx.x, gridDim.x, nullptr);
+                                                         int nrhs, T* loc) {
+    apply_p_body<T, DIM, P, DOT, LOC>(L, x, y, mask, dot, part, ticket, nrhs, blockIdx.x, gridDim.x, nullptr,
+                                 loc);
 }
 
 // Work-list form: item j (its own level, vectors and partials) owns the CTAs
@@ -208,8 +214,8 @@ __global__ void __launch_bounds__(256, 1) apply_p_list_kernel(const ApplyItem<T>
                                                               const int* __restrict__ start, int nitems, int mask) {
     const int j = work_item(start, nitems, blockIdx.x);
     const ApplyItem<T>& it = items[j];
-    apply_p_body<T, DIM, P, DOT>(it.L, it.x, it.y, mask, nullptr, it.part, nullptr, 1, blockIdx.x - start[j],
-                                 start[j + 1] - start[j], it.done);
+    apply_p_body<T, DIM, P, DOT, false>(it.L, it.x, it.y, mask, nullptr, it.part, nullptr, 1, blockIdx.x - start[j],
+                                 start[j + 1] - start[j], it.done, nullptr);
 }
 
 // Number of CTAs (= dot partials) the specialised apply launches for L.
@@ -223,30 +229,36 @@ int apply_blocks(const DevLevel<T>& L) {
 
 template <typename T, int DIM, int P>
 bool launch_p(const DevLevel<T>& L, const T* x, T* y, bool mask, double* dot, double* part, unsigned* ticket,
-              cudaStream_t st, int nrhs) {
+              cudaStream_t st, int nrhs, T* loc) {
     constexpr int N1 = P + 1;
     constexpr int NLOC = DIM == 2 ? N1 * N1 : N1 * N1 * N1;
     constexpr int EPB = NLOC >= 256 ? 1 : 256 / NLOC;
     const long long blocks = (L.E + EPB - 1) / EPB * nrhs;
     if (blocks > 0x7fffffffLL) return false;
-    if (dot) {
-        launch_k(apply_p_kernel<T, DIM, P, true>, (unsigned)blocks, 256, 0, st, L, x, y, mask ? 1 : 0, dot, part,
-                 ticket, nrhs);
-    } else {
-        launch_k(apply_p_kernel<T, DIM, P, false>, (unsigned)blocks, 256, 0, st, L, x, y, mask ? 1 : 0, nullptr,
-                 nullptr, nullptr, nrhs);
+    const int mk = mask ? 1 : 0;
+    if constexpr (sizeof(T) == 8) {
+        if (dot) {
+            if (loc) launch_k(apply_p_kernel<T, DIM, P, true, true>, (unsigned)blocks, 256, 0, st, L, x, y, mk, dot, part, ticket, nrhs, loc);
+            else launch_k(apply_p_kernel<T, DIM, P, true, false>, (unsigned)blocks, 256, 0, st, L, x, y, mk, dot, part, ticket, nrhs, loc);
+            return true;
+        }
     }
+    if (dot) return false;                   // x.(A x) is formed in FP64 only
+    double* nd = nullptr;
+    unsigned* nt = nullptr;
+    if (loc) launch_k(apply_p_kernel<T, DIM, P, false, true>, (unsigned)blocks, 256, 0, st, L, x, y, mk, nd, nd, nt, nrhs, loc);
+    else launch_k(apply_p_kernel<T, DIM, P, false, false>, (unsigned)blocks, 256, 0, st, L, x, y, mk, nd, nd, nt, nrhs, loc);
     return true;
 }
 
 template <typename T, int DIM, int P>
 bool dispatch(int p, const DevLevel<T>& L, const T* x, T* y, bool mask, double* dot, double* part, unsigned* ticket,
-              cudaStream_t st, int nrhs) {
+              cudaStream_t st, int nrhs, T* loc) {
     if constexpr (P == 0) {
         return false;
     } else {
-        if (p == P) return launch_p<T, DIM, P>(L, x, y, mask, dot, part, ticket, st, nrhs);
-        return dispatch<T, DIM, P - 1>(p, L, x, y, mask, dot, part, ticket, st, nrhs);
+        if (p == P) return launch_p<T, DIM, P>(L, x, y, mask, dot, part, ticket, st, nrhs, loc);
+        return dispatch<T, DIM, P - 1>(p, L, x, y, mask, dot, part, ticket, st, nrhs, loc);
     }
 }
 
@@ -257,12 +269,15 @@ bool launch_list_p(int p, const ApplyItem<T>* items, const int* start, int nitem
         return false;
     } else {
         if (p != P) return launch_list_p<T, P - 1>(p, items, start, nitems, blocks, mask, dot, st);
-        if (dot)
-            launch_k(apply_p_list_kernel<T, 2, P, true>, (unsigned)blocks, 256, 0, st, items, start, nitems,
-                     mask ? 1 : 0);
-        else
-            launch_k(apply_p_list_kernel<T, 2, P, false>, (unsigned)blocks, 256, 0, st, items, start, nitems,
-                     mask ? 1 : 0);
+        if constexpr (sizeof(T) == 8) {
+            if (dot) {
+                launch_k(apply_p_list_kernel<T, 2, P, true>, (unsigned)blocks, 256, 0, st, items, start, nitems,
+                         mask ? 1 : 0);
+                return true;
+            }
+        }
+        if (dot) return false;
+        launch_k(apply_p_list_kernel<T, 2, P, false>, (unsigned)blocks, 256, 0, st, items, start, nitems, mask ? 1 : 0);
         return true;
     }
 }
@@ -308,26 +323,27 @@ template int apply_dot_partials<double>(const DevLevel<double>&);
 // Returns false when the order has no specialisation (the caller falls back).
 template <typename T>
 bool launch_apply_fixed(const DevLevel<T>& L, const T* x, T* y, bool mask, double* dot, double* part,
-                        unsigned* ticket, cudaStream_t st, int nrhs) {
+                        unsigned* ticket, cudaStream_t st, int nrhs, T* loc) {
     if (L.N > (1LL << 31) - 1 || L.E * L.nloc * (L.dim == 2 ? 3 : 6) > (1LL << 31) - 1) return false;
     for (int a = 0; a < L.dim; ++a)
         if (L.ne[a] >= 1024) return false;   // element coordinates are packed in 10 bits
     // 3-D: the even-odd line kernel where it was measured fastest, then the
     // FP32 column kernel, else the node-per-thread kernel below
-    if (launch_apply_eo<T>(L, x, y, mask, dot, part, ticket, st, nrhs)) return true;
+    if (launch_apply_eo<T>(L, x, y, mask, dot, part, ticket, st, nrhs, loc)) return true;
     if constexpr (sizeof(T) == 4) {
-        if (L.dim == 3 && !dot && launch_apply_col(L, x, y, mask, st, nrhs)) return true;
+        if (L.dim == 3 && !dot && launch_apply_col(L, x, y, mask, st, nrhs, loc)) return true;
     }
-    if (L.dim == 2) return dispatch<T, 2, 16>(L.p, L, x, y, mask, dot, part, ticket, st, nrhs);
+    if (L.dim == 2) return dispatch<T, 2, 16>(L.p, L, x, y, mask, dot, part, ticket, st, nrhs, loc);
     // 3-D FP32 is served by the even-odd and column kernels above at every
     // order up to 8; this kernel keeps 3-D FP64
-    if constexpr (sizeof(T) == 8) return dispatch<T, 3, 8>(L.p, L, x, y, mask, dot, part, ticket, st, nrhs);
+    if constexpr (sizeof(T) == 8) return dispatch<T, 3, 8>(L.p, L, x, y, mask, dot, part, ticket, st, nrhs,
+                                                                  loc);
     return false;
 }
 
 template bool launch_apply_fixed<float>(const DevLevel<float>&, const float*, float*, bool, double*, double*,
-                                        unsigned*, cudaStream_t, int);
+                                        unsigned*, cudaStream_t, int, float*);
 template bool launch_apply_fixed<double>(const DevLevel<double>&, const double*, double*, bool, double*, double*,
-                                         unsigned*, cudaStream_t, int);
+                                         unsigned*, cudaStream_t, int, double*);
 
 }  // namespace glls

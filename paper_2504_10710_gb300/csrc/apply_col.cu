@@ -70,15 +70,16 @@ __device__ __forceinline__ float coldot(const float (&a)[N1], const float* col) 
     return s;
 }
 
-template <int P>
+template <int P, bool LOC>
 __global__ void __launch_bounds__(256, ColShape<P>::MINB) apply_col_kernel(DevLevel<float> L, DParam<P + 1> Dk,
                                                            const float* __restrict__ x, float* __restrict__ y,
-                                                           int mask, int nrhs) {
+                                                           int mask, int nrhs, float* loc) {
     grid_dep_sync();
     // right-hand side fastest in the CTA order (see device.cuh)
     const int rhs = blockIdx.x % nrhs, cta = blockIdx.x / nrhs;
     x += (long long)rhs * L.N;
     y += (long long)rhs * L.N;
+    if constexpr (LOC) loc += (long long)rhs * L.E * L.nloc;
     using S = ColShape<P>;
     constexpr int N1 = S::N1, NP = S::NP, NLOC = S::NLOC, EPB = S::EPB;
     constexpr bool VEC = S::VEC;
@@ -170,6 +171,10 @@ __global__ void __launch_bounds__(256, ColShape<P>::MINB) apply_col_kernel(DevLe
 #pragma unroll
             for (int m = 0; m < N1; ++m) vt += Dk.d[m * N1 + k] * wt[m];
             v += vt;
+            if constexpr (LOC) {         // element values; summed by gather_kernel in a fixed order
+                loc[e * NLOC + k * NP + c] = v;
+                continue;
+            }
             const int g = base + k * nplane;
             const bool inner = i > 0 && i < P && j > 0 && j < P && k > 0 && k < P;
             if (inner) {
@@ -198,21 +203,25 @@ const float* d_table(int p) {
 }
 
 template <int P>
-bool launch_col(const DevLevel<float>& L, const float* x, float* y, bool mask, cudaStream_t st, int nrhs) {
+bool launch_col(const DevLevel<float>& L, const float* x, float* y, bool mask, cudaStream_t st, int nrhs, float* loc) {
     DParam<P + 1> Dk;
     const float* d = d_table(P);
     for (int t = 0; t < (P + 1) * (P + 1); ++t) Dk.d[t] = d[t];
     constexpr int EPB = ColShape<P>::EPB;
     const long long nb = (L.E + EPB - 1) / EPB * nrhs;
     if (nb > 0x7fffffffLL) return false;
-    launch_k(apply_col_kernel<P>, (unsigned)nb, 256, 0, st, L, Dk, x, y, mask ? 1 : 0, nrhs);
+    if (loc) launch_k(apply_col_kernel<P, true>, (unsigned)nb, 256, 0, st, L, Dk, x, y, mask ? 1 : 0, nrhs, loc);
+    else launch_k(apply_col_kernel<P, false>, (unsigned)nb, 256, 0, st, L, Dk, x, y, mask ? 1 : 0, nrhs, loc);
     return true;
 }
 
 template <int P>
 bool prefer_shared() {
-    return cudaFuncSetAttribute((const void*)apply_col_kernel<P>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                (int)cudaSharedmemCarveoutMaxShared) == cudaSuccess;
+    const int c = (int)cudaSharedmemCarveoutMaxShared;
+    return cudaFuncSetAttribute((const void*)apply_col_kernel<P, false>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                c) == cudaSuccess &&
+           cudaFuncSetAttribute((const void*)apply_col_kernel<P, true>, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                c) == cudaSuccess;
 }
 
 }  // namespace
@@ -220,12 +229,13 @@ bool prefer_shared() {
 // Shared-memory carveout for the column apply (p <= 3: up to 27 KB per CTA).
 bool init_apply_col_attributes() { return prefer_shared<1>() && prefer_shared<2>() && prefer_shared<3>(); }
 
-bool launch_apply_col(const DevLevel<float>& L, const float* x, float* y, bool mask, cudaStream_t st, int nrhs) {
+bool launch_apply_col(const DevLevel<float>& L, const float* x, float* y, bool mask, cudaStream_t st, int nrhs,
+                      float* loc) {
     if (L.dim != 3 || L.p < 1 || L.p > 3) return false;
     switch (L.p) {
-        case 1: return launch_col<1>(L, x, y, mask, st, nrhs);
-        case 2: return launch_col<2>(L, x, y, mask, st, nrhs);
-        default: return launch_col<3>(L, x, y, mask, st, nrhs);
+        case 1: return launch_col<1>(L, x, y, mask, st, nrhs, loc);
+        case 2: return launch_col<2>(L, x, y, mask, st, nrhs, loc);
+        default: return launch_col<3>(L, x, y, mask, st, nrhs, loc);
     }
 }
 

@@ -107,10 +107,10 @@ __device__ __forceinline__ bool on_bd(int I, int J, int K, const int n[3]) {
 // FP64 (T = double).  epb elements per CTA (at most 256 threads), chosen at
 // launch so that small levels still spread over many CTAs per SM.  Two
 // resident CTAs per SM bound the registers (at most 128 per thread).
-template <typename T, int P, bool DOT>
+template <typename T, int P, bool DOT, bool LOC>
 __global__ void __launch_bounds__(256, 2)
     apply_eo3_kernel(DevLevel<T> L, const __grid_constant__ EoParams<T, P + 1> M, const T* __restrict__ x,
-                     T* __restrict__ y, int mask, double* dot, double* part, unsigned* ticket, int epb, int nrhs) {
+                     T* __restrict__ y, int mask, double* dot, double* part, unsigned* ticket, int epb, int nrhs, T* loc) {
     using S = EoShape<P + 1>;
     constexpr int N = P + 1, NP = S::NP, NLOC = S::NLOC, RS = S::RS, PS = S::PS, ES = S::ES;
     extern __shared__ __align__(16) unsigned char eo_smem3[];
@@ -122,6 +122,7 @@ __global__ void __launch_bounds__(256, 2)
     const int rhs = blockIdx.x % nrhs, bx = blockIdx.x / nrhs, nbx = gridDim.x / nrhs;
     x += (long long)rhs * L.N;
     y += (long long)rhs * L.N;
+    if constexpr (LOC) loc += (long long)rhs * L.E * NLOC;
     const int E = (int)L.E, n0 = L.n[0], n1 = L.n[1];
     const int nplane = n0 * n1;
     const int tid = threadIdx.x;
@@ -206,6 +207,10 @@ __global__ void __launch_bounds__(256, 2)
             const int s = k * PS + b * RS + a;
             const T v = yt[k] + U[s] + V[s];
             if (DOT) local += (double)xc[k] * (double)v;
+            if constexpr (LOC) {         // element values; summed by gather_kernel in a fixed order
+                loc[e * NLOC + k * NP + c] = v;
+                continue;
+            }
             const int g = base + k * nplane;
             if (a > 0 && a < P && b > 0 && b < P && k > 0 && k < P) {
                 y[g] = v;
@@ -283,10 +288,10 @@ __device__ __forceinline__ void eo_line2(const EoMat2<N>& M, const f32x2 (&u)[N]
 // Resident CTAs of 128 threads the registers must allow, as measured.
 constexpr int eo_pair_min_ctas(int P, bool rhs) { return rhs ? (P == 8 ? 4 : 5) : (P == 5 || P == 6 ? 5 : 4); }
 
-template <int P, bool RHS>
+template <int P, bool RHS, bool LOC>
 __global__ void __launch_bounds__(128, eo_pair_min_ctas(P, RHS))
     apply_eo3_pair_kernel(DevLevel<float> L, const __grid_constant__ EoParams2<P + 1> M, const float* __restrict__ x,
-                          float* __restrict__ y, int mask, int epb, int nrhs) {
+                          float* __restrict__ y, int mask, int epb, int nrhs, float* loc) {
     using S = EoShape<P + 1>;
     constexpr int N = P + 1, NP = S::NP, NLOC = S::NLOC, RS = S::RS, PS = S::PS, ES = S::ES;
     extern __shared__ __align__(16) unsigned char eo_smem2[];
@@ -414,12 +419,20 @@ __global__ void __launch_bounds__(128, eo_pair_min_ctas(P, RHS))
     __syncthreads();
     if (!act) return;
     const bool inner = a > 0 && a < P && b > 0 && b < P;
+    // element values of both halves; summed by gather_kernel in a fixed order
+    float* lA = LOC ? loc + ((long long)(RHS ? 2 * rg : rg) * E + eA) * NLOC + c : nullptr;
+    float* lB = LOC ? loc + ((long long)(RHS ? 2 * rg + 1 : rg) * E + eB) * NLOC + c : nullptr;
     const int last = L.n[2] - 1;
 #pragma unroll
     for (int k = 0; k < N; ++k) {
         const int s = at_t(k);
         float vA, vB;
         unpack2(add2(add2(yt[k], U[s]), V[s]), vA, vB);
+        if constexpr (LOC) {
+            lA[k * NP] = vA;
+            if (hasB) lB[k * NP] = vB;
+            continue;
+        }
         float* pA = yA + baseA + k * nplane;
         float* pB = yB + baseB + k * nplane;
         if (k > 0 && k < P && inner) {
@@ -486,7 +499,8 @@ int eo_pair_epb(int p, long long slots) {
 }
 
 template <int P>
-bool launch_eo_pair(const DevLevel<float>& L, const float* x, float* y, bool mask, cudaStream_t st, int nrhs) {
+bool launch_eo_pair(const DevLevel<float>& L, const float* x, float* y, bool mask, cudaStream_t st, int nrhs,
+                    float* loc) {
     using S = EoShape<P + 1>;
     const bool rhs = nrhs % 2 == 0;
     const EoParams2<P + 1> M = eo_params2<P + 1>();
@@ -496,14 +510,17 @@ bool launch_eo_pair(const DevLevel<float>& L, const float* x, float* y, bool mas
     if (nb > 0x7fffffffLL) return false;
     const int threads = (epb * S::NP + 31) / 32 * 32;
     const size_t smem = sizeof(f32x2) * S::NBUF * epb * S::ES;
-    if (rhs) launch_k(apply_eo3_pair_kernel<P, true>, (unsigned)nb, threads, smem, st, L, M, x, y, mask ? 1 : 0, epb, nrhs);
-    else launch_k(apply_eo3_pair_kernel<P, false>, (unsigned)nb, threads, smem, st, L, M, x, y, mask ? 1 : 0, epb, nrhs);
+    const int mk = mask ? 1 : 0;
+    if (rhs && loc) launch_k(apply_eo3_pair_kernel<P, true, true>, (unsigned)nb, threads, smem, st, L, M, x, y, mk, epb, nrhs, loc);
+    else if (rhs) launch_k(apply_eo3_pair_kernel<P, true, false>, (unsigned)nb, threads, smem, st, L, M, x, y, mk, epb, nrhs, loc);
+    else if (loc) launch_k(apply_eo3_pair_kernel<P, false, true>, (unsigned)nb, threads, smem, st, L, M, x, y, mk, epb, nrhs, loc);
+    else launch_k(apply_eo3_pair_kernel<P, false, false>, (unsigned)nb, threads, smem, st, L, M, x, y, mk, epb, nrhs, loc);
     return true;
 }
 
 template <typename T, int P>
 bool launch_eo(const DevLevel<T>& L, const T* x, T* y, bool mask, double* dot, double* part, unsigned* ticket,
-               cudaStream_t st, int nrhs) {
+               cudaStream_t st, int nrhs, T* loc) {
     using S = EoShape<P + 1>;
     const EoParams<T, P + 1> M = eo_params<T, P + 1>();
     const int epb = eo_epb(P, L.E);
@@ -512,10 +529,13 @@ bool launch_eo(const DevLevel<T>& L, const T* x, T* y, bool mask, double* dot, d
     const int blocks = (int)nb;
     const int threads = (epb * S::NP + 31) / 32 * 32;
     const size_t smem = sizeof(T) * S::NBUF * epb * S::ES;
-    if (dot) launch_k(apply_eo3_kernel<T, P, true>, blocks, threads, smem, st, L, M, x, y, mask ? 1 : 0, dot, part,
-                      ticket, epb, nrhs);
-    else launch_k(apply_eo3_kernel<T, P, false>, blocks, threads, smem, st, L, M, x, y, mask ? 1 : 0,
-                  (double*)nullptr, (double*)nullptr, (unsigned*)nullptr, epb, nrhs);
+    double* nd = nullptr;
+    unsigned* nt = nullptr;
+    const int mk = mask ? 1 : 0;
+    if (dot && loc) launch_k(apply_eo3_kernel<T, P, true, true>, blocks, threads, smem, st, L, M, x, y, mk, dot, part, ticket, epb, nrhs, loc);
+    else if (dot) launch_k(apply_eo3_kernel<T, P, true, false>, blocks, threads, smem, st, L, M, x, y, mk, dot, part, ticket, epb, nrhs, loc);
+    else if (loc) launch_k(apply_eo3_kernel<T, P, false, true>, blocks, threads, smem, st, L, M, x, y, mk, nd, nd, nt, epb, nrhs, loc);
+    else launch_k(apply_eo3_kernel<T, P, false, false>, blocks, threads, smem, st, L, M, x, y, mk, nd, nd, nt, epb, nrhs, loc);
     return true;
 }
 
@@ -523,10 +543,11 @@ template <typename T, int P>
 bool set_eo_attr() {
     using S = EoShape<P + 1>;
     const int smem = (int)(sizeof(T) * S::NBUF * (256 / S::NP) * S::ES);
-    return cudaFuncSetAttribute((const void*)apply_eo3_kernel<T, P, false>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess &&
-           cudaFuncSetAttribute((const void*)apply_eo3_kernel<T, P, true>,
-                                cudaFuncAttributeMaxDynamicSharedMemorySize, smem) == cudaSuccess;
+    const void* fns[] = {(const void*)apply_eo3_kernel<T, P, false, false>, (const void*)apply_eo3_kernel<T, P, false, true>,
+                         (const void*)apply_eo3_kernel<T, P, true, false>, (const void*)apply_eo3_kernel<T, P, true, true>};
+    for (const void* f : fns)
+        if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return false;
+    return true;
 }
 
 }  // namespace
@@ -549,28 +570,28 @@ int apply_eo_blocks(int p, long long E) {
 
 template <typename T>
 bool launch_apply_eo(const DevLevel<T>& L, const T* x, T* y, bool mask, double* dot, double* part,
-                     unsigned* ticket, cudaStream_t st, int nrhs) {
+                     unsigned* ticket, cudaStream_t st, int nrhs, T* loc) {
     if (!apply_eo_selected(L.dim, L.p, sizeof(T) == 8)) return false;
     if constexpr (sizeof(T) == 8) {
         switch (L.p) {
-            case 6: return launch_eo<T, 6>(L, x, y, mask, dot, part, ticket, st, nrhs);
-            default: return launch_eo<T, 7>(L, x, y, mask, dot, part, ticket, st, nrhs);
+            case 6: return launch_eo<T, 6>(L, x, y, mask, dot, part, ticket, st, nrhs, loc);
+            default: return launch_eo<T, 7>(L, x, y, mask, dot, part, ticket, st, nrhs, loc);
         }
     } else {
         if (dot) return false;               // x.(A x) is formed in FP64 only
         switch (L.p) {
-            case 4: return launch_eo_pair<4>(L, x, y, mask, st, nrhs);
-            case 5: return launch_eo_pair<5>(L, x, y, mask, st, nrhs);
-            case 6: return launch_eo_pair<6>(L, x, y, mask, st, nrhs);
-            case 7: return launch_eo_pair<7>(L, x, y, mask, st, nrhs);
-            default: return launch_eo_pair<8>(L, x, y, mask, st, nrhs);
+            case 4: return launch_eo_pair<4>(L, x, y, mask, st, nrhs, loc);
+            case 5: return launch_eo_pair<5>(L, x, y, mask, st, nrhs, loc);
+            case 6: return launch_eo_pair<6>(L, x, y, mask, st, nrhs, loc);
+            case 7: return launch_eo_pair<7>(L, x, y, mask, st, nrhs, loc);
+            default: return launch_eo_pair<8>(L, x, y, mask, st, nrhs, loc);
         }
     }
 }
 template bool launch_apply_eo<float>(const DevLevel<float>&, const float*, float*, bool, double*, double*,
-                                     unsigned*, cudaStream_t, int);
+                                     unsigned*, cudaStream_t, int, float*);
 template bool launch_apply_eo<double>(const DevLevel<double>&, const double*, double*, bool, double*, double*,
-                                      unsigned*, cudaStream_t, int);
+                                      unsigned*, cudaStream_t, int, double*);
 
 bool init_apply_eo_attributes() { return set_eo_attr<double, 6>() && set_eo_attr<double, 7>(); }
 

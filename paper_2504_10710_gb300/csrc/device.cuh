@@ -98,7 +98,7 @@ struct DevLevel {
     DevBand<T> P[3], R[3];
     int lpb[3] = {4, 4, 4};   // band-1 line-solve tile (lines per CTA) per direction, set by the autotuner
     int lbc[3] = {0, 0, 0};   // line-block lines per CTA per direction, set by the autotuner (0: launch heuristic)
-    int colored = 0;          // direct stiffness summation by element colours (bitwise reproducible; see launch_apply)
+    int colored = 0;          // direct stiffness summation in a fixed order (bitwise reproducible; see launch_apply)
     // float-float form of G (finest FP64 level, 2-D 2 <= p <= 16, 3-D
     // 2 <= p <= 8; null elsewhere): Ghi = the FP32 level's G (the FP64 factors rounded to
     // nearest), Glo = their FP32 rounding remainders (apply_ff.cu)
@@ -258,9 +258,11 @@ constexpr size_t kMaxDynSmemBytes = 200 * 1024;
 // dot: if non-null, also accumulate sum_e x_e^T (A_e x_e) = x.(A x) for x
 // zero on the boundary; the last block writes it to dot[0] using `part` and
 // `ticket` (see launch_dots).
+// loc: if non-null (nrhs x E (p+1)^dim values), the element results go there
+// instead of being summed into y (launch_apply then gathers them).
 template <typename T>
 bool launch_apply_fixed(const DevLevel<T>& L, const T* x, T* y, bool mask, double* dot, double* part,
-                        unsigned* ticket, cudaStream_t st, int nrhs = 1);
+                        unsigned* ticket, cudaStream_t st, int nrhs = 1, T* loc = nullptr);
 template <typename T>
 bool launch_line_warp(const DevLevel<T>& L, int s, int mode, const T* g, const T* r, T* y, T* x, T alpha,
                       cudaStream_t st, int nrhs = 1);
@@ -285,7 +287,7 @@ bool init_line_block_attributes<double>();
 // (the orders the even-odd kernel does not take); no x.(A x) product.
 // Returns false outside that range.
 bool launch_apply_col(const DevLevel<float>& L, const float* x, float* y, bool mask, cudaStream_t st,
-                      int nrhs = 1);
+                      int nrhs = 1, float* loc = nullptr);
 bool init_apply_col_attributes();
 // 3-D apply with one thread per element grid line and even-odd derivative
 // sweeps (apply_eo.cu), for the orders apply_eo_selected names, with the
@@ -293,7 +295,7 @@ bool init_apply_col_attributes();
 bool apply_eo_selected(int dim, int p, bool f64);
 template <typename T>
 bool launch_apply_eo(const DevLevel<T>& L, const T* x, T* y, bool mask, double* dot, double* part,
-                     unsigned* ticket, cudaStream_t st, int nrhs = 1);
+                     unsigned* ticket, cudaStream_t st, int nrhs = 1, T* loc = nullptr);
 int apply_eo_blocks(int p, long long E);
 bool init_apply_eo_attributes();
 
@@ -302,10 +304,15 @@ bool init_apply_eo_attributes();
 // guarantees y == 0 on entry (otherwise it is zeroed first).  dot, part,
 // ticket: optional x.(A x) into dot[0] (FP64 only).  Returns the status of
 // the zeroing (cudaSuccess when y_is_zero); launch errors are left to
-// cudaGetLastError.
+// cudaGetLastError.  Levels with fixed-order summation (L.colored): with
+// scratch loc (nrhs x E (p+1)^dim values of the instance) the specialised
+// kernels write the element results there and one gather sums them; without
+// it, or outside their range, one launch per element colour.  dot partials:
+// apply_dot_partials of them with loc, kDotBlocks without.
 template <typename T>
 cudaError_t launch_apply(const DevLevel<T>& L, const T* x, T* y, bool mask, cudaStream_t st, bool y_is_zero = false,
-                  double* dot = nullptr, double* part = nullptr, unsigned* ticket = nullptr, int nrhs = 1);
+                  double* dot = nullptr, double* part = nullptr, unsigned* ticket = nullptr, int nrhs = 1,
+                  T* loc = nullptr);
 
 // Line solves along axis s.  mode 0: x = B_s^-1 g; mode 1: x += alpha
 // B_s^-1 (r - y) and y is reset to 0 where read; mode 2: x += alpha B_s^-1 r;

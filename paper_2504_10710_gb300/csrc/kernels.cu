@@ -162,6 +162,43 @@ __global__ void __launch_bounds__(256) apply_kernel(DevLevel<T> L, const T* __re
     }
 }
 
+// y from the element results `loc` (element-major, nloc values each): every
+// node adds the contributions of the elements that hold it, lower elements
+// first along each axis, x fastest, so y is the same bits on every run.
+// Boundary nodes are set to 0 when mask is set.  One thread per node; bound by
+// the bytes of loc and y.
+template <typename T, int DIM>
+__global__ void __launch_bounds__(256) gather_kernel(DevLevel<T> L, const T* __restrict__ loc, T* __restrict__ y,
+                                                     int mask, int nrhs) {
+    grid_dep_sync();
+    const int p = L.p, n1 = L.n1, nloc = L.nloc, nx = L.n[0], ny = L.n[1], nz = L.n[2];
+    const int ne0 = L.ne[0], ne1 = L.ne[1], ne2 = L.ne[2], N = (int)L.N;
+    const long long EL = L.E * nloc, total = (long long)N * nrhs;
+    for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < total;
+         g += (long long)gridDim.x * blockDim.x) {
+        const int rhs = nrhs == 1 ? 0 : (int)(g / N), node = (int)(g - (long long)rhs * N);
+        const int row = node / nx, I = node - row * nx;
+        const int K = DIM == 3 ? row / ny : 0, J = row - K * ny;
+        if (mask && (I == 0 || I == nx - 1 || J == 0 || J == ny - 1 || (DIM == 3 && (K == 0 || K == nz - 1)))) {
+            y[g] = T(0);
+            continue;
+        }
+        // elements e with e p <= node index <= e p + p along each axis
+        const int ex1 = min(I / p, ne0 - 1), ex0 = I == ex1 * p && ex1 > 0 ? ex1 - 1 : ex1;
+        const int ey1 = min(J / p, ne1 - 1), ey0 = J == ey1 * p && ey1 > 0 ? ey1 - 1 : ey1;
+        const int ez1 = DIM == 3 ? min(K / p, ne2 - 1) : 0, ez0 = DIM == 3 && K == ez1 * p && ez1 > 0 ? ez1 - 1 : ez1;
+        const T* src = loc + rhs * EL;
+        T s = T(0);
+        for (int ez = ez0; ez <= ez1; ++ez)
+            for (int ey = ey0; ey <= ey1; ++ey)
+                for (int ex = ex0; ex <= ex1; ++ex) {
+                    const long long e = ((long long)ez * ne1 + ey) * ne0 + ex;
+                    s += src[e * nloc + ((K - ez * p) * n1 + (J - ey * p)) * n1 + I - ex * p];
+                }
+        y[g] = s;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // line solves by cyclic reduction
 // ---------------------------------------------------------------------------
@@ -1145,7 +1182,15 @@ constexpr int kMaxDynSmem = 200 * 1024;
 // ---------------------------------------------------------------------------
 template <typename T>
 cudaError_t launch_apply(const DevLevel<T>& L, const T* x, T* y, bool mask, cudaStream_t st, bool y_is_zero,
-                         double* dot, double* part, unsigned* ticket, int nrhs) {
+                         double* dot, double* part, unsigned* ticket, int nrhs, T* loc) {
+    // fixed-order summation: element results into loc, then one gather (2-D
+    // 45 x 28 elements, p = 11, FP32: 4 colour launches of the run-time-order
+    // kernel, 35 us, before)
+    if (L.colored && loc && launch_apply_fixed<T>(L, x, y, mask, dot, part, ticket, st, nrhs, loc)) {
+        const int g = grid_for(L.N * nrhs);
+        return L.dim == 2 ? launch_k(gather_kernel<T, 2>, g, 256, 0, st, L, (const T*)loc, y, mask ? 1 : 0, nrhs)
+                          : launch_k(gather_kernel<T, 3>, g, 256, 0, st, L, (const T*)loc, y, mask ? 1 : 0, nrhs);
+    }
     if (!y_is_zero) {
         const cudaError_t e = cudaMemsetAsync(y, 0, sizeof(T) * L.N * nrhs, st);
         if (e != cudaSuccess) return e;
@@ -1480,9 +1525,9 @@ bool init_kernel_attributes() {
 
 // explicit instantiations
 template cudaError_t launch_apply<double>(const DevLevel<double>&, const double*, double*, bool, cudaStream_t, bool, double*,
-                                   double*, unsigned*, int);
+                                   double*, unsigned*, int, double*);
 template cudaError_t launch_apply<float>(const DevLevel<float>&, const float*, float*, bool, cudaStream_t, bool, double*,
-                                  double*, unsigned*, int);
+                                  double*, unsigned*, int, float*);
 template void launch_line_solve<double>(const DevLevel<double>&, int, int, const double*, const double*, double*,
                                         double*, double, cudaStream_t, int);
 template void launch_line_solve<float>(const DevLevel<float>&, int, int, const float*, const float*, float*,
