@@ -501,30 +501,26 @@ void outer_iteration(glls_problem* P, const glls_solve_opts* o, cudaStream_t st)
     const int npq = ff ? apply_ff_partials(P->L64[L].dev) : apply_dot_partials<double>(P->L64[L].dev);
     launch_dots_rz_zq(P->rk, P->zk, mixed ? P->z32 : nullptr, P->qk, N, prz, pzq, st, k);
     const int nb = fcg_blocks(N);            // the dots' CTAs: partials of r.z, z.q, r.r per right-hand side
-    launch_fcg_direction(P->pk, P->zk, N, prz, pzq, nb, P->S, o->krylov == GLLS_KRYLOV_FCG ? 1 : 0, st, k);
+    launch_fcg_direction(P->pk, P->zk, mixed ? P->z32 : nullptr, N, prz, pzq, nb, P->S,
+                         o->krylov == GLLS_KRYLOV_FCG ? 1 : 0, st, k);
     if (ff) launch_apply_ff(P->L64[L].dev, P->pk, P->qk, true, ppq, st, k);
     else launch_apply<double>(P->L64[L].dev, P->pk, P->qk, true, st, true, P->S + S_PQ, ppq, nullptr, k,
                               P->L64[L].loc);
-    launch_fcg_update(P->xk, P->rk, P->pk, P->qk, N, ppq, npq, prz, nb, prr, P->S, P->ticket,
-                      mixed ? P->r32 : nullptr, st, k);
+    launch_fcg_update(P->xk, P->rk, P->pk, P->qk, N, ppq, npq, nb, prr, P->S, P->ticket, mixed ? P->r32 : nullptr, st,
+                      k);
 }
 
 // Lifting and Krylov initialisation (x = p = q = 0, r = f0, S_RR0 = r.r).
 // The lifting v of the (shared) Dirichlet data and A v are computed once;
 // f0 = M f - A v for every right-hand side.
 void solve_prologue(glls_problem* P, const glls_solve_opts* o, cudaStream_t st) {
-    const long long N = P->N, NK = P->N * P->nrhs;
     const int L = (int)P->L64.size() - 1;
     const DevLevel<double>& F = P->L64[L].dev;
-    launch_boundary_only(P->g, P->v, F.n, F.dim, st);
-    launch_apply<double>(F, P->v, P->yk, false, st, false, nullptr, nullptr, nullptr, 1, P->L64[L].loc);
-    launch_lift_rhs(P->mass, P->f, P->yk, P->f0, F.n, F.dim, st, P->nrhs);
-    cudaMemsetAsync(P->xk, 0, sizeof(double) * NK, st);
-    cudaMemsetAsync(P->pk, 0, sizeof(double) * NK, st);
-    cudaMemsetAsync(P->qk, 0, sizeof(double) * NK, st);
-    cudaMemcpyAsync(P->rk, P->f0, sizeof(double) * NK, cudaMemcpyDeviceToDevice, st);
-    launch_dots(P->rk, P->rk, nullptr, nullptr, 1, N, P->part, P->S, S_RR0, S_RR0, P->ticket, st, P->nrhs);
-    if (o->precision == GLLS_PREC_MIXED) launch_cast<double, float>(P->rk, P->r32, NK, st);
+    launch_boundary_only(P->g, P->v, P->yk, F.n, F.dim, st);
+    launch_apply<double>(F, P->v, P->yk, false, st, true, nullptr, nullptr, nullptr, 1, P->L64[L].loc);
+    launch_solve_start(P->mass, P->f, P->yk, P->f0, F.n, F.dim, P->rk,
+                       o->precision == GLLS_PREC_MIXED ? P->r32 : nullptr, P->xk, P->pk, P->qk, P->part, P->S,
+                       P->ticket, st, P->nrhs);
 }
 
 bool same_solve_key(const glls_solve_opts& a, const glls_solve_opts& b) {
@@ -579,10 +575,7 @@ cudaError_t capture_solve(glls_problem* P, const glls_solve_opts* o, cudaStream_
             if (e == cudaSuccess) P->kern_iter = count_kernel_nodes(body);
         }
     }
-    if (e == cudaSuccess) {   // u = w + v for every right-hand side
-        cudaMemcpyAsync(P->yk, P->xk, sizeof(double) * P->N * P->nrhs, cudaMemcpyDeviceToDevice, cs);
-        launch_axpy(P->yk, P->v, 1.0, P->N, cs, P->nrhs, true);
-    }
+    if (e == cudaSuccess) launch_sum(P->yk, P->xk, P->v, P->N, cs, P->nrhs);   // u = w + v
     return e;
 }
 
@@ -874,6 +867,7 @@ struct WlRecord {
     int p = 0, s = 0, cv = 1, wb = 0, ty = 0, l = 0, step = 0;
     bool mask = false, dot = false, add = false;
     bool ff = false;                   // the float-float form of the FP64 outer apply
+    bool mixed = false;                // outer-Krylov steps: z is z32
     int blocks = 0, threads = 256, nitems = 0;
     size_t smem = 0;
     std::vector<unsigned char> items;  // host copy of the item array
@@ -1183,7 +1177,7 @@ std::string build_group(WlGroup& G, const glls_solve_opts& o) {
     // every one: each CTA also sums all of its problem's partials
     long long nmax = 1;
     for (glls_problem* P : G.probs) nmax = std::max(nmax, P->N);
-    const int nblk = fcg_blocks(nmax);
+    const int nblk = fcg_list_blocks(nmax);
     for (int step : {0, 1, -1, 2}) {
         if (step == -1) {
             G.body.push_back(ap);
@@ -1191,6 +1185,7 @@ std::string build_group(WlGroup& G, const glls_solve_opts& o) {
         }
         WlRecord r;
         r.kind = WL_FCG;
+        r.mixed = mixed;
         r.step = step;
         r.dbl = true;
         r.blocks = nblk;
@@ -1270,7 +1265,7 @@ cudaError_t replay(const WlRecord& r, const unsigned char* base, int flexible, c
                 launch_coarse_list<float>((const CoarseItem<float>*)items, start, r.nitems, r.blocks, r.smem, st);
             break;
         default:
-            launch_fcg_list(r.step, (const FcgItem*)items, r.nitems, flexible, r.blocks, st);
+            launch_fcg_list(r.step, (const FcgItem*)items, r.nitems, flexible, r.blocks, r.mixed, st);
     }
     if (!ok) return cudaErrorInvalidConfiguration;
     return cudaGetLastError();
@@ -1348,8 +1343,7 @@ cudaError_t capture_plan(WlPlan* W, const glls_solve_opts* o) {
         }
         for (int j = 0; j < n && e == cudaSuccess; ++j) {   // u = w + v; the scalars back to the problem
             glls_problem* P = G.probs[j];
-            e = cudaMemcpyAsync(P->yk, P->xk, sizeof(double) * P->N, cudaMemcpyDeviceToDevice, G.s1);
-            launch_axpy(P->yk, P->v, 1.0, P->N, G.s1);
+            launch_sum(P->yk, P->xk, P->v, P->N, G.s1);
             if (e == cudaSuccess)
                 e = cudaMemcpyAsync(P->S, S + (size_t)j * S_COUNT, sizeof(double) * S_COUNT,
                                     cudaMemcpyDeviceToDevice, G.s1);
@@ -1715,8 +1709,8 @@ glls_status glls_lift_f64(glls_problem* P, const double* f, const double* g, dou
     cudaStream_t st = (cudaStream_t)stream;
     const int L = (int)P->L64.size() - 1;
     const DevLevel<double>& F = P->L64[L].dev;
-    launch_boundary_only(g, P->v, F.n, F.dim, st);
-    launch_apply<double>(F, P->v, P->yk, false, st, false, nullptr, nullptr, nullptr, 1, P->L64[L].loc);
+    launch_boundary_only(g, P->v, P->yk, F.n, F.dim, st);
+    launch_apply<double>(F, P->v, P->yk, false, st, true, nullptr, nullptr, nullptr, 1, P->L64[L].loc);
     launch_lift_rhs(P->mass, f, P->yk, f0, F.n, F.dim, st);
     CK(cudaGetLastError());
     return GLLS_OK;
@@ -1742,8 +1736,7 @@ static glls_status solve_impl(glls_problem* P, const glls_solve_opts* o, double*
     if (o->krylov == GLLS_KRYLOV_GMRES) {
         result = gmres_solve(P, o, st, &it, &rel);
         if (result != GLLS_OK && result != GLLS_ERR_NOT_CONVERGED) return result;
-        CK(cudaMemcpyAsync(P->yk, P->xk, sizeof(double) * N, cudaMemcpyDeviceToDevice, st));
-        launch_axpy(P->yk, P->v, 1.0, N, st);
+        launch_sum(P->yk, P->xk, P->v, N, st);
         CK(cudaMemcpyAsync(u, P->yk, sizeof(double) * N, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost,
                            st));
         CK(cudaStreamSynchronize(st));
@@ -1818,8 +1811,7 @@ static glls_status solve_impl(glls_problem* P, const glls_solve_opts* o, double*
     }
     CK(cudaGetLastError());
     // u = w + v
-    CK(cudaMemcpyAsync(P->yk, P->xk, sizeof(double) * N, cudaMemcpyDeviceToDevice, st));
-    launch_axpy(P->yk, P->v, 1.0, N, st);
+    launch_sum(P->yk, P->xk, P->v, N, st);
     CK(cudaMemcpyAsync(u, P->yk, sizeof(double) * N, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, st));
     if (!on_device || stats) CK(cudaStreamSynchronize(st));
     if (stats) {

@@ -189,7 +189,7 @@ __device__ __forceinline__ void apply_p_body(const DevLevel<T>& L, const T* __re
     if (DOT) {
         // per-block partial of x.(A x); with a ticket the last block also sums
         // them into dot[0], without one the consumer sums the partials
-        __shared__ double red[32];
+        __shared__ double red[kReduceThreads];
         const double tsum = block_sum(local, red);
         if (threadIdx.x == 0) part[(long long)rhs * nbx + bx] = tsum;
         if (ticket && last_block(ticket)) {   // single right-hand side, single launch only

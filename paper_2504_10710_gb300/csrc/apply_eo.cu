@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(256, 2)
         }
     }
     if (DOT) {
-        __shared__ double red[32];
+        __shared__ double red[kReduceThreads];
         const double tsum = block_sum(local, red);
         if (tid == 0) part[(long long)rhs * nbx + bx] = tsum;
         if (ticket && last_block(ticket)) {   // single right-hand side only

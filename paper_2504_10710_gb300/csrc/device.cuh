@@ -234,7 +234,8 @@ void launch_bcr_list(bool forward, int l, const BcrItem<T>* items, const int* st
                      size_t smem, cudaStream_t st);
 // blocks: CTAs per item (<= kDotBlocks), the same for every item: each item's
 // partial sums of r.z, z.q and r.r have that many entries
-void launch_fcg_list(int step, const FcgItem* items, int nitems, int flexible, int blocks, cudaStream_t st);
+void launch_fcg_list(int step, const FcgItem* items, int nitems, int flexible, int blocks, bool mixed,
+                     cudaStream_t st);
 template <typename T>
 size_t line_block_item_bytes();
 template <typename T>
@@ -357,49 +358,60 @@ void launch_zero_boundary(T* v, const int n[3], int dim, cudaStream_t st, int nr
 // kernel resets.
 constexpr int kDotBlocks = 304;   // 2 x 152 SMs
 // CTAs per right-hand side of the outer-iteration kernels (dots, direction,
-// update) for vectors of n values: about 16 values per thread, between 16
-// and kDotBlocks (each CTA also sums all of the apply's partials, so more
-// CTAs than the vector needs cost more than they hide)
-inline int fcg_blocks(long long n) {
-    const long long b = (n + 4095) / 4096;
+// update) for vectors of n values: a CTA also sums all of the apply's partials
+// and waits out a few memory latencies, so it pays to spread one problem's
+// vectors over the chip (1024 values a CTA; 2-D 64 x 64, p = 8 mixed solve
+// 1.62, 1.57, 1.53 ms with 4096, 2048, 1024), while the launches of a work
+// list have the CTAs of all their problems (4096; 24 uneven problems 16.7,
+// 17.1, 17.6 ms).
+inline int vector_blocks(long long n, int per_cta) {
+    const long long b = (n + per_cta - 1) / per_cta;
     return (int)(b < 16 ? 16 : b > kDotBlocks ? kDotBlocks : b);
 }
+inline int fcg_blocks(long long n) { return vector_blocks(n, 1024); }
+inline int fcg_list_blocks(long long n) { return vector_blocks(n, 4096); }
 constexpr int kMaxReduceBlocks = 8192;
 void launch_dots(const double* a0, const double* b0, const double* a1, const double* b1, int ndots,
                  long long n, double* part, double* S, int slot0, int slot1, unsigned* ticket, cudaStream_t st, int nrhs = 1);
 // Outer-iteration dots without a grid-wide finish: kDotBlocks per-block
-// partials of r.z into prz and of z.q into pzq; z is first taken from z32
-// when given (z = double(z32)); q is reset to 0 after it is read.
-void launch_dots_rz_zq(const double* r, double* z, const float* z32, double* q, long long n, double* prz, double* pzq,
-                       cudaStream_t st, int nrhs = 1);
+// partials of r.z into prz and of z.q into pzq; z is z32 when given; q is
+// reset to 0 after it is read.
+void launch_dots_rz_zq(const double* r, const double* z, const float* z32, double* q, long long n, double* prz,
+                       double* pzq, cudaStream_t st, int nrhs = 1);
 
 // Krylov scalar slots in the device array S.
 // Per right-hand side j the slots sit at S + j * S_COUNT.  S_DONE: 0 while
 // iterating, 1 converged, 2 broken down; S_ITS: iterations when it stopped.
 enum Slot { S_RZ = 0, S_PQ, S_RR, S_RZNEW, S_ZQ, S_RR0, S_ALPHA, S_FLAG, S_TOL2, S_ITER, S_DONE, S_ITS, S_COUNT };
 
-// q-independent update: p.q (npq partials from the apply) and r.z (nrz
-// partials) are summed in every block, alpha = r.z / p.q; x += alpha p;
-// r -= alpha q; r.r partials into prr; the last block writes S_RR, S_RZ,
-// S_ALPHA, S_PQ and flags breakdown in S_FLAG.  r32 (optional): also
-// r32 = float(r) for the FP32 gamma-cycle.
+// q-independent update on nb CTAs per right-hand side: p.q (npq partials from
+// the apply) is summed in every block, r.z taken from S_RZNEW, alpha = r.z /
+// p.q; x += alpha p; r -= alpha q; r.r partials into prr; the last block writes
+// S_RR, S_RZ, S_ALPHA, S_PQ and flags breakdown in S_FLAG.  r32 (optional):
+// also r32 = float(r) for the FP32 gamma-cycle.
 void launch_fcg_update(double* x, double* r, const double* p, const double* q, long long n, const double* ppq,
-                       int npq, const double* prz, int nrz, double* prr, double* S, unsigned* ticket, float* r32,
-                       cudaStream_t st, int nrhs = 1);
-// p = z + beta p with beta = -S_ALPHA zq / S_RZ (flexible) or rz_new / S_RZ,
-// rz_new and zq summed from the nd partials of launch_dots_rz_zq.
-void launch_fcg_direction(double* p, const double* z, long long n, const double* prz, const double* pzq, int nd,
-                          const double* S, int flexible, cudaStream_t st, int nrhs = 1);
+                       int npq, int nb, double* prr, double* S, unsigned* ticket, float* r32, cudaStream_t st,
+                       int nrhs = 1);
+// p = z + beta p (z is z32 when given) with beta = -S_ALPHA zq / S_RZ
+// (flexible) or rz_new / S_RZ, rz_new and zq summed from the nd partials of
+// launch_dots_rz_zq; rz_new into S_RZNEW.
+void launch_fcg_direction(double* p, const double* z, const float* z32, long long n, const double* prz,
+                          const double* pzq, int nd, double* S, int flexible, cudaStream_t st, int nrhs = 1);
 // Dot partials launch_apply writes for L when asked for x.(A x) without a ticket.
 template <typename T>
 int apply_dot_partials(const DevLevel<T>& L);
-// f0 = M f - y on interior nodes (0 on the boundary); v = g on the boundary, 0 inside.
+// f0 = M f - y on interior nodes (0 on the boundary); launch_solve_start also
+// sets r = f0, r32 (optional) = float(f0), x = p = q = 0 and S_RR0 = r.r for
+// every right-hand side (part: fcg_blocks partials each; ticket zero, reset).
 void launch_lift_rhs(const double* mass, const double* f, const double* y, double* f0, const int n[3], int dim,
-                     cudaStream_t st, int nrhs = 1);
-void launch_boundary_only(const double* g, double* v, const int n[3], int dim, cudaStream_t st);
-// y += a x; nrhs vectors of n values each, x the same for all when x_shared
-void launch_axpy(double* y, const double* x, double a, long long n, cudaStream_t st, int nrhs = 1,
-                 bool x_shared = false);
+                     cudaStream_t st);
+void launch_solve_start(const double* mass, const double* f, const double* y, double* f0, const int n[3], int dim,
+                        double* r, float* r32, double* x, double* p, double* q, double* part, double* S,
+                        unsigned* ticket, cudaStream_t st, int nrhs);
+// v = g on the boundary, 0 inside; y = 0
+void launch_boundary_only(const double* g, double* v, double* y, const int n[3], int dim, cudaStream_t st);
+// u = x + v for nrhs vectors of n values, v the same for all
+void launch_sum(double* u, const double* x, const double* v, long long n, cudaStream_t st, int nrhs = 1);
 // GMRES: h[j] = V_j . w (j < k1, deterministic, part holds 64 k1 partials);
 // w += sign sum_j h[j] V_j; out = in / sqrt(nrm2[0]).
 void launch_multidot(const double* V, long long ld, int k1, const double* w, long long n, double* part, double* h,

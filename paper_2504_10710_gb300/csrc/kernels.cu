@@ -773,6 +773,24 @@ __global__ void zero_boundary_kernel(T* v, int3 n, int dim, int nrhs) {
         if (on_boundary(i % total, nn, dim)) v[i] = T(0);
 }
 
+// Elements per thread per trip of the vector kernels' grid-stride loops.
+constexpr int kVecU = 4;
+
+// Load that stays where it is written.  The vector kernels read all values of
+// a trip before they use or overwrite any; left to itself the compiler moved
+// loads down to their uses, past stores that the later ones then had to wait
+// for (1.44 M nodes, 32 right-hand sides, the dots: 1263 against 307 us).
+__device__ __forceinline__ double ld_first(const double* p) {
+    double v;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ float ld_first(const float* p) {
+    float v;
+    asm volatile("ld.global.f32 %0, [%1];" : "=f"(v) : "l"(p) : "memory");
+    return v;
+}
+
 __global__ void __launch_bounds__(256) dots_kernel(const double* __restrict__ a0, const double* __restrict__ b0,
                                                    const double* __restrict__ a1, const double* __restrict__ b1,
                                                    int ndots, long long n, double* part, double* S, int slot0,
@@ -790,7 +808,7 @@ __global__ void __launch_bounds__(256) dots_kernel(const double* __restrict__ a0
     part += j * ndots * gridDim.x;
     S += j * S_COUNT;
     if (ticket) ticket += j;
-    __shared__ double red[32];
+    __shared__ double red[kReduceThreads];
     double s0 = 0.0, s1 = 0.0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
         s0 += a0[i] * b0[i];
@@ -811,8 +829,6 @@ __global__ void __launch_bounds__(256) dots_kernel(const double* __restrict__ a0
     }
 }
 
-// Elements per thread per trip of the FCG vector kernels' grid-stride loops.
-constexpr int kVecU = 4;
 
 // Sum of n partials in a fixed order (every block gets the same value);
 // valid in thread 0.
@@ -832,39 +848,57 @@ __device__ __forceinline__ double sum_partials(const double* part, int n, double
     return block_sum(s, red);
 }
 
-// Outer-iteration dots, grid-stride over kDotBlocks CTAs: per-block partials
-// of r.z into prz and of z.q into pzq (summed by the consumers); z is taken
-// from z32 when given (z = double(z32)); q is reset to 0 after it is read.
-__device__ __forceinline__ void dots_rz_zq_body(const double* __restrict__ r, double* __restrict__ z,
+// The values of one trip of up to M vectors.
+template <int M>
+struct Trip {
+    double v[M][kVecU];
+};
+
+// AHEAD (below): the next trip's values are loaded before the current ones are
+// used.  One right-hand side has two CTAs of these kernels per SM, and a
+// trip's latency is all it waits for (update, 1.44 M nodes: 53 us without);
+// with several the SMs are full and the registers are worth more resident CTAs
+// (32 right-hand sides: 463 against 662 us with it).  The sums are the same.
+
+// Outer-iteration dots, grid-stride over the CTAs: per-block partials of r.z
+// into prz and of z.q into pzq (summed by the consumers); z is z32 where given
+// (MIXED; double(z32) is exact, so no FP64 copy of it is kept); q is reset to 0
+// after it is read.
+template <bool MIXED, bool AHEAD>
+__device__ __forceinline__ void dots_rz_zq_body(const double* __restrict__ r, const double* __restrict__ z,
                                                 const float* __restrict__ z32, double* __restrict__ q, long long n,
                                                 double* __restrict__ prz, double* __restrict__ pzq) {
-    __shared__ double red[32];
+    __shared__ double red[kReduceThreads];
     double s0 = 0.0, s1 = 0.0;
     // kVecU elements per thread per trip, all loads issued before use (same
     // summation order as a plain grid-stride loop)
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i0 = blockIdx.x * (long long)blockDim.x + threadIdx.x; i0 < n; i0 += kVecU * stride) {
-        double rv[kVecU], zv[kVecU], qv[kVecU];
+    Trip<3> cur, nxt;
+    auto load = [&](Trip<3>& t, long long i0) {
 #pragma unroll
         for (int u = 0; u < kVecU; ++u) {
             const long long i = i0 + u * stride;
-            rv[u] = zv[u] = qv[u] = 0.0;
-            if (i < n) {
-                rv[u] = r[i];
-                zv[u] = z32 ? (double)z32[i] : z[i];
-                qv[u] = q[i];
-            }
+            const bool ok = i < n;
+            t.v[0][u] = ok ? ld_first(r + i) : 0.0;
+            t.v[1][u] = ok ? (MIXED ? (double)ld_first(z32 + i) : ld_first(z + i)) : 0.0;
+            t.v[2][u] = ok ? ld_first(q + i) : 0.0;
         }
+    };
+    const long long ifirst = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    if (AHEAD) load(cur, ifirst);
+    for (long long i0 = ifirst; i0 < n; i0 += kVecU * stride) {
+        if (AHEAD) load(nxt, i0 + kVecU * stride);
+        else load(cur, i0);
 #pragma unroll
         for (int u = 0; u < kVecU; ++u) {
             const long long i = i0 + u * stride;
             if (i < n) {
-                if (z32) z[i] = zv[u];
-                s0 += rv[u] * zv[u];
-                s1 += zv[u] * qv[u];
+                s0 += cur.v[0][u] * cur.v[1][u];
+                s1 += cur.v[1][u] * cur.v[2][u];
                 q[i] = 0.0;
             }
         }
+        if (AHEAD) cur = nxt;
     }
     const double t0 = block_sum(s0, red);
     if (threadIdx.x == 0) prz[blockIdx.x] = t0;
@@ -872,49 +906,48 @@ __device__ __forceinline__ void dots_rz_zq_body(const double* __restrict__ r, do
     if (threadIdx.x == 0) pzq[blockIdx.x] = t1;
 }
 
-__global__ void __launch_bounds__(256) dots_rz_zq_kernel(const double* __restrict__ r, double* __restrict__ z,
+template <bool MIXED, bool AHEAD>
+__global__ void __launch_bounds__(256, AHEAD ? 2 : 4) dots_rz_zq_kernel(const double* __restrict__ r, const double* __restrict__ z,
                                                          const float* __restrict__ z32, double* __restrict__ q,
                                                          long long n, double* __restrict__ prz,
                                                          double* __restrict__ pzq) {
     grid_dep_sync();
     const long long jr = blockIdx.y;       // right-hand side
-    dots_rz_zq_body(r + jr * n, z + jr * n, z32 ? z32 + jr * n : nullptr, q + jr * n, n, prz + jr * gridDim.x,
-                    pzq + jr * gridDim.x);
+    dots_rz_zq_body<MIXED, AHEAD>(r + jr * n, z + jr * n, MIXED ? z32 + jr * n : nullptr, q + jr * n, n,
+                           prz + jr * gridDim.x, pzq + jr * gridDim.x);
 }
 
 // q-independent update: every block sums the partials of p.q (npq, from the
-// apply) and of r.z (nrz), alpha = r.z / p.q; x += alpha p; r -= alpha q;
+// apply), takes r.z from S_RZNEW (published by the direction), alpha = r.z / p.q; x += alpha p; r -= alpha q;
 // partials of r.r into prr; the last block publishes S_RR, S_RZ (for the next
 // direction), S_ALPHA, S_PQ and the breakdown flag.
+template <bool MIXED, bool AHEAD>
 __device__ __forceinline__ void fcg_update_body(double* __restrict__ x, double* __restrict__ r,
                                                 const double* __restrict__ p, const double* __restrict__ q,
-                                                long long n, const double* ppq, int npq, const double* prz, int nrz,
-                                                double* prr, double* S, unsigned* ticket, float* __restrict__ r32) {
+                                                long long n, const double* ppq, int npq, double* prr, double* S, unsigned* ticket, float* __restrict__ r32) {
     // a right-hand side that has stopped keeps its x and r
     const bool active = S[S_DONE] == 0.0;
-    __shared__ double red[32];
+    __shared__ double red[kReduceThreads];
     __shared__ double sh[3];
     const long long stride = (long long)gridDim.x * blockDim.x;
     const long long ifirst = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    double xv[kVecU], rv[kVecU], pv[kVecU], qv[kVecU];
-    auto load = [&](long long i0) {
+    Trip<4> cur, nxt;
+    auto load = [&](Trip<4>& t, long long i0) {
 #pragma unroll
         for (int u = 0; u < kVecU; ++u) {
             const long long i = i0 + u * stride;
-            xv[u] = rv[u] = pv[u] = qv[u] = 0.0;
-            if (i < n) {
-                xv[u] = x[i];
-                rv[u] = r[i];
-                pv[u] = p[i];
-                qv[u] = q[i];
-            }
+            const bool ok = i < n;
+            t.v[0][u] = ok ? ld_first(x + i) : 0.0;
+            t.v[1][u] = ok ? ld_first(r + i) : 0.0;
+            t.v[2][u] = ok ? ld_first(p + i) : 0.0;
+            t.v[3][u] = ok ? ld_first(q + i) : 0.0;
         }
     };
     // the first trip's vectors are in flight while the partials are summed
-    if (active) load(ifirst);
+    if (active) load(cur, ifirst);
     const double pq = sum_partials(ppq, npq, red);
-    const double rz = sum_partials(prz, nrz, red);
     if (threadIdx.x == 0) {
+        const double rz = S[S_RZNEW];
         sh[0] = rz / pq;                    // FP64 division once per block
         sh[1] = pq;
         sh[2] = rz;
@@ -923,18 +956,20 @@ __device__ __forceinline__ void fcg_update_body(double* __restrict__ x, double* 
     const double alpha = sh[0];
     double s = 0.0;
     for (long long i0 = ifirst; active && i0 < n; i0 += kVecU * stride) {
-        if (i0 != ifirst) load(i0);
+        if (AHEAD) load(nxt, i0 + kVecU * stride);
+        else if (i0 != ifirst) load(cur, i0);
 #pragma unroll
         for (int u = 0; u < kVecU; ++u) {
             const long long i = i0 + u * stride;
             if (i < n) {
-                x[i] = xv[u] + alpha * pv[u];
-                const double ri = rv[u] - alpha * qv[u];
+                x[i] = cur.v[0][u] + alpha * cur.v[2][u];
+                const double ri = cur.v[1][u] - alpha * cur.v[3][u];
                 r[i] = ri;
-                if (r32) r32[i] = (float)ri;
+                if (MIXED) r32[i] = (float)ri;
                 s += ri * ri;
             }
         }
+        if (AHEAD) cur = nxt;
     }
     const double t = block_sum(s, red);
     if (threadIdx.x == 0) prr[blockIdx.x] = t;
@@ -952,77 +987,83 @@ __device__ __forceinline__ void fcg_update_body(double* __restrict__ x, double* 
     }
 }
 
-__global__ void __launch_bounds__(256) fcg_update_kernel(double* __restrict__ x, double* __restrict__ r,
+template <bool MIXED, bool AHEAD>
+__global__ void __launch_bounds__(256, AHEAD ? 2 : 4) fcg_update_kernel(double* __restrict__ x, double* __restrict__ r,
                                                          const double* __restrict__ p, const double* __restrict__ q,
-                                                         long long n, const double* ppq, int npq, const double* prz,
-                                                         int nrz, double* prr, double* S, unsigned* ticket,
-                                                         float* __restrict__ r32) {
+                                                         long long n, const double* ppq, int npq, double* prr, double* S,
+                                                         unsigned* ticket, float* __restrict__ r32) {
     grid_dep_sync();
     const long long jr = blockIdx.y;       // right-hand side
-    fcg_update_body(x + jr * n, r + jr * n, p + jr * n, q + jr * n, n, ppq + jr * npq, npq, prz + jr * nrz, nrz,
-                    prr + jr * gridDim.x, S + jr * S_COUNT, ticket + jr, r32 ? r32 + jr * n : nullptr);
+    fcg_update_body<MIXED, AHEAD>(x + jr * n, r + jr * n, p + jr * n, q + jr * n, n, ppq + jr * npq, npq, prr + jr * gridDim.x, S + jr * S_COUNT, ticket + jr, MIXED ? r32 + jr * n : nullptr);
 }
 
 // p = z + beta p, beta = -alpha zq / rz_old (flexible) or rz_new / rz_old
 // (Fletcher-Reeves), with rz_new and zq summed from the dots' partials in
 // every block and rz_old, alpha from the previous update.
+template <bool MIXED, bool AHEAD>
 __device__ __forceinline__ void fcg_direction_body(double* __restrict__ p, const double* __restrict__ z,
-                                                   long long n, const double* prz, const double* pzq, int nd,
-                                                   const double* __restrict__ S, int flexible) {
+                                                   const float* __restrict__ z32, long long n, const double* prz,
+                                                   const double* pzq, int nd, double* S, int flexible) {
     if (S[S_DONE] != 0.0) return;           // stopped: p is no longer used
-    __shared__ double red[32];
+    __shared__ double red[kReduceThreads];
     __shared__ double sh_beta;
     const long long stride = (long long)gridDim.x * blockDim.x;
     const long long ifirst = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    double zv[kVecU], pv[kVecU];
-    auto load = [&](long long i0) {
+    Trip<2> cur, nxt;
+    auto load = [&](Trip<2>& t, long long i0) {
 #pragma unroll
         for (int u = 0; u < kVecU; ++u) {
             const long long i = i0 + u * stride;
-            zv[u] = pv[u] = 0.0;
-            if (i < n) {
-                zv[u] = z[i];
-                pv[u] = p[i];
-            }
+            const bool ok = i < n;
+            t.v[0][u] = ok ? (MIXED ? (double)ld_first(z32 + i) : ld_first(z + i)) : 0.0;
+            t.v[1][u] = ok ? ld_first(p + i) : 0.0;
         }
     };
-    load(ifirst);      // in flight while the partials are summed
+    load(cur, ifirst);      // in flight while the partials are summed
     const double rz_new = sum_partials(prz, nd, red);
     const double zq = sum_partials(pzq, nd, red);
-    if (threadIdx.x == 0) sh_beta = flexible ? -S[S_ALPHA] * zq / S[S_RZ] : rz_new / S[S_RZ];
+    if (threadIdx.x == 0) {
+        sh_beta = flexible ? -S[S_ALPHA] * zq / S[S_RZ] : rz_new / S[S_RZ];
+        if (blockIdx.x == 0) S[S_RZNEW] = rz_new;    // for the update
+    }
     __syncthreads();
     const double beta = sh_beta;
     for (long long i0 = ifirst; i0 < n; i0 += kVecU * stride) {
-        if (i0 != ifirst) load(i0);
+        if (AHEAD) load(nxt, i0 + kVecU * stride);
+        else if (i0 != ifirst) load(cur, i0);
 #pragma unroll
         for (int u = 0; u < kVecU; ++u) {
             const long long i = i0 + u * stride;
-            if (i < n) p[i] = zv[u] + beta * pv[u];
+            if (i < n) p[i] = cur.v[0][u] + beta * cur.v[1][u];
         }
+        if (AHEAD) cur = nxt;
     }
 }
 
-__global__ void __launch_bounds__(256) fcg_direction_kernel(double* __restrict__ p, const double* __restrict__ z,
-                                                            long long n, const double* prz, const double* pzq, int nd,
-                                                            const double* __restrict__ S, int flexible) {
+template <bool MIXED, bool AHEAD>
+__global__ void __launch_bounds__(256, AHEAD ? 2 : 4) fcg_direction_kernel(double* __restrict__ p, const double* __restrict__ z,
+                                                            const float* __restrict__ z32, long long n,
+                                                            const double* prz, const double* pzq, int nd, double* S,
+                                                            int flexible) {
     grid_dep_sync();
     const long long jr = blockIdx.y;       // right-hand side
-    fcg_direction_body(p + jr * n, z + jr * n, n, prz + jr * nd, pzq + jr * nd, nd, S + jr * S_COUNT, flexible);
+    fcg_direction_body<MIXED, AHEAD>(p + jr * n, z + jr * n, MIXED ? z32 + jr * n : nullptr, n, prz + jr * nd,
+                              pzq + jr * nd, nd, S + jr * S_COUNT, flexible);
 }
 
 // Work-list form of the three outer-iteration kernels: item blockIdx.y is one
 // problem (its own vectors, length, partials and scalars), kDotBlocks CTAs
 // each.  step 0: dots r.z, z.q; 1: direction; 2: update.
-__global__ void __launch_bounds__(256) fcg_list_kernel(const FcgItem* __restrict__ items, int step, int flexible) {
+template <int STEP, bool MIXED>
+__global__ void __launch_bounds__(256) fcg_list_kernel(const FcgItem* __restrict__ items, int flexible) {
     grid_dep_sync();
     const FcgItem& it = items[blockIdx.y];
-    if (step == 0)
-        dots_rz_zq_body(it.r, it.z, it.z32, it.q, it.n, it.prz, it.pzq);
-    else if (step == 1)
-        fcg_direction_body(it.p, it.z, it.n, it.prz, it.pzq, (int)gridDim.x, it.S, flexible);
+    if constexpr (STEP == 0)
+        dots_rz_zq_body<MIXED, true>(it.r, it.z, it.z32, it.q, it.n, it.prz, it.pzq);
+    else if constexpr (STEP == 1)
+        fcg_direction_body<MIXED, true>(it.p, it.z, it.z32, it.n, it.prz, it.pzq, (int)gridDim.x, it.S, flexible);
     else
-        fcg_update_body(it.x, it.r, it.p, it.q, it.n, it.ppq, it.npq, it.prz, (int)gridDim.x, it.prr, it.S,
-                        it.ticket, it.r32);
+        fcg_update_body<MIXED, true>(it.x, it.r, it.p, it.q, it.n, it.ppq, it.npq, it.prr, it.S, it.ticket, it.r32);
 }
 
 // ---- GMRES helpers (Arnoldi with classical Gram-Schmidt, twice) ----------
@@ -1031,7 +1072,7 @@ __global__ void __launch_bounds__(256) multidot_kernel(const double* __restrict_
                                                        const double* __restrict__ w, long long n,
                                                        double* part, double* h, unsigned* ticket) {
     grid_dep_sync();
-    __shared__ double red[32];
+    __shared__ double red[kReduceThreads];
     const int j = blockIdx.y;
     const double* v = V + (long long)j * ld;
     double s = 0.0;
@@ -1078,12 +1119,13 @@ __global__ void scale_by_norm_kernel(double* __restrict__ out, const double* __r
 // ends every outer iteration.
 // With several right-hand sides the loop runs while any of them is still
 // iterating; each one stops (S_DONE, S_ITS) when it converges or breaks down.
-__global__ void solve_init_kernel(double* S0, cudaGraphConditionalHandle h, double tol, int maxit, int nrhs,
-                                  int set_cond) {
+// One thread per right-hand side (or problem of a work-list group).
+constexpr int kCondThreads = 128;
+__global__ void __launch_bounds__(kCondThreads) solve_init_kernel(double* S0, cudaGraphConditionalHandle h, double tol,
+                                                                  int maxit, int nrhs, int set_cond) {
     grid_dep_sync();
-    if (threadIdx.x != 0) return;
     bool go = false;
-    for (int j = 0; j < nrhs; ++j) {
+    for (int j = threadIdx.x; j < nrhs; j += kCondThreads) {
         double* S = S0 + (long long)j * S_COUNT;
         const double rr0 = S[S_RR0];
         S[S_RR] = rr0;
@@ -1096,71 +1138,138 @@ __global__ void solve_init_kernel(double* S0, cudaGraphConditionalHandle h, doub
         S[S_PQ] = 0.0;
         S[S_RZNEW] = 0.0;
         S[S_ITS] = 0.0;
-        S[S_DONE] = 0.0;
+        double done = 0.0;
         if (!isfinite(rr0)) {
             S[S_FLAG] = 1.0;
-            S[S_DONE] = 2.0;
+            done = 2.0;
         } else if (!(rr0 > 0.0)) {
-            S[S_DONE] = 1.0;
+            done = 1.0;
         }
-        go = go || S[S_DONE] == 0.0;
+        S[S_DONE] = done;
+        go = go || done == 0.0;
     }
-    if (set_cond) cudaGraphSetConditional(h, go && maxit > 0 ? 1u : 0u);
+    const int any = __syncthreads_or(go ? 1 : 0);
+    if (set_cond && threadIdx.x == 0) cudaGraphSetConditional(h, any && maxit > 0 ? 1u : 0u);
 }
 
-__global__ void solve_cond_kernel(double* S0, cudaGraphConditionalHandle h, int maxit, int nrhs, int set_cond) {
+__global__ void __launch_bounds__(kCondThreads) solve_cond_kernel(double* S0, cudaGraphConditionalHandle h, int maxit,
+                                                                  int nrhs, int set_cond) {
     grid_dep_sync();
-    if (threadIdx.x != 0) return;
-    bool any = false;
-    double it = 0.0;
-    for (int j = 0; j < nrhs; ++j) {
+    bool go = false;
+    for (int j = threadIdx.x; j < nrhs; j += kCondThreads) {
         double* S = S0 + (long long)j * S_COUNT;
-        it = S[S_ITER] + 1.0;
+        const double it = S[S_ITER] + 1.0, done = S[S_DONE], rr = S[S_RR], flag = S[S_FLAG], tol2 = S[S_TOL2];
         S[S_ITER] = it;
-        if (S[S_DONE] != 0.0) continue;
-        const double rr = S[S_RR];
-        if (!isfinite(rr) || S[S_FLAG] != 0.0) {
+        if (done != 0.0) continue;
+        if (!isfinite(rr) || flag != 0.0) {
             S[S_FLAG] = 1.0;
             S[S_DONE] = 2.0;
             S[S_ITS] = it;
-        } else if (rr <= S[S_TOL2]) {
+        } else if (rr <= tol2) {
             S[S_DONE] = 1.0;
             S[S_ITS] = it;
         } else {
-            any = true;
+            go = go || it < (double)maxit;
         }
     }
-    if (set_cond) cudaGraphSetConditional(h, any && it < (double)maxit ? 1u : 0u);
+    const int any = __syncthreads_or(go ? 1 : 0);
+    if (set_cond && threadIdx.x == 0) cudaGraphSetConditional(h, any ? 1u : 0u);
 }
 
 // f and f0 hold nrhs vectors; mass and y (A v of the shared lifting) one.
-__global__ void lift_rhs_kernel(const double* __restrict__ mass, const double* __restrict__ f,
-                                const double* __restrict__ y, double* __restrict__ f0, int3 n, int dim, int nrhs) {
+// With r given (the start of a solve) also r = f0, r32 = float(f0), x = p = q
+// = 0 and the partials of r.r per right-hand side blockIdx.y, added by its
+// last block into S_RR0: one pass instead of a copy, a cast, three memsets and
+// a dot.
+struct SolveStart {
+    double *r = nullptr, *x = nullptr, *p = nullptr, *q = nullptr;
+    float* r32 = nullptr;
+    double *part = nullptr, *S = nullptr;
+    unsigned* ticket = nullptr;
+};
+__global__ void __launch_bounds__(256) lift_rhs_kernel(const double* __restrict__ mass, const double* __restrict__ f,
+                                                       const double* __restrict__ y, double* __restrict__ f0, int3 n,
+                                                       int dim, SolveStart st) {
+    __shared__ double red[kReduceThreads];
     grid_dep_sync();
-    const long long total = (long long)n.x * n.y * n.z;
-    const int nn[3] = {n.x, n.y, n.z};
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total * nrhs;
-         i += (long long)gridDim.x * blockDim.x) {
-        const long long li = i % total;
-        f0[i] = on_boundary(li, nn, dim) ? 0.0 : mass[li] * f[i] - y[li];
+    const int total = n.x * n.y * n.z;
+    const long long o = (long long)blockIdx.y * total;
+    const int stride = (int)(gridDim.x * blockDim.x);
+    double s = 0.0;
+    for (int i0 = blockIdx.x * (int)blockDim.x + threadIdx.x; i0 < total; i0 += kVecU * stride) {
+        double m[kVecU], fv[kVecU], yv[kVecU];
+#pragma unroll
+        for (int u = 0; u < kVecU; ++u) {
+            const int i = i0 + u * stride;
+            m[u] = fv[u] = yv[u] = 0.0;
+            if (i < total) {
+                m[u] = ld_first(mass + i);
+                fv[u] = ld_first(f + o + i);
+                yv[u] = ld_first(y + i);
+            }
+        }
+#pragma unroll
+        for (int u = 0; u < kVecU; ++u) {
+            const int i = i0 + u * stride;
+            if (i >= total) break;
+            const int row = i / n.x, I = i - row * n.x, K = row / n.y, J = row - K * n.y;
+            const bool bd = I == 0 || I == n.x - 1 || J == 0 || J == n.y - 1 || (dim == 3 && (K == 0 || K == n.z - 1));
+            const double v = bd ? 0.0 : m[u] * fv[u] - yv[u];
+            f0[o + i] = v;
+            if (st.r) {
+                st.r[o + i] = v;
+                st.x[o + i] = 0.0;
+                st.p[o + i] = 0.0;
+                st.q[o + i] = 0.0;
+                if (st.r32) st.r32[o + i] = (float)v;
+                s += v * v;
+            }
+        }
+    }
+    if (!st.r) return;
+    double* part = st.part + (long long)blockIdx.y * gridDim.x;
+    const double t = block_sum(s, red);
+    if (threadIdx.x == 0) part[blockIdx.x] = t;
+    unsigned* ticket = st.ticket + blockIdx.y;
+    if (last_block(ticket)) {
+        finalize_partials(part, 1, gridDim.x, st.S + (long long)blockIdx.y * S_COUNT, S_RR0, S_RR0, red);
+        if (threadIdx.x == 0) *ticket = 0u;
     }
 }
 
-__global__ void boundary_only_kernel(const double* __restrict__ g, double* __restrict__ v, int3 n, int dim) {
+// v = g on the boundary, 0 inside; y = 0 (the lifting's A v accumulates there)
+__global__ void boundary_only_kernel(const double* __restrict__ g, double* __restrict__ v, double* __restrict__ y,
+                                     int3 n, int dim) {
     grid_dep_sync();
-    const long long total = (long long)n.x * n.y * n.z;
-    const int nn[3] = {n.x, n.y, n.z};
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x)
-        v[i] = on_boundary(i, nn, dim) ? g[i] : 0.0;
+    const int total = n.x * n.y * n.z;
+    for (int i = blockIdx.x * (int)blockDim.x + threadIdx.x; i < total; i += (int)(gridDim.x * blockDim.x)) {
+        const int row = i / n.x, I = i - row * n.x, K = row / n.y, J = row - K * n.y;
+        const bool bd = I == 0 || I == n.x - 1 || J == 0 || J == n.y - 1 || (dim == 3 && (K == 0 || K == n.z - 1));
+        v[i] = bd ? g[i] : 0.0;
+        y[i] = 0.0;
+    }
 }
 
-// y (nrhs vectors of n values) += a x; x one vector for all when x_shared
-__global__ void axpy_kernel(double* __restrict__ y, const double* __restrict__ x, double a, long long n, int nrhs,
-                            int x_shared) {
+// u = x + v for nrhs vectors of n values (v one vector for all)
+__global__ void sum_kernel(double* __restrict__ u, const double* __restrict__ x, const double* __restrict__ v,
+                           int n) {
     grid_dep_sync();
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n * nrhs;
-         i += (long long)gridDim.x * blockDim.x)
-        y[i] += a * x[x_shared ? i % n : i];
+    const long long o = (long long)blockIdx.y * n;
+    const int stride = (int)(gridDim.x * blockDim.x);
+    for (int i0 = blockIdx.x * (int)blockDim.x + threadIdx.x; i0 < n; i0 += kVecU * stride) {
+        double xv[kVecU], vv[kVecU];
+#pragma unroll
+        for (int k = 0; k < kVecU; ++k) {
+            const int i = i0 + k * stride;
+            xv[k] = i < n ? ld_first(x + o + i) : 0.0;
+            vv[k] = i < n ? ld_first(v + i) : 0.0;
+        }
+#pragma unroll
+        for (int k = 0; k < kVecU; ++k) {
+            const int i = i0 + k * stride;
+            if (i < n) u[o + i] = xv[k] + vv[k];
+        }
+    }
 }
 
 inline int grid_for(long long n, int threads = 256) {
@@ -1366,9 +1475,13 @@ void launch_bcr_list(bool forward, int l, const BcrItem<T>* items, const int* st
     launch_k(bcr_list_kernel<T>, blocks, 256, smem, st, items, start, nitems, l, forward ? 1 : 0);
 }
 
-void launch_fcg_list(int step, const FcgItem* items, int nitems, int flexible, int blocks, cudaStream_t st) {
+void launch_fcg_list(int step, const FcgItem* items, int nitems, int flexible, int blocks, bool mixed,
+                     cudaStream_t st) {
     if (nitems < 1) return;
-    launch_k(fcg_list_kernel, dim3(blocks, nitems), 256, 0, st, items, step, flexible);
+    const dim3 grid(blocks, nitems);
+    if (step == 0) launch_k(mixed ? fcg_list_kernel<0, true> : fcg_list_kernel<0, false>, grid, 256, 0, st, items, flexible);
+    else if (step == 1) launch_k(mixed ? fcg_list_kernel<1, true> : fcg_list_kernel<1, false>, grid, 256, 0, st, items, flexible);
+    else launch_k(mixed ? fcg_list_kernel<2, true> : fcg_list_kernel<2, false>, grid, 256, 0, st, items, flexible);
 }
 
 template bool transfer2_list_config<float>(const DevBand<float>&, const DevBand<float>&, const int*, int*, int*, int*,
@@ -1429,33 +1542,55 @@ void launch_dots(const double* a0, const double* b0, const double* a1, const dou
              0);
 }
 
+// The instance for MIXED (mixed) and AHEAD (ahead).
+template <typename K>
+K* pick_vector(bool mixed, bool ahead, K* none, K* m, K* a, K* both) {
+    return mixed ? (ahead ? both : m) : (ahead ? a : none);
+}
+
 void launch_fcg_update(double* x, double* r, const double* p, const double* q, long long n, const double* ppq,
-                       int npq, const double* prz, int nrz, double* prr, double* S, unsigned* ticket, float* r32,
-                       cudaStream_t st, int nrhs) {
-    // nrz: the dots' CTA count, the same grid here (prr gets one partial per CTA)
-    launch_k(fcg_update_kernel, dim3(nrz, nrhs), 256, 0, st, x, r, p, q, n, ppq, npq, prz, nrz, prr, S, ticket, r32);
+                       int npq, int nb, double* prr, double* S, unsigned* ticket, float* r32, cudaStream_t st,
+                       int nrhs) {
+    launch_k(pick_vector(r32 != nullptr, nrhs == 1, fcg_update_kernel<false, false>, fcg_update_kernel<true, false>,
+                         fcg_update_kernel<false, true>, fcg_update_kernel<true, true>), dim3(nb, nrhs), 256, 0, st, x, r, p, q, n, ppq,
+             npq, prr, S, ticket, r32);
 }
 
-void launch_dots_rz_zq(const double* r, double* z, const float* z32, double* q, long long n, double* prz, double* pzq,
-                       cudaStream_t st, int nrhs) {
-    launch_k(dots_rz_zq_kernel, dim3(fcg_blocks(n), nrhs), 256, 0, st, r, z, z32, q, n, prz, pzq);
+void launch_dots_rz_zq(const double* r, const double* z, const float* z32, double* q, long long n, double* prz,
+                       double* pzq, cudaStream_t st, int nrhs) {
+    launch_k(pick_vector(z32 != nullptr, nrhs == 1, dots_rz_zq_kernel<false, false>, dots_rz_zq_kernel<true, false>,
+                         dots_rz_zq_kernel<false, true>, dots_rz_zq_kernel<true, true>), dim3(fcg_blocks(n), nrhs), 256, 0, st, r, z, z32,
+             q, n, prz, pzq);
 }
 
-void launch_fcg_direction(double* p, const double* z, long long n, const double* prz, const double* pzq, int nd,
-                          const double* S, int flexible, cudaStream_t st, int nrhs) {
-    launch_k(fcg_direction_kernel, dim3(nd, nrhs), 256, 0, st, p, z, n, prz, pzq, nd, S, flexible);
+void launch_fcg_direction(double* p, const double* z, const float* z32, long long n, const double* prz,
+                          const double* pzq, int nd, double* S, int flexible, cudaStream_t st, int nrhs) {
+    launch_k(pick_vector(z32 != nullptr, nrhs == 1, fcg_direction_kernel<false, false>, fcg_direction_kernel<true, false>,
+                         fcg_direction_kernel<false, true>, fcg_direction_kernel<true, true>), dim3(nd, nrhs), 256, 0, st, p, z, z32, n, prz,
+             pzq, nd, S, flexible);
 }
 
 void launch_lift_rhs(const double* mass, const double* f, const double* y, double* f0, const int n[3], int dim,
-                     cudaStream_t st, int nrhs) {
-    const long long total = (long long)n[0] * n[1] * n[2];
-    launch_k(lift_rhs_kernel, grid_for(total * nrhs), 256, 0, st, mass, f, y, f0, make_int3(n[0], n[1], n[2]), dim,
-             nrhs);
+                     cudaStream_t st) {
+    launch_k(lift_rhs_kernel, grid_for((long long)n[0] * n[1] * n[2]), 256, 0, st, mass, f, y, f0,
+             make_int3(n[0], n[1], n[2]), dim, SolveStart());
 }
 
-void launch_boundary_only(const double* g, double* v, const int n[3], int dim, cudaStream_t st) {
-    const long long total = (long long)n[0] * n[1] * n[2];
-    launch_k(boundary_only_kernel, grid_for(total), 256, 0, st, g, v, make_int3(n[0], n[1], n[2]), dim);
+void launch_solve_start(const double* mass, const double* f, const double* y, double* f0, const int n[3], int dim,
+                        double* r, float* r32, double* x, double* p, double* q, double* part, double* S,
+                        unsigned* ticket, cudaStream_t st, int nrhs) {
+    const SolveStart s{r, x, p, q, r32, part, S, ticket};
+    launch_k(lift_rhs_kernel, dim3(fcg_blocks((long long)n[0] * n[1] * n[2]), nrhs), 256, 0, st, mass, f, y, f0,
+             make_int3(n[0], n[1], n[2]), dim, s);
+}
+
+void launch_boundary_only(const double* g, double* v, double* y, const int n[3], int dim, cudaStream_t st) {
+    launch_k(boundary_only_kernel, grid_for((long long)n[0] * n[1] * n[2]), 256, 0, st, g, v, y,
+             make_int3(n[0], n[1], n[2]), dim);
+}
+
+void launch_sum(double* u, const double* x, const double* v, long long n, cudaStream_t st, int nrhs) {
+    launch_k(sum_kernel, dim3(grid_for(n), nrhs), 256, 0, st, u, x, v, (int)n);
 }
 
 void launch_multidot(const double* V, long long ld, int k1, const double* w, long long n, double* part, double* h,
@@ -1476,16 +1611,12 @@ void launch_scale_by_norm(double* out, const double* in, const double* nrm2, lon
 
 void launch_solve_init(double* S, cudaGraphConditionalHandle h, double tol, int maxit, cudaStream_t st, int nrhs,
                        bool set_cond) {
-    launch_k(solve_init_kernel, 1, 32, 0, st, S, h, tol, maxit, nrhs, set_cond ? 1 : 0);
+    launch_k(solve_init_kernel, 1, kCondThreads, 0, st, S, h, tol, maxit, nrhs, set_cond ? 1 : 0);
 }
 
 void launch_solve_cond(double* S, cudaGraphConditionalHandle h, int maxit, cudaStream_t st, int nrhs,
                        bool set_cond) {
-    launch_k(solve_cond_kernel, 1, 32, 0, st, S, h, maxit, nrhs, set_cond ? 1 : 0);
-}
-
-void launch_axpy(double* y, const double* x, double a, long long n, cudaStream_t st, int nrhs, bool x_shared) {
-    launch_k(axpy_kernel, grid_for(n * nrhs), 256, 0, st, y, x, a, n, nrhs, x_shared ? 1 : 0);
+    launch_k(solve_cond_kernel, 1, kCondThreads, 0, st, S, h, maxit, nrhs, set_cond ? 1 : 0);
 }
 
 bool pdl_enabled() {

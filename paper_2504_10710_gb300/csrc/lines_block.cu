@@ -250,16 +250,13 @@ struct SegOp {
     }
 };
 
-// The right-hand side of a CTA (fastest in the CTA order, see device.cuh: the
-// nrhs CTAs of one line group read the same segment operators) and its lines.
+// First line of CTA `blk` and the offset of its right-hand side's vectors (the
+// right-hand side fastest in the CTA order, see device.cuh: the nrhs CTAs of
+// one line group read the same segment operators).
 template <typename T>
-__device__ __forceinline__ int enter(BlockLineArgs<T>& A, int blk) {
+__device__ __forceinline__ int enter(const BlockLineArgs<T>& A, int blk, long long& vo) {
     const int rhs = A.nrhs == 1 ? 0 : blk % A.nrhs, bx = A.nrhs == 1 ? blk : blk / A.nrhs;
-    const long long vo = (long long)rhs * A.N;
-    if (A.g) A.g += vo;
-    if (A.r) A.r += vo;
-    if (A.y) A.y += vo;
-    A.x += vo;
+    vo = (long long)rhs * A.N;
     return bx * A.lpc;
 }
 
@@ -268,14 +265,18 @@ __device__ __forceinline__ int enter(BlockLineArgs<T>& A, int blk) {
 // interior nodes and adds into element-boundary ones).  MODE 2: x += alpha
 // B^-1 r.  MODE 3: x = alpha B^-1 r.
 template <typename T, int P, int C, bool CONTIG>
-__device__ __forceinline__ void line_seg_body(BlockLineArgs<T>& A, int blk) {
+__device__ __forceinline__ void line_seg_body(const BlockLineArgs<T>& A, int blk) {
     constexpr int MI = SegOp<T, P>::MI;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int E = A.E, LPC = A.lpc, SE = E | 1, mode = A.mode;
     T* sh = reinterpret_cast<T*>(smem_raw);   // [LPC][SE]
     T* sdr = sh + LPC * SE;                   // [LPC][SE]
     T* so = sdr + LPC * SE;                   // [padk(LPC n)]: new x (CONTIG)
-    const int l0 = enter(A, blk);
+    long long vo;
+    const int l0 = enter(A, blk, vo);
+    const T* src = (mode == 0 ? A.g : A.r) + vo;
+    T* const yp = mode == 1 ? A.y + vo : nullptr;
+    T* const xp = A.x + vo;
     const int Wc = min(LPC, A.nlines - l0);
     const int tid = threadIdx.x;
     // this thread's line w and segment e: segments adjacent for x-lines,
@@ -305,7 +306,6 @@ __device__ __forceinline__ void line_seg_body(BlockLineArgs<T>& A, int blk) {
     T gi[MI], xi[MI], gv = T(0), xv = T(0);
     const bool vertex = act && e > 0;
     // one branch per mode, so that a thread's loads are issued back to back
-    const T* src = mode == 0 ? A.g : A.r;
 #pragma unroll
     for (int i = 0; i < MI; ++i) gi[i] = xi[i] = T(0);
     if (act) {
@@ -314,19 +314,19 @@ __device__ __forceinline__ void line_seg_body(BlockLineArgs<T>& A, int blk) {
         for (int i = 0; i < MI; ++i) gi[i] = src[v0 + (i + 1) * stride];
         if (mode == 1) {
             T yi[MI], yv = T(0);
-            if (vertex) yv = A.y[v0];
+            if (vertex) yv = yp[v0];
 #pragma unroll
-            for (int i = 0; i < MI; ++i) yi[i] = A.y[v0 + (i + 1) * stride];
-            if (vertex) xv = A.x[v0];
+            for (int i = 0; i < MI; ++i) yi[i] = yp[v0 + (i + 1) * stride];
+            if (vertex) xv = xp[v0];
 #pragma unroll
-            for (int i = 0; i < MI; ++i) xi[i] = A.x[v0 + (i + 1) * stride];
+            for (int i = 0; i < MI; ++i) xi[i] = xp[v0 + (i + 1) * stride];
             gv -= yv;
 #pragma unroll
             for (int i = 0; i < MI; ++i) gi[i] -= yi[i];
         } else if (mode == 2) {
-            if (vertex) xv = A.x[v0];
+            if (vertex) xv = xp[v0];
 #pragma unroll
-            for (int i = 0; i < MI; ++i) xi[i] = A.x[v0 + (i + 1) * stride];
+            for (int i = 0; i < MI; ++i) xi[i] = xp[v0 + (i + 1) * stride];
         }
     }
     T z[MI], nl = T(0), nr = T(0);
@@ -354,12 +354,12 @@ __device__ __forceinline__ void line_seg_body(BlockLineArgs<T>& A, int blk) {
 #pragma unroll
         for (int i = 0; i < MI; ++i) {
             const int node = v0 + (i + 1) * stride;
-            A.x[node] = xi[i] + scale * (z[i] - (op.left(i) * nl + op.right(i) * nr));
-            if (seam) A.y[node] = T(0);
+            xp[node] = xi[i] + scale * (z[i] - (op.left(i) * nl + op.right(i) * nr));
+            if (seam) yp[node] = T(0);
         }
         if (vertex) {
-            A.x[v0] = xv + scale * nl;
-            if (mode == 1) A.y[v0] = T(0);
+            xp[v0] = xv + scale * nl;
+            if (mode == 1) yp[v0] = T(0);
         }
     } else {
         // a segment's nodes are adjacent: through shared memory, so that whole
@@ -371,11 +371,11 @@ __device__ __forceinline__ void line_seg_body(BlockLineArgs<T>& A, int blk) {
                 so[padk(k0 + i)] = xi[i] + scale * (z[i] - (op.left(i) * nl + op.right(i) * nr));
             if (vertex) {
                 so[padk(k0 - 1)] = xv + scale * nl;
-                if (mode == 1) A.y[v0] = T(0);
+                if (mode == 1) yp[v0] = T(0);
             }
             if (seam) {
 #pragma unroll
-                for (int i = 0; i < MI; ++i) A.y[v0 + i + 1] = T(0);
+                for (int i = 0; i < MI; ++i) yp[v0 + i + 1] = T(0);
             }
         }
         __syncthreads();
@@ -394,7 +394,7 @@ __device__ __forceinline__ void line_seg_body(BlockLineArgs<T>& A, int blk) {
                     row -= A.m1;
                     ++plane;
                 }
-                A.x[(row + 1) * A.st1 + (plane + 1) * A.st2 + 1 + idx - wl * n] = so[padk(idx)];
+                xp[(row + 1) * A.st1 + (plane + 1) * A.st2 + 1 + idx - wl * n] = so[padk(idx)];
             }
         }
     }
@@ -403,7 +403,7 @@ __device__ __forceinline__ void line_seg_body(BlockLineArgs<T>& A, int blk) {
 // Any order and line length: the line values and the segment operators in
 // shared memory (cp.async), z accumulated there.
 template <typename T, int C>
-__device__ __forceinline__ void line_any_body(BlockLineArgs<T>& A, int blk) {
+__device__ __forceinline__ void line_any_body(BlockLineArgs<T> A, int blk) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n = A.n, E = A.E, span = A.span, mode = A.mode, LPC = A.lpc, SE = E | 1;
     const int p = A.p, mi = p - 1, npk = mi * (mi + 1) / 2;
@@ -415,7 +415,12 @@ __device__ __forceinline__ void line_any_body(BlockLineArgs<T>& A, int blk) {
     T* sh = sz + LPC * span;                  // [LPC][SE]
     T* sdr = sh + LPC * SE;                   // [LPC][SE]
     T* sop = sdr + LPC * SE;                  // [ncoef][threads of the item]: segment operators
-    const int l0 = enter(A, blk);
+    long long vo;
+    const int l0 = enter(A, blk, vo);
+    if (A.g) A.g += vo;
+    if (A.r) A.r += vo;
+    if (A.y) A.y += vo;
+    A.x += vo;
     const int Wc = min(LPC, A.nlines - l0);
     const int tid = threadIdx.x;
     auto line_base = [&](int w) {
@@ -535,7 +540,7 @@ __device__ __forceinline__ void line_any_body(BlockLineArgs<T>& A, int blk) {
 }
 
 template <typename T, int P, int CV, bool CONTIG>
-__device__ __forceinline__ void line_block_body(BlockLineArgs<T>& A, int blk) {
+__device__ __forceinline__ void line_block_body(const BlockLineArgs<T>& A, int blk) {
     if constexpr (P == 0) line_any_body<T, CV>(A, blk);
     else line_seg_body<T, P, CV, CONTIG>(A, blk);
 }
@@ -548,8 +553,7 @@ constexpr int line_min_ctas() {
 
 template <typename T, int P, int CV, bool CONTIG>
 __global__ void __launch_bounds__(kBlockThreads, line_min_ctas<T, P>())
-    line_block_kernel(const __grid_constant__ BlockLineArgs<T> A0) {
-    BlockLineArgs<T> A = A0;
+    line_block_kernel(const __grid_constant__ BlockLineArgs<T> A) {
     line_block_body<T, P, CV, CONTIG>(A, blockIdx.x);
 }
 
@@ -559,8 +563,7 @@ template <typename T, int P, int CV, bool CONTIG>
 __global__ void __launch_bounds__(kBlockThreads, line_min_ctas<T, P>())
     line_block_list_kernel(const BlockLineArgs<T>* __restrict__ items, const int* __restrict__ start, int nitems) {
     const int j = work_item(start, nitems, blockIdx.x);
-    BlockLineArgs<T> A = items[j];
-    line_block_body<T, P, CV, CONTIG>(A, blockIdx.x - start[j]);
+    line_block_body<T, P, CV, CONTIG>(items[j], blockIdx.x - start[j]);
 }
 
 // Shared memory of a CTA of lpc lines: the vertex arrays, with the line

@@ -1,5 +1,4 @@
-// Block-level FP64 reductions shared by the kernels: a warp-shuffle block
-// sum, the "last block" ticket, and the fixed-order sum of block partials
+// Block-level FP64 reductions shared by the kernels: a block sum, the "last block" ticket, and the fixed-order sum of block partials
 // (results do not depend on block scheduling).
 #pragma once
 #include <cuda_runtime.h>
@@ -7,15 +6,22 @@
 namespace glls {
 namespace {
 
+// Block sum of one FP64 value per thread (blockDim.x a multiple of 32, at most
+// kReduceThreads; red: as many doubles).  The values go through shared memory
+// and warp 0 adds lane l's values l, l + 32, ... in that order, then its
+// shuffle tree: GB300 issues a warp's FP64 add over 16 cycles, and a shuffle
+// tree in every warp (40 adds for 256 threads instead of 13) was a visible
+// share of the outer-iteration kernels.
+constexpr int kReduceThreads = 256;
 __device__ __forceinline__ double block_sum(double v, double* red) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    __syncthreads();
-    if (lane == 0) red[warp] = v;
+    __syncthreads();                        // red may still be read from the last sum
+    red[threadIdx.x] = v;
     __syncthreads();
     double s = 0.0;
-    if (threadIdx.x == 0)
-        for (int w = 0; w < (int)(blockDim.x / 32); ++w) s += red[w];
+    if (threadIdx.x < 32) {
+        for (int i = threadIdx.x; i < (int)blockDim.x; i += 32) s += red[i];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    }
     return s;   // valid in thread 0
 }
 
