@@ -294,6 +294,8 @@ glls_status upload_levels(glls_problem* P, const std::vector<LevelHost>& H, bool
                     ds[k]->width = bs[k]->width;
                     ds[k]->span32 = band_span(*bs[k], 32);
                     ds[k]->span8 = band_span(*bs[k], 8);
+                    ds[k]->chunk = std::max(1, (bs[k]->rows - 1) / h.ne[a]);
+                    ds[k]->spanc = band_span(*bs[k], ds[k]->chunk);
                     CK(P->upload(&ds[k]->start, bs[k]->start));
                     CK(P->upload(&ds[k]->coef, bs[k]->coef));
                 }
@@ -355,12 +357,14 @@ void restrict_residual(glls_problem* P, int l, const T* r, const T* y, T* rc, cu
     auto& Ls = levels_of<T>(P);
     const DevLevel<T>& F = Ls[l].dev;
     const DevLevel<T>& C = Ls[l - 1].dev;
-    // axes 0 and 1 in one fused launch (then axis 2 in 3-D)
-    const int mid[3] = {C.n[0], C.n[1], F.n[2]};
-    const bool only2 = F.dim == 2;
-    if (launch_transfer2<T>(F.R[0], F.R[1], F.n, mid, r, y, only2 ? rc : Ls[l].t1, false, only2, st, nullptr,
-                            nrhs)) {
-        if (!only2) launch_transfer<T>(F.R[2], 2, mid, C.n, Ls[l].t1, nullptr, rc, false, true, st, nullptr, nrhs);
+    // axes 0 and 1 in one fused launch; in 3-D axis 2 before them, which reads r
+    // and y once in whole planes and leaves them the coarse planes only
+    if (F.dim == 2) {
+        if (launch_transfer2<T>(F.R[0], F.R[1], F.n, C.n, r, y, rc, false, true, st, nullptr, nrhs)) return;
+    } else if (transfer2_fits<T>(F.R[0], F.R[1])) {
+        const int mid[3] = {F.n[0], F.n[1], C.n[2]};
+        launch_transfer<T>(F.R[2], 2, F.n, mid, r, y, Ls[l].t1, false, false, st, nullptr, nrhs);
+        launch_transfer2<T>(F.R[0], F.R[1], mid, C.n, Ls[l].t1, nullptr, rc, false, true, st, nullptr, nrhs, true);
         return;
     }
     int cur[3] = {F.n[0], F.n[1], F.n[2]};

@@ -21,6 +21,7 @@
 #include "device.cuh"
 #include "reduce.cuh"
 
+#include <algorithm>
 #include <climits>
 #include <cstdio>
 #include <cstdlib>
@@ -359,6 +360,62 @@ __global__ void transfer_kernel(DevBand<T> M, int a, int3 nin, int3 nout, const 
     }
 }
 
+// One factor along the slowest axis (axis 2 of a 3-D grid): a thread owns one
+// in-plane node and the rows of one element of the output grid (M.chunk of
+// them).  The inputs those rows touch (at most WB, in - in2) are read into
+// registers once, all loads in flight together and coalesced in the plane; the
+// rows' coefficients, laid out over that window, are the same for the whole
+// CTA and come from shared memory.  The row-per-thread kernel above reads every
+// input once per row that touches it and divides out three indices per output
+// (3-D 16^3 elements, p = 7, 32 right-hand sides: 191 us for the prolongation).
+template <typename T, int WB>
+__global__ void __launch_bounds__(128) axis_kernel(DevBand<T> M, int plane, const T* __restrict__ in,
+                                                   const T* __restrict__ in2, T* __restrict__ out, int add, int mask,
+                                                   int nx, T* __restrict__ clear) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    T* cf = reinterpret_cast<T*>(smem_raw);          // [chunk][WB]
+    const int K0 = blockIdx.y * M.chunk, K1 = min(K0 + M.chunk, M.rows), rows = K1 - K0;
+    int w0 = M.start[K0], w1 = 0;
+    for (int K = K0; K < K1; ++K) {
+        w0 = min(w0, M.start[K]);
+        w1 = max(w1, M.start[K] + M.width);
+    }
+    for (int i = threadIdx.x; i < rows * WB; i += blockDim.x) {
+        const int r = i / WB, k = i - r * WB - (M.start[K0 + r] - w0);
+        cf[i] = k >= 0 && k < M.width ? M.coef[(size_t)(K0 + r) * M.width + k] : T(0);
+    }
+    __syncthreads();
+    grid_dep_sync();                                 // the bands above are mesh data
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= plane) return;
+    const size_t rhs = blockIdx.z;
+    const int W = w1 - w0;
+    const size_t at = rhs * M.cols * plane + (size_t)w0 * plane + c;
+    T v[WB];
+#pragma unroll
+    for (int k = 0; k < WB; ++k) v[k] = k < W ? in[at + (size_t)k * plane] : T(0);
+    if (in2) {
+#pragma unroll
+        for (int k = 0; k < WB; ++k)
+            if (k < W) v[k] -= in2[at + (size_t)k * plane];
+    }
+    const int ny = plane / nx, J = c / nx, I = c - J * nx;
+    const bool edge = mask && (I == 0 || I == nx - 1 || J == 0 || J == ny - 1);
+    const size_t o0 = rhs * M.rows * plane + (size_t)K0 * plane + c;
+    for (int r = 0; r < rows; ++r) {
+        const size_t o = o0 + (size_t)r * plane;
+        T s = T(0);
+#pragma unroll
+        for (int k = 0; k < WB; ++k) s += cf[r * WB + k] * v[k];
+        if (clear) clear[o] = T(0);
+        if (edge || (mask && (K0 + r == 0 || K0 + r == M.rows - 1))) {
+            if (!add) out[o] = T(0);
+        } else {
+            out[o] = add ? out[o] + s : s;
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------
 // coarsest solve: dense inverse times vector, one warp per row
 // ---------------------------------------------------------------------------
@@ -674,6 +731,8 @@ __device__ __forceinline__ void transfer2_body(const DevBand<T>& M0, const DevBa
     // staged in rounds of U loads per thread, all issued before any is used
     constexpr int U = 4;
     const int total = nrow * ncol;
+    // idx / ncol by the rounded-up reciprocal: exact for idx < 2^16, ncol < 2^16
+    const unsigned magic = ncol > 1 ? 0xffffffffu / (unsigned)ncol + 1u : 0u;
     for (int base = threadIdx.x; base < total; base += 256 * U) {
         T a[U], b[U];
 #pragma unroll
@@ -682,7 +741,7 @@ __device__ __forceinline__ void transfer2_body(const DevBand<T>& M0, const DevBa
             a[u] = T(0);
             b[u] = T(0);
             if (idx < total) {
-                const int r = idx / ncol, c = idx - r * ncol;
+                const int r = ncol > 1 ? (int)__umulhi((unsigned)idx, magic) : idx, c = idx - r * ncol;
                 const size_t g = (size_t)(rlo + r) * nin.x + clo + c;
                 a[u] = inz[g];
                 if (in2z) b[u] = in2z[g];
@@ -713,7 +772,8 @@ __device__ __forceinline__ void transfer2_body(const DevBand<T>& M0, const DevBa
         if (J >= nout.y) break;
         const size_t o = z * pout + (size_t)J * nout.x + I;
         if (clear) clear[o] = T(0);
-        if (mask && (I == 0 || I == nout.x - 1 || J == 0 || J == nout.y - 1)) {
+        if (mask && (I == 0 || I == nout.x - 1 || J == 0 || J == nout.y - 1 ||
+                     (mask == 2 && (z % nout.z == 0 || z % nout.z == nout.z - 1)))) {
             if (!add) out[o] = T(0);
             continue;
         }
@@ -1400,6 +1460,20 @@ void launch_transfer(const DevBand<T>& M, int a, const int nin[3], const int nou
     const int3 ni = make_int3(nin[0], nin[1], nin[2]), no = make_int3(nout[0], nout[1], nout[2]);
     const int g = grid_for(total * nrhs);
     const int ad = add ? 1 : 0, mk = mask ? 1 : 0;
+    const int plane = nout[0] * nout[1];
+    const long long chunks = M.chunk > 0 ? (M.rows + M.chunk - 1) / M.chunk : 0;
+    if (a == 2 && M.spanc > 0 && M.spanc <= 32 && chunks <= 65535 && nrhs <= 65535) {
+        const int WB = M.spanc <= 4 ? 4 : M.spanc <= 8 ? 8 : M.spanc <= 16 ? 16 : M.spanc <= 20 ? 20 : 32;
+        const dim3 grid((unsigned)((plane + 127) / 128), (unsigned)chunks, (unsigned)nrhs);
+        const size_t sm = sizeof(T) * (size_t)M.chunk * WB;
+        auto go = [&](auto kern) { launch_k(kern, grid, 128, sm, st, M, plane, in, in2, out, ad, mk, nout[0], clear); };
+        if (WB == 4) go(axis_kernel<T, 4>);
+        else if (WB == 8) go(axis_kernel<T, 8>);
+        else if (WB == 16) go(axis_kernel<T, 16>);
+        else if (WB == 20) go(axis_kernel<T, 20>);
+        else go(axis_kernel<T, 32>);
+        return;
+    }
     if (M.width <= 4)
         launch_k(transfer_kernel<T, 4>, g, 256, 0, st, M, a, ni, no, in, in2, out, ad, mk, dim, clear, nrhs);
     else if (M.width <= 8)
@@ -1412,16 +1486,22 @@ void launch_transfer(const DevBand<T>& M, int a, const int nin[3], const int nou
 }
 
 template <typename T>
+bool transfer2_fits(const DevBand<T>& M0, const DevBand<T>& M1) {
+    const size_t smem = sizeof(T) * (size_t)M1.span8 * (M0.span32 + 32);
+    return M0.span32 > 0 && M1.span8 > 0 && smem <= (size_t)kMaxDynSmem && std::max(M0.width, M1.width) <= 32;
+}
+
+template <typename T>
 bool launch_transfer2(const DevBand<T>& M0, const DevBand<T>& M1, const int nin[3], const int nout[3], const T* in,
-                      const T* in2, T* out, bool add, bool mask, cudaStream_t st, T* clear, int nrhs) {
+                      const T* in2, T* out, bool add, bool mask, cudaStream_t st, T* clear, int nrhs, bool planes) {
+    if (!transfer2_fits<T>(M0, M1)) return false;
     constexpr int TY = 8;
     const size_t smem = sizeof(T) * (size_t)M1.span8 * (M0.span32 + 32);
     const int W = M0.width > M1.width ? M0.width : M1.width;
-    if (M0.span32 <= 0 || M1.span8 <= 0 || smem > kMaxDynSmem || W > 32) return false;
     // the nrhs right-hand sides follow one another: nrhs x nout[2] planes of axis 2
     const dim3 grid((unsigned)((nout[0] + 31) / 32), (unsigned)((nout[1] + TY - 1) / TY), (unsigned)(nout[2] * nrhs));
     const int3 ni = make_int3(nin[0], nin[1], nin[2]), no = make_int3(nout[0], nout[1], nout[2]);
-    const int ad = add ? 1 : 0, mk = mask ? 1 : 0;
+    const int ad = add ? 1 : 0, mk = mask ? (planes ? 2 : 1) : 0;   // 2: the end planes of axis 2 too
     if (W <= 4) launch_k(transfer2_kernel<T, 4, TY>, grid, 256, smem, st, M0, M1, ni, no, in, in2, out, ad, mk, clear);
     else if (W <= 8) launch_k(transfer2_kernel<T, 8, TY>, grid, 256, smem, st, M0, M1, ni, no, in, in2, out, ad, mk, clear);
     else if (W <= 16) launch_k(transfer2_kernel<T, 16, TY>, grid, 256, smem, st, M0, M1, ni, no, in, in2, out, ad, mk, clear);
@@ -1672,9 +1752,12 @@ template void launch_coarse<double>(const DevCoarse<double>&, long long, const d
 template void launch_coarse<float>(const DevCoarse<float>&, long long, const float*, float*, float*, cudaStream_t, bool,
                                    int);
 template bool launch_transfer2<double>(const DevBand<double>&, const DevBand<double>&, const int*, const int*,
-                                       const double*, const double*, double*, bool, bool, cudaStream_t, double*, int);
+                                       const double*, const double*, double*, bool, bool, cudaStream_t, double*, int,
+                                       bool);
+template bool transfer2_fits<double>(const DevBand<double>&, const DevBand<double>&);
+template bool transfer2_fits<float>(const DevBand<float>&, const DevBand<float>&);
 template bool launch_transfer2<float>(const DevBand<float>&, const DevBand<float>&, const int*, const int*,
-                                      const float*, const float*, float*, bool, bool, cudaStream_t, float*, int);
+                                      const float*, const float*, float*, bool, bool, cudaStream_t, float*, int, bool);
 template void launch_cast<double, float>(const double*, float*, long long, cudaStream_t);
 template void launch_cast<float, double>(const float*, double*, long long, cudaStream_t);
 template void launch_zero_boundary<double>(double*, const int*, int, cudaStream_t, int);
