@@ -28,6 +28,7 @@
 #include "setup.h"
 
 #include <algorithm>
+#include <cstring>
 #include <mutex>
 #include <vector>
 
@@ -219,48 +220,57 @@ int eo_ff_epb(int p, long long E) {
     return (int)std::max(1LL, std::min(most, fill));
 }
 
-// D (f) and D^T (t) in even-odd form, float-float (H = N / 2)
+// D (f) and D^T (t) in even-odd form, float-float (H = N / 2): the even and odd
+// coefficient of (i, m) side by side in one pair.
+struct EoCoef2 {
+    ffloat2 v;
+    f32x2 nhi;   // -v.hi
+};
 template <int N>
 struct EoMatFF {
     static constexpr int H = N / 2;
-    ffloat e[H * H];   // (M[i][m] + M[i][N-1-m]) / 2, i, m < H
-    ffloat o[H * H];   // (M[i][m] - M[i][N-1-m]) / 2
-    ffloat c[H];       // M[i][h], N odd
-    ffloat r[H];       // M[h][m], N odd
+    EoCoef2 eo[H * H];   // (M[i][m] +- M[i][N-1-m]) / 2, i, m < H
+    EoCoef2 c[H];        // (M[i][h], 0), N odd
+    ffloat r[H];         // M[h][m], N odd
 };
 template <int N>
 struct EoParamsFF {
     EoMatFF<N> f, t;
 };
 
+// out = M u for one line.  The even sum a_i and the odd sum b_i take the same
+// steps on different data, so they run in the two halves of FP32 pairs, and so
+// do the sum and difference that lead in and out of them: about 350
+// instructions a line at N = 8 instead of 584.  (3-D, 16^3 elements, p = 7:
+// see the kernel.)
 template <int N>
 __device__ __forceinline__ void eo_line_ff(const EoMatFF<N>& M, const ffloat (&u)[N], ffloat (&out)[N]) {
     constexpr int H = N / 2;
     constexpr bool ODD = (N & 1) != 0;
-    ffloat ue[H], uo[H];
+    ffloat2 w[H];                            // (u[m] + u[N-1-m], u[m] - u[N-1-m])
 #pragma unroll
-    for (int m = 0; m < H; ++m) {
-        ue[m] = ff_add(u[m], u[N - 1 - m]);
-        uo[m] = ff_sub(u[m], u[N - 1 - m]);
-    }
+    for (int m = 0; m < H; ++m)
+        w[m] = ff_add(ff_pack(u[m], u[m]), ff_pack(u[N - 1 - m], ff_neg(u[N - 1 - m])));
 #pragma unroll
     for (int i = 0; i < H; ++i) {
-        ffloat a = {0.f, 0.f}, b = {0.f, 0.f};
-        if constexpr (ODD) ff_mac(a, M.c[i], u[H]);
+        const f32x2 zero = pack2(0.f, 0.f);
+        ffloat2 ab = {zero, zero};
+        if constexpr (ODD) ff_mac(ab, M.c[i].v, M.c[i].nhi, ff_pack(u[H], u[H]));
 #pragma unroll
-        for (int m = 0; m < H; ++m) {
-            ff_mac(a, M.e[i * H + m], ue[m]);
-            ff_mac(b, M.o[i * H + m], uo[m]);
-        }
-        a = ff_norm(a);
-        b = ff_norm(b);
-        out[i] = ff_add(a, b);
-        out[N - 1 - i] = ff_sub(b, a);
+        for (int m = 0; m < H; ++m) ff_mac(ab, M.eo[i * H + m].v, M.eo[i * H + m].nhi, w[m]);
+        ab = ff_norm(ab);
+        ffloat a, b;
+        ff_unpack(ab, a, b);
+        ff_unpack(ff_add(ab, ff_pack(b, ff_neg(a))), out[i], out[N - 1 - i]);   // (a + b, b - a)
     }
     if constexpr (ODD) {
         ffloat sum = {0.f, 0.f};
 #pragma unroll
-        for (int m = 0; m < H; ++m) ff_mac(sum, M.r[m], uo[m]);
+        for (int m = 0; m < H; ++m) {
+            ffloat e, o;
+            ff_unpack(w[m], e, o);
+            ff_mac(sum, M.r[m], o);
+        }
         out[H] = ff_norm(sum);
     }
 }
@@ -276,11 +286,17 @@ struct EoShapeFF {
     static constexpr int ES = N == 3 ? 27 : N == 4 ? 76 : N == 5 ? 125 : N == 6 ? 324 : N == 7 ? 369 : N == 8 ? 576 : 801;
 };
 
+// Measured (graph replay): 16^3 elements, p = 7: 75.2 -> 65.7 us with the packed
+// sweeps above, 20^3 p = 4: 33.0 -> 30.0, p = 6: 95 -> 83, 14^3 p = 8: 92.6 ->
+// 89.4 (order 8 spills at three CTAs per SM and takes two).  What is left is
+// the FP64 conversions and additions (38 % of that pipe) and the latency of 18
+// resident warps.
+//
 // Thread (a, b) of an element owns the t-line (i, j) = (a, b) in registers
 // and the r-line (j, k) = (a, b) and s-line (i, k) = (a, b) through shared
 // memory (X: x, U, V: the r and s work buffers).
 template <int P>
-__global__ void __launch_bounds__(kEoFfThreads, 3)
+__global__ void __launch_bounds__(kEoFfThreads, P == 8 ? 2 : 3)
     apply_eo3_ff_kernel(DevLevel<double> L, const __grid_constant__ EoParamsFF<P + 1> M, const double* __restrict__ x,
                         double* __restrict__ y, int mask, double* part, int epb, int nrhs) {
     using S = EoShapeFF<P + 1>;
@@ -412,15 +428,23 @@ EoParamsFF<N> eo_ff_params() {
             const float hi = (float)v;
             return ffloat{hi, (float)(v - (double)hi)};
         };
+        auto halves = [](float x, float y) {
+            f32x2 p;
+            const float v[2] = {x, y};
+            std::memcpy(&p, v, sizeof(p));
+            return p;
+        };
+        auto pair = [&](ffloat e, ffloat o) {
+            return EoCoef2{{halves(e.hi, o.hi), halves(e.lo, o.lo)}, halves(-e.hi, -o.hi)};
+        };
         for (int tr = 0; tr < 2; ++tr) {
             EoMatFF<N>& T = tr ? M.t : M.f;
             auto Mv = [&](int i, int m) { return tr ? D[m * N + i] : D[i * N + m]; };
             for (int i = 0; i < H; ++i)
-                for (int m = 0; m < H; ++m) {
-                    T.e[i * H + m] = split(0.5 * (Mv(i, m) + Mv(i, N - 1 - m)));
-                    T.o[i * H + m] = split(0.5 * (Mv(i, m) - Mv(i, N - 1 - m)));
-                }
-            for (int i = 0; i < H; ++i) T.c[i] = split(Mv(i, H));
+                for (int m = 0; m < H; ++m)
+                    T.eo[i * H + m] = pair(split(0.5 * (Mv(i, m) + Mv(i, N - 1 - m))),
+                                           split(0.5 * (Mv(i, m) - Mv(i, N - 1 - m))));
+            for (int i = 0; i < H; ++i) T.c[i] = pair(split(Mv(i, H)), ffloat{0.f, 0.f});
             for (int m = 0; m < H; ++m) T.r[m] = split(Mv(H, m));
         }
     });

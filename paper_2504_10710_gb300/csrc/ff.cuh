@@ -7,6 +7,7 @@
 // free operation).  The _rn intrinsics are never contracted or reassociated
 // by the compiler, which the transformations rely on.
 #pragma once
+#include "f32x2.cuh"
 
 namespace glls {
 
@@ -57,5 +58,43 @@ __device__ __forceinline__ ffloat ff_add(ffloat a, ffloat b) {
     return ff_norm({s, __fadd_rn(e, __fadd_rn(a.lo, b.lo))});
 }
 __device__ __forceinline__ ffloat ff_sub(ffloat a, ffloat b) { return ff_add(a, {-b.hi, -b.lo}); }
+
+// ---- two float-float values in the halves of FP32 pairs --------------------
+// Every operation does to each half what the scalar one above does, in the
+// same order, so the halves carry the same bits.
+struct ffloat2 {
+    f32x2 hi, lo;
+};
+
+__device__ __forceinline__ ffloat2 ff_pack(ffloat a, ffloat b) { return {pack2(a.hi, b.hi), pack2(a.lo, b.lo)}; }
+__device__ __forceinline__ void ff_unpack(ffloat2 p, ffloat& a, ffloat& b) {
+    unpack2(p.hi, a.hi, b.hi);
+    unpack2(p.lo, a.lo, b.lo);
+}
+__device__ __forceinline__ ffloat ff_neg(ffloat a) { return {-a.hi, -a.lo}; }
+
+__device__ __forceinline__ ffloat2 ff_norm(ffloat2 a) {
+    const f32x2 s = add2(a.hi, a.lo);
+    return {s, sub2(a.lo, sub2(s, a.hi))};
+}
+
+__device__ __forceinline__ ffloat2 ff_add(ffloat2 a, ffloat2 b) {
+    const f32x2 s = add2(a.hi, b.hi), bb = sub2(s, a.hi);
+    const f32x2 e = add2(sub2(a.hi, sub2(s, bb)), sub2(b.hi, bb));
+    return ff_norm(ffloat2{s, add2(e, add2(a.lo, b.lo))});
+}
+
+// acc += a b, nahi = -a.hi: the product is formed with its sign turned (m =
+// -fl(a.hi b.hi), exact negation), so that its error term needs no negation.
+__device__ __forceinline__ void ff_mac(ffloat2& acc, ffloat2 a, f32x2 nahi, ffloat2 b) {
+    const f32x2 m = mul2(nahi, b.hi);
+    f32x2 e = fma2(a.hi, b.hi, m);
+    e = fma2(a.hi, b.lo, e);
+    e = fma2(a.lo, b.hi, e);
+    const f32x2 s = sub2(acc.hi, m), bb = sub2(s, acc.hi);
+    const f32x2 es = sub2(sub2(acc.hi, sub2(s, bb)), add2(m, bb));
+    acc.hi = s;
+    acc.lo = add2(acc.lo, add2(es, e));
+}
 
 }  // namespace glls
