@@ -15,7 +15,7 @@ __device__ __forceinline__ bool on_boundary32(int I, int J, int K, const int n[3
 }
 
 // DOT: also sum_e x_e^T (A_e x_e) over all elements into *dot (last block).
-// Each thread owns ITEMS local nodes (t = threadIdx.x + 256 * it); its
+// Each thread owns ITEMS local nodes (t = threadIdx.x + THREADS * it); its
 // geometry factors and D are loaded before the wait on the preceding kernel,
 // so that only the x gather's latency follows it.
 // sum_m a[m] b[m] and sum_m a[m] b[m * stride] over N terms with a (and, in
@@ -66,8 +66,9 @@ __device__ __forceinline__ void apply_p_body(const DevLevel<T>& L, const T* __re
     if constexpr (LOC) loc += (long long)rhs * L.E * L.nloc;
     constexpr int N1 = P + 1;
     constexpr int NLOC = DIM == 2 ? N1 * N1 : N1 * N1 * N1;
-    constexpr int EPB = NLOC >= 256 ? 1 : 256 / NLOC;
-    constexpr int ITEMS = (EPB * NLOC + 255) / 256;
+    constexpr int EPB = apply_epb(NLOC);
+    constexpr int THREADS = apply_threads(NLOC);
+    constexpr int ITEMS = (EPB * NLOC + THREADS - 1) / THREADS;
     constexpr int NC = DIM == 2 ? 3 : 6;
     // FP32 with N1 a multiple of 4: rows of D, D^T, x and w are 16-byte
     // aligned, so the contractions read them with float4 loads
@@ -93,14 +94,14 @@ __device__ __forceinline__ void apply_p_body(const DevLevel<T>& L, const T* __re
     T gk[ITEMS][NC];
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
-        const int t = threadIdx.x + 256 * it;
+        const int t = threadIdx.x + THREADS * it;
         if (t < total) {
             const int gq = e0 * NLOC + t;          // = (e0 + el) * NLOC + q
 #pragma unroll
             for (int c = 0; c < NC; ++c) gk[it][c] = __ldg(L.G + c * EN + gq);
         }
     }
-    for (int t = threadIdx.x; t < N1 * N1; t += 256) {
+    for (int t = threadIdx.x; t < N1 * N1; t += THREADS) {
         sD[t] = L.D[t];
         if constexpr (VEC) sDT[t] = L.D[(t % N1) * N1 + t / N1];
     }
@@ -108,7 +109,7 @@ __device__ __forceinline__ void apply_p_body(const DevLevel<T>& L, const T* __re
     if (!grid_dep_ready(done)) return;
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
-        const int t = threadIdx.x + 256 * it;
+        const int t = threadIdx.x + THREADS * it;
         if (t < total) {
             const int el = t / NLOC, q = t - el * NLOC;
             const int i = q % N1, j = (q / N1) % N1, k = DIM == 3 ? q / (N1 * N1) : 0;
@@ -119,7 +120,7 @@ __device__ __forceinline__ void apply_p_body(const DevLevel<T>& L, const T* __re
 
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
-        const int t = threadIdx.x + 256 * it;
+        const int t = threadIdx.x + THREADS * it;
         if (t >= total) break;
         const int el = t / NLOC, q = t - el * NLOC;
         const int i = q % N1, j = (q / N1) % N1, k = DIM == 3 ? q / (N1 * N1) : 0;
@@ -152,7 +153,7 @@ __device__ __forceinline__ void apply_p_body(const DevLevel<T>& L, const T* __re
     double local = 0.0;
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
-        const int t = threadIdx.x + 256 * it;
+        const int t = threadIdx.x + THREADS * it;
         if (t >= total) break;
         const int el = t / NLOC, q = t - el * NLOC;
         const int i = q % N1, j = (q / N1) % N1, k = DIM == 3 ? q / (N1 * N1) : 0;
@@ -199,8 +200,13 @@ __device__ __forceinline__ void apply_p_body(const DevLevel<T>& L, const T* __re
     }
 }
 
+template <int DIM, int P>
+constexpr int threads_of() {
+    return apply_threads(DIM == 2 ? (P + 1) * (P + 1) : (P + 1) * (P + 1) * (P + 1));
+}
+
 template <typename T, int DIM, int P, bool DOT, bool LOC>
-__global__ void __launch_bounds__(256, 1) apply_p_kernel(DevLevel<T> L, const T* __restrict__ x, T* __restrict__ y,
+__global__ void __launch_bounds__(threads_of<DIM, P>(), 1) apply_p_kernel(DevLevel<T> L, const T* __restrict__ x, T* __restrict__ y,
                                                          int mask, double* dot, double* part, unsigned* ticket,
                                                          int nrhs, T* loc) {
     apply_p_body<T, DIM, P, DOT, LOC>(L, x, y, mask, dot, part, ticket, nrhs, blockIdx.x, gridDim.x, nullptr,
@@ -210,7 +216,7 @@ __global__ void __launch_bounds__(256, 1) apply_p_kernel(DevLevel<T> L, const T*
 // Work-list form: item j (its own level, vectors and partials) owns the CTAs
 // [start[j], start[j + 1]) of the launch.
 template <typename T, int DIM, int P, bool DOT>
-__global__ void __launch_bounds__(256, 1) apply_p_list_kernel(const ApplyItem<T>* __restrict__ items,
+__global__ void __launch_bounds__(threads_of<DIM, P>(), 1) apply_p_list_kernel(const ApplyItem<T>* __restrict__ items,
                                                               const int* __restrict__ start, int nitems, int mask) {
     const int j = work_item(start, nitems, blockIdx.x);
     const ApplyItem<T>& it = items[j];
@@ -223,7 +229,7 @@ template <typename T, int DIM, int P>
 int apply_blocks(const DevLevel<T>& L) {
     constexpr int N1 = P + 1;
     constexpr int NLOC = DIM == 2 ? N1 * N1 : N1 * N1 * N1;
-    constexpr int EPB = NLOC >= 256 ? 1 : 256 / NLOC;
+    constexpr int EPB = apply_epb(NLOC);
     return (int)((L.E + EPB - 1) / EPB);
 }
 
@@ -232,22 +238,22 @@ bool launch_p(const DevLevel<T>& L, const T* x, T* y, bool mask, double* dot, do
               cudaStream_t st, int nrhs, T* loc) {
     constexpr int N1 = P + 1;
     constexpr int NLOC = DIM == 2 ? N1 * N1 : N1 * N1 * N1;
-    constexpr int EPB = NLOC >= 256 ? 1 : 256 / NLOC;
+    constexpr int EPB = apply_epb(NLOC);
     const long long blocks = (L.E + EPB - 1) / EPB * nrhs;
     if (blocks > 0x7fffffffLL) return false;
     const int mk = mask ? 1 : 0;
     if constexpr (sizeof(T) == 8) {
         if (dot) {
-            if (loc) launch_k(apply_p_kernel<T, DIM, P, true, true>, (unsigned)blocks, 256, 0, st, L, x, y, mk, dot, part, ticket, nrhs, loc);
-            else launch_k(apply_p_kernel<T, DIM, P, true, false>, (unsigned)blocks, 256, 0, st, L, x, y, mk, dot, part, ticket, nrhs, loc);
+            if (loc) launch_k(apply_p_kernel<T, DIM, P, true, true>, (unsigned)blocks, threads_of<DIM, P>(), 0, st, L, x, y, mk, dot, part, ticket, nrhs, loc);
+            else launch_k(apply_p_kernel<T, DIM, P, true, false>, (unsigned)blocks, threads_of<DIM, P>(), 0, st, L, x, y, mk, dot, part, ticket, nrhs, loc);
             return true;
         }
     }
     if (dot) return false;                   // x.(A x) is formed in FP64 only
     double* nd = nullptr;
     unsigned* nt = nullptr;
-    if (loc) launch_k(apply_p_kernel<T, DIM, P, false, true>, (unsigned)blocks, 256, 0, st, L, x, y, mk, nd, nd, nt, nrhs, loc);
-    else launch_k(apply_p_kernel<T, DIM, P, false, false>, (unsigned)blocks, 256, 0, st, L, x, y, mk, nd, nd, nt, nrhs, loc);
+    if (loc) launch_k(apply_p_kernel<T, DIM, P, false, true>, (unsigned)blocks, threads_of<DIM, P>(), 0, st, L, x, y, mk, nd, nd, nt, nrhs, loc);
+    else launch_k(apply_p_kernel<T, DIM, P, false, false>, (unsigned)blocks, threads_of<DIM, P>(), 0, st, L, x, y, mk, nd, nd, nt, nrhs, loc);
     return true;
 }
 
@@ -271,13 +277,13 @@ bool launch_list_p(int p, const ApplyItem<T>* items, const int* start, int nitem
         if (p != P) return launch_list_p<T, P - 1>(p, items, start, nitems, blocks, mask, dot, st);
         if constexpr (sizeof(T) == 8) {
             if (dot) {
-                launch_k(apply_p_list_kernel<T, 2, P, true>, (unsigned)blocks, 256, 0, st, items, start, nitems,
+                launch_k(apply_p_list_kernel<T, 2, P, true>, (unsigned)blocks, threads_of<2, P>(), 0, st, items, start, nitems,
                          mask ? 1 : 0);
                 return true;
             }
         }
         if (dot) return false;
-        launch_k(apply_p_list_kernel<T, 2, P, false>, (unsigned)blocks, 256, 0, st, items, start, nitems, mask ? 1 : 0);
+        launch_k(apply_p_list_kernel<T, 2, P, false>, (unsigned)blocks, threads_of<2, P>(), 0, st, items, start, nitems, mask ? 1 : 0);
         return true;
     }
 }
@@ -288,7 +294,7 @@ bool launch_list_p(int p, const ApplyItem<T>* items, const int* start, int nitem
 // (one dot partial each).
 int apply_list_blocks(int p, long long E) {
     const int nloc = (p + 1) * (p + 1);
-    const int epb = nloc >= 256 ? 1 : 256 / nloc;
+    const int epb = apply_epb(nloc);
     return (int)((E + epb - 1) / epb);
 }
 
@@ -315,7 +321,7 @@ int apply_dot_partials(const DevLevel<T>& L) {
     if (apply_eo_selected(L.dim, L.p, true)) return apply_eo_blocks(L.p, L.E);
     long long nloc = 1;
     for (int a = 0; a < L.dim; ++a) nloc *= L.p + 1;
-    const long long epb = nloc >= 256 ? 1 : 256 / nloc;
+    const long long epb = apply_epb((int)nloc);
     return (int)((L.E + epb - 1) / epb);
 }
 template int apply_dot_partials<double>(const DevLevel<double>&);

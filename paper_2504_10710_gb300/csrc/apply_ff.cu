@@ -35,8 +35,7 @@
 namespace glls {
 namespace {
 
-// Block sum of one FP64 value per thread (blockDim.x <= 256, a multiple of
-// 32) with few FP64 adds: the values go through shared memory, lane l of
+// Block sum of one FP64 value per thread (blockDim.x a multiple of 32) with few FP64 adds: the values go through shared memory, lane l of
 // warp 0 adds values l, l + 32, ... in that order, then warp 0's shuffle
 // tree.  A shuffle tree over every warp would cost each thread five FP64
 // adds, which on GB300's FP64 pipe is a visible share of these kernels.
@@ -60,8 +59,9 @@ __device__ __forceinline__ void apply_ff_body(const DevLevel<double>& L, const d
     y += (long long)rhs * L.N;
     constexpr int N1 = P + 1;
     constexpr int NLOC = N1 * N1;
-    constexpr int EPB = NLOC >= 256 ? 1 : 256 / NLOC;
-    constexpr int ITEMS = (EPB * NLOC + 255) / 256;
+    constexpr int EPB = apply_epb(NLOC);
+    constexpr int THREADS = apply_threads(NLOC);
+    constexpr int ITEMS = (EPB * NLOC + THREADS - 1) / THREADS;
     __shared__ ffloat sD[N1 * N1];
     __shared__ ffloat sx[EPB * NLOC];
     __shared__ ffloat sw[2 * EPB * NLOC];
@@ -81,20 +81,20 @@ __device__ __forceinline__ void apply_ff_body(const DevLevel<double>& L, const d
     ffloat gk[ITEMS][3];
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
-        const int t = threadIdx.x + 256 * it;
+        const int t = threadIdx.x + THREADS * it;
         if (t < total) {
             const int gq = e0 * NLOC + t;
 #pragma unroll
             for (int c = 0; c < 3; ++c) gk[it][c] = {__ldg(L.Ghi + c * EN + gq), __ldg(L.Glo + c * EN + gq)};
         }
     }
-    for (int t = threadIdx.x; t < N1 * N1; t += 256) sD[t] = ff_from_double(L.D[t]);
+    for (int t = threadIdx.x; t < N1 * N1; t += THREADS) sD[t] = ff_from_double(L.D[t]);
     __syncthreads();
     if (!grid_dep_ready(done)) return;   // G and D above are mesh data: loaded ahead of the wait
     double xd[ITEMS];
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
-        const int t = threadIdx.x + 256 * it;
+        const int t = threadIdx.x + THREADS * it;
         xd[it] = 0.0;
         if (t < total) {
             const int el = t / NLOC, q = t - el * NLOC;
@@ -107,7 +107,7 @@ __device__ __forceinline__ void apply_ff_body(const DevLevel<double>& L, const d
 
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
-        const int t = threadIdx.x + 256 * it;
+        const int t = threadIdx.x + THREADS * it;
         if (t >= total) break;
         const int el = t / NLOC, q = t - el * NLOC;
         const int i = q % N1, j = q / N1;
@@ -134,7 +134,7 @@ __device__ __forceinline__ void apply_ff_body(const DevLevel<double>& L, const d
     double local = 0.0;
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
-        const int t = threadIdx.x + 256 * it;
+        const int t = threadIdx.x + THREADS * it;
         if (t >= total) break;
         const int el = t / NLOC, q = t - el * NLOC;
         const int i = q % N1, j = q / N1;
@@ -159,20 +159,20 @@ __device__ __forceinline__ void apply_ff_body(const DevLevel<double>& L, const d
             atomicAdd(&y[g], vd);
         }
     }
-    __shared__ double sv[256];
+    __shared__ double sv[THREADS];
     const double tsum = block_sum_lean(local, sv);
     if (threadIdx.x == 0) part[(long long)rhs * nbx + bx] = tsum;
 }
 
 template <int P>
-__global__ void __launch_bounds__(256, 1) apply_ff_kernel(DevLevel<double> L, const double* __restrict__ x,
+__global__ void __launch_bounds__(apply_threads((P + 1) * (P + 1)), 1) apply_ff_kernel(DevLevel<double> L, const double* __restrict__ x,
                                                           double* __restrict__ y, int mask, double* part, int nrhs) {
     apply_ff_body<P>(L, x, y, mask, part, nrhs, blockIdx.x, gridDim.x, nullptr);
 }
 
 // Work-list form: item j owns the CTAs [start[j], start[j + 1]).
 template <int P>
-__global__ void __launch_bounds__(256, 1) apply_ff_list_kernel(const ApplyItem<double>* __restrict__ items,
+__global__ void __launch_bounds__(apply_threads((P + 1) * (P + 1)), 1) apply_ff_list_kernel(const ApplyItem<double>* __restrict__ items,
                                                                const int* __restrict__ start, int nitems, int mask) {
     const int j = work_item(start, nitems, blockIdx.x);
     const ApplyItem<double>& it = items[j];
@@ -187,10 +187,10 @@ bool launch_ff(int p, const DevLevel<double>& L, const double* x, double* y, boo
     } else {
         if (p != P) return launch_ff<P - 1>(p, L, x, y, mask, part, st, nrhs);
         constexpr int NLOC = (P + 1) * (P + 1);
-        constexpr int EPB = NLOC >= 256 ? 1 : 256 / NLOC;
+        constexpr int EPB = apply_epb(NLOC);
         const long long blocks = (L.E + EPB - 1) / EPB * nrhs;
         if (blocks > 0x7fffffffLL) return false;
-        return launch_k(apply_ff_kernel<P>, (unsigned)blocks, 256, 0, st, L, x, y, mask ? 1 : 0, part, nrhs) ==
+        return launch_k(apply_ff_kernel<P>, (unsigned)blocks, apply_threads(NLOC), 0, st, L, x, y, mask ? 1 : 0, part, nrhs) ==
                cudaSuccess;
     }
 }
@@ -202,7 +202,7 @@ bool launch_ff_list(int p, const ApplyItem<double>* items, const int* start, int
         return false;
     } else {
         if (p != P) return launch_ff_list<P - 1>(p, items, start, nitems, blocks, mask, st);
-        return launch_k(apply_ff_list_kernel<P>, (unsigned)blocks, 256, 0, st, items, start, nitems,
+        return launch_k(apply_ff_list_kernel<P>, (unsigned)blocks, apply_threads((P + 1) * (P + 1)), 0, st, items, start, nitems,
                         mask ? 1 : 0) == cudaSuccess;
     }
 }
@@ -497,7 +497,7 @@ int apply_ff_partials(const DevLevel<double>& L) {
         return (int)((L.E + epb - 1) / epb);
     }
     const long long nloc = (long long)(L.p + 1) * (L.p + 1);
-    const long long epb = nloc >= 256 ? 1 : 256 / nloc;
+    const long long epb = apply_epb((int)nloc);
     return (int)((L.E + epb - 1) / epb);
 }
 

@@ -206,6 +206,27 @@ struct FcgItem {                 // one problem's outer Krylov vectors, partial 
     unsigned* ticket;
 };
 
+// Threads of a CTA of the node-per-thread applies (2-D, and 3-D FP64) for
+// elements of nloc nodes, and its elements.  256 threads, unless whole elements
+// fill a CTA of 192 to 352 threads better by 15 %: at 256, the orders 9, 11, 12
+// and 16 in 2-D left 22 to 44 % of the threads idle (24 uneven problems: 17.27
+// -> 16.69 ms).
+__host__ __device__ constexpr int apply_threads(int nloc) {
+    if (nloc < 96 || nloc > 352) return 256;
+    // share of busy threads, in 1/1000 (256 threads take nloc > 256 in two rounds)
+    const int base = nloc > 256 ? nloc * 1000 / 512 : 256 / nloc * nloc * 1000 / 256;
+    int best = 256, most = base * 115 / 100;
+    for (int t = 192; t <= 352; t += 32) {
+        const int u = t / nloc * nloc * 1000 / t;
+        if (u > most) {
+            best = t;
+            most = u;
+        }
+    }
+    return best;
+}
+__host__ __device__ constexpr int apply_epb(int nloc) { return nloc >= apply_threads(nloc) ? 1 : apply_threads(nloc) / nloc; }
+
 int apply_list_blocks(int p, long long E);
 template <typename T>
 bool launch_apply_list(int p, const ApplyItem<T>* items, const int* start, int nitems, int blocks, bool mask,

@@ -12,7 +12,7 @@ namespace {
 // shuffle tree: GB300 issues a warp's FP64 add over 16 cycles, and a shuffle
 // tree in every warp (40 adds for 256 threads instead of 13) was a visible
 // share of the outer-iteration kernels.
-constexpr int kReduceThreads = 256;
+constexpr int kReduceThreads = 352;
 __device__ __forceinline__ double block_sum(double v, double* red) {
     __syncthreads();                        // red may still be read from the last sum
     red[threadIdx.x] = v;
