@@ -479,10 +479,8 @@ def line_roofline(prob, glls, torch):
 def _fp32_apply_kernel(d, p):
     """Name and traffic key of the FP32 apply kernel the library launches for
     a level of dimension d and order p (the dispatch in csrc/apply.cu)."""
-    if d == 3 and p >= 4:
-        return f"apply_eo3_kernel<float, {p}> (even-odd line apply)", f"apply_eo3_kernel<float,{p}>"
     if d == 3:
-        return f"apply_col_kernel<{p}> (column apply)", f"apply_col_kernel<{p}>"
+        return f"apply_eo3_pair_kernel<{p}> (even-odd line apply, packed FP32)", f"apply_eo3_pair_kernel<{p}>"
     return f"apply_p_kernel<float, {d}, {p}>", f"apply_p_kernel<float,{d},{p}>"
 
 

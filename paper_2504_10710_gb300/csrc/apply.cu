@@ -333,15 +333,12 @@ bool launch_apply_fixed(const DevLevel<T>& L, const T* x, T* y, bool mask, doubl
     if (L.N > (1LL << 31) - 1 || L.E * L.nloc * (L.dim == 2 ? 3 : 6) > (1LL << 31) - 1) return false;
     for (int a = 0; a < L.dim; ++a)
         if (L.ne[a] >= 1024) return false;   // element coordinates are packed in 10 bits
-    // 3-D: the even-odd line kernel where it was measured fastest, then the
-    // FP32 column kernel, else the node-per-thread kernel below
+    // 3-D: the even-odd line kernels (FP32, and FP64 where they were measured
+    // fastest), else the node-per-thread kernel below
     if (launch_apply_eo<T>(L, x, y, mask, dot, part, ticket, st, nrhs, loc)) return true;
-    if constexpr (sizeof(T) == 4) {
-        if (L.dim == 3 && !dot && launch_apply_col(L, x, y, mask, st, nrhs, loc)) return true;
-    }
     if (L.dim == 2) return dispatch<T, 2, 16>(L.p, L, x, y, mask, dot, part, ticket, st, nrhs, loc);
-    // 3-D FP32 is served by the even-odd and column kernels above at every
-    // order up to 8; this kernel keeps 3-D FP64
+    // 3-D FP32 is served by the even-odd kernel above at every order up to 8;
+    // this kernel keeps 3-D FP64
     if constexpr (sizeof(T) == 8) return dispatch<T, 3, 8>(L.p, L, x, y, mask, dot, part, ticket, st, nrhs,
                                                                   loc);
     return false;

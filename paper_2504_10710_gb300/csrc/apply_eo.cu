@@ -95,8 +95,8 @@ template <int N>
 struct EoShape {
     static constexpr int NP = N * N, NLOC = NP * N;
     static constexpr int RS = N == 8 ? 9 : N == 7 ? 7 : N == 6 ? 9 : N;
-    static constexpr int PS = N == 5 ? 25 : N == 6 ? 54 : N == 7 ? 52 : N == 8 ? 72 : 89;
-    static constexpr int ES = N == 5 ? 125 : N == 6 ? 324 : N == 7 ? 369 : N == 8 ? 576 : 801;
+    static constexpr int PS = N == 2 ? 5 : N == 3 ? 9 : N == 4 ? 19 : N == 5 ? 25 : N == 6 ? 54 : N == 7 ? 52 : N == 8 ? 72 : 89;
+    static constexpr int ES = N == 2 ? 12 : N == 3 ? 27 : N == 4 ? 76 : N == 5 ? 125 : N == 6 ? 324 : N == 7 ? 369 : N == 8 ? 576 : 801;
     static constexpr int NBUF = 3;                           // x, and two work buffers
 };
 
@@ -355,6 +355,22 @@ __global__ void __launch_bounds__(128, eo_pair_min_ctas(P, RHS))
         baseB = (KB * n1 + J) * n0 + I;
         bdB = I == 0 || I == n0 - 1 || J == 0 || J == n1 - 1;
     }
+    // low orders hold their geometric factors before the preceding kernel has
+    // ended (mesh data)
+    constexpr bool HELD = N <= 4;
+    const int EN = E * NLOC;
+    const float* GA = L.G + eA * NLOC + c;
+    const float* GB = L.G + eB * NLOC + c;
+    f32x2 gh[HELD ? N : 1][6];
+    if (HELD && act) {
+#pragma unroll
+        for (int k = 0; k < N; ++k)
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                const float ga = __ldg(GA + q * EN + k * NP);
+                gh[HELD ? k : 0][q] = pack2(ga, RHS ? ga : __ldg(GB + q * EN + k * NP));
+            }
+    }
     grid_dep_sync();
     f32x2 ut[N];
     if (act) {
@@ -382,17 +398,18 @@ __global__ void __launch_bounds__(128, eo_pair_min_ctas(P, RHS))
     __syncthreads();
     f32x2 yt[N];
     if (act) {
-        const int EN = E * NLOC;
-        const float* GA = L.G + eA * NLOC + c;
-        const float* GB = L.G + eB * NLOC + c;
         f32x2 wt[N];
 #pragma unroll
         for (int k = 0; k < N; ++k) {
             f32x2 g[6];
 #pragma unroll
             for (int q = 0; q < 6; ++q) {
-                const float ga = __ldg(GA + q * EN + k * NP);
-                g[q] = pack2(ga, RHS ? ga : __ldg(GB + q * EN + k * NP));
+                if constexpr (HELD) {
+                    g[q] = gh[k][q];
+                } else {
+                    const float ga = __ldg(GA + q * EN + k * NP);
+                    g[q] = pack2(ga, RHS ? ga : __ldg(GB + q * EN + k * NP));
+                }
             }
             const int s = at_t(k);
             const f32x2 dr = U[s], ds = V[s], dt = ut[k];
@@ -492,10 +509,11 @@ EoParams2<N> eo_params2() {
 }
 
 // Element slots per CTA of the pair kernel: at most 128 threads, and no more
-// than keep about eight CTAs per SM on the level.
+// than keep about eight CTAs per SM on the level, but at least two warps' worth.
 int eo_pair_epb(int p, long long slots) {
-    const long long most = std::max(1, 128 / ((p + 1) * (p + 1)));
-    return (int)std::max(1LL, std::min(most, slots / (152 * 8)));
+    const int np = (p + 1) * (p + 1);
+    const long long most = std::max(1, 128 / np), least = std::max(1, 64 / np);
+    return (int)std::max(least, std::min(most, slots / (152 * 8)));
 }
 
 template <int P>
@@ -552,14 +570,15 @@ bool set_eo_attr() {
 
 }  // namespace
 
-// Orders measured faster with these kernels than with the node-per-thread and
-// column kernels on 16^3-element levels (graph replay and L2-cold launches):
-// FP32 p >= 4 (one line per thread, p = 7: 15.1 against 16.4 and 24.4 us),
-// FP64 p = 6, 7 (p = 7: 193 against 218 us).  FP64 elsewhere: the 2N adds per
-// line and the lower thread count cost more than the saved multiply-adds.
+// FP32 takes this kernel at every order (p <= 3: 16^3 elements, p = 3, 32
+// right-hand sides 46.5 us with one thread per element column, 32.4 here; 20^3,
+// one, 5.2 and 4.5 us), FP64 where it was measured faster than the node-per-
+// thread kernel on 16^3-element levels: p = 6, 7 (p = 7: 193 against 218 us).
+// FP64 elsewhere: the 2N adds per line and the lower thread count cost more
+// than the saved multiply-adds.
 bool apply_eo_selected(int dim, int p, bool f64) {
     if (dim != 3) return false;
-    return f64 ? (p == 6 || p == 7) : (p >= 4 && p <= 8);
+    return f64 ? (p == 6 || p == 7) : (p >= 1 && p <= 8);
 }
 
 // Number of CTAs (= dot partials) of the even-odd kernel for L.
@@ -580,6 +599,9 @@ bool launch_apply_eo(const DevLevel<T>& L, const T* x, T* y, bool mask, double* 
     } else {
         if (dot) return false;               // x.(A x) is formed in FP64 only
         switch (L.p) {
+            case 1: return launch_eo_pair<1>(L, x, y, mask, st, nrhs, loc);
+            case 2: return launch_eo_pair<2>(L, x, y, mask, st, nrhs, loc);
+            case 3: return launch_eo_pair<3>(L, x, y, mask, st, nrhs, loc);
             case 4: return launch_eo_pair<4>(L, x, y, mask, st, nrhs, loc);
             case 5: return launch_eo_pair<5>(L, x, y, mask, st, nrhs, loc);
             case 6: return launch_eo_pair<6>(L, x, y, mask, st, nrhs, loc);

@@ -277,8 +277,7 @@ bool launch_line_block_list(int p, int s, int cv, const void* items, const int* 
 bool init_kernel_attributes();
 constexpr size_t kMaxDynSmemBytes = 200 * 1024;
 
-// Specialised fast paths (apply.cu with apply_eo.cu and apply_col.cu for
-// 3-D, lines.cu); they return false when the case is outside their compiled
+// Specialised fast paths (apply.cu with apply_eo.cu for 3-D, lines.cu); they return false when the case is outside their compiled
 // range and the generic kernels take over.
 // dot: if non-null, also accumulate sum_e x_e^T (A_e x_e) = x.(A x) for x
 // zero on the boundary; the last block writes it to dot[0] using `part` and
@@ -308,12 +307,6 @@ template <>
 bool init_line_block_attributes<float>();
 template <>
 bool init_line_block_attributes<double>();
-// 3-D FP32 apply with one thread per element column (apply_col.cu), p <= 3
-// (the orders the even-odd kernel does not take); no x.(A x) product.
-// Returns false outside that range.
-bool launch_apply_col(const DevLevel<float>& L, const float* x, float* y, bool mask, cudaStream_t st,
-                      int nrhs = 1, float* loc = nullptr);
-bool init_apply_col_attributes();
 // 3-D apply with one thread per element grid line and even-odd derivative
 // sweeps (apply_eo.cu), for the orders apply_eo_selected names, with the
 // optional x.(A x) partials (one per CTA, apply_eo_blocks of them).

@@ -1730,8 +1730,7 @@ bool init_kernel_attributes() {
         if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem) != cudaSuccess)
             return false;
     return init_line_warp_attributes() && init_line_block_attributes<float>() &&
-           init_line_block_attributes<double>() && init_apply_col_attributes() &&
-           init_apply_eo_attributes();
+           init_line_block_attributes<double>() && init_apply_eo_attributes();
 }
 
 // explicit instantiations
