@@ -893,9 +893,21 @@ struct WlRecord {
     }
 };
 
+// Finest-level nodes per group of a chain (a chain below twice that stays one
+// group).  A group's problems advance in lockstep, so once its launches fill
+// the chip further problems only lengthen every phase, while a second group
+// runs its phases beside the first one's.  Measured with 200, 300, 400 and 500
+// thousand nodes and with one group per chain: 128 problems (n x n elements,
+// n ~ U{4..64}, p ~ U{4..12}) 70.2, 70.1, 73.0, 73.8, 81.0 ms; four batches of
+// 24: 50.9, 51.8, 52.5, 52.7, 52.8 ms together, but with 300 thousand one of
+// them and one of 16 were 3-4 % slower than with one group per chain, with
+// 200 thousand one of 12 by 5 %; with 400 thousand none was.
+constexpr long long kGroupNodes = 400000;
+
 struct WlGroup {
     std::vector<glls_problem*> probs;
     std::vector<int> index;            // position of each problem in the batch
+    long long nodes = 0;               // of all its problems' finest levels
     std::vector<WlRecord> body;        // one outer iteration
     size_t off_S = 0;                  // [n][S_COUNT] scalars in the plan's block
     cudaStream_t s1 = nullptr, s2 = nullptr;
@@ -1371,6 +1383,7 @@ glls_status make_plan(glls_problem* const* probs, int n, const glls_solve_opts* 
     std::unique_ptr<WlPlan, void (*)(WlPlan*)> W(new WlPlan(), destroy_plan);
     W->probs.assign(probs, probs + n);
     W->key = *o;
+    std::vector<std::vector<int>> chains;   // problems with the same orders, by position
     for (int i = 0; i < n; ++i) {
         glls_problem* P = probs[i];
         if (P->dim != 2) return fail(GLLS_ERR_INVALID, "work-list batch: 2-D problems only");
@@ -1382,11 +1395,26 @@ glls_status make_plan(glls_problem* const* probs, int n, const glls_solve_opts* 
             if (l > 0 && (!L.blk[0] || !L.blk[1]))
                 return fail(GLLS_ERR_INVALID, "work-list batch: a level without line blocks");
         }
-        size_t gi = 0;
-        while (gi < W->groups.size() && W->groups[gi].probs[0]->orders != P->orders) ++gi;
-        if (gi == W->groups.size()) W->groups.emplace_back();
-        W->groups[gi].probs.push_back(P);
-        W->groups[gi].index.push_back(i);
+        size_t ci = 0;
+        while (ci < chains.size() && probs[chains[ci][0]]->orders != P->orders) ++ci;
+        if (ci == chains.size()) chains.emplace_back();
+        chains[ci].push_back(i);
+    }
+    // each chain in one group per kGroupNodes nodes, its problems dealt out
+    // largest first to the group with the fewest nodes
+    for (auto& C : chains) {
+        std::stable_sort(C.begin(), C.end(), [&](int a, int b) { return probs[a]->N > probs[b]->N; });
+        long long nodes = 0;
+        for (int i : C) nodes += probs[i]->N;
+        const size_t first = W->groups.size();
+        W->groups.resize(first + (size_t)std::max(1LL, std::min((long long)C.size(), nodes / kGroupNodes)));
+        for (int i : C) {
+            auto G = std::min_element(W->groups.begin() + first, W->groups.end(),
+                                      [](const WlGroup& a, const WlGroup& b) { return a.nodes < b.nodes; });
+            G->probs.push_back(probs[i]);
+            G->index.push_back(i);
+            G->nodes += probs[i]->N;
+        }
     }
     // records, then one device block for every item array, start array and
     // group scalar array
