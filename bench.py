@@ -487,14 +487,14 @@ def _fp32_apply_kernel(d, p):
 def _line_operator_bytes(shape, p, s, block):
     """FP32 bytes of the line operator along axis s read by one line solve:
     the Def. 3.2 line blocks (per element segment (p-1)p/2 + 2(p-1) values,
-    per element-boundary vertex 2) or the band-1 (diag, off) pairs."""
+    per element-boundary vertex 3) or the band-1 (diag, off) pairs."""
     d = len(shape)
     n = shape[d - 1 - s]                      # nodes along s
     lines = int(np.prod([shape[d - 1 - a] - 2 for a in range(d) if a != s]))
     if not block:
         return 8 * lines * (n - 2)
     E = (n - 1) // p
-    return 4 * lines * E * ((p - 1) * p // 2 + 2 * (p - 1)) + 8 * lines * (E - 1)
+    return 4 * lines * E * ((p - 1) * p // 2 + 2 * (p - 1)) + 12 * lines * (E - 1)
 
 
 def smoother_rooflines(prob, glls, torch, inputs, flush, large=True):
@@ -747,9 +747,9 @@ def batch_run(glls, inputs, torch, reps=3):
                        "converged": int(sum(x.status == glls.OK for x in st_w)),
                        "iterations": {"median": float(np.median(its_w)), "max": int(its_w.max())},
                        "kernels_per_launch": int(st_w[0].kernels),
-                       "groups": len({tuple(p.info.order[:p.info.levels]) for p in probs}),
+                       "order_chains": len({tuple(p.info.order[:p.info.levels]) for p in probs}),
                        "plan_s": plan_s, "max_rel_diff_vs_branches": diff,
-                       "form": "glls_solve_batch_worklist: problems grouped by order chain, one launch per step "
+                       "form": "glls_solve_batch_worklist: problems grouped by order chain and size, one launch per step "
                                "over each group's work list of (problem, level, tile range) items, one graph "
                                "branch and device-side loop per group"}
     for p in probs:
