@@ -412,15 +412,14 @@ void prolong_add(glls_problem* P, int l, const T* e, T* x, cudaStream_t st, T* c
 // the apply.  The level scratch y is zero on entry and on exit: the apply
 // accumulates into it and the line solve resets what it reads.
 template <typename T>
-void smooth(glls_problem* P, int l, int s, T alpha, const T* r, T* x, bool x_is_zero, cudaStream_t st,
-            int nrhs = 1) {
+cudaError_t smooth(glls_problem* P, int l, int s, T alpha, const T* r, T* x, bool x_is_zero, cudaStream_t st,
+                   int nrhs = 1) {
     auto& Ls = levels_of<T>(P);
-    if (x_is_zero) {
-        launch_line_solve<T>(Ls[l].dev, s, 3, nullptr, r, nullptr, x, alpha, st, nrhs);
-    } else {
+    if (x_is_zero) return launch_line_solve<T>(Ls[l].dev, s, 3, nullptr, r, nullptr, x, alpha, st, nrhs);
+    const cudaError_t e =
         launch_apply<T>(Ls[l].dev, x, Ls[l].y, true, st, true, nullptr, nullptr, nullptr, nrhs, Ls[l].loc);
-        launch_line_solve<T>(Ls[l].dev, s, 1, nullptr, r, Ls[l].y, x, alpha, st, nrhs);
-    }
+    if (e != cudaSuccess) return e;
+    return launch_line_solve<T>(Ls[l].dev, s, 1, nullptr, r, Ls[l].y, x, alpha, st, nrhs);
 }
 
 // Algorithm 2: x = M_l^-1 r from x0 = 0
@@ -724,10 +723,10 @@ glls_status tune_levels(glls_problem* P, std::vector<LevelStore<T>>& Ls, int pre
                 if (blocks) Ls[l].dev.lbc[s] = c;
                 else Ls[l].dev.lpb[s] = c;
                 for (int w = 0; w < 3; ++w)
-                    launch_line_solve<T>(Ls[l].dev, s, 0, Ls[l].r, nullptr, nullptr, Ls[l].t2, T(1), st);
+                    CK(launch_line_solve<T>(Ls[l].dev, s, 0, Ls[l].r, nullptr, nullptr, Ls[l].t2, T(1), st));
                 CK(cudaEventRecord(a, st));
                 for (int w = 0; w < 10; ++w)
-                    launch_line_solve<T>(Ls[l].dev, s, 0, Ls[l].r, nullptr, nullptr, Ls[l].t2, T(1), st);
+                    CK(launch_line_solve<T>(Ls[l].dev, s, 0, Ls[l].r, nullptr, nullptr, Ls[l].t2, T(1), st));
                 CK(cudaEventRecord(b, st));
                 CK(cudaEventSynchronize(b));
                 float ms = 0.f;
@@ -2220,8 +2219,8 @@ glls_status glls_apply_partials_ff(glls_problem* P, int level, const double* x, 
         if (!g || !x) return fail(GLLS_ERR_INVALID, "null vector");                                             \
         DeviceScope scope(P->device);                                                                           \
         CK(scope.err);                                                                                          \
-        launch_line_solve<T>(levels_of<T>(P)[level].dev, axis, 0, g, nullptr, nullptr, x, T(1),                 \
-                             (cudaStream_t)stream);                                                             \
+        CK(launch_line_solve<T>(levels_of<T>(P)[level].dev, axis, 0, g, nullptr, nullptr, x, T(1),              \
+                                (cudaStream_t)stream));                                                         \
         CK(cudaGetLastError());                                                                                 \
         return GLLS_OK;                                                                                         \
     }                                                                                                           \
@@ -2233,7 +2232,7 @@ glls_status glls_apply_partials_ff(glls_problem* P, int level, const double* x, 
         if (!r || !x) return fail(GLLS_ERR_INVALID, "null vector");                                             \
         DeviceScope scope(P->device);                                                                           \
         CK(scope.err);                                                                                          \
-        smooth<T>(P, level, axis, alpha, r, x, false, (cudaStream_t)stream);                                    \
+        CK(smooth<T>(P, level, axis, alpha, r, x, false, (cudaStream_t)stream));                                \
         CK(cudaGetLastError());                                                                                 \
         return GLLS_OK;                                                                                         \
     }                                                                                                           \
@@ -2245,7 +2244,8 @@ glls_status glls_apply_partials_ff(glls_problem* P, int level, const double* x, 
         if (!r || !y || !x) return fail(GLLS_ERR_INVALID, "null vector");                                       \
         DeviceScope scope(P->device);                                                                           \
         CK(scope.err);                                                                                          \
-        launch_line_solve<T>(levels_of<T>(P)[level].dev, axis, 1, nullptr, r, y, x, alpha, (cudaStream_t)stream); \
+        CK(launch_line_solve<T>(levels_of<T>(P)[level].dev, axis, 1, nullptr, r, y, x, alpha,                   \
+                                (cudaStream_t)stream));                                                         \
         CK(cudaGetLastError());                                                                                 \
         return GLLS_OK;                                                                                         \
     }                                                                                                           \

@@ -334,9 +334,10 @@ cudaError_t launch_apply(const DevLevel<T>& L, const T* x, T* y, bool mask, cuda
 
 // Line solves along axis s.  mode 0: x = B_s^-1 g; mode 1: x += alpha
 // B_s^-1 (r - y) and y is reset to 0 where read; mode 2: x += alpha B_s^-1 r;
-// mode 3: x = alpha B_s^-1 r.  Only interior entries of x are written.
+// mode 3: x = alpha B_s^-1 r.  Only interior entries of x are written.  Returns
+// the launch's status.
 template <typename T>
-void launch_line_solve(const DevLevel<T>& L, int s, int mode, const T* g, const T* r, T* y,
+cudaError_t launch_line_solve(const DevLevel<T>& L, int s, int mode, const T* g, const T* r, T* y,
                        T* x, T alpha, cudaStream_t st, int nrhs = 1);
 
 // One tensor-product factor of a transfer: out = M in (or in - in2) along

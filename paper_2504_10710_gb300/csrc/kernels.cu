@@ -1399,34 +1399,34 @@ cudaError_t launch_apply(const DevLevel<T>& L, const T* x, T* y, bool mask, cuda
 }
 
 template <typename T>
-void launch_line_solve(const DevLevel<T>& L, int s, int mode, const T* g, const T* r, T* y, T* x, T alpha,
-                       cudaStream_t st, int nrhs) {
+cudaError_t launch_line_solve(const DevLevel<T>& L, int s, int mode, const T* g, const T* r, T* y, T* x, T alpha,
+                              cudaStream_t st, int nrhs) {
     // levels with Def. 3.2 line blocks: the condensed block solve (set-up
     // guarantees the sizes it takes)
-    if (L.blk[s] != nullptr) {
-        launch_line_block<T>(L, s, mode, g, r, y, x, alpha, st, nrhs);
-        return;
-    }
-    if (launch_line_warp<T>(L, s, mode, g, r, y, x, alpha, st, nrhs)) return;
+    if (L.blk[s] != nullptr)
+        return launch_line_block<T>(L, s, mode, g, r, y, x, alpha, st, nrhs) ? cudaSuccess
+                                                                             : cudaErrorInvalidConfiguration;
+    if (launch_line_warp<T>(L, s, mode, g, r, y, x, alpha, st, nrhs)) return cudaSuccess;
     // long band-1 lines: the shared-memory kernel, one launch per right-hand side
     if (nrhs > 1) {
         for (int j = 0; j < nrhs; ++j) {
             const long long o = (long long)j * L.N;
-            launch_line_solve<T>(L, s, mode, g ? g + o : nullptr, r ? r + o : nullptr, y ? y + o : nullptr, x + o,
-                                 alpha, st, 1);
+            const cudaError_t e = launch_line_solve<T>(L, s, mode, g ? g + o : nullptr, r ? r + o : nullptr,
+                                                       y ? y + o : nullptr, x + o, alpha, st, 1);
+            if (e != cudaSuccess) return e;
         }
-        return;
+        return cudaSuccess;
     }
     LineArgs<T> A;
     A.n = L.n[s] - 2;
-    if (A.n <= 0) return;
+    if (A.n <= 0) return cudaSuccess;
     int o1, o2;
     if (s == 0) { o1 = 1; o2 = 2; } else if (s == 1) { o1 = 0; o2 = 2; } else { o1 = 0; o2 = 1; }
     const long long strides[3] = {1, L.n[0], (long long)L.n[0] * L.n[1]};
     A.m1 = L.n[o1] - 2;
     const int m2 = L.dim == 3 ? L.n[o2] - 2 : 1;
     A.nlines = (long long)A.m1 * m2;
-    if (A.nlines <= 0) return;
+    if (A.nlines <= 0) return cudaSuccess;
     A.stride = strides[s];
     A.st1 = strides[o1];
     A.st2 = L.dim == 3 ? strides[o2] : 0;
@@ -1449,7 +1449,7 @@ void launch_line_solve(const DevLevel<T>& L, int s, int mode, const T* g, const 
     A.W = (int)W;
     const size_t smem = per_line * W;
     const long long blocks = (A.nlines + W - 1) / W;
-    launch_k(line_kernel<T>, (unsigned)blocks, 256, smem, st, A);
+    return launch_k(line_kernel<T>, (unsigned)blocks, 256, smem, st, A);
 }
 
 template <typename T>
@@ -1738,9 +1738,9 @@ template cudaError_t launch_apply<double>(const DevLevel<double>&, const double*
                                    double*, unsigned*, int, double*);
 template cudaError_t launch_apply<float>(const DevLevel<float>&, const float*, float*, bool, cudaStream_t, bool, double*,
                                   double*, unsigned*, int, float*);
-template void launch_line_solve<double>(const DevLevel<double>&, int, int, const double*, const double*, double*,
+template cudaError_t launch_line_solve<double>(const DevLevel<double>&, int, int, const double*, const double*, double*,
                                         double*, double, cudaStream_t, int);
-template void launch_line_solve<float>(const DevLevel<float>&, int, int, const float*, const float*, float*,
+template cudaError_t launch_line_solve<float>(const DevLevel<float>&, int, int, const float*, const float*, float*,
                                        float*, float, cudaStream_t, int);
 template void launch_transfer<double>(const DevBand<double>&, int, const int*, const int*, const double*, const double*,
                                       double*, bool, bool, cudaStream_t, double*, int);

@@ -31,7 +31,7 @@
 // kernel writes, so they are loaded before the wait on the preceding kernel
 // and overlap its end.
 // P is the compile-time order (2..12); line_any_body takes the order at run
-// time with the operators in shared memory.
+// time, with the operators in shared memory where one line's fit there.
 #include "async_copy.cuh"
 #include "cr_warp.cuh"
 #include "device.cuh"
@@ -401,8 +401,11 @@ __device__ __forceinline__ void line_seg_body(const BlockLineArgs<T>& A, int blk
 }
 
 // Any order and line length: the line values and the segment operators in
-// shared memory (cp.async), z accumulated there.
-template <typename T, int C>
+// shared memory (cp.async), z accumulated there.  STAGED = false reads the
+// operators from global memory where they are used: the form of the lines
+// whose operators alone pass the shared-memory limit (FP64 from p = 39 on one
+// element, p = 16 on 97 elements a line; FP32 from p = 55).
+template <typename T, int C, bool STAGED>
 __device__ __forceinline__ void line_any_body(BlockLineArgs<T> A, int blk) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n = A.n, E = A.E, span = A.span, mode = A.mode, LPC = A.lpc, SE = E | 1;
@@ -439,11 +442,14 @@ __device__ __forceinline__ void line_any_body(BlockLineArgs<T> A, int blk) {
         const int wg = tid / A.sub;
         vc.load(A, l0 + wg, wg < Wc, tid & (A.sub - 1));
     }
-    if (has_task) {
+    if (STAGED && has_task) {
         const int ncoef = npk + 2 * mi;
         for (int c = 0; c < ncoef; ++c) cp_async(sop + c * opstride + tid, bp + (long long)c * ntask);
     }
-    auto opc = [&](int c) { return sop[c * opstride + tid]; };   // coefficient c of this thread's segment
+    auto opc = [&](int c) {   // coefficient c of this thread's segment
+        if constexpr (STAGED) return sop[c * opstride + tid];
+        else return __ldg(bp + (long long)c * ntask);
+    };
     if (!grid_dep_ready(A.done)) {
         cp_async_wait_all();
         return;
@@ -539,10 +545,11 @@ __device__ __forceinline__ void line_any_body(BlockLineArgs<T> A, int blk) {
     }
 }
 
-template <typename T, int P, int CV, bool CONTIG>
+// FORM: x-lines (P > 0); operators in shared memory (P == 0, any direction).
+template <typename T, int P, int CV, bool FORM>
 __device__ __forceinline__ void line_block_body(const BlockLineArgs<T>& A, int blk) {
-    if constexpr (P == 0) line_any_body<T, CV>(A, blk);
-    else line_seg_body<T, P, CV, CONTIG>(A, blk);
+    if constexpr (P == 0) line_any_body<T, CV, FORM>(A, blk);
+    else line_seg_body<T, P, CV, FORM>(A, blk);
 }
 
 // Resident CTAs the registers must allow.
@@ -551,19 +558,19 @@ constexpr int line_min_ctas() {
     return sizeof(T) == 8 ? 2 : P == 0 ? 2 : P >= 9 ? 1 : 3;
 }
 
-template <typename T, int P, int CV, bool CONTIG>
+template <typename T, int P, int CV, bool FORM>
 __global__ void __launch_bounds__(kBlockThreads, line_min_ctas<T, P>())
     line_block_kernel(const __grid_constant__ BlockLineArgs<T> A) {
-    line_block_body<T, P, CV, CONTIG>(A, blockIdx.x);
+    line_block_body<T, P, CV, FORM>(A, blockIdx.x);
 }
 
 // Work-list form: item j (one problem's level, direction and vectors) owns
 // the CTAs [start[j], start[j + 1]).
-template <typename T, int P, int CV, bool CONTIG>
+template <typename T, int P, int CV, bool FORM>
 __global__ void __launch_bounds__(kBlockThreads, line_min_ctas<T, P>())
     line_block_list_kernel(const BlockLineArgs<T>* __restrict__ items, const int* __restrict__ start, int nitems) {
     const int j = work_item(start, nitems, blockIdx.x);
-    line_block_body<T, P, CV, CONTIG>(items[j], blockIdx.x - start[j]);
+    line_block_body<T, P, CV, FORM>(items[j], blockIdx.x - start[j]);
 }
 
 // Shared memory of a CTA of lpc lines: the vertex arrays, with the line
@@ -610,18 +617,21 @@ bool launch_pc(BlockLineArgs<T> A, cudaStream_t st) {
         const int least = A.contiguous ? 1 : 4;
         while (lpc > least && (long long)(A.nlines + lpc - 1) / lpc * A.nrhs < 4 * sm_count()) lpc /= 2;
     }
-    auto sm = [&](int c) {
+    // the run-time order's operators: in shared memory unless those of a
+    // single line do not fit beside its values
+    auto sm = [&](int c, bool staged) {
         return block_smem<T>(c, A.n, A.span, A.E, A.contiguous != 0, P == 0) +
-               (P == 0 ? op_smem<T>(A.p, block_threads(c, A.E)) : 0);
+               (staged ? op_smem<T>(A.p, block_threads(c, A.E)) : 0);
     };
-    while (lpc > 1 && sm(lpc) > kMaxDynSmemBytes) lpc /= 2;
-    const size_t smem = sm(lpc);
-    if (smem > kMaxDynSmemBytes) return false;
+    const bool staged = P == 0 && sm(1, true) <= kMaxDynSmemBytes;
+    while (lpc > 1 && sm(lpc, staged) > kMaxDynSmemBytes) lpc /= 2;
+    const size_t smem = sm(lpc, staged);
+    if (smem > kMaxDynSmemBytes) return false;   // not reached: kMaxBlockLine, kMaxBlockSegments
     A.lpc = lpc;
     const int threads = block_threads(lpc, A.E);
     const long long blocks = (long long)(A.nlines + lpc - 1) / lpc * A.nrhs;
     if (blocks > 0x7fffffffLL) return false;
-    if (P > 0 && !A.contiguous)
+    if (P > 0 ? !A.contiguous : !staged)
         return launch_k(line_block_kernel<T, P, CV, false>, (unsigned)blocks, threads, smem, st, A) == cudaSuccess;
     return launch_k(line_block_kernel<T, P, CV, true>, (unsigned)blocks, threads, smem, st, A) == cudaSuccess;
 }
@@ -648,6 +658,8 @@ bool set_attr_any() {
     const int lim = (int)kMaxDynSmemBytes;
     const void* fns[] = {(const void*)line_block_kernel<T, 0, 1, true>, (const void*)line_block_kernel<T, 0, 2, true>,
                          (const void*)line_block_kernel<T, 0, 4, true>, (const void*)line_block_kernel<T, 0, 8, true>,
+                         (const void*)line_block_kernel<T, 0, 1, false>, (const void*)line_block_kernel<T, 0, 2, false>,
+                         (const void*)line_block_kernel<T, 0, 4, false>, (const void*)line_block_kernel<T, 0, 8, false>,
                          (const void*)line_block_list_kernel<T, 0, 1, true>,
                          (const void*)line_block_list_kernel<T, 0, 2, true>,
                          (const void*)line_block_list_kernel<T, 0, 4, true>,
