@@ -876,8 +876,8 @@ struct WlRecord {
     std::vector<unsigned char> items;  // host copy of the item array
     std::vector<int> start{0};         // CTA offsets, nitems + 1
     std::vector<int> owner;            // the group position of each item's problem
-    size_t item_bytes = 0, done_at = 0;   // item size and offset of its stop-flag pointer
-    size_t off_items = 0, off_start = 0;
+    size_t off_items = 0, off_start = 0, off_owner = 0, off_S = 0;   // in the plan's block
+    bool own = true;                   // item j belongs to the group's problem j
 
     template <class Item>
     void put(const Item& it, int nblocks, int who) {
@@ -885,8 +885,7 @@ struct WlRecord {
         items.insert(items.end(), b, b + sizeof(Item));
         start.push_back(start.back() + nblocks);
         owner.push_back(who);
-        item_bytes = sizeof(Item);
-        done_at = offsetof(Item, done);
+        own = own && who == nitems;
         ++nitems;
         blocks = start.back();
     }
@@ -971,7 +970,7 @@ struct WlBuilder {
             glls_problem* P = G.probs[j];
             const DevLevel<T>& L = levels_of<T>(P)[l].dev;
             r.p = L.p;
-            ApplyItem<T> it{L, xv(P, l), levels_of<T>(P)[l].y, nullptr, nullptr};
+            ApplyItem<T> it{L, xv(P, l), levels_of<T>(P)[l].y, nullptr};
             r.put(it, apply_list_blocks(L.p, L.E), (int)j);
         }
         G.body.push_back(std::move(r));
@@ -986,8 +985,6 @@ struct WlBuilder {
         r.threads = 32;
         std::vector<size_t> sm0, sm1;
         std::vector<unsigned char> buf(line_block_item_bytes<T>());
-        r.item_bytes = buf.size();
-        r.done_at = line_block_item_done_offset<T>();
         for (size_t j = 0; j < G.probs.size(); ++j) {
             glls_problem* P = G.probs[j];
             auto& Ls = levels_of<T>(P);
@@ -1001,6 +998,7 @@ struct WlBuilder {
             r.items.insert(r.items.end(), buf.begin(), buf.end());
             r.start.push_back(r.start.back() + blocks);
             r.owner.push_back((int)j);
+            r.own = r.own && (int)j == r.nitems;
             ++r.nitems;
             r.blocks = r.start.back();
             r.threads = std::max(r.threads, threads);
@@ -1184,7 +1182,7 @@ std::string build_group(WlGroup& G, const glls_solve_opts& o) {
         items.push_back(it);
         ap.p = F.p;
         ap.ff = ap.ff && F.dim == 2 && apply_ff_supported(F);
-        ApplyItem<double> ai{F, P->pk, P->qk, ppq, nullptr};
+        ApplyItem<double> ai{F, P->pk, P->qk, ppq};
         ap.put(ai, apply_list_blocks(F.p, F.E), (int)j);
     }
     // CTAs per problem of the outer-Krylov kernels: enough for the largest
@@ -1218,66 +1216,58 @@ std::string build_group(WlGroup& G, const glls_solve_opts& o) {
 }
 
 // Problem j of a group uses S = (plan block) + off_S + j S_COUNT: the FCG
-// items get that pointer, every other item a pointer to its S_DONE flag,
-// once the block is allocated.
+// items get that pointer once the block is allocated (the other kernels find
+// their problem's stop flag through their WorkList).
 void bind_scalars(WlGroup& G, unsigned char* base) {
     double* S = reinterpret_cast<double*>(base + G.off_S);
-    for (auto& r : G.body)
+    for (auto& r : G.body) {
+        if (r.kind != WL_FCG) continue;
         for (int i = 0; i < r.nitems; ++i) {
-            double* Sj = S + (size_t)r.owner[i] * S_COUNT;
-            if (r.kind == WL_FCG) {
-                FcgItem it;
-                std::memcpy(&it, r.items.data() + sizeof(FcgItem) * i, sizeof(FcgItem));
-                it.S = Sj;
-                std::memcpy(r.items.data() + sizeof(FcgItem) * i, &it, sizeof(FcgItem));
-            } else {
-                const double* done = Sj + S_DONE;
-                std::memcpy(r.items.data() + r.item_bytes * i + r.done_at, &done, sizeof(done));
-            }
+            FcgItem it;
+            std::memcpy(&it, r.items.data() + sizeof(FcgItem) * i, sizeof(FcgItem));
+            it.S = S + (size_t)r.owner[i] * S_COUNT;
+            std::memcpy(r.items.data() + sizeof(FcgItem) * i, &it, sizeof(FcgItem));
         }
+    }
 }
 
 cudaError_t replay(const WlRecord& r, const unsigned char* base, int flexible, cudaStream_t st) {
     const void* items = base + r.off_items;
-    const int* start = reinterpret_cast<const int*>(base + r.off_start);
+    const WorkList w{reinterpret_cast<const int*>(base + r.off_start), r.nitems,
+                     reinterpret_cast<const double*>(base + r.off_S),
+                     r.own ? nullptr : reinterpret_cast<const int*>(base + r.off_owner)};
     bool ok = true;
     switch (r.kind) {
         case WL_APPLY:
             if (r.ff) {
-                ok = launch_apply_ff_list(r.p, (const ApplyItem<double>*)items, start, r.nitems, r.blocks, r.mask, st);
+                ok = launch_apply_ff_list(r.p, (const ApplyItem<double>*)items, w, r.blocks, r.mask, st);
                 break;
             }
-            ok = r.dbl ? launch_apply_list<double>(r.p, (const ApplyItem<double>*)items, start, r.nitems, r.blocks,
-                                                   r.mask, r.dot, st)
-                       : launch_apply_list<float>(r.p, (const ApplyItem<float>*)items, start, r.nitems, r.blocks,
-                                                  r.mask, r.dot, st);
+            ok = r.dbl ? launch_apply_list<double>(r.p, (const ApplyItem<double>*)items, w, r.blocks, r.mask, r.dot, st)
+                       : launch_apply_list<float>(r.p, (const ApplyItem<float>*)items, w, r.blocks, r.mask, r.dot, st);
             break;
         case WL_LINE:
-            ok = r.dbl ? launch_line_block_list<double>(r.p, r.s, r.cv, items, start, r.nitems, r.blocks, r.threads, r.smem,
-                                                        st)
-                       : launch_line_block_list<float>(r.p, r.s, r.cv, items, start, r.nitems, r.blocks, r.threads, r.smem,
-                                                       st);
+            ok = r.dbl ? launch_line_block_list<double>(r.p, r.s, r.cv, items, w, r.blocks, r.threads, r.smem, st)
+                       : launch_line_block_list<float>(r.p, r.s, r.cv, items, w, r.blocks, r.threads, r.smem, st);
             break;
         case WL_T2:
-            ok = r.dbl ? launch_transfer2_list<double>(r.wb, r.ty, (const Transfer2Item<double>*)items, start,
-                                                       r.nitems, r.blocks, r.smem, r.add, r.mask, st)
-                       : launch_transfer2_list<float>(r.wb, r.ty, (const Transfer2Item<float>*)items, start, r.nitems,
-                                                      r.blocks, r.smem, r.add, r.mask, st);
+            ok = r.dbl ? launch_transfer2_list<double>(r.wb, r.ty, (const Transfer2Item<double>*)items, w, r.blocks,
+                                                       r.smem, r.add, r.mask, st)
+                       : launch_transfer2_list<float>(r.wb, r.ty, (const Transfer2Item<float>*)items, w, r.blocks,
+                                                      r.smem, r.add, r.mask, st);
             break;
         case WL_BCR_F:
         case WL_BCR_B:
             if (r.dbl)
-                launch_bcr_list<double>(r.kind == WL_BCR_F, r.l, (const BcrItem<double>*)items, start, r.nitems,
-                                        r.blocks, r.smem, st);
+                launch_bcr_list<double>(r.kind == WL_BCR_F, r.l, (const BcrItem<double>*)items, w, r.blocks, r.smem, st);
             else
-                launch_bcr_list<float>(r.kind == WL_BCR_F, r.l, (const BcrItem<float>*)items, start, r.nitems,
-                                       r.blocks, r.smem, st);
+                launch_bcr_list<float>(r.kind == WL_BCR_F, r.l, (const BcrItem<float>*)items, w, r.blocks, r.smem, st);
             break;
         case WL_COARSE:
             if (r.dbl)
-                launch_coarse_list<double>((const CoarseItem<double>*)items, start, r.nitems, r.blocks, r.smem, st);
+                launch_coarse_list<double>((const CoarseItem<double>*)items, w, r.blocks, r.smem, st);
             else
-                launch_coarse_list<float>((const CoarseItem<float>*)items, start, r.nitems, r.blocks, r.smem, st);
+                launch_coarse_list<float>((const CoarseItem<float>*)items, w, r.blocks, r.smem, st);
             break;
         default:
             launch_fcg_list(r.step, (const FcgItem*)items, r.nitems, flexible, r.blocks, r.mixed, st);
@@ -1318,10 +1308,19 @@ cudaError_t capture_plan(WlPlan* W, const glls_solve_opts* o) {
             // profiling form: `unroll` passes of the body inline, no
             // conditional node (ncu lists the kernels of the passes)
             launch_solve_init(S, 0, o->tol, o->max_iter, G.s1, n, false);
+            // the work-list kernels read the stop flags ahead of their wait: a
+            // copy after the kernel that writes them makes the dependency on it
+            // a full one, as the conditional node does
+            auto fence = [&] {
+                if (e == cudaSuccess)
+                    e = cudaMemcpyAsync(G.probs[0]->S, S, sizeof(double) * S_COUNT, cudaMemcpyDeviceToDevice, G.s1);
+            };
+            fence();
             for (int k = 0; k < unroll && e == cudaSuccess; ++k) {
                 for (const WlRecord& r : G.body)
                     if (e == cudaSuccess) e = replay(r, base, flexible, G.s1);
                 launch_solve_cond(S, 0, o->max_iter, G.s1, n, false);
+                fence();
             }
         } else {
             cudaStreamCaptureStatus stt;
@@ -1430,6 +1429,8 @@ glls_status make_plan(glls_problem* const* probs, int n, const glls_solve_opts* 
         for (auto& r : G.body) {
             r.off_items = take(r.items.size());
             r.off_start = take(sizeof(int) * r.start.size());
+            r.off_owner = r.own ? 0 : take(sizeof(int) * r.owner.size());
+            r.off_S = G.off_S;
         }
     }
     CK(dev_malloc(&W->dev, bytes));
@@ -1439,6 +1440,7 @@ glls_status make_plan(glls_problem* const* probs, int n, const glls_solve_opts* 
         for (auto& r : G.body) {
             std::memcpy(host.data() + r.off_items, r.items.data(), r.items.size());
             std::memcpy(host.data() + r.off_start, r.start.data(), sizeof(int) * r.start.size());
+            if (!r.own) std::memcpy(host.data() + r.off_owner, r.owner.data(), sizeof(int) * r.owner.size());
         }
     }
     CK(cudaMemcpy(W->dev, host.data(), bytes, cudaMemcpyHostToDevice));

@@ -59,7 +59,7 @@ __device__ __forceinline__ float dot_cs(const float* a, const float* b) {
 template <typename T, int DIM, int P, bool DOT, bool LOC>
 __device__ __forceinline__ void apply_p_body(const DevLevel<T>& L, const T* __restrict__ x, T* __restrict__ y,
                                              int mask, double* dot, double* part, unsigned* ticket, int nrhs, int blk,
-                                             int nblk, const double* done, T* loc) {
+                                             int nblk, double stopped, T* loc) {
     const int rhs = blk % nrhs, bx = blk / nrhs, nbx = nblk / nrhs;
     x += (long long)rhs * L.N;
     y += (long long)rhs * L.N;
@@ -91,6 +91,7 @@ __device__ __forceinline__ void apply_p_body(const DevLevel<T>& L, const T* __re
         sxyz[threadIdx.x] = ex | (ey << 10) | (ez << 20);
     }
 
+    if (skip_item(stopped)) return;
     T gk[ITEMS][NC];
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
@@ -106,7 +107,7 @@ __device__ __forceinline__ void apply_p_body(const DevLevel<T>& L, const T* __re
         if constexpr (VEC) sDT[t] = L.D[(t % N1) * N1 + t / N1];
     }
     __syncthreads();
-    if (!grid_dep_ready(done)) return;
+    grid_dep_sync();
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
         const int t = threadIdx.x + THREADS * it;
@@ -209,19 +210,19 @@ template <typename T, int DIM, int P, bool DOT, bool LOC>
 __global__ void __launch_bounds__(threads_of<DIM, P>(), 1) apply_p_kernel(DevLevel<T> L, const T* __restrict__ x, T* __restrict__ y,
                                                          int mask, double* dot, double* part, unsigned* ticket,
                                                          int nrhs, T* loc) {
-    apply_p_body<T, DIM, P, DOT, LOC>(L, x, y, mask, dot, part, ticket, nrhs, blockIdx.x, gridDim.x, nullptr,
-                                 loc);
+    apply_p_body<T, DIM, P, DOT, LOC>(L, x, y, mask, dot, part, ticket, nrhs, blockIdx.x, gridDim.x, 0.0,
+                                      loc);
 }
 
-// Work-list form: item j (its own level, vectors and partials) owns the CTAs
-// [start[j], start[j + 1]) of the launch.
+// Work-list form: item j is one problem's level, vectors and partials.
 template <typename T, int DIM, int P, bool DOT>
-__global__ void __launch_bounds__(threads_of<DIM, P>(), 1) apply_p_list_kernel(const ApplyItem<T>* __restrict__ items,
-                                                              const int* __restrict__ start, int nitems, int mask) {
-    const int j = work_item(start, nitems, blockIdx.x);
+__global__ void __launch_bounds__(threads_of<DIM, P>(), 1)
+    apply_p_list_kernel(const ApplyItem<T>* __restrict__ items, WorkList w, int mask) {
+    const int j = work_item(w, blockIdx.x);
+    const double stopped = item_stopped(w, j);
     const ApplyItem<T>& it = items[j];
-    apply_p_body<T, DIM, P, DOT, false>(it.L, it.x, it.y, mask, nullptr, it.part, nullptr, 1, blockIdx.x - start[j],
-                                 start[j + 1] - start[j], it.done, nullptr);
+    apply_p_body<T, DIM, P, DOT, false>(it.L, it.x, it.y, mask, nullptr, it.part, nullptr, 1, blockIdx.x - w.start[j],
+                                        w.start[j + 1] - w.start[j], stopped, nullptr);
 }
 
 // Number of CTAs (= dot partials) the specialised apply launches for L.
@@ -269,21 +270,21 @@ bool dispatch(int p, const DevLevel<T>& L, const T* x, T* y, bool mask, double* 
 }
 
 template <typename T, int P>
-bool launch_list_p(int p, const ApplyItem<T>* items, const int* start, int nitems, int blocks, bool mask, bool dot,
+bool launch_list_p(int p, const ApplyItem<T>* items, const WorkList& w, int blocks, bool mask, bool dot,
                    cudaStream_t st) {
     if constexpr (P == 0) {
         return false;
     } else {
-        if (p != P) return launch_list_p<T, P - 1>(p, items, start, nitems, blocks, mask, dot, st);
+        if (p != P) return launch_list_p<T, P - 1>(p, items, w, blocks, mask, dot, st);
+        constexpr int threads = threads_of<2, P>();
         if constexpr (sizeof(T) == 8) {
             if (dot) {
-                launch_k(apply_p_list_kernel<T, 2, P, true>, (unsigned)blocks, threads_of<2, P>(), 0, st, items, start, nitems,
-                         mask ? 1 : 0);
+                launch_k(apply_p_list_kernel<T, 2, P, true>, (unsigned)blocks, threads, 0, st, items, w, mask ? 1 : 0);
                 return true;
             }
         }
         if (dot) return false;
-        launch_k(apply_p_list_kernel<T, 2, P, false>, (unsigned)blocks, threads_of<2, P>(), 0, st, items, start, nitems, mask ? 1 : 0);
+        launch_k(apply_p_list_kernel<T, 2, P, false>, (unsigned)blocks, threads, 0, st, items, w, mask ? 1 : 0);
         return true;
     }
 }
@@ -300,13 +301,13 @@ int apply_list_blocks(int p, long long E) {
 
 // 2-D work-list apply (orders 1..16): every item's level has order p.
 template <typename T>
-bool launch_apply_list(int p, const ApplyItem<T>* items, const int* start, int nitems, int blocks, bool mask,
-                       bool dot, cudaStream_t st) {
-    if (nitems < 1 || blocks < 1) return true;
-    return launch_list_p<T, 16>(p, items, start, nitems, blocks, mask, dot, st);
+bool launch_apply_list(int p, const ApplyItem<T>* items, const WorkList& w, int blocks, bool mask, bool dot,
+                       cudaStream_t st) {
+    if (w.nitems < 1 || blocks < 1) return true;
+    return launch_list_p<T, 16>(p, items, w, blocks, mask, dot, st);
 }
-template bool launch_apply_list<float>(int, const ApplyItem<float>*, const int*, int, int, bool, bool, cudaStream_t);
-template bool launch_apply_list<double>(int, const ApplyItem<double>*, const int*, int, int, bool, bool,
+template bool launch_apply_list<float>(int, const ApplyItem<float>*, const WorkList&, int, bool, bool, cudaStream_t);
+template bool launch_apply_list<double>(int, const ApplyItem<double>*, const WorkList&, int, bool, bool,
                                         cudaStream_t);
 
 // Dot partials that launch_apply writes for L (one per CTA of the

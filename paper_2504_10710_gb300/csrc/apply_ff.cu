@@ -53,7 +53,7 @@ __device__ __forceinline__ double block_sum_lean(double v, double* sv) {
 template <int P>
 __device__ __forceinline__ void apply_ff_body(const DevLevel<double>& L, const double* __restrict__ x,
                                               double* __restrict__ y, int mask, double* part, int nrhs, int blk,
-                                              int nblk, const double* done) {
+                                              int nblk, double stopped) {
     const int rhs = blk % nrhs, bx = blk / nrhs, nbx = nblk / nrhs;
     x += (long long)rhs * L.N;
     y += (long long)rhs * L.N;
@@ -78,6 +78,7 @@ __device__ __forceinline__ void apply_ff_body(const DevLevel<double>& L, const d
         sbase[threadIdx.x] = ey * P * n0 + ex * P;
         sxy[threadIdx.x] = ex | (ey << 16);
     }
+    if (skip_item(stopped)) return;
     ffloat gk[ITEMS][3];
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
@@ -90,7 +91,7 @@ __device__ __forceinline__ void apply_ff_body(const DevLevel<double>& L, const d
     }
     for (int t = threadIdx.x; t < N1 * N1; t += THREADS) sD[t] = ff_from_double(L.D[t]);
     __syncthreads();
-    if (!grid_dep_ready(done)) return;   // G and D above are mesh data: loaded ahead of the wait
+    grid_dep_sync();             // G and D above are mesh data: loaded ahead of the wait
     double xd[ITEMS];
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
@@ -167,16 +168,18 @@ __device__ __forceinline__ void apply_ff_body(const DevLevel<double>& L, const d
 template <int P>
 __global__ void __launch_bounds__(apply_threads((P + 1) * (P + 1)), 1) apply_ff_kernel(DevLevel<double> L, const double* __restrict__ x,
                                                           double* __restrict__ y, int mask, double* part, int nrhs) {
-    apply_ff_body<P>(L, x, y, mask, part, nrhs, blockIdx.x, gridDim.x, nullptr);
+    apply_ff_body<P>(L, x, y, mask, part, nrhs, blockIdx.x, gridDim.x, 0.0);
 }
 
-// Work-list form: item j owns the CTAs [start[j], start[j + 1]).
+// Work-list form.
 template <int P>
-__global__ void __launch_bounds__(apply_threads((P + 1) * (P + 1)), 1) apply_ff_list_kernel(const ApplyItem<double>* __restrict__ items,
-                                                               const int* __restrict__ start, int nitems, int mask) {
-    const int j = work_item(start, nitems, blockIdx.x);
+__global__ void __launch_bounds__(apply_threads((P + 1) * (P + 1)), 1)
+    apply_ff_list_kernel(const ApplyItem<double>* __restrict__ items, WorkList w, int mask) {
+    const int j = work_item(w, blockIdx.x);
+    const double stopped = item_stopped(w, j);
     const ApplyItem<double>& it = items[j];
-    apply_ff_body<P>(it.L, it.x, it.y, mask, it.part, 1, blockIdx.x - start[j], start[j + 1] - start[j], it.done);
+    apply_ff_body<P>(it.L, it.x, it.y, mask, it.part, 1, blockIdx.x - w.start[j], w.start[j + 1] - w.start[j],
+                     stopped);
 }
 
 template <int P>
@@ -196,13 +199,13 @@ bool launch_ff(int p, const DevLevel<double>& L, const double* x, double* y, boo
 }
 
 template <int P>
-bool launch_ff_list(int p, const ApplyItem<double>* items, const int* start, int nitems, int blocks, bool mask,
+bool launch_ff_list(int p, const ApplyItem<double>* items, const WorkList& w, int blocks, bool mask,
                     cudaStream_t st) {
     if constexpr (P < 2) {
         return false;
     } else {
-        if (p != P) return launch_ff_list<P - 1>(p, items, start, nitems, blocks, mask, st);
-        return launch_k(apply_ff_list_kernel<P>, (unsigned)blocks, apply_threads((P + 1) * (P + 1)), 0, st, items, start, nitems,
+        if (p != P) return launch_ff_list<P - 1>(p, items, w, blocks, mask, st);
+        return launch_k(apply_ff_list_kernel<P>, (unsigned)blocks, apply_threads((P + 1) * (P + 1)), 0, st, items, w,
                         mask ? 1 : 0) == cudaSuccess;
     }
 }
@@ -508,10 +511,10 @@ bool launch_apply_ff(const DevLevel<double>& L, const double* x, double* y, bool
     return launch_ff<16>(L.p, L, x, y, mask, part, st, nrhs);
 }
 
-bool launch_apply_ff_list(int p, const ApplyItem<double>* items, const int* start, int nitems, int blocks, bool mask,
+bool launch_apply_ff_list(int p, const ApplyItem<double>* items, const WorkList& w, int blocks, bool mask,
                           cudaStream_t st) {
-    if (nitems < 1 || blocks < 1) return true;
-    return launch_ff_list<16>(p, items, start, nitems, blocks, mask, st);
+    if (w.nitems < 1 || blocks < 1) return true;
+    return launch_ff_list<16>(p, items, w, blocks, mask, st);
 }
 
 }  // namespace glls

@@ -39,15 +39,6 @@ __device__ __forceinline__ void grid_dep_sync() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
-// grid_dep_sync() for a CTA body that has already loaded mesh data (arrays no
-// kernel writes: geometry factors, operators, transfer bands, work-list
-// items), so that those loads overlap the end of the preceding kernel; false
-// when the work-list item's problem has stopped (done: its stop flag or null).
-__device__ __forceinline__ bool grid_dep_ready(const double* done) {
-    grid_dep_sync();
-    return !(done && *done != 0.0);
-}
-
 // False when GLLS_PDL=0 is set in the environment (plain stream order).
 bool pdl_enabled();
 
@@ -136,14 +127,27 @@ struct DevCoarse {
     const T* agk[kMaxCrLevels] = {};    // level l: [elim][3][m][ldm]: A_j^-1, A_j^-1 L_j, A_j^-1 U_j
 };
 
+// Krylov scalar slots in the device array S.
+// Per right-hand side j the slots sit at S + j * S_COUNT.  S_DONE: 0 while
+// iterating, 1 converged, 2 broken down; S_ITS: iterations when it stopped.
+enum Slot { S_RZ = 0, S_PQ, S_RR, S_RZNEW, S_ZQ, S_RR0, S_ALPHA, S_FLAG, S_TOL2, S_ITER, S_DONE, S_ITS, S_COUNT };
+
 // ---- work lists: one launch over the tiles of several problems ----------
 // Item j of a work-list launch owns the CTAs [start[j], start[j + 1]) of a
 // one-dimensional grid (start has nitems + 1 entries, start[0] = 0); every
 // item carries its own level data and vectors, so problems of different
-// sizes share a launch; an item whose problem has stopped (done flag set)
-// returns at once.  Returns the item of CTA b by bisection.
-__device__ __forceinline__ int work_item(const int* __restrict__ start, int nitems, int b) {
-    int lo = 0, hi = nitems - 1;
+// sizes share a launch.
+struct WorkList {
+    const int* start = nullptr;
+    int nitems = 0;
+    const double* S = nullptr;   // Krylov scalars of the group's problems, S_COUNT each
+    const int* owner = nullptr;  // the position in S of each item's problem; null: the item's own
+};
+
+// The item of CTA b, by bisection.
+__device__ __forceinline__ int work_item(const WorkList& w, int b) {
+    const int* __restrict__ start = w.start;
+    int lo = 0, hi = w.nitems - 1;
     while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (start[mid] <= b) lo = mid;
@@ -152,13 +156,37 @@ __device__ __forceinline__ int work_item(const int* __restrict__ start, int nite
     return lo;
 }
 
+// The stop flag of item j's problem (0: it iterates), read as soon as j is
+// known, beside the item's own fields.  It may be read before the wait on the
+// preceding kernel: the flags are written by the last kernel of a pass and by
+// the start of a solve only, and neither is followed by a work-list kernel
+// without a full dependency (the loop's condition lies between them).
+__device__ __forceinline__ double item_stopped(const WorkList& w, int j) {
+    double v;
+    const double* p = w.S + (long long)(w.owner ? w.owner[j] : j) * S_COUNT + S_DONE;
+    asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+
+// In a kernel body ahead of its mesh-data loads: true when the item's problem
+// has stopped, so that its CTAs load nothing more.  They still wait, which
+// keeps the ordering along the stream transitive.  (Two stopped problems of
+// 64 x 64 elements, p = 8, beside an active one of 6 x 6, mixed: 1.76 ms with
+// the flag read after the loads, 1.50 here; 24 uneven problems 16.5 and 16.1.
+// A flag read once by every thread from L2, again after the wait, cost the 24
+// problems 7 %.)
+__device__ __forceinline__ bool skip_item(double stopped) {
+    if (stopped == 0.0) return false;
+    grid_dep_sync();
+    return true;
+}
+
 template <typename T>
 struct ApplyItem {               // y (+)= A x on one problem's level; dot partials (FP64 outer apply) in part
     DevLevel<T> L;
     const T* x;
     T* y;
     double* part;
-    const double* done;          // the problem's stop flag (nonzero: its CTAs return at once), or null
 };
 
 template <typename T>
@@ -170,7 +198,6 @@ struct Transfer2Item {           // both in-plane factors of a restriction or pr
     T* out;
     T* clear;
     int gx, gy;                  // the item's tile grid (x: 32 outputs of axis 0, y: TY outputs of axis 1)
-    const double* done;
 };
 
 template <typename T>
@@ -182,7 +209,6 @@ struct CoarseItem {              // dense part of the coarsest solve (coarse_ker
     const long long* src_index;
     int m, H;
     T* e;
-    const double* done;
 };
 
 template <typename T>
@@ -193,7 +219,6 @@ struct BcrItem {                 // one block-CR level of one problem (bcr_forwa
     const T* src;                // forward: r; backward: w
     T* dst;                      // forward: w; backward: e
     int gx, rows;                // the item's CTA grid
-    const double* done;
 };
 
 struct FcgItem {                 // one problem's outer Krylov vectors, partial sums and scalars
@@ -229,8 +254,8 @@ __host__ __device__ constexpr int apply_epb(int nloc) { return nloc >= apply_thr
 
 int apply_list_blocks(int p, long long E);
 template <typename T>
-bool launch_apply_list(int p, const ApplyItem<T>* items, const int* start, int nitems, int blocks, bool mask,
-                       bool dot, cudaStream_t st);
+bool launch_apply_list(int p, const ApplyItem<T>* items, const WorkList& w, int blocks, bool mask, bool dot,
+                       cudaStream_t st);
 // Float-float outer apply with p.(A p) partials (apply_ff.cu): the finest
 // level of 2-D problems with 2 <= p <= 16 and of 3-D problems with
 // 2 <= p <= 8 (false elsewhere).  y seams zero on entry.
@@ -238,7 +263,7 @@ bool apply_ff_supported(const DevLevel<double>& L);
 int apply_ff_partials(const DevLevel<double>& L);   // dot partials (CTAs) per right-hand side
 bool launch_apply_ff(const DevLevel<double>& L, const double* x, double* y, bool mask, double* part,
                      cudaStream_t st, int nrhs);
-bool launch_apply_ff_list(int p, const ApplyItem<double>* items, const int* start, int nitems, int blocks, bool mask,
+bool launch_apply_ff_list(int p, const ApplyItem<double>* items, const WorkList& w, int blocks, bool mask,
                           cudaStream_t st);
 // The float-float apply serves solves with tol >= kFfMinTol: its rounding
 // (about 2^-44 relative per contraction) parts the recurrence residual from
@@ -248,14 +273,13 @@ template <typename T>
 bool transfer2_list_config(const DevBand<T>& M0, const DevBand<T>& M1, const int nout[3], int* gx, int* gy,
                            int* wb, int* ty, size_t* smem);
 template <typename T>
-bool launch_transfer2_list(int wb, int ty, const Transfer2Item<T>* items, const int* start, int nitems, int blocks,
+bool launch_transfer2_list(int wb, int ty, const Transfer2Item<T>* items, const WorkList& w, int blocks,
                            size_t smem, bool add, bool mask, cudaStream_t st);
 template <typename T>
-void launch_coarse_list(const CoarseItem<T>* items, const int* start, int nitems, int blocks, size_t smem,
-                        cudaStream_t st);
+void launch_coarse_list(const CoarseItem<T>* items, const WorkList& w, int blocks, size_t smem, cudaStream_t st);
 template <typename T>
-void launch_bcr_list(bool forward, int l, const BcrItem<T>* items, const int* start, int nitems, int blocks,
-                     size_t smem, cudaStream_t st);
+void launch_bcr_list(bool forward, int l, const BcrItem<T>* items, const WorkList& w, int blocks, size_t smem,
+                     cudaStream_t st);
 // blocks: CTAs per item (<= kDotBlocks), the same for every item: each item's
 // partial sums of r.z, z.q and r.r have that many entries
 void launch_fcg_list(int step, const FcgItem* items, int nitems, int flexible, int blocks, bool mixed,
@@ -263,13 +287,11 @@ void launch_fcg_list(int step, const FcgItem* items, int nitems, int flexible, i
 template <typename T>
 size_t line_block_item_bytes();
 template <typename T>
-size_t line_block_item_done_offset();
-template <typename T>
 int line_block_list_item(const DevLevel<T>& L, int s, int mode, const T* g, const T* r, T* y, T* x, T alpha,
                          void* item, int* blocks, int* threads, size_t smem[2], int* cv);
 bool line_block_list_specialised(int p, int cv);
 template <typename T>
-bool launch_line_block_list(int p, int s, int cv, const void* items, const int* start, int nitems, int blocks, int threads,
+bool launch_line_block_list(int p, int s, int cv, const void* items, const WorkList& w, int blocks, int threads,
                             size_t smem, cudaStream_t st);
 
 // Opt every kernel into up to 200 KB of dynamic shared memory (call once per
@@ -401,11 +423,6 @@ void launch_dots(const double* a0, const double* b0, const double* a1, const dou
 // reset to 0 after it is read.
 void launch_dots_rz_zq(const double* r, const double* z, const float* z32, double* q, long long n, double* prz,
                        double* pzq, cudaStream_t st, int nrhs = 1);
-
-// Krylov scalar slots in the device array S.
-// Per right-hand side j the slots sit at S + j * S_COUNT.  S_DONE: 0 while
-// iterating, 1 converged, 2 broken down; S_ITS: iterations when it stopped.
-enum Slot { S_RZ = 0, S_PQ, S_RR, S_RZNEW, S_ZQ, S_RR0, S_ALPHA, S_FLAG, S_TOL2, S_ITER, S_DONE, S_ITS, S_COUNT };
 
 // q-independent update on nb CTAs per right-hand side: p.q (npq partials from
 // the apply) is summed in every block, r.z taken from S_RZNEW, alpha = r.z /

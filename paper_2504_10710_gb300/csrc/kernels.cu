@@ -433,7 +433,7 @@ template <typename T>
 __device__ __forceinline__ void coarse_body(long long n, long long ld, const long long* __restrict__ index,
                                             const T* __restrict__ inv, const T* __restrict__ src,
                                             const long long* __restrict__ src_index, int m, int H, T* __restrict__ e,
-                                            int nrhs, long long vstride, int blk, int nblk, const double* done) {
+                                            int nrhs, long long vstride, int blk, int nblk, double stopped) {
     // right-hand side fastest in the CTA order (see device.cuh); src and e
     // hold vstride values per right-hand side
     const int rhs = blk % nrhs;
@@ -461,8 +461,9 @@ __device__ __forceinline__ void coarse_body(long long n, long long ld, const lon
         }
     };
     const long long row0 = bx * wpb + warp;
+    if (skip_item(stopped)) return;
     if (row0 < n) fetch(reinterpret_cast<const Vec*>(inv + row0 * ld), lane);
-    if (!grid_dep_ready(done)) return;
+    grid_dep_sync();
     for (long long t = threadIdx.x; t < ld; t += blockDim.x) {
         T w = T(0);
         if (t < n) {
@@ -503,16 +504,16 @@ __global__ void __launch_bounds__(256) coarse_kernel(long long n, long long ld, 
                                                      const T* __restrict__ inv, const T* __restrict__ src,
                                                      const long long* __restrict__ src_index, int m, int H,
                                                      T* __restrict__ e, int nrhs, long long vstride) {
-    coarse_body<T>(n, ld, index, inv, src, src_index, m, H, e, nrhs, vstride, blockIdx.x, gridDim.x, nullptr);
+    coarse_body<T>(n, ld, index, inv, src, src_index, m, H, e, nrhs, vstride, blockIdx.x, gridDim.x, 0.0);
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) coarse_list_kernel(const CoarseItem<T>* __restrict__ items,
-                                                          const int* __restrict__ start, int nitems) {
-    const int j = work_item(start, nitems, blockIdx.x);
+__global__ void __launch_bounds__(256) coarse_list_kernel(const CoarseItem<T>* __restrict__ items, WorkList w) {
+    const int j = work_item(w, blockIdx.x);
+    const double stopped = item_stopped(w, j);
     const CoarseItem<T>& it = items[j];
     coarse_body<T>(it.n, it.ld, it.index, it.inv, it.src, it.src_index, it.m, it.H, it.e, 1, 0,
-                   blockIdx.x - start[j], start[j + 1] - start[j], it.done);
+                   blockIdx.x - w.start[j], w.start[j + 1] - w.start[j], stopped);
 }
 
 // Rows of a block per CTA in the block-CR kernels: one per warp, so that a
@@ -532,7 +533,7 @@ constexpr int kBcrAhead = 4;
 template <typename T>
 __device__ __forceinline__ void bcr_forward_body(const T* __restrict__ FH, int l, int nb, int m, int ldm,
                                                  const long long* __restrict__ index, const T* __restrict__ r, T* w,
-                                                 int nrhs, long long nvec, int bx, int by, const double* done) {
+                                                 int nrhs, long long nvec, int bx, int by, double stopped) {
     const int rhs = bx % nrhs;
     r += rhs * nvec;
     w += rhs * nvec;
@@ -543,8 +544,9 @@ __device__ __forceinline__ void bcr_forward_body(const T* __restrict__ FH, int l
     const int row0 = by * kBcrRows;
     const bool lvl0 = l == 0;
     const int q = bx / nrhs;
+    if (skip_item(stopped)) return;
     if (q >= nk) {                                   // level 0: copy eliminated block 2 (q - nk)
-        if (!grid_dep_ready(done)) return;
+        grid_dep_sync();
         const long long b = 2LL * (q - nk);
         for (int rr = threadIdx.x; rr < kBcrRows; rr += blockDim.x) {
             const int row = row0 + rr;
@@ -567,7 +569,7 @@ __device__ __forceinline__ void bcr_forward_body(const T* __restrict__ FH, int l
         f[u] = ok ? __ldg(F + (size_t)row * ldm + c) : T(0);
         hh[u] = ok ? __ldg(Hm + (size_t)row * ldm + c) : T(0);
     }
-    if (!grid_dep_ready(done)) return;
+    grid_dep_sync();
     for (int c = threadIdx.x; c < m; c += blockDim.x) {
         xl[c] = lvl0 ? r[index[lb * m + c]] : w[lb * m + c];
         xr[c] = right ? (lvl0 ? r[index[rb * m + c]] : w[rb * m + c]) : T(0);
@@ -593,7 +595,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) bcr_forward_kernel(const T* __restrict__ FH, int l, int nb, int m, int ldm,
                                                           const long long* __restrict__ index,
                                                           const T* __restrict__ r, T* w, int nrhs, long long nvec) {
-    bcr_forward_body<T>(FH, l, nb, m, ldm, index, r, w, nrhs, nvec, blockIdx.x, blockIdx.y, nullptr);
+    bcr_forward_body<T>(FH, l, nb, m, ldm, index, r, w, nrhs, nvec, blockIdx.x, blockIdx.y, 0.0);
 }
 
 // Block CR back substitution at level l, one CTA per (eliminated block,
@@ -604,7 +606,7 @@ __global__ void __launch_bounds__(256) bcr_forward_kernel(const T* __restrict__ 
 template <typename T>
 __device__ __forceinline__ void bcr_backward_body(const T* __restrict__ AGK, int l, int nb, int m, int ldm,
                                                   const long long* __restrict__ index, const T* __restrict__ w, T* e,
-                                                  int nrhs, long long nvec, int bx, int by, const double* done) {
+                                                  int nrhs, long long nvec, int bx, int by, double stopped) {
     const int rhs = bx % nrhs;
     w += rhs * nvec;
     e += rhs * nvec;
@@ -622,6 +624,7 @@ __device__ __forceinline__ void bcr_backward_body(const T* __restrict__ AGK, int
     const T* K = G + (size_t)m * ldm;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int row = row0 + warp;                      // one row per warp
+    if (skip_item(stopped)) return;
     T fa[kBcrAhead], fg[kBcrAhead], fk[kBcrAhead];    // as in the forward step
 #pragma unroll
     for (int u = 0; u < kBcrAhead; ++u) {
@@ -633,7 +636,7 @@ __device__ __forceinline__ void bcr_backward_body(const T* __restrict__ AGK, int
         fk[u] = ok ? __ldg(K + o) : T(0);
     }
     const long long out = row < m ? index[b * m + row] : 0;
-    if (!grid_dep_ready(done)) return;
+    grid_dep_sync();
     for (int c = threadIdx.x; c < m; c += blockDim.x) {
         xw[c] = w[b * m + c];
         xl[c] = left ? e[index[lb * m + c]] : T(0);
@@ -659,22 +662,23 @@ template <typename T>
 __global__ void __launch_bounds__(256) bcr_backward_kernel(const T* __restrict__ AGK, int l, int nb, int m, int ldm,
                                                            const long long* __restrict__ index,
                                                            const T* __restrict__ w, T* e, int nrhs, long long nvec) {
-    bcr_backward_body<T>(AGK, l, nb, m, ldm, index, w, e, nrhs, nvec, blockIdx.x, blockIdx.y, nullptr);
+    bcr_backward_body<T>(AGK, l, nb, m, ldm, index, w, e, nrhs, nvec, blockIdx.x, blockIdx.y, 0.0);
 }
 
 // Work-list forms of both block-CR steps: item j owns the CTAs [start[j],
 // start[j + 1]) (its gx x rows grid, x fastest).
 template <typename T>
-__global__ void __launch_bounds__(256) bcr_list_kernel(const BcrItem<T>* __restrict__ items,
-                                                       const int* __restrict__ start, int nitems, int l, int forward) {
-    const int j = work_item(start, nitems, blockIdx.x);
+__global__ void __launch_bounds__(256) bcr_list_kernel(const BcrItem<T>* __restrict__ items, WorkList w, int l,
+                                                       int forward) {
+    const int j = work_item(w, blockIdx.x);
+    const double stopped = item_stopped(w, j);
     const BcrItem<T>& it = items[j];
-    const int local = blockIdx.x - start[j];
+    const int local = blockIdx.x - w.start[j];
     const int bx = local % it.gx, by = local / it.gx;
     if (forward)
-        bcr_forward_body<T>(it.ops, l, it.nb, it.m, it.ldm, it.index, it.src, it.dst, 1, 0, bx, by, it.done);
+        bcr_forward_body<T>(it.ops, l, it.nb, it.m, it.ldm, it.index, it.src, it.dst, 1, 0, bx, by, stopped);
     else
-        bcr_backward_body<T>(it.ops, l, it.nb, it.m, it.ldm, it.index, it.src, it.dst, 1, 0, bx, by, it.done);
+        bcr_backward_body<T>(it.ops, l, it.nb, it.m, it.ldm, it.index, it.src, it.dst, 1, 0, bx, by, stopped);
 }
 
 // Fused two-factor transfer: a CTA of 32 x 8 threads computes a 32 x TY tile
@@ -687,7 +691,7 @@ template <typename T, int WB, int TY>
 __device__ __forceinline__ void transfer2_body(const DevBand<T>& M0, const DevBand<T>& M1, int3 nin, int3 nout,
                                                const T* __restrict__ in, const T* __restrict__ in2,
                                                T* __restrict__ out, int add, int mask, T* __restrict__ clear, int bx,
-                                               int by, int z, const double* done) {
+                                               int by, int z, double stopped) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int win[4];                       // column lo, column count, row lo, row count
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
@@ -695,6 +699,7 @@ __device__ __forceinline__ void transfer2_body(const DevBand<T>& M0, const DevBa
     const int W0 = M0.width, W1 = M1.width;
     const int I = I0 + tx;
     const bool okI = I < nout.x;
+    if (skip_item(stopped)) return;
     const int s0 = okI ? M0.start[I] : 0;
     T c0[WB];
 #pragma unroll
@@ -721,7 +726,7 @@ __device__ __forceinline__ void transfer2_body(const DevBand<T>& M0, const DevBa
         }
     }
     __syncthreads();
-    if (!grid_dep_ready(done)) return;            // the bands above are mesh data
+    grid_dep_sync();                              // the bands above are mesh data
     const int clo = win[0], ncol = win[1], rlo = win[2], nrow = win[3];
     T* sin = reinterpret_cast<T*>(smem_raw);      // nrow x ncol
     T* st = sin + (size_t)M1.span8 * M0.span32;   // nrow x 32
@@ -796,21 +801,21 @@ __global__ void __launch_bounds__(256) transfer2_kernel(DevBand<T> M0, DevBand<T
                                                         const T* __restrict__ in, const T* __restrict__ in2,
                                                         T* __restrict__ out, int add, int mask, T* __restrict__ clear) {
     transfer2_body<T, WB, TY>(M0, M1, nin, nout, in, in2, out, add, mask, clear, blockIdx.x, blockIdx.y, blockIdx.z,
-                              nullptr);
+                              0.0);
 }
 
 // Work-list form: item j owns the CTAs [start[j], start[j + 1]), its
 // gx x gy x (planes) tile grid, x fastest.
 template <typename T, int WB, int TY>
-__global__ void __launch_bounds__(256) transfer2_list_kernel(const Transfer2Item<T>* __restrict__ items,
-                                                             const int* __restrict__ start, int nitems, int add,
-                                                             int mask) {
-    const int j = work_item(start, nitems, blockIdx.x);
+__global__ void __launch_bounds__(256) transfer2_list_kernel(const Transfer2Item<T>* __restrict__ items, WorkList w,
+                                                             int add, int mask) {
+    const int j = work_item(w, blockIdx.x);
+    const double stopped = item_stopped(w, j);
     const Transfer2Item<T>& it = items[j];
-    const int local = blockIdx.x - start[j];
+    const int local = blockIdx.x - w.start[j];
     const int bx = local % it.gx, rest = local / it.gx;
     transfer2_body<T, WB, TY>(it.M0, it.M1, it.nin, it.nout, it.in, it.in2, it.out, add, mask, it.clear, bx,
-                              rest % it.gy, rest / it.gy, it.done);
+                              rest % it.gy, rest / it.gy, stopped);
 }
 
 // ---------------------------------------------------------------------------
@@ -1527,32 +1532,30 @@ bool transfer2_list_config(const DevBand<T>& M0, const DevBand<T>& M1, const int
 }
 
 template <typename T>
-bool launch_transfer2_list(int wb, int ty, const Transfer2Item<T>* items, const int* start, int nitems, int blocks,
+bool launch_transfer2_list(int wb, int ty, const Transfer2Item<T>* items, const WorkList& w, int blocks,
                            size_t smem, bool add, bool mask, cudaStream_t st) {
-    if (nitems < 1 || blocks < 1) return true;
+    if (w.nitems < 1 || blocks < 1) return true;
     if (ty != 8) return false;
     const int ad = add ? 1 : 0, mk = mask ? 1 : 0;
     cudaError_t e;
-    if (wb == 4) e = launch_k(transfer2_list_kernel<T, 4, 8>, blocks, 256, smem, st, items, start, nitems, ad, mk);
-    else if (wb == 8) e = launch_k(transfer2_list_kernel<T, 8, 8>, blocks, 256, smem, st, items, start, nitems, ad, mk);
-    else if (wb == 16)
-        e = launch_k(transfer2_list_kernel<T, 16, 8>, blocks, 256, smem, st, items, start, nitems, ad, mk);
-    else e = launch_k(transfer2_list_kernel<T, 32, 8>, blocks, 256, smem, st, items, start, nitems, ad, mk);
+    if (wb == 4) e = launch_k(transfer2_list_kernel<T, 4, 8>, blocks, 256, smem, st, items, w, ad, mk);
+    else if (wb == 8) e = launch_k(transfer2_list_kernel<T, 8, 8>, blocks, 256, smem, st, items, w, ad, mk);
+    else if (wb == 16) e = launch_k(transfer2_list_kernel<T, 16, 8>, blocks, 256, smem, st, items, w, ad, mk);
+    else e = launch_k(transfer2_list_kernel<T, 32, 8>, blocks, 256, smem, st, items, w, ad, mk);
     return e == cudaSuccess;
 }
 
 template <typename T>
-void launch_coarse_list(const CoarseItem<T>* items, const int* start, int nitems, int blocks, size_t smem,
-                        cudaStream_t st) {
-    if (nitems < 1 || blocks < 1) return;
-    launch_k(coarse_list_kernel<T>, blocks, 256, smem, st, items, start, nitems);
+void launch_coarse_list(const CoarseItem<T>* items, const WorkList& w, int blocks, size_t smem, cudaStream_t st) {
+    if (w.nitems < 1 || blocks < 1) return;
+    launch_k(coarse_list_kernel<T>, blocks, 256, smem, st, items, w);
 }
 
 template <typename T>
-void launch_bcr_list(bool forward, int l, const BcrItem<T>* items, const int* start, int nitems, int blocks,
-                     size_t smem, cudaStream_t st) {
-    if (nitems < 1 || blocks < 1) return;
-    launch_k(bcr_list_kernel<T>, blocks, 256, smem, st, items, start, nitems, l, forward ? 1 : 0);
+void launch_bcr_list(bool forward, int l, const BcrItem<T>* items, const WorkList& w, int blocks, size_t smem,
+                     cudaStream_t st) {
+    if (w.nitems < 1 || blocks < 1) return;
+    launch_k(bcr_list_kernel<T>, blocks, 256, smem, st, items, w, l, forward ? 1 : 0);
 }
 
 void launch_fcg_list(int step, const FcgItem* items, int nitems, int flexible, int blocks, bool mixed,
@@ -1568,14 +1571,14 @@ template bool transfer2_list_config<float>(const DevBand<float>&, const DevBand<
                                            int*, size_t*);
 template bool transfer2_list_config<double>(const DevBand<double>&, const DevBand<double>&, const int*, int*, int*,
                                             int*, int*, size_t*);
-template bool launch_transfer2_list<float>(int, int, const Transfer2Item<float>*, const int*, int, int, size_t, bool,
+template bool launch_transfer2_list<float>(int, int, const Transfer2Item<float>*, const WorkList&, int, size_t, bool,
                                            bool, cudaStream_t);
-template bool launch_transfer2_list<double>(int, int, const Transfer2Item<double>*, const int*, int, int, size_t, bool,
+template bool launch_transfer2_list<double>(int, int, const Transfer2Item<double>*, const WorkList&, int, size_t, bool,
                                             bool, cudaStream_t);
-template void launch_coarse_list<float>(const CoarseItem<float>*, const int*, int, int, size_t, cudaStream_t);
-template void launch_coarse_list<double>(const CoarseItem<double>*, const int*, int, int, size_t, cudaStream_t);
-template void launch_bcr_list<float>(bool, int, const BcrItem<float>*, const int*, int, int, size_t, cudaStream_t);
-template void launch_bcr_list<double>(bool, int, const BcrItem<double>*, const int*, int, int, size_t, cudaStream_t);
+template void launch_coarse_list<float>(const CoarseItem<float>*, const WorkList&, int, size_t, cudaStream_t);
+template void launch_coarse_list<double>(const CoarseItem<double>*, const WorkList&, int, size_t, cudaStream_t);
+template void launch_bcr_list<float>(bool, int, const BcrItem<float>*, const WorkList&, int, size_t, cudaStream_t);
+template void launch_bcr_list<double>(bool, int, const BcrItem<double>*, const WorkList&, int, size_t, cudaStream_t);
 
 template <typename T>
 void launch_coarse(const DevCoarse<T>& C, long long N0, const T* r, T* e, T* w, cudaStream_t st, bool e_boundary_zero,

@@ -37,7 +37,6 @@
 #include "device.cuh"
 
 #include <algorithm>
-#include <cstddef>
 #include <cstring>
 
 namespace glls {
@@ -66,7 +65,6 @@ struct BlockLineArgs {
     const T* r;
     T* y;
     T* x;
-    const double* done;                        // work lists: the problem's stop flag, or null
 };
 
 constexpr int kBlockThreads = 256;
@@ -265,7 +263,7 @@ __device__ __forceinline__ int enter(const BlockLineArgs<T>& A, int blk, long lo
 // interior nodes and adds into element-boundary ones).  MODE 2: x += alpha
 // B^-1 r.  MODE 3: x = alpha B^-1 r.
 template <typename T, int P, int C, bool CONTIG>
-__device__ __forceinline__ void line_seg_body(const BlockLineArgs<T>& A, int blk) {
+__device__ __forceinline__ void line_seg_body(const BlockLineArgs<T>& A, int blk, double stopped) {
     constexpr int MI = SegOp<T, P>::MI;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int E = A.E, LPC = A.lpc, SE = E | 1, mode = A.mode;
@@ -291,6 +289,7 @@ __device__ __forceinline__ void line_seg_body(const BlockLineArgs<T>& A, int blk
     }
     const bool act = w < Wc && e < E;
     const int li = l0 + (act ? w : 0);
+    if (skip_item(stopped)) return;
     SegOp<T, P> op;
     op.load(A.blk + (CONTIG ? (long long)li * E + e : (long long)(act ? e : 0) * A.nlines + li), A.ntask, act);
     VertexCr<T, C> vc;
@@ -301,7 +300,7 @@ __device__ __forceinline__ void line_seg_body(const BlockLineArgs<T>& A, int blk
     const int stride = CONTIG ? 1 : A.stride;
     const int c2 = li / A.m1 + 1, c1 = li - (c2 - 1) * A.m1 + 1;
     const int v0 = c1 * A.st1 + c2 * A.st2 + e * P * stride;   // the segment's left vertex
-    if (!grid_dep_ready(A.done)) return;
+    grid_dep_sync();
 
     T gi[MI], xi[MI], gv = T(0), xv = T(0);
     const bool vertex = act && e > 0;
@@ -406,7 +405,7 @@ __device__ __forceinline__ void line_seg_body(const BlockLineArgs<T>& A, int blk
 // whose operators alone pass the shared-memory limit (FP64 from p = 39 on one
 // element, p = 16 on 97 elements a line; FP32 from p = 55).
 template <typename T, int C, bool STAGED>
-__device__ __forceinline__ void line_any_body(BlockLineArgs<T> A, int blk) {
+__device__ __forceinline__ void line_any_body(BlockLineArgs<T> A, int blk, double stopped) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int n = A.n, E = A.E, span = A.span, mode = A.mode, LPC = A.lpc, SE = E | 1;
     const int p = A.p, mi = p - 1, npk = mi * (mi + 1) / 2;
@@ -437,6 +436,7 @@ __device__ __forceinline__ void line_any_body(BlockLineArgs<T> A, int blk) {
     // operator rows are as long as this launch item's own thread count (a
     // work-list block may be larger; its extra threads have no segment)
     const int opstride = block_threads(LPC, E);
+    if (skip_item(stopped)) return;
     VertexCr<T, C> vc;
     {
         const int wg = tid / A.sub;
@@ -450,10 +450,7 @@ __device__ __forceinline__ void line_any_body(BlockLineArgs<T> A, int blk) {
         if constexpr (STAGED) return sop[c * opstride + tid];
         else return __ldg(bp + (long long)c * ntask);
     };
-    if (!grid_dep_ready(A.done)) {
-        cp_async_wait_all();
-        return;
-    }
+    grid_dep_sync();
     // x-lines are walked along the line by whole warps; strided directions by
     // threads that each keep one line of the CTA and step over its rows,
     // adjacent threads on adjacent lines
@@ -547,9 +544,9 @@ __device__ __forceinline__ void line_any_body(BlockLineArgs<T> A, int blk) {
 
 // FORM: x-lines (P > 0); operators in shared memory (P == 0, any direction).
 template <typename T, int P, int CV, bool FORM>
-__device__ __forceinline__ void line_block_body(const BlockLineArgs<T>& A, int blk) {
-    if constexpr (P == 0) line_any_body<T, CV, FORM>(A, blk);
-    else line_seg_body<T, P, CV, FORM>(A, blk);
+__device__ __forceinline__ void line_block_body(const BlockLineArgs<T>& A, int blk, double stopped) {
+    if constexpr (P == 0) line_any_body<T, CV, FORM>(A, blk, stopped);
+    else line_seg_body<T, P, CV, FORM>(A, blk, stopped);
 }
 
 // Resident CTAs the registers must allow.
@@ -561,16 +558,16 @@ constexpr int line_min_ctas() {
 template <typename T, int P, int CV, bool FORM>
 __global__ void __launch_bounds__(kBlockThreads, line_min_ctas<T, P>())
     line_block_kernel(const __grid_constant__ BlockLineArgs<T> A) {
-    line_block_body<T, P, CV, FORM>(A, blockIdx.x);
+    line_block_body<T, P, CV, FORM>(A, blockIdx.x, 0.0);
 }
 
-// Work-list form: item j (one problem's level, direction and vectors) owns
-// the CTAs [start[j], start[j + 1]).
+// Work-list form: item j is one problem's level, direction and vectors.
 template <typename T, int P, int CV, bool FORM>
 __global__ void __launch_bounds__(kBlockThreads, line_min_ctas<T, P>())
-    line_block_list_kernel(const BlockLineArgs<T>* __restrict__ items, const int* __restrict__ start, int nitems) {
-    const int j = work_item(start, nitems, blockIdx.x);
-    line_block_body<T, P, CV, FORM>(items[j], blockIdx.x - start[j]);
+    line_block_list_kernel(const BlockLineArgs<T>* __restrict__ items, WorkList w) {
+    const int j = work_item(w, blockIdx.x);
+    const double stopped = item_stopped(w, j);
+    line_block_body<T, P, CV, FORM>(items[j], blockIdx.x - w.start[j], stopped);
 }
 
 // Shared memory of a CTA of lpc lines: the vertex arrays, with the line
@@ -725,34 +722,32 @@ int make_args(BlockLineArgs<T>& A, const DevLevel<T>& L, int s, int mode, const 
     A.r = r;
     A.y = y;
     A.x = x;
-    A.done = nullptr;
     return 1;
 }
 
 template <typename T, int P, int CV>
-bool launch_list_pc(int s, const void* items, const int* start, int nitems, int blocks, int threads, size_t smem,
+bool launch_list_pc(int s, const void* items, const WorkList& w, int blocks, int threads, size_t smem,
                     cudaStream_t st) {
     const BlockLineArgs<T>* it = static_cast<const BlockLineArgs<T>*>(items);
     if (P > 0 && s != 0)
-        return launch_k(line_block_list_kernel<T, P, CV, false>, (unsigned)blocks, threads, smem, st, it, start,
-                        nitems) == cudaSuccess;
-    return launch_k(line_block_list_kernel<T, P, CV, true>, (unsigned)blocks, threads, smem, st, it, start, nitems) ==
-           cudaSuccess;
+        return launch_k(line_block_list_kernel<T, P, CV, false>, (unsigned)blocks, threads, smem, st, it, w) ==
+               cudaSuccess;
+    return launch_k(line_block_list_kernel<T, P, CV, true>, (unsigned)blocks, threads, smem, st, it, w) == cudaSuccess;
 }
 
 template <typename T, int P>
-bool launch_list_p(int s, int cv, const void* items, const int* start, int nitems, int blocks, int threads, size_t smem,
+bool launch_list_p(int s, int cv, const void* items, const WorkList& w, int blocks, int threads, size_t smem,
                    cudaStream_t st) {
     if constexpr (P > 0) {
-        if (cv == 1) return launch_list_pc<T, P, 1>(s, items, start, nitems, blocks, threads, smem, st);
-        if (cv == 2) return launch_list_pc<T, P, 2>(s, items, start, nitems, blocks, threads, smem, st);
-        return launch_list_p<T, 0>(s, cv, items, start, nitems, blocks, threads, smem, st);
+        if (cv == 1) return launch_list_pc<T, P, 1>(s, items, w, blocks, threads, smem, st);
+        if (cv == 2) return launch_list_pc<T, P, 2>(s, items, w, blocks, threads, smem, st);
+        return launch_list_p<T, 0>(s, cv, items, w, blocks, threads, smem, st);
     } else {
         switch (cv) {
-            case 1: return launch_list_pc<T, 0, 1>(s, items, start, nitems, blocks, threads, smem, st);
-            case 2: return launch_list_pc<T, 0, 2>(s, items, start, nitems, blocks, threads, smem, st);
-            case 4: return launch_list_pc<T, 0, 4>(s, items, start, nitems, blocks, threads, smem, st);
-            default: return launch_list_pc<T, 0, 8>(s, items, start, nitems, blocks, threads, smem, st);
+            case 1: return launch_list_pc<T, 0, 1>(s, items, w, blocks, threads, smem, st);
+            case 2: return launch_list_pc<T, 0, 2>(s, items, w, blocks, threads, smem, st);
+            case 4: return launch_list_pc<T, 0, 4>(s, items, w, blocks, threads, smem, st);
+            default: return launch_list_pc<T, 0, 8>(s, items, w, blocks, threads, smem, st);
         }
     }
 }
@@ -762,11 +757,6 @@ bool launch_list_p(int s, int cv, const void* items, const int* start, int nitem
 template <typename T>
 size_t line_block_item_bytes() {
     return sizeof(BlockLineArgs<T>);
-}
-
-template <typename T>
-size_t line_block_item_done_offset() {
-    return offsetof(BlockLineArgs<T>, done);
 }
 
 // One work-list item: the line solve of L along s (as launch_line_block,
@@ -803,30 +793,29 @@ int line_block_list_item(const DevLevel<T>& L, int s, int mode, const T* g, cons
 // One launch over the items (all along axis s and of order p; cv: the largest
 // vertex chunk of the items).
 template <typename T>
-bool launch_line_block_list(int p, int s, int cv, const void* items, const int* start, int nitems, int blocks, int threads,
+bool launch_line_block_list(int p, int s, int cv, const void* items, const WorkList& w, int blocks, int threads,
                             size_t smem, cudaStream_t st) {
-    if (nitems < 1 || blocks < 1) return true;
+    if (w.nitems < 1 || blocks < 1) return true;
     switch (line_block_list_specialised(p, cv) ? p : 0) {
-        case 2: return launch_list_p<T, 2>(s, cv, items, start, nitems, blocks, threads, smem, st);
-        case 3: return launch_list_p<T, 3>(s, cv, items, start, nitems, blocks, threads, smem, st);
-        case 4: return launch_list_p<T, 4>(s, cv, items, start, nitems, blocks, threads, smem, st);
-        case 5: return launch_list_p<T, 5>(s, cv, items, start, nitems, blocks, threads, smem, st);
-        case 6: return launch_list_p<T, 6>(s, cv, items, start, nitems, blocks, threads, smem, st);
-        case 7: return launch_list_p<T, 7>(s, cv, items, start, nitems, blocks, threads, smem, st);
-        case 8: return launch_list_p<T, 8>(s, cv, items, start, nitems, blocks, threads, smem, st);
-        case 9: return launch_list_p<T, 9>(s, cv, items, start, nitems, blocks, threads, smem, st);
-        case 10: return launch_list_p<T, 10>(s, cv, items, start, nitems, blocks, threads, smem, st);
-        case 11: return launch_list_p<T, 11>(s, cv, items, start, nitems, blocks, threads, smem, st);
-        case 12: return launch_list_p<T, 12>(s, cv, items, start, nitems, blocks, threads, smem, st);
-        default: return launch_list_p<T, 0>(s, cv, items, start, nitems, blocks, threads, smem, st);
+        case 2: return launch_list_p<T, 2>(s, cv, items, w, blocks, threads, smem, st);
+        case 3: return launch_list_p<T, 3>(s, cv, items, w, blocks, threads, smem, st);
+        case 4: return launch_list_p<T, 4>(s, cv, items, w, blocks, threads, smem, st);
+        case 5: return launch_list_p<T, 5>(s, cv, items, w, blocks, threads, smem, st);
+        case 6: return launch_list_p<T, 6>(s, cv, items, w, blocks, threads, smem, st);
+        case 7: return launch_list_p<T, 7>(s, cv, items, w, blocks, threads, smem, st);
+        case 8: return launch_list_p<T, 8>(s, cv, items, w, blocks, threads, smem, st);
+        case 9: return launch_list_p<T, 9>(s, cv, items, w, blocks, threads, smem, st);
+        case 10: return launch_list_p<T, 10>(s, cv, items, w, blocks, threads, smem, st);
+        case 11: return launch_list_p<T, 11>(s, cv, items, w, blocks, threads, smem, st);
+        case 12: return launch_list_p<T, 12>(s, cv, items, w, blocks, threads, smem, st);
+        default: return launch_list_p<T, 0>(s, cv, items, w, blocks, threads, smem, st);
     }
 }
 
 template size_t line_block_item_bytes<LineT>();
-template size_t line_block_item_done_offset<LineT>();
 template int line_block_list_item<LineT>(const DevLevel<LineT>&, int, int, const LineT*, const LineT*, LineT*, LineT*,
                                          LineT, void*, int*, int*, size_t*, int*);
-template bool launch_line_block_list<LineT>(int, int, int, const void*, const int*, int, int, int, size_t,
+template bool launch_line_block_list<LineT>(int, int, int, const void*, const WorkList&, int, int, size_t,
                                             cudaStream_t);
 
 template <typename T>
