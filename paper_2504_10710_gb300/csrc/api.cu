@@ -189,7 +189,7 @@ glls_status alloc_level_vectors(glls_problem* P, std::vector<LevelStore<T>>& Ls)
         CK(P->alloc(&s.y, n));
         CK(P->alloc(&s.t1, n));
         CK(P->alloc(&s.t2, n));
-        if (s.dev.colored) CK(P->alloc(&s.loc, (size_t)s.dev.E * s.dev.nloc * P->nrhs));
+        if (s.dev.colored && apply_is_fixed(s.dev)) CK(P->alloc(&s.loc, (size_t)s.dev.E * s.dev.nloc * P->nrhs));
         CK(cudaMemset(s.r, 0, sizeof(T) * n));
         CK(cudaMemset(s.x, 0, sizeof(T) * n));
         CK(cudaMemset(s.y, 0, sizeof(T) * n));
@@ -1911,7 +1911,8 @@ glls_status glls_estimate_bytes(const glls_mesh_desc* desc, size_t* bytes) {
         // vectors in each precision; transfer bands
         total += 12.0 * ((double)ncomp * E * nloc + (1 + d) * (double)N + (p + 1) * (p + 1)) + 12.0 * 5 * N;
         total += 24.0 * d * (double)N;
-        if (desc->summation == GLLS_SUM_COLORED) total += 12.0 * E * nloc;   // element results, both precisions
+        if (desc->summation == GLLS_SUM_COLORED && p <= (d == 2 ? 16 : 8) && std::max({ne[0], ne[1], ne[2]}) < 1024)
+            total += 12.0 * E * nloc;                                        // element results, both precisions
         if (c == 0 && p >= 2 && p <= (d == 2 ? 16 : 8)) total += 4.0 * ncomp * E * nloc;   // float-float G remainders
         total += 2.0 * d * (12.0 * (2 * p + 2) * (double)(ne[0] * p + 1) + 4.0 * (ne[0] * p + 1));
         if (desc->smoother == GLLS_SMOOTHER_GLL && p >= 2) {

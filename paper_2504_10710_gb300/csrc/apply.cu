@@ -310,15 +310,21 @@ template bool launch_apply_list<float>(int, const ApplyItem<float>*, const WorkL
 template bool launch_apply_list<double>(int, const ApplyItem<double>*, const WorkList&, int, bool, bool,
                                         cudaStream_t);
 
+template <typename T>
+bool apply_is_fixed(const DevLevel<T>& L) {
+    if (L.N > (1LL << 31) - 1 || L.E * L.nloc * (L.dim == 2 ? 3 : 6) > (1LL << 31) - 1) return false;
+    for (int a = 0; a < L.dim; ++a)
+        if (L.ne[a] >= 1024) return false;   // element coordinates are packed in 10 bits
+    return L.p >= 1 && L.p <= (L.dim == 2 ? 16 : 8);
+}
+template bool apply_is_fixed<double>(const DevLevel<double>&);
+template bool apply_is_fixed<float>(const DevLevel<float>&);
+
 // Dot partials that launch_apply writes for L (one per CTA of the
 // specialised kernel, else one per block of the separate dot launch).
 template <typename T>
 int apply_dot_partials(const DevLevel<T>& L) {
-    bool fixed = L.N <= (1LL << 31) - 1 && L.E * L.nloc * (L.dim == 2 ? 3 : 6) <= (1LL << 31) - 1 && L.p >= 1 &&
-                 L.p <= (L.dim == 2 ? 16 : 8);
-    for (int a = 0; a < L.dim; ++a)
-        if (L.ne[a] >= 1024) fixed = false;
-    if (!fixed) return kDotBlocks;
+    if (!apply_is_fixed(L)) return kDotBlocks;
     if (apply_eo_selected(L.dim, L.p, true)) return apply_eo_blocks(L.p, L.E);
     long long nloc = 1;
     for (int a = 0; a < L.dim; ++a) nloc *= L.p + 1;
@@ -331,9 +337,7 @@ template int apply_dot_partials<double>(const DevLevel<double>&);
 template <typename T>
 bool launch_apply_fixed(const DevLevel<T>& L, const T* x, T* y, bool mask, double* dot, double* part,
                         unsigned* ticket, cudaStream_t st, int nrhs, T* loc) {
-    if (L.N > (1LL << 31) - 1 || L.E * L.nloc * (L.dim == 2 ? 3 : 6) > (1LL << 31) - 1) return false;
-    for (int a = 0; a < L.dim; ++a)
-        if (L.ne[a] >= 1024) return false;   // element coordinates are packed in 10 bits
+    if (!apply_is_fixed(L)) return false;
     // 3-D: the even-odd line kernels (FP32, and FP64 where they were measured
     // fastest), else the node-per-thread kernel below
     if (launch_apply_eo<T>(L, x, y, mask, dot, part, ticket, st, nrhs, loc)) return true;

@@ -309,6 +309,9 @@ constexpr size_t kMaxDynSmemBytes = 200 * 1024;
 template <typename T>
 bool launch_apply_fixed(const DevLevel<T>& L, const T* x, T* y, bool mask, double* dot, double* part,
                         unsigned* ticket, cudaStream_t st, int nrhs = 1, T* loc = nullptr);
+// Whether L is in that range (else loc is never used).
+template <typename T>
+bool apply_is_fixed(const DevLevel<T>& L);
 template <typename T>
 bool launch_line_warp(const DevLevel<T>& L, int s, int mode, const T* g, const T* r, T* y, T* x, T alpha,
                       cudaStream_t st, int nrhs = 1);
