@@ -25,6 +25,7 @@
 // parameters, the three line directions of an element through shared memory.
 #include "device.cuh"
 #include "ff.cuh"
+#include "reduce.cuh"
 #include "setup.h"
 
 #include <algorithm>
@@ -34,21 +35,6 @@
 
 namespace glls {
 namespace {
-
-// Block sum of one FP64 value per thread (blockDim.x a multiple of 32) with few FP64 adds: the values go through shared memory, lane l of
-// warp 0 adds values l, l + 32, ... in that order, then warp 0's shuffle
-// tree.  A shuffle tree over every warp would cost each thread five FP64
-// adds, which on GB300's FP64 pipe is a visible share of these kernels.
-__device__ __forceinline__ double block_sum_lean(double v, double* sv) {
-    sv[threadIdx.x] = v;
-    __syncthreads();
-    double s = 0.0;
-    if (threadIdx.x < 32) {
-        for (int i = threadIdx.x; i < (int)blockDim.x; i += 32) s += sv[i];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-    }
-    return s;   // valid in thread 0
-}
 
 template <int P>
 __device__ __forceinline__ void apply_ff_body(const DevLevel<double>& L, const double* __restrict__ x,
@@ -161,7 +147,7 @@ __device__ __forceinline__ void apply_ff_body(const DevLevel<double>& L, const d
         }
     }
     __shared__ double sv[THREADS];
-    const double tsum = block_sum_lean(local, sv);
+    const double tsum = block_sum_once(local, sv);
     if (threadIdx.x == 0) part[(long long)rhs * nbx + bx] = tsum;
 }
 
@@ -415,7 +401,7 @@ __global__ void __launch_bounds__(kEoFfThreads, P == 8 ? 2 : 3)
         }
     }
     __shared__ double sv[kEoFfThreads];
-    const double tsum = block_sum_lean(local, sv);
+    const double tsum = block_sum_once(local, sv);
     if (tid == 0) part[(long long)rhs * nbx + bx] = tsum;
 }
 

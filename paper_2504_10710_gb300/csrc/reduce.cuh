@@ -1,5 +1,6 @@
-// Block-level FP64 reductions shared by the kernels: a block sum, the "last block" ticket, and the fixed-order sum of block partials
-// (results do not depend on block scheduling).
+// Block-level FP64 reductions shared by the kernels: a block sum, the "last
+// block" ticket, and the fixed-order sum of block partials (results do not
+// depend on block scheduling).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -7,14 +8,14 @@ namespace glls {
 namespace {
 
 // Block sum of one FP64 value per thread (blockDim.x a multiple of 32, at most
-// kReduceThreads; red: as many doubles).  The values go through shared memory
+// kReduceThreads; red: blockDim.x doubles).  The values go through shared memory
 // and warp 0 adds lane l's values l, l + 32, ... in that order, then its
 // shuffle tree: GB300 issues a warp's FP64 add over 16 cycles, and a shuffle
 // tree in every warp (40 adds for 256 threads instead of 13) was a visible
 // share of the outer-iteration kernels.
+// block_sum_once: red holds nothing that another thread may still read.
 constexpr int kReduceThreads = 352;
-__device__ __forceinline__ double block_sum(double v, double* red) {
-    __syncthreads();                        // red may still be read from the last sum
+__device__ __forceinline__ double block_sum_once(double v, double* red) {
     red[threadIdx.x] = v;
     __syncthreads();
     double s = 0.0;
@@ -23,6 +24,10 @@ __device__ __forceinline__ double block_sum(double v, double* red) {
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     }
     return s;   // valid in thread 0
+}
+__device__ __forceinline__ double block_sum(double v, double* red) {
+    __syncthreads();                        // red may still be read from the last sum
+    return block_sum_once(v, red);
 }
 
 // Ticket increment with acquire-release semantics at GPU scope: the calling
@@ -55,8 +60,8 @@ __device__ __forceinline__ bool last_block_of(unsigned* ticket, unsigned total) 
     return is_last_n;
 }
 
-__device__ __forceinline__ void finalize_partials(const double* part, int ndots, int nblocks, double* S, int slot0, int slot1,
-                                  double* red) {
+__device__ __forceinline__ void finalize_partials(const double* part, int ndots, int nblocks, double* S, int slot0,
+                                                  int slot1, double* red) {
     for (int d = 0; d < ndots; ++d) {
         double s = 0.0;
         for (int i = threadIdx.x; i < nblocks; i += blockDim.x) s += __ldcg(part + d * nblocks + i);
