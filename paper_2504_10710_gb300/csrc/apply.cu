@@ -207,11 +207,10 @@ constexpr int threads_of() {
 }
 
 template <typename T, int DIM, int P, bool DOT, bool LOC>
-__global__ void __launch_bounds__(threads_of<DIM, P>(), 1) apply_p_kernel(DevLevel<T> L, const T* __restrict__ x, T* __restrict__ y,
-                                                         int mask, double* dot, double* part, unsigned* ticket,
-                                                         int nrhs, T* loc) {
-    apply_p_body<T, DIM, P, DOT, LOC>(L, x, y, mask, dot, part, ticket, nrhs, blockIdx.x, gridDim.x, 0.0,
-                                      loc);
+__global__ void __launch_bounds__(threads_of<DIM, P>(), 1)
+    apply_p_kernel(DevLevel<T> L, const T* __restrict__ x, T* __restrict__ y, int mask, double* dot, double* part,
+                   unsigned* ticket, int nrhs, T* loc) {
+    apply_p_body<T, DIM, P, DOT, LOC>(L, x, y, mask, dot, part, ticket, nrhs, blockIdx.x, gridDim.x, 0.0, loc);
 }
 
 // Work-list form: item j is one problem's level, vectors and partials.
@@ -225,15 +224,6 @@ __global__ void __launch_bounds__(threads_of<DIM, P>(), 1)
                                         w.start[j + 1] - w.start[j], stopped, nullptr);
 }
 
-// Number of CTAs (= dot partials) the specialised apply launches for L.
-template <typename T, int DIM, int P>
-int apply_blocks(const DevLevel<T>& L) {
-    constexpr int N1 = P + 1;
-    constexpr int NLOC = DIM == 2 ? N1 * N1 : N1 * N1 * N1;
-    constexpr int EPB = apply_epb(NLOC);
-    return (int)((L.E + EPB - 1) / EPB);
-}
-
 template <typename T, int DIM, int P>
 bool launch_p(const DevLevel<T>& L, const T* x, T* y, bool mask, double* dot, double* part, unsigned* ticket,
               cudaStream_t st, int nrhs, T* loc) {
@@ -242,20 +232,16 @@ bool launch_p(const DevLevel<T>& L, const T* x, T* y, bool mask, double* dot, do
     constexpr int EPB = apply_epb(NLOC);
     const long long blocks = (L.E + EPB - 1) / EPB * nrhs;
     if (blocks > 0x7fffffffLL) return false;
-    const int mk = mask ? 1 : 0;
+    auto go = [&](auto kern) {
+        launch_k(kern, (unsigned)blocks, threads_of<DIM, P>(), 0, st, L, x, y, mask ? 1 : 0, dot, part, ticket, nrhs,
+                 loc);
+        return true;
+    };
     if constexpr (sizeof(T) == 8) {
-        if (dot) {
-            if (loc) launch_k(apply_p_kernel<T, DIM, P, true, true>, (unsigned)blocks, threads_of<DIM, P>(), 0, st, L, x, y, mk, dot, part, ticket, nrhs, loc);
-            else launch_k(apply_p_kernel<T, DIM, P, true, false>, (unsigned)blocks, threads_of<DIM, P>(), 0, st, L, x, y, mk, dot, part, ticket, nrhs, loc);
-            return true;
-        }
+        if (dot) return loc ? go(apply_p_kernel<T, DIM, P, true, true>) : go(apply_p_kernel<T, DIM, P, true, false>);
     }
     if (dot) return false;                   // x.(A x) is formed in FP64 only
-    double* nd = nullptr;
-    unsigned* nt = nullptr;
-    if (loc) launch_k(apply_p_kernel<T, DIM, P, false, true>, (unsigned)blocks, threads_of<DIM, P>(), 0, st, L, x, y, mk, nd, nd, nt, nrhs, loc);
-    else launch_k(apply_p_kernel<T, DIM, P, false, false>, (unsigned)blocks, threads_of<DIM, P>(), 0, st, L, x, y, mk, nd, nd, nt, nrhs, loc);
-    return true;
+    return loc ? go(apply_p_kernel<T, DIM, P, false, true>) : go(apply_p_kernel<T, DIM, P, false, false>);
 }
 
 template <typename T, int DIM, int P>

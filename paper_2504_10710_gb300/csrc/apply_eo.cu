@@ -95,8 +95,9 @@ template <int N>
 struct EoShape {
     static constexpr int NP = N * N, NLOC = NP * N;
     static constexpr int RS = N == 8 ? 9 : N == 7 ? 7 : N == 6 ? 9 : N;
-    static constexpr int PS = N == 2 ? 5 : N == 3 ? 9 : N == 4 ? 19 : N == 5 ? 25 : N == 6 ? 54 : N == 7 ? 52 : N == 8 ? 72 : 89;
-    static constexpr int ES = N == 2 ? 12 : N == 3 ? 27 : N == 4 ? 76 : N == 5 ? 125 : N == 6 ? 324 : N == 7 ? 369 : N == 8 ? 576 : 801;
+    static constexpr int kPlane[8] = {5, 9, 19, 25, 54, 52, 72, 89};              // N = 2 .. 9
+    static constexpr int kElement[8] = {12, 27, 76, 125, 324, 369, 576, 801};
+    static constexpr int PS = kPlane[N - 2], ES = kElement[N - 2];
     static constexpr int NBUF = 3;                           // x, and two work buffers
 };
 
@@ -110,7 +111,8 @@ __device__ __forceinline__ bool on_bd(int I, int J, int K, const int n[3]) {
 template <typename T, int P, bool DOT, bool LOC>
 __global__ void __launch_bounds__(256, 2)
     apply_eo3_kernel(DevLevel<T> L, const __grid_constant__ EoParams<T, P + 1> M, const T* __restrict__ x,
-                     T* __restrict__ y, int mask, double* dot, double* part, unsigned* ticket, int epb, int nrhs, T* loc) {
+                     T* __restrict__ y, int mask, double* dot, double* part, unsigned* ticket, int epb, int nrhs,
+                     T* loc) {
     using S = EoShape<P + 1>;
     constexpr int N = P + 1, NP = S::NP, NLOC = S::NLOC, RS = S::RS, PS = S::PS, ES = S::ES;
     extern __shared__ __align__(16) unsigned char eo_smem3[];
@@ -285,7 +287,12 @@ __device__ __forceinline__ void eo_line2(const EoMat2<N>& M, const f32x2 (&u)[N]
 // conflicts that a pair of strides leaves.  Measured on 16^3 elements, p = 7:
 // 12.7 -> 10.9 us (9.1 us at the measured copy bandwidth), 32 right-hand
 // sides 359 -> 237 us; 24^3, p = 8: 74 -> 71 us.
-// Resident CTAs of 128 threads the registers must allow, as measured.
+//
+// Resident CTAs of 128 threads the registers must allow: 4 (at most 128
+// registers a thread) or 5 (96).  us per apply with 4 and with 5, 1 to 2 M
+// nodes: one right-hand side p = 4 14.5 and 14.4, p = 5 18.3 and 18.3, p = 6
+// 22.6 and 21.1, p = 7 20.5 and 20.4, p = 8 22.6 and 24.6; eight p = 5 88.1 and
+// 88.1, p = 6 114.7 and 115.3, p = 7 108.4 and 102.3, p = 8 127.0 and 119.9.
 constexpr int eo_pair_min_ctas(int P, bool rhs) { return rhs ? (P == 8 ? 4 : 5) : (P == 5 || P == 6 ? 5 : 4); }
 
 template <int P, bool RHS, bool LOC>
@@ -528,12 +535,12 @@ bool launch_eo_pair(const DevLevel<float>& L, const float* x, float* y, bool mas
     if (nb > 0x7fffffffLL) return false;
     const int threads = (epb * S::NP + 31) / 32 * 32;
     const size_t smem = sizeof(f32x2) * S::NBUF * epb * S::ES;
-    const int mk = mask ? 1 : 0;
-    if (rhs && loc) launch_k(apply_eo3_pair_kernel<P, true, true>, (unsigned)nb, threads, smem, st, L, M, x, y, mk, epb, nrhs, loc);
-    else if (rhs) launch_k(apply_eo3_pair_kernel<P, true, false>, (unsigned)nb, threads, smem, st, L, M, x, y, mk, epb, nrhs, loc);
-    else if (loc) launch_k(apply_eo3_pair_kernel<P, false, true>, (unsigned)nb, threads, smem, st, L, M, x, y, mk, epb, nrhs, loc);
-    else launch_k(apply_eo3_pair_kernel<P, false, false>, (unsigned)nb, threads, smem, st, L, M, x, y, mk, epb, nrhs, loc);
-    return true;
+    auto go = [&](auto kern) {
+        launch_k(kern, (unsigned)nb, threads, smem, st, L, M, x, y, mask ? 1 : 0, epb, nrhs, loc);
+        return true;
+    };
+    if (rhs) return loc ? go(apply_eo3_pair_kernel<P, true, true>) : go(apply_eo3_pair_kernel<P, true, false>);
+    return loc ? go(apply_eo3_pair_kernel<P, false, true>) : go(apply_eo3_pair_kernel<P, false, false>);
 }
 
 template <typename T, int P>
@@ -547,22 +554,22 @@ bool launch_eo(const DevLevel<T>& L, const T* x, T* y, bool mask, double* dot, d
     const int blocks = (int)nb;
     const int threads = (epb * S::NP + 31) / 32 * 32;
     const size_t smem = sizeof(T) * S::NBUF * epb * S::ES;
-    double* nd = nullptr;
-    unsigned* nt = nullptr;
-    const int mk = mask ? 1 : 0;
-    if (dot && loc) launch_k(apply_eo3_kernel<T, P, true, true>, blocks, threads, smem, st, L, M, x, y, mk, dot, part, ticket, epb, nrhs, loc);
-    else if (dot) launch_k(apply_eo3_kernel<T, P, true, false>, blocks, threads, smem, st, L, M, x, y, mk, dot, part, ticket, epb, nrhs, loc);
-    else if (loc) launch_k(apply_eo3_kernel<T, P, false, true>, blocks, threads, smem, st, L, M, x, y, mk, nd, nd, nt, epb, nrhs, loc);
-    else launch_k(apply_eo3_kernel<T, P, false, false>, blocks, threads, smem, st, L, M, x, y, mk, nd, nd, nt, epb, nrhs, loc);
-    return true;
+    auto go = [&](auto kern) {
+        launch_k(kern, blocks, threads, smem, st, L, M, x, y, mask ? 1 : 0, dot, part, ticket, epb, nrhs, loc);
+        return true;
+    };
+    if (dot) return loc ? go(apply_eo3_kernel<T, P, true, true>) : go(apply_eo3_kernel<T, P, true, false>);
+    return loc ? go(apply_eo3_kernel<T, P, false, true>) : go(apply_eo3_kernel<T, P, false, false>);
 }
 
 template <typename T, int P>
 bool set_eo_attr() {
     using S = EoShape<P + 1>;
     const int smem = (int)(sizeof(T) * S::NBUF * (256 / S::NP) * S::ES);
-    const void* fns[] = {(const void*)apply_eo3_kernel<T, P, false, false>, (const void*)apply_eo3_kernel<T, P, false, true>,
-                         (const void*)apply_eo3_kernel<T, P, true, false>, (const void*)apply_eo3_kernel<T, P, true, true>};
+    const void* fns[] = {(const void*)apply_eo3_kernel<T, P, false, false>,
+                         (const void*)apply_eo3_kernel<T, P, false, true>,
+                         (const void*)apply_eo3_kernel<T, P, true, false>,
+                         (const void*)apply_eo3_kernel<T, P, true, true>};
     for (const void* f : fns)
         if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return false;
     return true;

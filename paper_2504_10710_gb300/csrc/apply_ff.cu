@@ -152,8 +152,9 @@ __device__ __forceinline__ void apply_ff_body(const DevLevel<double>& L, const d
 }
 
 template <int P>
-__global__ void __launch_bounds__(apply_threads((P + 1) * (P + 1)), 1) apply_ff_kernel(DevLevel<double> L, const double* __restrict__ x,
-                                                          double* __restrict__ y, int mask, double* part, int nrhs) {
+__global__ void __launch_bounds__(apply_threads((P + 1) * (P + 1)), 1)
+    apply_ff_kernel(DevLevel<double> L, const double* __restrict__ x, double* __restrict__ y, int mask, double* part,
+                    int nrhs) {
     apply_ff_body<P>(L, x, y, mask, part, nrhs, blockIdx.x, gridDim.x, 0.0);
 }
 

@@ -30,10 +30,15 @@ namespace glls {
 // Programmatic dependent launch.  Kernels are launched with programmatic
 // stream serialisation, so the CTAs of the next kernel in a stream (or graph)
 // may be scheduled while the previous kernel drains.  Every kernel therefore
-// starts with grid_dep_sync(): it waits until the preceding kernel has
-// completed and its writes are visible, then lets the following kernel begin
-// launching.  Because each kernel waits before it touches memory, ordering is
-// transitive along the stream exactly as without the attribute.
+// calls grid_dep_sync() before it touches a vector or a scalar that any kernel
+// writes: it waits until the preceding kernel has completed and its writes are
+// visible, then lets the following kernel begin launching.  Ahead of it a kernel
+// may read only what no kernel writes: mesh data (geometry factors, operators,
+// transfer bands, coarse inverse) and work-list items, uploaded before the
+// problem or plan is handed out; and a work list's stop flags (item_stopped).
+// Every CTA waits, also one that has nothing to do, so a kernel completes only
+// after the one before it: ordering is transitive along the stream exactly as
+// without the attribute.
 __device__ __forceinline__ void grid_dep_sync() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -250,7 +255,9 @@ __host__ __device__ constexpr int apply_threads(int nloc) {
     }
     return best;
 }
-__host__ __device__ constexpr int apply_epb(int nloc) { return nloc >= apply_threads(nloc) ? 1 : apply_threads(nloc) / nloc; }
+__host__ __device__ constexpr int apply_epb(int nloc) {
+    return nloc >= apply_threads(nloc) ? 1 : apply_threads(nloc) / nloc;
+}
 
 int apply_list_blocks(int p, long long E);
 template <typename T>
@@ -299,8 +306,9 @@ bool launch_line_block_list(int p, int s, int cv, const void* items, const WorkL
 bool init_kernel_attributes();
 constexpr size_t kMaxDynSmemBytes = 200 * 1024;
 
-// Specialised fast paths (apply.cu with apply_eo.cu for 3-D, lines.cu); they return false when the case is outside their compiled
-// range and the generic kernels take over.
+// Specialised fast paths (apply.cu with apply_eo.cu for 3-D, lines.cu); they
+// return false when the case is outside their compiled range and the generic
+// kernels take over.
 // dot: if non-null, also accumulate sum_e x_e^T (A_e x_e) = x.(A x) for x
 // zero on the boundary; the last block writes it to dot[0] using `part` and
 // `ticket` (see launch_dots).
@@ -379,13 +387,13 @@ void launch_transfer(const DevBand<T>& M, int a, const int nin[3], const int nou
 // planes for a restriction whose axis 2 came first).
 // Returns false when the tile window does not fit in shared memory (the
 // caller then runs the two passes separately).
-// Whether launch_transfer2 takes these factors.
-template <typename T>
-bool transfer2_fits(const DevBand<T>& M0, const DevBand<T>& M1);
 template <typename T>
 bool launch_transfer2(const DevBand<T>& M0, const DevBand<T>& M1, const int nin[3], const int nout[3], const T* in,
                       const T* in2, T* out, bool add, bool mask, cudaStream_t st, T* clear = nullptr, int nrhs = 1,
                       bool planes = false);
+// Whether launch_transfer2 takes these factors.
+template <typename T>
+bool transfer2_fits(const DevBand<T>& M0, const DevBand<T>& M1);
 
 // e = A_0^-1 r on the interior of the coarsest level; e's boundary entries
 // are zeroed first unless e_boundary_zero.  w: scratch of C.n values (used
@@ -421,7 +429,7 @@ inline int fcg_list_blocks(long long n) { return vector_blocks(n, 4096); }
 constexpr int kMaxReduceBlocks = 8192;
 void launch_dots(const double* a0, const double* b0, const double* a1, const double* b1, int ndots,
                  long long n, double* part, double* S, int slot0, int slot1, unsigned* ticket, cudaStream_t st, int nrhs = 1);
-// Outer-iteration dots without a grid-wide finish: kDotBlocks per-block
+// Outer-iteration dots without a grid-wide finish: fcg_blocks(n) per-block
 // partials of r.z into prz and of z.q into pzq; z is z32 when given; q is
 // reset to 0 after it is read.
 void launch_dots_rz_zq(const double* r, const double* z, const float* z32, double* q, long long n, double* prz,

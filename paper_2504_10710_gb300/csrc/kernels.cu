@@ -922,8 +922,10 @@ struct Trip {
 // AHEAD (below): the next trip's values are loaded before the current ones are
 // used.  One right-hand side has two CTAs of these kernels per SM, and a
 // trip's latency is all it waits for (update, 1.44 M nodes: 53 us without);
-// with several the SMs are full and the registers are worth more resident CTAs
-// (32 right-hand sides: 463 against 662 us with it).  The sums are the same.
+// with 32 the SMs are full and the registers are worth more resident CTAs (463
+// against 662 us with it).  A work list's launch, with far fewer CTAs per
+// problem, is of the first kind: 24 uneven problems 16.5 ms with it, 17.1 with
+// four resident CTAs instead, 128 problems 72.9 and 75.1.  The sums are the same.
 
 // Outer-iteration dots, grid-stride over the CTAs: per-block partials of r.z
 // into prz and of z.q into pzq (summed by the consumers); z is z32 where given
@@ -972,24 +974,25 @@ __device__ __forceinline__ void dots_rz_zq_body(const double* __restrict__ r, co
 }
 
 template <bool MIXED, bool AHEAD>
-__global__ void __launch_bounds__(256, AHEAD ? 2 : 4) dots_rz_zq_kernel(const double* __restrict__ r, const double* __restrict__ z,
-                                                         const float* __restrict__ z32, double* __restrict__ q,
-                                                         long long n, double* __restrict__ prz,
-                                                         double* __restrict__ pzq) {
+__global__ void __launch_bounds__(256, AHEAD ? 2 : 4)
+    dots_rz_zq_kernel(const double* __restrict__ r, const double* __restrict__ z, const float* __restrict__ z32,
+                      double* __restrict__ q, long long n, double* __restrict__ prz, double* __restrict__ pzq) {
     grid_dep_sync();
     const long long jr = blockIdx.y;       // right-hand side
     dots_rz_zq_body<MIXED, AHEAD>(r + jr * n, z + jr * n, MIXED ? z32 + jr * n : nullptr, q + jr * n, n,
-                           prz + jr * gridDim.x, pzq + jr * gridDim.x);
+                                  prz + jr * gridDim.x, pzq + jr * gridDim.x);
 }
 
 // q-independent update: every block sums the partials of p.q (npq, from the
-// apply), takes r.z from S_RZNEW (published by the direction), alpha = r.z / p.q; x += alpha p; r -= alpha q;
-// partials of r.r into prr; the last block publishes S_RR, S_RZ (for the next
-// direction), S_ALPHA, S_PQ and the breakdown flag.
+// apply) and takes r.z from S_RZNEW (published by the direction); alpha = r.z /
+// p.q; x += alpha p; r -= alpha q; partials of r.r into prr; the last block
+// publishes S_RR, S_RZ (for the next direction), S_ALPHA, S_PQ and the
+// breakdown flag.
 template <bool MIXED, bool AHEAD>
 __device__ __forceinline__ void fcg_update_body(double* __restrict__ x, double* __restrict__ r,
                                                 const double* __restrict__ p, const double* __restrict__ q,
-                                                long long n, const double* ppq, int npq, double* prr, double* S, unsigned* ticket, float* __restrict__ r32) {
+                                                long long n, const double* ppq, int npq, double* prr, double* S,
+                                                unsigned* ticket, float* __restrict__ r32) {
     // a right-hand side that has stopped keeps its x and r
     const bool active = S[S_DONE] == 0.0;
     __shared__ double red[kReduceThreads];
@@ -1053,13 +1056,15 @@ __device__ __forceinline__ void fcg_update_body(double* __restrict__ x, double* 
 }
 
 template <bool MIXED, bool AHEAD>
-__global__ void __launch_bounds__(256, AHEAD ? 2 : 4) fcg_update_kernel(double* __restrict__ x, double* __restrict__ r,
-                                                         const double* __restrict__ p, const double* __restrict__ q,
-                                                         long long n, const double* ppq, int npq, double* prr, double* S,
-                                                         unsigned* ticket, float* __restrict__ r32) {
+__global__ void __launch_bounds__(256, AHEAD ? 2 : 4)
+    fcg_update_kernel(double* __restrict__ x, double* __restrict__ r, const double* __restrict__ p,
+                      const double* __restrict__ q, long long n, const double* ppq, int npq, double* prr, double* S,
+                      unsigned* ticket, float* __restrict__ r32) {
     grid_dep_sync();
     const long long jr = blockIdx.y;       // right-hand side
-    fcg_update_body<MIXED, AHEAD>(x + jr * n, r + jr * n, p + jr * n, q + jr * n, n, ppq + jr * npq, npq, prr + jr * gridDim.x, S + jr * S_COUNT, ticket + jr, MIXED ? r32 + jr * n : nullptr);
+    fcg_update_body<MIXED, AHEAD>(x + jr * n, r + jr * n, p + jr * n, q + jr * n, n, ppq + jr * npq, npq,
+                                  prr + jr * gridDim.x, S + jr * S_COUNT, ticket + jr,
+                                  MIXED ? r32 + jr * n : nullptr);
 }
 
 // p = z + beta p, beta = -alpha zq / rz_old (flexible) or rz_new / rz_old
@@ -1106,19 +1111,19 @@ __device__ __forceinline__ void fcg_direction_body(double* __restrict__ p, const
 }
 
 template <bool MIXED, bool AHEAD>
-__global__ void __launch_bounds__(256, AHEAD ? 2 : 4) fcg_direction_kernel(double* __restrict__ p, const double* __restrict__ z,
-                                                            const float* __restrict__ z32, long long n,
-                                                            const double* prz, const double* pzq, int nd, double* S,
-                                                            int flexible) {
+__global__ void __launch_bounds__(256, AHEAD ? 2 : 4)
+    fcg_direction_kernel(double* __restrict__ p, const double* __restrict__ z, const float* __restrict__ z32,
+                         long long n, const double* prz, const double* pzq, int nd, double* S, int flexible) {
     grid_dep_sync();
     const long long jr = blockIdx.y;       // right-hand side
     fcg_direction_body<MIXED, AHEAD>(p + jr * n, z + jr * n, MIXED ? z32 + jr * n : nullptr, n, prz + jr * nd,
-                              pzq + jr * nd, nd, S + jr * S_COUNT, flexible);
+                                     pzq + jr * nd, nd, S + jr * S_COUNT, flexible);
 }
 
 // Work-list form of the three outer-iteration kernels: item blockIdx.y is one
-// problem (its own vectors, length, partials and scalars), kDotBlocks CTAs
-// each.  step 0: dots r.z, z.q; 1: direction; 2: update.
+// problem (its own vectors, length, partials and scalars) on gridDim.x CTAs
+// (fcg_list_blocks of the group's longest vectors).  STEP 0: dots r.z, z.q;
+// 1: direction; 2: update.
 template <int STEP, bool MIXED>
 __global__ void __launch_bounds__(256) fcg_list_kernel(const FcgItem* __restrict__ items, int flexible) {
     grid_dep_sync();
@@ -1507,10 +1512,11 @@ bool launch_transfer2(const DevBand<T>& M0, const DevBand<T>& M1, const int nin[
     const dim3 grid((unsigned)((nout[0] + 31) / 32), (unsigned)((nout[1] + TY - 1) / TY), (unsigned)(nout[2] * nrhs));
     const int3 ni = make_int3(nin[0], nin[1], nin[2]), no = make_int3(nout[0], nout[1], nout[2]);
     const int ad = add ? 1 : 0, mk = mask ? (planes ? 2 : 1) : 0;   // 2: the end planes of axis 2 too
-    if (W <= 4) launch_k(transfer2_kernel<T, 4, TY>, grid, 256, smem, st, M0, M1, ni, no, in, in2, out, ad, mk, clear);
-    else if (W <= 8) launch_k(transfer2_kernel<T, 8, TY>, grid, 256, smem, st, M0, M1, ni, no, in, in2, out, ad, mk, clear);
-    else if (W <= 16) launch_k(transfer2_kernel<T, 16, TY>, grid, 256, smem, st, M0, M1, ni, no, in, in2, out, ad, mk, clear);
-    else launch_k(transfer2_kernel<T, 32, TY>, grid, 256, smem, st, M0, M1, ni, no, in, in2, out, ad, mk, clear);
+    auto go = [&](auto kern) { launch_k(kern, grid, 256, smem, st, M0, M1, ni, no, in, in2, out, ad, mk, clear); };
+    if (W <= 4) go(transfer2_kernel<T, 4, TY>);
+    else if (W <= 8) go(transfer2_kernel<T, 8, TY>);
+    else if (W <= 16) go(transfer2_kernel<T, 16, TY>);
+    else go(transfer2_kernel<T, 32, TY>);
     return true;
 }
 
@@ -1562,9 +1568,10 @@ void launch_fcg_list(int step, const FcgItem* items, int nitems, int flexible, i
                      cudaStream_t st) {
     if (nitems < 1) return;
     const dim3 grid(blocks, nitems);
-    if (step == 0) launch_k(mixed ? fcg_list_kernel<0, true> : fcg_list_kernel<0, false>, grid, 256, 0, st, items, flexible);
-    else if (step == 1) launch_k(mixed ? fcg_list_kernel<1, true> : fcg_list_kernel<1, false>, grid, 256, 0, st, items, flexible);
-    else launch_k(mixed ? fcg_list_kernel<2, true> : fcg_list_kernel<2, false>, grid, 256, 0, st, items, flexible);
+    auto go = [&](auto kern) { launch_k(kern, grid, 256, 0, st, items, flexible); };
+    if (step == 0) go(mixed ? fcg_list_kernel<0, true> : fcg_list_kernel<0, false>);
+    else if (step == 1) go(mixed ? fcg_list_kernel<1, true> : fcg_list_kernel<1, false>);
+    else go(mixed ? fcg_list_kernel<2, true> : fcg_list_kernel<2, false>);
 }
 
 template bool transfer2_list_config<float>(const DevBand<float>&, const DevBand<float>&, const int*, int*, int*, int*,
@@ -1625,32 +1632,38 @@ void launch_dots(const double* a0, const double* b0, const double* a1, const dou
              0);
 }
 
-// The instance for MIXED (mixed) and AHEAD (ahead).
-template <typename K>
-K* pick_vector(bool mixed, bool ahead, K* none, K* m, K* a, K* both) {
-    return mixed ? (ahead ? both : m) : (ahead ? a : none);
+// MIXED as given, AHEAD for one right-hand side: launch(MIXED, AHEAD) with both
+// as types.
+template <typename F>
+void pick_vector(bool mixed, int nrhs, F launch) {
+    using Yes = std::true_type;
+    using No = std::false_type;
+    if (nrhs == 1) mixed ? launch(Yes(), Yes()) : launch(No(), Yes());
+    else mixed ? launch(Yes(), No()) : launch(No(), No());
 }
 
 void launch_fcg_update(double* x, double* r, const double* p, const double* q, long long n, const double* ppq,
                        int npq, int nb, double* prr, double* S, unsigned* ticket, float* r32, cudaStream_t st,
                        int nrhs) {
-    launch_k(pick_vector(r32 != nullptr, nrhs == 1, fcg_update_kernel<false, false>, fcg_update_kernel<true, false>,
-                         fcg_update_kernel<false, true>, fcg_update_kernel<true, true>), dim3(nb, nrhs), 256, 0, st, x, r, p, q, n, ppq,
-             npq, prr, S, ticket, r32);
+    pick_vector(r32 != nullptr, nrhs, [&](auto m, auto a) {
+        launch_k(fcg_update_kernel<m.value, a.value>, dim3(nb, nrhs), 256, 0, st, x, r, p, q, n, ppq, npq, prr, S,
+                 ticket, r32);
+    });
 }
 
 void launch_dots_rz_zq(const double* r, const double* z, const float* z32, double* q, long long n, double* prz,
                        double* pzq, cudaStream_t st, int nrhs) {
-    launch_k(pick_vector(z32 != nullptr, nrhs == 1, dots_rz_zq_kernel<false, false>, dots_rz_zq_kernel<true, false>,
-                         dots_rz_zq_kernel<false, true>, dots_rz_zq_kernel<true, true>), dim3(fcg_blocks(n), nrhs), 256, 0, st, r, z, z32,
-             q, n, prz, pzq);
+    pick_vector(z32 != nullptr, nrhs, [&](auto m, auto a) {
+        launch_k(dots_rz_zq_kernel<m.value, a.value>, dim3(fcg_blocks(n), nrhs), 256, 0, st, r, z, z32, q, n, prz, pzq);
+    });
 }
 
 void launch_fcg_direction(double* p, const double* z, const float* z32, long long n, const double* prz,
                           const double* pzq, int nd, double* S, int flexible, cudaStream_t st, int nrhs) {
-    launch_k(pick_vector(z32 != nullptr, nrhs == 1, fcg_direction_kernel<false, false>, fcg_direction_kernel<true, false>,
-                         fcg_direction_kernel<false, true>, fcg_direction_kernel<true, true>), dim3(nd, nrhs), 256, 0, st, p, z, z32, n, prz,
-             pzq, nd, S, flexible);
+    pick_vector(z32 != nullptr, nrhs, [&](auto m, auto a) {
+        launch_k(fcg_direction_kernel<m.value, a.value>, dim3(nd, nrhs), 256, 0, st, p, z, z32, n, prz, pzq, nd, S,
+                 flexible);
+    });
 }
 
 void launch_lift_rhs(const double* mass, const double* f, const double* y, double* f0, const int n[3], int dim,

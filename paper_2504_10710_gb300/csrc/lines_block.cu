@@ -549,7 +549,14 @@ __device__ __forceinline__ void line_block_body(const BlockLineArgs<T>& A, int b
     else line_seg_body<T, P, CV, FORM>(A, blk, stopped);
 }
 
-// Resident CTAs the registers must allow.
+// Resident CTAs the registers must allow.  us per line update along the first
+// and the second axis, with one fewer, as chosen and with one more: FP32 p = 8
+// 2-D 64 x 64 4.1 4.7, 4.4 5.3, 5.2 7.1; 3-D 16^3 15.7 13.2, 14.0 12.5, 15.2
+// 15.1; p = 6 20^3 12.4 14.2, 12.2 14.2, 12.0 12.9.  FP32 2-D 60 x 60 as chosen
+// and with two: p = 9 4.3 4.9, 4.1 4.9; p = 11 4.5 9.8, 5.2 7.5; p = 12 7.4 10.8,
+// 6.1 9.1.  FP64 p = 8 16^3 91 86, 80 75, 76 77; p = 6 20^3 71 72, 71 72, 73 78;
+// 2-D 64 x 64 13.0 12.8, 12.8 13.2, 14.2 14.7.  Run-time order, FP32 2-D 200 x
+// 200, p = 2: 11.7 9.1, 11.5 9.0, 7.7 7.2.
 template <typename T, int P>
 constexpr int line_min_ctas() {
     return sizeof(T) == 8 ? 2 : P == 0 ? 2 : P >= 9 ? 1 : 3;
