@@ -270,7 +270,7 @@ def run_ours(args, rank, world):
 
 
 def _top_kernel_roofline(roof_hbm):
-    """The top kernel of the bench workload's ncu launch list (13 % of the
+    """The top kernel of the bench workload's ncu launch list (14 % of the
     solve): the fine-level FP32 apply of the smoothing steps,
     apply_p_kernel<float, 2, 8>, as measured in roofline_hbm (graph replay,
     the level L2-resident as inside a solve)."""
@@ -379,9 +379,8 @@ def _fp64_peak_gflops(torch):
 
 
 def fp64_apply_roofline(prob, glls, torch):
-    """The bench workload's top kernel in the ncu launch list (13 % of the
-    solve): the FP64 fine-level stiffness apply of the outer iteration, in
-    the form the solve launches it: y = A p with the per-CTA partials of
+    """The FP64-plain solve's outer apply: the FP64 fine-level stiffness apply
+    of the outer iteration, in the form that solve launches it: y = A p with the per-CTA partials of
     p.(A p) fused (flexible CG's p.Ap).  FP64-ALU bound.  FLOPs per launch from the
     sum-factorised algorithm: per element 4 (p+1)^3 FMA for the four 1-D
     contraction sweeps and 4 (p+1)^2 for the geometric factors, plus 2 (p+1)^2

@@ -899,7 +899,10 @@ struct WlRecord {
 // n ~ U{4..64}, p ~ U{4..12}) 70.2, 70.1, 73.0, 73.8, 81.0 ms; four batches of
 // 24: 50.9, 51.8, 52.5, 52.7, 52.8 ms together, but with 300 thousand one of
 // them and one of 16 were 3-4 % slower than with one group per chain, with
-// 200 thousand one of 12 by 5 %; with 400 thousand none was.
+// 200 thousand one of 12 by 5 %; with 400 thousand none was.  Many groups cost
+// plan time, not speed: 512 problems of 64 x 64 elements, p = 8, in 336 groups
+// instead of one 454 -> 414 ms with 77 ms of plan instead of 13; 1000 of 16 x 16
+// elements in 41 groups 87 -> 71 ms.
 constexpr long long kGroupNodes = 400000;
 
 struct WlGroup {

@@ -286,7 +286,8 @@ __device__ __forceinline__ void eo_line2(const EoMat2<N>& M, const f32x2 (&u)[N]
 // neighbouring elements; at p = 7 the swizzled slots below remove the bank
 // conflicts that a pair of strides leaves.  Measured on 16^3 elements, p = 7:
 // 12.7 -> 10.9 us (9.1 us at the measured copy bandwidth), 32 right-hand
-// sides 359 -> 237 us; 24^3, p = 8: 74 -> 71 us.
+// sides 359 -> 237 us (L1 and shared memory then 84 % busy, issue 51 %); 24^3,
+// p = 8: 74 -> 71 us.
 //
 // Resident CTAs of 128 threads the registers must allow: 4 (at most 128
 // registers a thread) or 5 (96).  us per apply with 4 and with 5, 1 to 2 M

@@ -279,7 +279,7 @@ struct EoShapeFF {
 // Measured (graph replay): 16^3 elements, p = 7: 75.2 -> 65.7 us with the packed
 // sweeps above, 20^3 p = 4: 33.0 -> 30.0, p = 6: 95 -> 83, 14^3 p = 8: 92.6 ->
 // 89.4 (order 8 spills at three CTAs per SM and takes two).  What is left is
-// the FP64 conversions and additions (38 % of that pipe) and the latency of 18
+// the FP64 conversions and additions (44 % of that pipe) and the latency of 16
 // resident warps.
 //
 // Thread (a, b) of an element owns the t-line (i, j) = (a, b) in registers
